@@ -349,6 +349,17 @@ qec_status qec_debug_blocks(const qec_params* params, uint64_t seed, uint64_t tr
                             double* kraus, double* u);
 
 /*
+ * Host-only test hook (no GPU needed): the factored form of round `round`'s (>= 1) blocks for
+ * trajectory `traj`, by the code the device runs: block b's Kraus operator of outcome m is, on the
+ * register read at indices flipped by *flips, one rotation per data qubit j of the block,
+ * o_0 = x - t* y, o_1 = y + t x with t = rot[b][j] (complex), then a multiplication by
+ * diag[b][m][z], z the block's data bits.  rot: [blocks][4][2], diag: [blocks][2][16][2].
+ * *flips: the flipped data qubits before the round in, after it out.
+ */
+qec_status qec_debug_factors(const qec_params* params, uint64_t seed, uint64_t traj, int32_t round, uint32_t* flips,
+                             double* rot, double* diag);
+
+/*
  * Host-only test hook (no GPU needed): the FP64-exact emulated product that the tensor-core
  * complex128 pass computes, run on the CPU with the same slicing and recombination code.
  * out[m][32] = A[m][32] . B[32][32]^T (row-major FP64); each entry is the dot product of

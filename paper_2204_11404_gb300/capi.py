@@ -71,6 +71,8 @@ SIGNATURES = {
                            _P, ctypes.c_uint32, ctypes.POINTER(ctypes.c_uint32)], ctypes.c_int),
     "qec_debug_blocks": ([ctypes.POINTER(qec_params), ctypes.c_uint64, ctypes.c_uint64, ctypes.c_int32, _P, _P],
                          ctypes.c_int),
+    "qec_debug_factors": ([ctypes.POINTER(qec_params), ctypes.c_uint64, ctypes.c_uint64, ctypes.c_int32, _P, _P, _P],
+                          ctypes.c_int),
     "qec_debug_ozaki_gemm": ([_P, _P, ctypes.c_int32, ctypes.c_int32, _P], ctypes.c_int),
     "qec_debug_exact_probability": ([_P, ctypes.c_int32, _P], ctypes.c_int),
     "qec_debug_speculation": ([_P, ctypes.c_int32, _P], ctypes.c_int),
@@ -251,6 +253,18 @@ def qec_debug_unreduced_plan(gates, k, cap=512):
 
 def qec_debug_blocks(params, seed, traj, rnd, kraus_ptr, u_ptr):
     return check(lib().qec_debug_blocks(ctypes.byref(params), seed, traj, rnd, kraus_ptr, u_ptr))
+
+
+def qec_debug_factors(params, seed, traj, rnd, flips, n_blocks):
+    """(flips after the round, rotations [blocks][4], diagonals [blocks][2][16]) of one noisy round."""
+    import numpy as np
+
+    rot = np.zeros((n_blocks, 4), np.complex128)
+    diag = np.zeros((n_blocks, 2, 16), np.complex128)
+    f = ctypes.c_uint32(flips)
+    check(lib().qec_debug_factors(ctypes.byref(params), seed, traj, rnd, ctypes.cast(ctypes.pointer(f), _P),
+                                  rot.ctypes.data, diag.ctypes.data))
+    return int(f.value), rot, diag
 
 
 def qec_debug_exact_probability(sim, force):

@@ -13,7 +13,9 @@
 
 #include "../../include/qecsv.h"
 #include "common.cuh"
+#include "factor.cuh"
 #include "kernels.hpp"
+#include "onchip.hpp"
 #include "ozaki.cuh"
 #include "program.hpp"
 
@@ -56,6 +58,11 @@ struct qec_sim {
   cudaEvent_t kev[3] = {nullptr, nullptr, nullptr};   // event-record nodes around the instrumented block
   int timed_block = -1;
   Program init_prog, prog;
+  FactorProgram fprog;                  // prog's blocks in factored form (the speculative and on-chip engines)
+  unsigned char* d_factor = nullptr;    // its arrays on the device, at factor_off
+  size_t factor_off[5] = {};
+  double fm[FM_COUNT][4][2] = {};
+  uint8_t* h_out = nullptr;             // pinned outputs of an on-chip batch, written by the kernel
   int D = 0, nstab = 0, R = 0, S = 0;
   size_t amp = 16;
   void* psi = nullptr;
@@ -87,6 +94,7 @@ struct qec_sim {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   bool ran = false;
+  bool ran_onchip = false;              // the last trajectories ran on chip: their state is in psi
   int blk_cap = 0;      // blocks the Kraus/measurement buffers hold
   int syn_cap = 0;      // bytes per trajectory the syndrome buffer holds
 
@@ -120,6 +128,52 @@ qec_status upload_program(qec_sim* s, int which, const Program& P) {
   QEC_CUDA(cudaMemcpy(s->d_blocks[which], P.blocks.data(), sizeof(BlockInfo) * P.blocks.size(), cudaMemcpyHostToDevice));
   QEC_CUDA(cudaMemcpy(s->d_mats[which], P.mats, sizeof(P.mats), cudaMemcpyHostToDevice));
   return QEC_OK;
+}
+
+// The factored program's arrays behind each other; room for every noise site, so that qec_reconfigure
+// never reallocates.
+qec_status alloc_factor(qec_sim* s) {
+  qec_params full = s->p;
+  full.noise = qec_noise{1, 1, 1, 1, 1, 1, 1, 1, 1, 0};
+  Program P;
+  FactorProgram F;
+  std::string err;
+  if (!build_program(full, true, P, err, true) || !build_factor(P, F, err)) return fail(QEC_EINVAL, err);
+  const size_t bytes[5] = {sizeof(FSite) * F.sites.size(), sizeof(FItem) * F.items.size(),
+                           sizeof(FTouch) * F.touches.size(), sizeof(FBlock) * F.blocks.size(),
+                           sizeof(uint16_t) * F.order.size()};
+  size_t off = 0;
+  for (int i = 0; i < 5; ++i) {
+    s->factor_off[i] = off;
+    off += (bytes[i] + 255) / 256 * 256;
+  }
+  return dmalloc(&s->d_factor, off);
+}
+
+// Builds prog's factored form and uploads it on the work stream (the caller waits before s->fprog changes).
+qec_status upload_factor(qec_sim* s) {
+  std::string err;
+  if (!build_factor(s->prog, s->fprog, err)) return fail(QEC_EINVAL, err);
+  factor_mats(s->prog.mats, s->p.gates == QEC_GATES_CR, s->p.noise.twirl != 0.0, s->fm);
+  const FactorProgram& F = s->fprog;
+  const void* src[5] = {F.sites.data(), F.items.data(), F.touches.data(), F.blocks.data(), F.order.data()};
+  const size_t bytes[5] = {sizeof(FSite) * F.sites.size(), sizeof(FItem) * F.items.size(),
+                           sizeof(FTouch) * F.touches.size(), sizeof(FBlock) * F.blocks.size(),
+                           sizeof(uint16_t) * F.order.size()};
+  for (int i = 0; i < 5; ++i)
+    if (bytes[i])
+      QEC_CUDA(cudaMemcpyAsync(s->d_factor + s->factor_off[i], src[i], bytes[i], cudaMemcpyHostToDevice, s->work));
+  return QEC_OK;
+}
+
+FactorView device_factor(const qec_sim* s) {
+  FactorView v = view_of(s->fprog);
+  v.sites = reinterpret_cast<const FSite*>(s->d_factor + s->factor_off[0]);
+  v.items = reinterpret_cast<const FItem*>(s->d_factor + s->factor_off[1]);
+  v.touches = reinterpret_cast<const FTouch*>(s->d_factor + s->factor_off[2]);
+  v.blocks = reinterpret_cast<const FBlock*>(s->d_factor + s->factor_off[3]);
+  v.order = reinterpret_cast<const uint16_t*>(s->d_factor + s->factor_off[4]);
+  return v;
 }
 
 InstArgs inst_args(const qec_sim* s, int which, int round_base, int nblk, bool with_ctl) {
@@ -205,11 +259,22 @@ PassArgs spec_pass(const qec_sim* s, int b) {
 
 bool spec_applies(const qec_sim*) { return true; }
 
-// The state the last block wrote (the init state when there are no noisy rounds).
-const void* final_state(const qec_sim* s) {
+// Registers of up to 13 qubits run whole trajectories on chip (onchip.cu), one SM each, unless the
+// passes that compute each probability first were asked for.  2^13 complex128 amplitudes are enough
+// FP64 work for one or two trajectories to be faster as passes over the whole GPU (three rounds of the
+// repetition code: 1.45 ms on one SM, 0.74 ms per trajectory in passes; 16 trajectories 1.46 and 10.9 ms).
+bool on_chip(const qec_sim* s, uint32_t n) {
+  return s->spec && onchip_applies(s->D) && (s->D < 13 || !is_f64(s->p.precision) || n >= 3);
+}
+
+// The state that a trajectory's graph ends in (the init state when there are no noisy rounds).
+const void* graph_state(const qec_sim* s) {
   if (s->S == 0) return s->psi0;
   return s->spec ? spec_out(s, s->S - 1) : s->psi;
 }
+
+// Where the last run left its final state.
+const void* final_state(const qec_sim* s) { return s->ran_onchip ? s->psi : graph_state(s); }
 
 // Block b's apply pass is fused with block b+1's probability pass (one HBM read + write per
 // stabilizer) in the complex64 forms (k_fused, k_fused_tc) and in the tensor-core complex128 form
@@ -242,7 +307,7 @@ qec_status record(qec_sim* s, int i) {
 
 qec_status enqueue_readout(qec_sim* s) {
   ReadArgs r;
-  r.src = final_state(s);
+  r.src = graph_state(s);
   r.D = s->D;
   r.k1 = hist_k1(s->D);
   r.d = s->p.d;
@@ -342,7 +407,8 @@ void drop_graph(qec_sim* s) {
 
 void free_all(qec_sim* s) {
   drop_graph(s);
-  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_kraus, s->d_u, s->d_A, s->d_N, s->d_m, s->d_partials, s->d_ctl,
+  if (s->h_out) cudaFreeHost(s->h_out);
+  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_factor, s->d_kraus, s->d_u, s->d_A, s->d_N, s->d_m, s->d_partials, s->d_ctl,
                   s->d_hist_part, s->d_hist, s->d_syn, s->d_bits, s->d_log, s->d_events,
                   s->d_ops[0], s->d_ops[1], s->d_blocks[0], s->d_blocks[1], s->d_mats[0], s->d_mats[1]};
   for (void* p : ptrs) if (p) cudaFree(p);
@@ -386,6 +452,7 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   for (int i = 0; i < kCtlRing && e == cudaSuccess; ++i)
     e = cudaEventCreateWithFlags(&s->ctl_ev[i], cudaEventDisableTiming);
   if (e == cudaSuccess) e = setup_kernels(s->p.precision, s->D);
+  if (e == cudaSuccess && onchip_applies(s->D)) e = setup_onchip();
   if (e != cudaSuccess) return bail(fail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e)));
   const size_t state_bytes = ((size_t)1 << s->D) * s->amp;
   const int nblk = s->nstab * kMaxRounds;   // room for any round count (qec_reconfigure)
@@ -411,15 +478,81 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   e = cudaMemcpy(s->d_ctl, s->h_ctl, sizeof(Ctl), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return bail(fail(QEC_ECUDA, cudaGetErrorString(e)));
   if ((st = upload_program(s, 0, s->init_prog)) || (st = upload_program(s, 1, s->prog))) return bail(st);
+  if ((st = alloc_factor(s)) || (st = upload_factor(s))) return bail(st);
+  if (onchip_applies(s->D)) {
+    e = cudaMallocHost((void**)&s->h_out, (size_t)kBatchCap * (s->syn_cap + s->D + 1));
+    if (e != cudaSuccess) return bail(fail(QEC_ENOMEM, "pinned allocation failed"));
+  }
   if ((st = run_init_round(s))) return bail(st);
   *out = s;
+  return QEC_OK;
+}
+
+// The control header (seed, trajectory range, event capacity) of the next launches.  The events restart
+// with each call (reset_events).
+qec_status send_header(qec_sim* s, uint64_t seed, uint64_t first, bool reset_events) {
+  const int slot = s->ctl_next;
+  s->ctl_next = (s->ctl_next + 1) % kCtlRing;
+  QEC_CUDA(cudaEventSynchronize(s->ctl_ev[slot]));          // this header's previous copy is done
+  Ctl* h = s->h_ctl + slot;
+  h->seed = seed;
+  h->first = first;
+  h->traj = first;
+  h->ticket = 0;
+  h->ev_cap = s->ev_cap;
+  if (reset_events) h->n_events = 0;
+  const size_t head = reset_events ? offsetof(Ctl, prob_uncertain) : offsetof(Ctl, ticket);
+  QEC_CUDA(cudaMemcpyAsync(s->d_ctl, h, head, cudaMemcpyHostToDevice, s->work));
+  QEC_CUDA(cudaEventRecord(s->ctl_ev[slot], s->work));
+  return QEC_OK;
+}
+
+// Trajectories on chip: one launch per kBatchCap of them.  Host outputs are written by the kernel
+// straight into pinned memory, device outputs into the caller's buffers.
+qec_status run_onchip(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8_t* syn, uint8_t* bits,
+                      uint8_t* logical, bool host_out) {
+  const size_t ss = (size_t)s->syn_stride(), bs = (size_t)s->D;
+  OnchipArgs a;
+  a.F = device_factor(s);
+  for (int i = 0; i < PR_COUNT; ++i) a.thr[i] = fac::draw_threshold(s->prog.prob[i]);
+  std::memcpy(a.fm, s->fm, sizeof(a.fm));
+  a.seed = seed;
+  a.rounds = s->R;
+  a.nl = s->p.d;
+  a.psi0 = s->psi0;
+  a.ctl = s->d_ctl;
+  a.events = s->ev_cap ? s->d_events : nullptr;
+  for (uint32_t done = 0; done < n;) {
+    const uint32_t chunk = host_out && n - done > kBatchCap ? kBatchCap : n - done;
+    if (s->ev_cap && done == 0) {
+      qec_status st = send_header(s, seed, first, true);
+      if (st) return st;
+    }
+    a.first = first + done;
+    a.n = chunk;
+    a.psi_out = done + chunk == n ? s->psi : nullptr;
+    a.syn = !syn ? nullptr : host_out ? s->h_out : syn + done * ss;
+    a.bits = !bits ? nullptr : host_out ? s->h_out + chunk * ss : bits + done * bs;
+    a.logical = !logical ? nullptr : host_out ? s->h_out + chunk * (ss + bs) : logical + done;
+    if (done == 0) QEC_CUDA(cudaEventRecord(s->kev[1], s->work));
+    QEC_CUDA(launch_onchip(s->p.precision, a, s->num_sms, s->work));
+    if (done == 0) QEC_CUDA(cudaEventRecord(s->kev[2], s->work));
+    if (host_out) {
+      QEC_CUDA(cudaStreamSynchronize(s->work));
+      if (syn) std::memcpy(syn + done * ss, a.syn, chunk * ss);
+      if (bits) std::memcpy(bits + done * bs, a.bits, chunk * bs);
+      if (logical) std::memcpy(logical + done, a.logical, chunk);
+    }
+    done += chunk;
+  }
   return QEC_OK;
 }
 
 qec_status run_impl(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8_t* syn, uint8_t* bits,
                     uint8_t* logical, bool host_out) {
   if (!s) return fail(QEC_EINVAL, "null handle");
-  qec_status st = ensure_graph(s);
+  const bool oc = on_chip(s, n);
+  qec_status st = oc ? QEC_OK : ensure_graph(s);
   if (st) return st;
   if (s->user) {
     QEC_CUDA(cudaEventRecord(s->ev_in, s->user));
@@ -427,22 +560,11 @@ qec_status run_impl(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8
   }
   const cudaMemcpyKind kind = host_out ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   const size_t ss = (size_t)s->syn_stride(), bs = (size_t)s->D;
-  for (uint32_t done = 0; done < n;) {
+  if (oc && (st = run_onchip(s, seed, first, n, syn, bits, logical, host_out))) return st;
+  for (uint32_t done = 0; done < n && !oc;) {
     const uint32_t chunk = (n - done) < kBatchCap ? (n - done) : kBatchCap;
     if (done > 0) QEC_CUDA(cudaStreamSynchronize(s->work));   // the device output batch is reused
-    const int slot = s->ctl_next;
-    s->ctl_next = (s->ctl_next + 1) % kCtlRing;
-    QEC_CUDA(cudaEventSynchronize(s->ctl_ev[slot]));          // this header's previous copy is done
-    Ctl* h = s->h_ctl + slot;
-    h->seed = seed;
-    h->first = first + done;
-    h->traj = first + done;
-    h->ticket = 0;
-    h->ev_cap = s->ev_cap;
-    const size_t head = done == 0 ? offsetof(Ctl, prob_uncertain) : offsetof(Ctl, ticket);   // events reset per call
-    if (done == 0) h->n_events = 0;
-    QEC_CUDA(cudaMemcpyAsync(s->d_ctl, h, head, cudaMemcpyHostToDevice, s->work));
-    QEC_CUDA(cudaEventRecord(s->ctl_ev[slot], s->work));
+    if ((st = send_header(s, seed, first + done, done == 0))) return st;
     for (uint32_t t = 0; t < chunk; ++t) {
       st = launch_trajectory(s);
       if (st) return st;
@@ -456,14 +578,17 @@ qec_status run_impl(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8
     QEC_CUDA(cudaEventRecord(s->ev_out, s->work));
     QEC_CUDA(cudaStreamWaitEvent(s->user, s->ev_out, 0));
   }
-  if (host_out) {
+  if (host_out && !oc) {   // (the on-chip trajectories have no bounded waits and have been waited for)
     QEC_CUDA(cudaStreamSynchronize(s->work));
     unsigned int status = 0;
     QEC_CUDA(cudaMemcpy(&status, &s->d_ctl->status, sizeof(status), cudaMemcpyDeviceToHost));
     if (status) return fail(QEC_ETIMEOUT, "a bounded device wait gave up; results are invalid");
   }
   QEC_CUDA(cudaGetLastError());
-  if (n) s->ran = true;
+  if (n) {
+    s->ran = true;
+    s->ran_onchip = oc;
+  }
   return QEC_OK;
 }
 
@@ -571,8 +696,10 @@ qec_status qec_reconfigure(qec_sim* s, const qec_params* params) {
   QEC_CUDA(cudaMemcpyAsync(s->d_blocks[1], s->prog.blocks.data(), sizeof(BlockInfo) * P.blocks.size(),
                            cudaMemcpyHostToDevice, s->work));
   QEC_CUDA(cudaMemcpyAsync(s->d_mats[1], s->prog.mats, sizeof(P.mats), cudaMemcpyHostToDevice, s->work));
-  QEC_CUDA(cudaStreamSynchronize(s->work));   // the host copies in s->prog must outlive the uploads
   s->p = *params;
+  qec_status fst = upload_factor(s);
+  if (fst) return fst;
+  QEC_CUDA(cudaStreamSynchronize(s->work));   // the host copies in s->prog must outlive the uploads
   s->R = params->rounds;
   s->S = S;
   s->timed_block = s->R > 0 ? pick_timed_block(s) : -1;
@@ -599,7 +726,8 @@ qec_status qec_kernel_times(qec_sim* s, float* ms, int32_t* block) {
   if (!s || !ms || !block) return fail(QEC_EINVAL, "null argument");
   if (!s->ran || s->timed_block < 0) return fail(QEC_EINVAL, "no instrumented trajectory has run");
   QEC_CUDA(cudaStreamSynchronize(s->work));
-  QEC_CUDA(cudaEventElapsedTime(&ms[0], s->kev[0], s->kev[1]));
+  ms[0] = 0.f;   // on chip: the launch of the whole trajectories
+  if (!s->ran_onchip) QEC_CUDA(cudaEventElapsedTime(&ms[0], s->kev[0], s->kev[1]));
   QEC_CUDA(cudaEventElapsedTime(&ms[1], s->kev[1], s->kev[2]));
   *block = s->timed_block;
   return QEC_OK;
@@ -862,6 +990,38 @@ qec_status qec_debug_speculation(qec_sim* sim, int32_t enable, uint64_t* misses)
                         cudaMemcpyDeviceToHost));
     *misses = c;
   }
+  return QEC_OK;
+}
+
+qec_status qec_debug_factors(const qec_params* params, uint64_t seed, uint64_t traj, int32_t round, uint32_t* flips,
+                             double* rot, double* diag) {
+  if (!params || !flips || !rot || !diag) return fail(QEC_EINVAL, "null argument");
+  std::string err;
+  Program P;
+  FactorProgram FP;
+  if (round < 1 || !build_program(*params, true, P, err) || !build_factor(P, FP, err))
+    return fail(QEC_EINVAL, err.empty() ? "bad round" : err);
+  double2 fm[FM_COUNT][4];
+  factor_mats(P.mats, params->gates == QEC_GATES_CR, params->noise.twirl != 0.0,
+              reinterpret_cast<double (*)[4][2]>(&fm[0][0]));
+  const size_t nt = 4 * (size_t)P.nstab;
+  std::vector<uint8_t> code(FP.sites.size() + 1), swap(nt);
+  std::vector<fac::Touch> T(nt);
+  uint32_t mask = 0;
+  const fac::Rounds R{1, code.data(), T.data(), swap.data(), &mask};
+  std::memset(rot, 0, sizeof(double) * 2 * nt);
+  std::memset(diag, 0, sizeof(double) * 64 * P.nstab);
+  const FactorView F = view_of(FP);
+  uint64_t thr[PR_COUNT];
+  for (int i = 0; i < PR_COUNT; ++i) thr[i] = fac::draw_threshold(P.prob[i]);
+  fac::compile_merge(fac::OneThread{}, F, thr, seed, traj, (uint64_t)round, fm, R, [](int, int, int) {});
+  fac::compile_emit(fac::OneThread{}, F, fm, R, *flips,
+                    [&](int, int t, double2 v) { rot[2 * t] = v.x; rot[2 * t + 1] = v.y; },
+                    [&](int, int b, int z, double2 d0, double2 d1) {
+                      double* o = diag + 64 * (size_t)b + 2 * z;
+                      o[0] = d0.x; o[1] = d0.y; o[32] = d1.x; o[33] = d1.y;
+                    });
+  *flips ^= mask;
   return QEC_OK;
 }
 

@@ -4,9 +4,8 @@
 // owns every byte of device memory through its own pool or arena, code on a
 // latency-critical path where cudaMalloc's implicit device synchronisation is
 // not acceptable, or plug-ins that are handed a stream and output buffers but
-// no allocator.  All device working memory of the call (circuit program,
-// state vectors, Kraus blocks, reduction partials, readout histogram, control
-// word) lives in one file-scope static device array below; the caller passes
+// no allocator.  All device working memory of the call (circuit program, init
+// state, the init round's Kraus blocks and reduction partials, control word) lives in one file-scope static device array below; the caller passes
 // only the inputs (parameters, seed, trajectory range) and the device output
 // buffers.  The array is sized for the d = 3 register (2^9 amplitudes) with at
 // most kNoAllocMaxRounds noisy rounds, and every GPU that loads this library
@@ -20,7 +19,9 @@
 
 #include "../../include/qecsv.h"
 #include "common.cuh"
+#include "factor.cuh"
 #include "kernels.hpp"
+#include "onchip.hpp"
 #include "program.hpp"
 
 using namespace qec;
@@ -70,7 +71,7 @@ qec_status run_noalloc(const qec_params* params, uint64_t seed, uint64_t first_t
   Program init_prog, prog;
   if (!build_program(*params, false, init_prog, err) || !build_program(*params, true, prog, err))
     return nfail(QEC_EINVAL, err);
-  const int D = prog.nd, nstab = prog.nstab, R = params->rounds, S = nstab * R;
+  const int D = prog.nd, nstab = prog.nstab, R = params->rounds;
   const int prec = params->precision;
   const size_t amp = is_f64(prec) ? 16 : 8;
 
@@ -92,42 +93,41 @@ qec_status run_noalloc(const qec_params* params, uint64_t seed, uint64_t first_t
     base = static_cast<unsigned char*>(g_scratch_ptr[dev]);
   }
 
-  const int nblk = S > nstab ? S : nstab;
-  const int k1 = hist_k1(D), hgrid = hist_grid(D, sms);
+  FactorProgram fprog;
+  if (!build_factor(prog, fprog, err)) return nfail(QEC_EINVAL, err);
   int pgrid = pass_grid(D, 2, sms);
   const int pg4 = pass_grid(D, 4, sms);
   if (pg4 > pgrid) pgrid = pg4;
   Carve c;
-  const size_t o_psi = c.take(((size_t)1 << D) * amp), o_psi0 = c.take(((size_t)1 << D) * amp);
-  const size_t o_psi2 = c.take(((size_t)1 << D) * amp);   // second working state (speculative passes)
-  const size_t o_ops0 = c.take(sizeof(ProgOp) * (init_prog.ops.size() + 1));
-  const size_t o_ops1 = c.take(sizeof(ProgOp) * (prog.ops.size() + 1));
-  const size_t o_blk0 = c.take(sizeof(BlockInfo) * nstab), o_blk1 = c.take(sizeof(BlockInfo) * nstab);
-  const size_t o_mat0 = c.take(sizeof(prog.mats)), o_mat1 = c.take(sizeof(prog.mats));
-  const size_t o_kraus = c.take((size_t)nblk * KRAUS_STRIDE * amp);
-  const size_t o_u = c.take(sizeof(double) * nblk), o_A = c.take(sizeof(double) * nblk);
-  const size_t o_N = c.take(sizeof(double) * nblk), o_m = c.take(sizeof(int) * nblk);
+  const size_t o_psi0 = c.take(((size_t)1 << D) * amp);
+  const size_t o_ops = c.take(sizeof(ProgOp) * (init_prog.ops.size() + 1));
+  const size_t o_blk = c.take(sizeof(BlockInfo) * nstab), o_mat = c.take(sizeof(prog.mats));
+  const void* fac_src[5] = {fprog.sites.data(), fprog.items.data(), fprog.touches.data(), fprog.blocks.data(),
+                            fprog.order.data()};
+  const size_t fac_bytes[5] = {sizeof(FSite) * fprog.sites.size(), sizeof(FItem) * fprog.items.size(),
+                               sizeof(FTouch) * fprog.touches.size(), sizeof(FBlock) * fprog.blocks.size(),
+                               sizeof(uint16_t) * fprog.order.size()};
+  size_t o_fac[5];
+  for (int i = 0; i < 5; ++i) o_fac[i] = c.take(fac_bytes[i]);
+  const size_t o_kraus = c.take((size_t)nstab * KRAUS_STRIDE * amp);
+  const size_t o_u = c.take(sizeof(double) * nstab), o_A = c.take(sizeof(double) * nstab);
+  const size_t o_N = c.take(sizeof(double) * nstab), o_m = c.take(sizeof(int) * nstab);
   const size_t o_part = c.take(sizeof(double) * 2 * (pgrid > MAX_PASS_GRID ? pgrid : MAX_PASS_GRID));
   const size_t o_ctl = c.take(sizeof(Ctl));
-  const size_t o_hp = c.take(sizeof(double) * ((size_t)hgrid << k1)), o_h = c.take(sizeof(double) << k1);
   if (c.off > kNoAllocBytes) return nfail(QEC_EINVAL, "request does not fit the 2 MiB static scratch");
 
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  void* psi = base + o_psi;
   void* psi0 = base + o_psi0;
-  void* psi2 = base + o_psi2;
-  ProgOp* ops[2] = {reinterpret_cast<ProgOp*>(base + o_ops0), reinterpret_cast<ProgOp*>(base + o_ops1)};
-  BlockInfo* blks[2] = {reinterpret_cast<BlockInfo*>(base + o_blk0), reinterpret_cast<BlockInfo*>(base + o_blk1)};
-  double* mats[2] = {reinterpret_cast<double*>(base + o_mat0), reinterpret_cast<double*>(base + o_mat1)};
-  const Program* progs[2] = {&init_prog, &prog};
-  for (int i = 0; i < 2; ++i) {
-    const Program& P = *progs[i];
-    if (!P.ops.empty() && e == cudaSuccess)
-      e = cudaMemcpyAsync(ops[i], P.ops.data(), sizeof(ProgOp) * P.ops.size(), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(blks[i], P.blocks.data(), sizeof(BlockInfo) * nstab, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(mats[i], P.mats, sizeof(P.mats), cudaMemcpyHostToDevice, st);
-  }
+  ProgOp* ops = reinterpret_cast<ProgOp*>(base + o_ops);
+  BlockInfo* blks = reinterpret_cast<BlockInfo*>(base + o_blk);
+  double* mats = reinterpret_cast<double*>(base + o_mat);
+  if (!init_prog.ops.empty())
+    e = cudaMemcpyAsync(ops, init_prog.ops.data(), sizeof(ProgOp) * init_prog.ops.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(blks, init_prog.blocks.data(), sizeof(BlockInfo) * nstab, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(mats, init_prog.mats, sizeof(init_prog.mats), cudaMemcpyHostToDevice, st);
+  for (int i = 0; i < 5 && e == cudaSuccess; ++i)
+    if (fac_bytes[i]) e = cudaMemcpyAsync(base + o_fac[i], fac_src[i], fac_bytes[i], cudaMemcpyHostToDevice, st);
   // The control word is the only scratch that must start from known values (the reduction
   // ticket at 0); everything else is written before it is read.
   Ctl h_ctl;
@@ -139,94 +139,82 @@ qec_status run_noalloc(const qec_params* params, uint64_t seed, uint64_t first_t
   if (e == cudaSuccess) e = cudaMemcpyAsync(ctl, &h_ctl, sizeof(Ctl), cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return nfail(QEC_ECUDA, std::string("scratch upload: ") + cudaGetErrorString(e));
 
-  auto inst = [&](int which, int round_base, int nb, bool with_ctl) {
-    const Program& P = *progs[which];
+  auto inst = [&]() {
+    const Program& P = init_prog;
     InstArgs a;
-    a.ops = ops[which];
-    a.blocks = blks[which];
-    a.mats = mats[which];
+    a.ops = ops;
+    a.blocks = blks;
+    a.mats = mats;
     for (int i = 0; i < PR_COUNT; ++i) a.prob[i] = P.prob[i];
     a.nstab = nstab;
     a.nd = D;
-    a.round_base = round_base;
-    a.nblk = nb;
+    a.round_base = 0;
+    a.nblk = nstab;
     a.kraus = base + o_kraus;
     a.u = reinterpret_cast<double*>(base + o_u);
-    a.ctl = with_ctl ? ctl : nullptr;
+    a.ctl = nullptr;
     a.events = nullptr;
     return a;
   };
-  auto pass = [&](const Program& P, int blk, const void* src, bool forced, uint8_t* syn, int syn_idx) {
-    const BlockInfo& bi = P.blocks[blk % nstab];
+  auto pass = [&](int blk) {
+    const BlockInfo& bi = init_prog.blocks[blk];
     PassArgs a;
-    a.src = src;
-    a.dst = psi;
+    a.src = psi0;
+    a.dst = psi0;
     a.D = D;
     a.w = bi.w;
     for (int j = 0; j < 4; ++j) a.q[j] = bi.q[j] < 0 ? 0 : bi.q[j];
     a.kraus = base + o_kraus + (size_t)blk * KRAUS_STRIDE * amp;
     a.u = reinterpret_cast<double*>(base + o_u) + blk;
-    a.forced = forced ? bi.offset : -1;
+    a.forced = bi.offset;
     a.A = reinterpret_cast<double*>(base + o_A) + blk;
     a.N = reinterpret_cast<double*>(base + o_N) + blk;
     a.m = reinterpret_cast<int*>(base + o_m) + blk;
     a.ctl = ctl;
     a.partials = reinterpret_cast<double*>(base + o_part);
-    a.syn = syn;
+    a.syn = nullptr;
     a.syn_stride = (R + 1) * nstab;
-    a.syn_idx = syn_idx;
+    a.syn_idx = 0;
     a.offset = bi.offset;
     return a;
   };
 
-  // The same launches, grids and kernel sequence as qec_create / qec_run_trajectories, so that the
-  // reductions add in the same order and the results are identical: per block the speculative pass
-  // and its corrective launch, alternating between two working states.  (At d <= 3 the tensor-core
-  // passes do not apply: their tiles are larger than the register.)
+  // The same launches and kernels as qec_create / qec_run_trajectories, so that the results are
+  // identical: the init round's passes, then every trajectory on chip in one launch.
   auto prob = [&](const PassArgs& a) { return launch_prob(prec, a, pass_grid_for(prec, true, D, a.w, sms), st); };
   auto apply = [&](const PassArgs& a) { return launch_apply(prec, a, pass_grid_for(prec, false, D, a.w, sms), st); };
-  auto spec_out = [&](int b) { return (b & 1) ? psi2 : psi; };
   // Noise-free init round with outcomes forced to the zero syndrome (Sec. III.B), in psi0.
   e = launch_set_basis0(prec, psi0, D, st);
-  if (e == cudaSuccess) e = launch_instantiate(prec, inst(0, 0, nstab, false), st);
+  if (e == cudaSuccess) e = launch_instantiate(prec, inst(), st);
   for (int k = 0; k < nstab && e == cudaSuccess; ++k) {
-    PassArgs a = pass(init_prog, k, psi0, true, nullptr, 0);
-    a.dst = psi0;
+    const PassArgs a = pass(k);
     e = prob(a);
     if (e == cudaSuccess) e = apply(a);
   }
-  auto traj_pass = [&](int b) {
-    const int rnd = 1 + b / nstab, k = b % nstab;
-    return pass(prog, b, b == 0 ? psi0 : spec_out(b - 1), false, d_syndromes, rnd * nstab + k);
-  };
-  for (uint32_t t = 0; t < n && e == cudaSuccess; ++t) {
-    if (S > 0) e = launch_instantiate(prec, inst(1, 1, S, true), st);
-    for (int b = 0; b < S && e == cudaSuccess; ++b) {
-      PassArgs a = traj_pass(b);
-      a.src = b == 0 ? psi0 : spec_out(b - 1);
-      a.dst = spec_out(b);
-      a.spec_prev = b >= nstab ? a.syn_idx - nstab : -1;
-      double* n_next = b + 1 < S ? reinterpret_cast<double*>(base + o_N) + b + 1 : nullptr;
-      e = launch_spec(prec, a, n_next, b == 0, sms, st);
-      if (e == cudaSuccess) e = launch_spec_fix(prec, a, n_next, b == 0, sms, st);
-    }
-    if (e != cudaSuccess) break;
-    ReadArgs r;
-    r.src = S > 0 ? spec_out(S - 1) : psi0;
-    r.D = D;
-    r.k1 = k1;
-    r.d = params->d;
-    r.rounds = R;
-    r.grid_hist = hgrid;
-    r.hist_part = reinterpret_cast<double*>(base + o_hp);
-    r.hist = reinterpret_cast<double*>(base + o_h);
-    r.ctl = ctl;
-    r.bits = d_data_bits;
-    r.logical = d_raw_logical;
-    r.syn = d_syndromes;
-    r.syn_stride = (R + 1) * nstab;
-    r.nstab = nstab;
-    e = launch_readout(prec, r, st);
+  if (e == cudaSuccess) e = setup_onchip();
+  if (e == cudaSuccess) {
+    OnchipArgs a;
+    a.F = view_of(fprog);
+    a.F.sites = reinterpret_cast<const FSite*>(base + o_fac[0]);
+    a.F.items = reinterpret_cast<const FItem*>(base + o_fac[1]);
+    a.F.touches = reinterpret_cast<const FTouch*>(base + o_fac[2]);
+    a.F.blocks = reinterpret_cast<const FBlock*>(base + o_fac[3]);
+    a.F.order = reinterpret_cast<const uint16_t*>(base + o_fac[4]);
+    for (int i = 0; i < PR_COUNT; ++i) a.thr[i] = fac::draw_threshold(prog.prob[i]);
+    factor_mats(prog.mats, params->gates == QEC_GATES_CR, params->noise.twirl != 0.0, a.fm);
+    a.seed = seed;
+    a.first = first_traj;
+    a.n = n;
+    a.rounds = R;
+    a.nl = params->d;
+    a.psi0 = psi0;
+    a.psi_out = nullptr;
+    a.syn = d_syndromes;
+    a.bits = d_data_bits;
+    a.logical = d_raw_logical;
+    a.ctl = nullptr;
+    a.events = nullptr;
+    e = launch_onchip(prec, a, sms, st);
   }
   if (e != cudaSuccess) return nfail(QEC_ECUDA, std::string("launch: ") + cudaGetErrorString(e));
   return QEC_OK;
