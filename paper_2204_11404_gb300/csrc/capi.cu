@@ -18,6 +18,7 @@
 #include "onchip.hpp"
 #include "ozaki.cuh"
 #include "program.hpp"
+#include "rounds.hpp"
 
 using namespace qec;
 
@@ -62,13 +63,25 @@ struct qec_sim {
   unsigned char* d_factor = nullptr;    // its arrays on the device, at factor_off
   size_t factor_off[5] = {};
   double fm[FM_COUNT][4][2] = {};
+  // factored passes (rounds.cu): up to r_groups trajectories of r_G CTAs each
+  int r_groups = 0, r_G = 0;
+  std::vector<ChainDesc> chains;
+  ChainDesc* d_chains = nullptr;
+  void* d_cblocks = nullptr;
+  unsigned char* d_scratch = nullptr;
+  uint32_t* d_masks = nullptr;
+  double* d_norm = nullptr;
+  double* d_rparts = nullptr;
+  unsigned int* d_bar = nullptr;
+  const void* last_state = nullptr;     // of the last run in factored passes: its state and flips
+  const uint32_t* last_masks = nullptr;
   uint8_t* h_out = nullptr;             // pinned outputs of an on-chip batch, written by the kernel
   int D = 0, nstab = 0, R = 0, S = 0;
   size_t amp = 16;
   void* psi = nullptr;
   void* psi0 = nullptr;
   void* psi2 = nullptr;                        // second working state of the speculative passes
-  bool spec = false;                           // QEC_C128_TC with every block on the speculative pass
+  bool spec = false;                           // outcomes guessed (every form's default), or each probability first
   ProgOp* d_ops[2] = {nullptr, nullptr};       // [0] init, [1] noisy
   BlockInfo* d_blocks[2] = {nullptr, nullptr};
   double* d_mats[2] = {nullptr, nullptr};
@@ -94,7 +107,7 @@ struct qec_sim {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   bool ran = false;
-  bool ran_onchip = false;              // the last trajectories ran on chip: their state is in psi
+  enum Engine { GRAPH, ONCHIP, ROUNDS } ran_on = GRAPH;   // what the last trajectories ran on
   int blk_cap = 0;      // blocks the Kraus/measurement buffers hold
   int syn_cap = 0;      // bytes per trajectory the syndrome buffer holds
 
@@ -132,13 +145,14 @@ qec_status upload_program(qec_sim* s, int which, const Program& P) {
 
 // The factored program's arrays behind each other; room for every noise site, so that qec_reconfigure
 // never reallocates.
-qec_status alloc_factor(qec_sim* s) {
+qec_status alloc_factor(qec_sim* s, size_t* scratch) {
   qec_params full = s->p;
   full.noise = qec_noise{1, 1, 1, 1, 1, 1, 1, 1, 1, 0};
   Program P;
   FactorProgram F;
   std::string err;
   if (!build_program(full, true, P, err, true) || !build_factor(P, F, err)) return fail(QEC_EINVAL, err);
+  *scratch = compile_scratch_bytes(F);
   const size_t bytes[5] = {sizeof(FSite) * F.sites.size(), sizeof(FItem) * F.items.size(),
                            sizeof(FTouch) * F.touches.size(), sizeof(FBlock) * F.blocks.size(),
                            sizeof(uint16_t) * F.order.size()};
@@ -257,14 +271,25 @@ PassArgs spec_pass(const qec_sim* s, int b) {
   return a;
 }
 
-bool spec_applies(const qec_sim*) { return true; }
-
 // Registers of up to 13 qubits run whole trajectories on chip (onchip.cu), one SM each, unless the
 // passes that compute each probability first were asked for.  2^13 complex128 amplitudes are enough
 // FP64 work for one or two trajectories to be faster as passes over the whole GPU (three rounds of the
 // repetition code: 1.45 ms on one SM, 0.74 ms per trajectory in passes; 16 trajectories 1.46 and 10.9 ms).
 bool on_chip(const qec_sim* s, uint32_t n) {
   return s->spec && onchip_applies(s->D) && (s->D < 13 || !is_f64(s->p.precision) || n >= 3);
+}
+
+// Everything else runs in factored passes (rounds.cu), but for the tensor-core complex128 form on large
+// registers, where its dense slices beat the FP64 pipe (five rounds of the repetition code, 25 qubits:
+// 47.0 and 52.1 ms, 21 qubits: 5.1 and 6.2, 17 qubits: 2.0 and 0.89).
+// Blocks per pass.  complex64 passes are bound by memory and shared-memory sweeps: four blocks share a
+// read and a write.  complex128 ones are bound by the FP64 pipe, where a pass that runs again costs
+// all its blocks: one block each on large registers (d = 5, five rounds: 94.8, 101, 107, 112 ms for 1 to
+// 4); on small ones the barrier between passes counts (17 qubits: 1.25, 1.01, 0.94, 0.89 ms).
+int chain_limit(const qec_params& p, int D) { return is_f64(p.precision) && D > 21 ? 1 : 4; }
+bool rounds_apply(const qec_params& p, int D) {
+  if (D < 13 || (D == 13 && !is_f64(p.precision))) return false;   // on chip
+  return p.precision != QEC_C128_TC || D < 21;
 }
 
 // The state that a trajectory's graph ends in (the init state when there are no noisy rounds).
@@ -274,7 +299,10 @@ const void* graph_state(const qec_sim* s) {
 }
 
 // Where the last run left its final state.
-const void* final_state(const qec_sim* s) { return s->ran_onchip ? s->psi : graph_state(s); }
+const void* final_state(const qec_sim* s) {
+  if (s->ran_on == qec_sim::ROUNDS) return s->last_state;
+  return s->ran_on == qec_sim::ONCHIP ? s->psi : graph_state(s);
+}
 
 // Block b's apply pass is fused with block b+1's probability pass (one HBM read + write per
 // stabilizer) in the complex64 forms (k_fused, k_fused_tc) and in the tensor-core complex128 form
@@ -305,7 +333,7 @@ qec_status record(qec_sim* s, int i) {
   return QEC_OK;
 }
 
-qec_status enqueue_readout(qec_sim* s) {
+ReadArgs read_args(const qec_sim* s) {
   ReadArgs r;
   r.src = graph_state(s);
   r.D = s->D;
@@ -321,7 +349,11 @@ qec_status enqueue_readout(qec_sim* s) {
   r.syn = s->d_syn;
   r.syn_stride = s->syn_stride();
   r.nstab = s->nstab;
-  QEC_CUDA(launch_readout(s->p.precision, r, s->work));
+  return r;
+}
+
+qec_status enqueue_readout(qec_sim* s) {
+  QEC_CUDA(launch_readout(s->p.precision, read_args(s), s->work));
   return QEC_OK;
 }
 
@@ -342,9 +374,9 @@ qec_status enqueue_trajectory(qec_sim* s) {
       const PassArgs a = spec_pass(s, b);
       double* n_next = b + 1 < s->S ? s->d_N + b + 1 : nullptr;
       if (timed && ((st = record(s, 0)) || (st = record(s, 1)))) return st;
-      QEC_CUDA(launch_spec(s->p.precision, a, n_next, b == 0, s->num_sms, s->work));
+      QEC_CUDA(launch_spec(a, n_next, b == 0, s->num_sms, s->work));
       if (timed && (st = record(s, 2))) return st;
-      QEC_CUDA(launch_spec_fix(s->p.precision, a, n_next, b == 0, s->num_sms, s->work));
+      QEC_CUDA(launch_spec_fix(a, n_next, b == 0, s->num_sms, s->work));
     }
     return st == QEC_OK ? enqueue_readout(s) : st;
   }
@@ -408,7 +440,8 @@ void drop_graph(qec_sim* s) {
 void free_all(qec_sim* s) {
   drop_graph(s);
   if (s->h_out) cudaFreeHost(s->h_out);
-  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_factor, s->d_kraus, s->d_u, s->d_A, s->d_N, s->d_m, s->d_partials, s->d_ctl,
+  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_factor, s->d_chains, s->d_cblocks, s->d_scratch, s->d_masks,
+                  s->d_norm, s->d_rparts, s->d_bar, s->d_kraus, s->d_u, s->d_A, s->d_N, s->d_m, s->d_partials, s->d_ctl,
                   s->d_hist_part, s->d_hist, s->d_syn, s->d_bits, s->d_log, s->d_events,
                   s->d_ops[0], s->d_ops[1], s->d_blocks[0], s->d_blocks[1], s->d_mats[0], s->d_mats[1]};
   for (void* p : ptrs) if (p) cudaFree(p);
@@ -457,16 +490,25 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   const size_t state_bytes = ((size_t)1 << s->D) * s->amp;
   const int nblk = s->nstab * kMaxRounds;   // room for any round count (qec_reconfigure)
   const int k1 = hist_k1(s->D);
-  s->spec = spec_applies(s);
-  if (s->spec && (st = dmalloc(&s->psi2, state_bytes))) return bail(st);
-  if ((st = dmalloc(&s->psi, state_bytes)) || (st = dmalloc(&s->psi0, state_bytes)) ||
+  s->spec = true;
+  s->r_groups = 1;
+  if (rounds_apply(s->p, s->D)) {
+    if ((e = setup_rounds(s->p.precision)) != cudaSuccess)
+      return bail(fail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e)));
+    const int wave = round_wave(s->p.precision, s->num_sms), tiles = round_ctas(s->D);
+    if (wave < 1) return bail(fail(QEC_ECUDA, "the factored pass does not fit an SM"));
+    s->r_G = std::min(wave, tiles);
+    s->r_groups = s->D == 13 ? 2 : wave / s->r_G;   // trajectories side by side where one does not fill the GPU
+  }
+  const size_t groups = (size_t)s->r_groups;
+  if ((st = dmalloc(&s->psi2, state_bytes * groups)) || (st = dmalloc(&s->psi, state_bytes * groups)) || (st = dmalloc(&s->psi0, state_bytes)) ||
       (st = dmalloc(&s->d_kraus, (size_t)nblk * KRAUS_STRIDE * s->amp)) ||
       (st = dmalloc(&s->d_u, sizeof(double) * nblk)) || (st = dmalloc(&s->d_A, sizeof(double) * nblk)) ||
       (st = dmalloc(&s->d_N, sizeof(double) * nblk)) || (st = dmalloc(&s->d_m, sizeof(int) * nblk)) ||
       (st = dmalloc(&s->d_partials, sizeof(double) * 2 * MAX_PASS_GRID)) ||
       (st = dmalloc(&s->d_ctl, sizeof(Ctl))) ||
-      (st = dmalloc(&s->d_hist_part, sizeof(double) * ((size_t)hist_grid(s->D, s->num_sms) << k1))) ||
-      (st = dmalloc(&s->d_hist, sizeof(double) << k1)) ||
+      (st = dmalloc(&s->d_hist_part, sizeof(double) * groups * ((size_t)hist_grid(s->D, s->num_sms) << k1))) ||
+      (st = dmalloc(&s->d_hist, (sizeof(double) * groups) << k1)) ||
       (st = dmalloc(&s->d_syn, (size_t)kBatchCap * (kMaxRounds + 1) * s->nstab)) ||
       (st = dmalloc(&s->d_bits, (size_t)kBatchCap * s->D)) || (st = dmalloc(&s->d_log, kBatchCap)))
     return bail(st);
@@ -478,7 +520,24 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   e = cudaMemcpy(s->d_ctl, s->h_ctl, sizeof(Ctl), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return bail(fail(QEC_ECUDA, cudaGetErrorString(e)));
   if ((st = upload_program(s, 0, s->init_prog)) || (st = upload_program(s, 1, s->prog))) return bail(st);
-  if ((st = alloc_factor(s)) || (st = upload_factor(s))) return bail(st);
+  size_t scratch = 0;
+  if ((st = alloc_factor(s, &scratch)) || (st = upload_factor(s))) return bail(st);
+  if (rounds_apply(s->p, s->D)) {
+    s->chains = plan_chains(s->fprog, s->p.precision, chain_limit(s->p, s->D));
+    const size_t nr = groups * kMaxRounds;
+    if ((st = dmalloc(&s->d_chains, sizeof(ChainDesc) * s->chains.size())) ||
+        (st = dmalloc(&s->d_cblocks, nr * s->nstab * compiled_block_bytes(s->p.precision))) ||
+        (st = dmalloc(&s->d_scratch, nr * scratch)) || (st = dmalloc(&s->d_masks, nr * sizeof(uint32_t))) ||
+        (st = dmalloc(&s->d_norm, groups * sizeof(double))) ||
+        (st = dmalloc(&s->d_rparts, 2 * groups * s->r_G * kMaxChain * sizeof(double))) ||
+        (st = dmalloc(&s->d_bar, 2 * groups * sizeof(unsigned int))))
+      return bail(st);
+    e = cudaMemsetAsync(s->d_bar, 0, 2 * groups * sizeof(unsigned int), s->work);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(s->d_chains, s->chains.data(), sizeof(ChainDesc) * s->chains.size(), cudaMemcpyHostToDevice,
+                          s->work);
+    if (e != cudaSuccess) return bail(fail(QEC_ECUDA, cudaGetErrorString(e)));
+  }
   if (onchip_applies(s->D)) {
     e = cudaMallocHost((void**)&s->h_out, (size_t)kBatchCap * (s->syn_cap + s->D + 1));
     if (e != cudaSuccess) return bail(fail(QEC_ENOMEM, "pinned allocation failed"));
@@ -548,11 +607,73 @@ qec_status run_onchip(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uin
   return QEC_OK;
 }
 
+// A batch of `chunk` trajectories from `first` on, in factored passes, into the device output batch:
+// r_groups of them side by side, a launch per round (larger registers: other streams' work gets in
+// between) or for all rounds.
+qec_status run_rounds(qec_sim* s, uint64_t seed, uint64_t first, uint32_t chunk) {
+  RoundArgs a;
+  a.F = device_factor(s);
+  for (int i = 0; i < PR_COUNT; ++i) a.thr[i] = fac::draw_threshold(s->prog.prob[i]);
+  std::memcpy(a.fm, s->fm, sizeof(a.fm));
+  a.seed = seed;
+  a.G = s->r_G;
+  a.D = s->D;
+  a.rounds = s->R;
+  a.chains = s->d_chains;
+  a.nc = (int)s->chains.size();
+  a.psi0 = s->psi0;
+  a.buf[0] = s->psi;
+  a.buf[1] = s->psi2;
+  a.blocks = s->d_cblocks;
+  a.scratch = s->d_scratch;
+  a.masks = s->d_masks;
+  a.norm = s->d_norm;
+  a.partials = s->d_rparts;
+  a.bar = s->d_bar;
+  a.ctl = s->d_ctl;
+  a.events = s->ev_cap ? s->d_events : nullptr;
+  ReadArgs r = read_args(s);
+  r.direct = 1;
+  r.seed = seed;
+  if (s->R > 0) {
+    r.src = ((s->R * a.nc - 1) & 1) ? s->psi2 : s->psi;
+    r.src_stride = (size_t)1 << s->D;
+    r.masks = s->d_masks;
+  }
+  const int per = s->D >= 21 ? 1 : std::max(s->R, 1);   // rounds per launch
+  const int timed = s->timed_block < 0 ? 0 : 1 + s->timed_block / s->nstab;
+  for (uint32_t t = 0; t < chunk; t += (uint32_t)a.groups) {
+    a.groups = (int)std::min<uint32_t>((uint32_t)s->r_groups, chunk - t);
+    a.first = first + t;
+    a.syn = s->d_syn + (size_t)t * s->syn_stride();
+    if (s->R > 0) QEC_CUDA(launch_compile(s->p.precision, a, s->work));
+    for (int r0 = 1; r0 <= s->R; r0 += per) {
+      const int r1 = std::min(s->R, r0 + per - 1);
+      const bool tm = t == 0 && timed >= r0 && timed <= r1;
+      if (tm) {
+        QEC_CUDA(cudaEventRecord(s->kev[0], s->work));
+        QEC_CUDA(cudaEventRecord(s->kev[1], s->work));
+      }
+      QEC_CUDA(launch_rounds(s->p.precision, a, r0, r1, s->work));
+      if (tm) QEC_CUDA(cudaEventRecord(s->kev[2], s->work));
+    }
+    r.groups = a.groups;
+    r.first = a.first;
+    r.syn = a.syn;
+    r.bits = s->d_bits + (size_t)t * s->D;
+    r.logical = s->d_log + t;
+    QEC_CUDA(launch_readout(s->p.precision, r, s->work));
+  }
+  s->last_state = static_cast<const char*>(r.src) + (size_t)(a.groups - 1) * r.src_stride * s->amp;
+  s->last_masks = r.masks ? r.masks + (size_t)(a.groups - 1) * s->R : nullptr;
+  return QEC_OK;
+}
+
 qec_status run_impl(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8_t* syn, uint8_t* bits,
                     uint8_t* logical, bool host_out) {
   if (!s) return fail(QEC_EINVAL, "null handle");
-  const bool oc = on_chip(s, n);
-  qec_status st = oc ? QEC_OK : ensure_graph(s);
+  const bool oc = on_chip(s, n), rd = !oc && s->spec && rounds_apply(s->p, s->D);
+  qec_status st = oc || rd ? QEC_OK : ensure_graph(s);
   if (st) return st;
   if (s->user) {
     QEC_CUDA(cudaEventRecord(s->ev_in, s->user));
@@ -565,7 +686,8 @@ qec_status run_impl(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8
     const uint32_t chunk = (n - done) < kBatchCap ? (n - done) : kBatchCap;
     if (done > 0) QEC_CUDA(cudaStreamSynchronize(s->work));   // the device output batch is reused
     if ((st = send_header(s, seed, first + done, done == 0))) return st;
-    for (uint32_t t = 0; t < chunk; ++t) {
+    if (rd && (st = run_rounds(s, seed, first + done, chunk))) return st;
+    for (uint32_t t = 0; t < chunk && !rd; ++t) {
       st = launch_trajectory(s);
       if (st) return st;
     }
@@ -587,7 +709,7 @@ qec_status run_impl(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8
   QEC_CUDA(cudaGetLastError());
   if (n) {
     s->ran = true;
-    s->ran_onchip = oc;
+    s->ran_on = oc ? qec_sim::ONCHIP : rd ? qec_sim::ROUNDS : qec_sim::GRAPH;
   }
   return QEC_OK;
 }
@@ -633,15 +755,28 @@ qec_status qec_get_state(qec_sim* s, void* host_buf, size_t bytes) {
   Ctl c;
   QEC_CUDA(cudaMemcpy(&c, s->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
   const void* src = final_state(s);
+  uint32_t flips = 0;   // the register holds data index x at x ^ flips
+  if (s->ran_on == qec_sim::ROUNDS && s->last_masks) {
+    std::vector<uint32_t> masks(s->R);
+    QEC_CUDA(cudaMemcpy(masks.data(), s->last_masks, sizeof(uint32_t) * masks.size(), cudaMemcpyDeviceToHost));
+    for (uint32_t m : masks) flips ^= m;
+  }
   double* out = static_cast<double*>(host_buf);
   const double scale = 1.0 / std::sqrt(c.final_norm);
   if (is_f64(s->p.precision)) {
     QEC_CUDA(cudaMemcpy(out, src, 16 * n, cudaMemcpyDeviceToHost));
     for (size_t i = 0; i < 2 * n; ++i) out[i] *= scale;
+    for (size_t i = 0; i < n && flips; ++i) {
+      const size_t k = i ^ flips;
+      if (k > i) {
+        std::swap(out[2 * i], out[2 * k]);
+        std::swap(out[2 * i + 1], out[2 * k + 1]);
+      }
+    }
   } else {
     std::vector<float> tmp(2 * n);
     QEC_CUDA(cudaMemcpy(tmp.data(), src, 8 * n, cudaMemcpyDeviceToHost));
-    for (size_t i = 0; i < 2 * n; ++i) out[i] = (double)tmp[i] * scale;
+    for (size_t i = 0; i < 2 * n; ++i) out[i] = (double)tmp[i ^ (2 * (size_t)flips)] * scale;
   }
   return QEC_OK;
 }
@@ -727,7 +862,7 @@ qec_status qec_kernel_times(qec_sim* s, float* ms, int32_t* block) {
   if (!s->ran || s->timed_block < 0) return fail(QEC_EINVAL, "no instrumented trajectory has run");
   QEC_CUDA(cudaStreamSynchronize(s->work));
   ms[0] = 0.f;   // on chip: the launch of the whole trajectories
-  if (!s->ran_onchip) QEC_CUDA(cudaEventElapsedTime(&ms[0], s->kev[0], s->kev[1]));
+  if (s->ran_on != qec_sim::ONCHIP) QEC_CUDA(cudaEventElapsedTime(&ms[0], s->kev[0], s->kev[1]));
   QEC_CUDA(cudaEventElapsedTime(&ms[1], s->kev[1], s->kev[2]));
   *block = s->timed_block;
   return QEC_OK;

@@ -406,16 +406,15 @@ __device__ __forceinline__ int spec_guess(const PassArgs& a) {
   return (int)(a.syn[t * (unsigned long long)a.syn_stride + a.spec_prev] & 1u) ^ a.offset;
 }
 
-// End of a speculative (FIX = false) or corrective (FIX = true) pass (Sec. II.B, evaluated as the
-// tensor-core k_ozs below describes): block sums of (Nin^ = |input|^2, its bound) and (Y^ = |output|^2,
+// End of a speculative (FIX = false) or corrective (FIX = true) pass (Sec. II.B, evaluated as k_ozs
+// below describes): block sums of (Nin^ = |input|^2, its bound) and (Y^ = |output|^2,
 // its bound) into 4 partials per CTA; the last CTA sums them in a fixed order and stores Y^ as the
 // next block's N.  The speculative pass then decides where |u N' - P(1) N'| exceeds twice the summed
 // bounds plus 1e-10 (N' + Y^), N' = Nin^ / N, P(1) N' = Y^ for g = 1 and N' - Y^ for g = 0, and
-// otherwise flags the exact pass.  exact: the sums are FP64 sums of the FP64 values themselves (the
-// CUDA-core pass) and decide every outcome directly, as the FP64 probability pass does.
+// otherwise flags the exact pass.
 template <bool FIX>
 __device__ void spec_finish(const FusedArgs& f, int g, double nI, double rI, double nO, double rO, double* sred,
-                            int* s_last, bool exact = false) {
+                            int* s_last) {
   const PassArgs& a = f.ap;
   block_sum2(nI, rI, sred);
   block_sum2(nO, rO, sred);
@@ -453,7 +452,7 @@ __device__ void spec_finish(const FusedArgs& f, int g, double nI, double rI, dou
       int m = a.forced;
       if (m < 0) {
         const double u = *a.u;
-        decided = exact || (!a.ctl->prob_force_exact && fabs(u * Np - A1) > 2.0 * (rNp + sRO) + 1e-10 * (Np + sO));
+        decided = !a.ctl->prob_force_exact && fabs(u * Np - A1) > 2.0 * (rNp + sRO) + 1e-10 * (Np + sO);
         m = u * Np < A1 ? 1 : 0;
       }
       a.ctl->prob_uncertain = decided ? 0u : 1u;
@@ -468,67 +467,6 @@ __device__ void spec_finish(const FusedArgs& f, int g, double nI, double rI, dou
     }
     a.ctl->ticket = 0u;
   }
-}
-
-// ---- speculative FP64 pass (QEC_C128, and QEC_C128_TC where the tensor-core tile does not fit) ----
-// The order of evaluation of the tensor-core k_ozs (Sec. II.B; guess = the same stabilizer's outcome
-// one round earlier): y = K_g psi / sqrt(N) out of place, with Nin = sum |psi|^2 and Y = sum |y|^2
-// summed in FP64 per thread; the last CTA decides u N' < P(1) N' (N' = Nin / N; P(1) N' = Y for
-// g = 1, N' - Y for g = 0) and stores Y as the next block's N.  FIX: the corrective apply of the
-// decided K_m from the untouched input, only where m != g.  Grid-stride over groups as k_apply, so
-// every sum and outcome is the same in every run for a fixed grid.
-template <int W, bool FIX>
-__global__ void __launch_bounds__(256) k_apply_spec(FusedArgs f) {
-  const PassArgs& a = f.ap;
-  const int gs = spec_guess(a);
-  const int m = FIX ? *a.m : gs;
-  if (FIX && m == gs) return;
-  constexpr int C = 1 << W;
-  __shared__ double2 sK[C * C];
-  __shared__ double sred[64];
-  __shared__ int s_last;
-  const double scale = f.spec_unit ? 1.0 : 1.0 / sqrt(*a.N);
-  const double2* Kg = reinterpret_cast<const double2*>(a.kraus) + (m ? 256 : 0);
-  for (int i = threadIdx.x; i < C * C; i += blockDim.x) {
-    double2 kv = Kg[(i / C) * 16 + (i % C)];
-    kv.x *= scale;
-    kv.y *= scale;
-    sK[i] = kv;
-  }
-  __syncthreads();
-  int q[4];
-  load_q<W>(a, q);
-  uint32_t off[C];
-#pragma unroll
-  for (int l = 0; l < C; ++l) off[l] = member_off<W>(l, q);
-  const double2* src = reinterpret_cast<const double2*>(a.src);
-  double2* dst = reinterpret_cast<double2*>(a.dst);
-  const uint32_t G = 1u << (a.D - W);
-  double accI = 0.0, accO = 0.0;
-  for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
-    const uint32_t base = group_base<W>(g, q);
-    double2 v[C];
-#pragma unroll
-    for (int l = 0; l < C; ++l) {
-      v[l] = src[base + off[l]];
-      accI = fma(v[l].x, v[l].x, fma(v[l].y, v[l].y, accI));
-    }
-#pragma unroll
-    for (int r = 0; r < C; ++r) {
-      double sr = 0, si = 0;
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        const double2 k = lds_v2(&sK[r * C + c]);
-        sr = fma(k.x, v[c].x, sr);
-        sr = fma(-k.y, v[c].y, sr);
-        si = fma(k.x, v[c].y, si);
-        si = fma(k.y, v[c].x, si);
-      }
-      dst[base + off[r]] = make_double2(sr, si);
-      accO = fma(sr, sr, fma(si, si, accO));
-    }
-  }
-  spec_finish<FIX>(f, gs, accI, 0.0, accO, 0.0, sred, &s_last, true);
 }
 
 // ---- fused pass: apply block s, then probability of block s+1, per shared-memory tile ----
@@ -704,116 +642,6 @@ __global__ void __launch_bounds__(256) k_fused(FusedArgs f) {
   }
   cp_async_wait<0>();
   prob_finish(f.pr, accA, accN, sred, &s_last);
-}
-
-// ---- speculative complex64 pass (QEC_C64), per shared-memory tile -------------------------------
-// The order of evaluation of k_apply_spec (Sec. II.B; guess = the same stabilizer's outcome one round
-// earlier) on k_fused's double-buffered tiles of block a's qubits and the low register bits: the
-// tile's groups are multiplied by K_g / sqrt(N) in FP32, in shared memory, with |in|^2 and |out|^2
-// summed per thread in FP32 over the tile and in FP64 across tiles (as k_fused sums its
-// probabilities); the tile is stored to the other working state.  The last CTA decides
-// u N' < P(1) N' directly, as the complex64 probability pass does.  FIX: the corrective apply where
-// the drawn outcome differs from g.
-template <int W, bool FIX>
-__global__ void __launch_bounds__(256) k_fused_spec(FusedArgs f) {
-  const int gs = spec_guess(f.ap);
-  const int m = FIX ? *f.ap.m : gs;
-  if (FIX && m == gs) return;
-  constexpr int C = 1 << W;
-  constexpr int CH = 2;   // complex64 amplitudes per 16-byte copy
-  extern __shared__ __align__(16) unsigned char fsm[];
-  const uint32_t tsz = 1u << f.nt, lmask = (1u << f.lb) - 1u;
-  float2* buf0 = reinterpret_cast<float2*>(fsm);
-  float2* buf1 = buf0 + tsz;
-  uint32_t* hoff = reinterpret_cast<uint32_t*>(buf1 + tsz);
-  __shared__ __align__(16) float2 sK[C * C];
-  __shared__ double sred[64];
-  __shared__ int s_last;
-  {
-    const double scale = f.spec_unit ? 1.0 : 1.0 / sqrt(*f.ap.N);
-    const float2* Kg = reinterpret_cast<const float2*>(f.ap.kraus) + (m ? 256 : 0);
-    for (int i = threadIdx.x; i < C * C; i += blockDim.x) {
-      float2 kv = Kg[(i / C) * 16 + (i % C)];
-      kv.x = (float)((double)kv.x * scale);
-      kv.y = (float)((double)kv.y * scale);
-      sK[i] = kv;
-    }
-    const int nh = f.nt - f.lb;
-    for (int h = threadIdx.x; h < (1 << nh); h += blockDim.x) {
-      uint32_t o = 0;
-      for (int j = 0; j < nh; ++j) o |= (uint32_t)((h >> j) & 1) << f.hbits[j];
-      hoff[h] = o;
-    }
-  }
-  __syncthreads();
-  int qa[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) qa[j] = j < W ? f.qa[j] : 0;
-  uint32_t offa[C];
-#pragma unroll
-  for (int l = 0; l < C; ++l) offa[l] = member_off<W>(l, qa);
-  const float2* src = reinterpret_cast<const float2*>(f.ap.src);
-  float2* dst = reinterpret_cast<float2*>(f.ap.dst);
-  const uint32_t ntile = 1u << f.nout;
-  const int obit = (threadIdx.x & 31) < (unsigned)f.nout ? f.obits[threadIdx.x & 31] : 0;
-  auto tile_base = [&](uint32_t tix) { return tile_base_warp(tix, f.nout, obit); };
-  auto issue = [&](uint32_t tix, float2* buf) {
-    const uint32_t tb = tile_base(tix);
-    for (uint32_t e = threadIdx.x * CH; e < tsz; e += blockDim.x * CH)
-      cp_async16(buf + e, src + (tb | hoff[e >> f.lb] | (e & lmask)));
-    cp_async_commit();
-  };
-  double accI = 0.0, accO = 0.0;
-  uint32_t tix = blockIdx.x;
-  if (tix < ntile) issue(tix, buf0);
-  int cur = 0;
-  for (; tix < ntile; tix += gridDim.x) {
-    float2* tile = cur ? buf1 : buf0;
-    const uint32_t nxt = tix + gridDim.x;
-    if (nxt < ntile) issue(nxt, cur ? buf0 : buf1);
-    else cp_async_commit();
-    cp_async_wait<1>();
-    __syncthreads();
-    float tI = 0.f, tO = 0.f;   // this thread's sums over its groups of the tile
-    for (uint32_t g = threadIdx.x; g < (tsz >> W); g += blockDim.x) {
-      const uint32_t b = local_base<W>(g, qa);
-      float2 v[C];
-#pragma unroll
-      for (int l = 0; l < C; ++l) {
-        v[l] = tile[b + offa[l]];
-        tI = fmaf(v[l].x, v[l].x, fmaf(v[l].y, v[l].y, tI));
-      }
-#pragma unroll
-      for (int r = 0; r < C; ++r) {
-        float sr = 0.f, si = 0.f;
-#pragma unroll
-        for (int c = 0; c < C; c += 2) {
-          float2 k0, k1;
-          lds_pair(&sK[r * C + c], k0, k1);
-          sr = fmaf(k0.x, v[c].x, sr);
-          sr = fmaf(-k0.y, v[c].y, sr);
-          si = fmaf(k0.x, v[c].y, si);
-          si = fmaf(k0.y, v[c].x, si);
-          sr = fmaf(k1.x, v[c + 1].x, sr);
-          sr = fmaf(-k1.y, v[c + 1].y, sr);
-          si = fmaf(k1.x, v[c + 1].y, si);
-          si = fmaf(k1.y, v[c + 1].x, si);
-        }
-        tile[b + offa[r]] = make_float2(sr, si);
-        tO = fmaf(sr, sr, fmaf(si, si, tO));
-      }
-    }
-    accI += (double)tI;
-    accO += (double)tO;
-    __syncthreads();
-    const uint32_t tb = tile_base(tix);
-    for (uint32_t e = threadIdx.x * CH; e < tsz; e += blockDim.x * CH)
-      *reinterpret_cast<float4*>(dst + (tb | hoff[e >> f.lb] | (e & lmask))) = *reinterpret_cast<const float4*>(tile + e);
-    __syncthreads();
-    cur ^= 1;
-  }
-  cp_async_wait<0>();
-  spec_finish<FIX>(f, gs, accI, 0.0, accO, 0.0, sred, &s_last, true);
 }
 
 // ---- tensor-core complex64 fused pass (tcgen05, 3xTF32, FP32 accumulation in TMEM) --------
@@ -1158,158 +986,6 @@ __global__ void __launch_bounds__(256, 2) k_fused_tc(FusedArgs f) {
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem));
   if (s_err && tid == 0) atomicOr(&f.pr.ctl->status, 1u);
   prob_finish(f.pr, accA, accN, sred, &s_last);
-}
-
-// Speculative complex64 pass on the tensor cores (QEC_C64_TC, weight-4 blocks): the order of
-// evaluation of k_apply_spec (Sec. II.B; guess = the same stabilizer's outcome one round earlier)
-// with k_fused_tc's 3xTF32 apply.  Per 4096-amplitude tile (256 groups of 16, one per thread):
-//  1. gather the thread's group from the input tile, split hi + lo in TF32 straight into tensor memory
-//     as the GEMM's A operand (the layout of k_fused_tc's probability GEMM), summing |in|^2;
-//  2. the input buffer takes the copy of the tile two ahead (two input buffers, so that two tile
-//     copies are in flight while one tile is computed);
-//  3. the apply GEMM, A from tensor memory, B (K_g / sqrt(N)) from shared memory, D in columns 0..63;
-//  4. its outputs into the updated tile in shared memory, summing |out|^2, then stored to the other
-//     working state in whole 16-byte chunks.
-// Sums in FP32 per tile, FP64 across tiles; the last CTA decides directly, as the complex64
-// probability pass does.  FIX: the corrective apply where the drawn outcome differs from g.
-// Shared memory: two input tiles and the updated tile (3 x 32 KiB) and B (8 KiB): 104 KiB, two CTAs
-// per SM; tensor memory: 256 columns per CTA.
-template <bool FIX>
-__global__ void __launch_bounds__(256, 2) k_fused_tc_spec(FusedArgs f) {
-  const int gs = spec_guess(f.ap);
-  const int m = FIX ? *f.ap.m : gs;
-  if (FIX && m == gs) return;
-  constexpr int C = 16;
-  extern __shared__ __align__(128) unsigned char tsm[];
-  const uint32_t tsz = 1u << f.nt, lmask = (1u << f.lb) - 1u;     // tsz = 4096 (checked by the launcher)
-  float2* tiles = reinterpret_cast<float2*>(tsm);                 // input tiles i even / odd
-  float2* outt = tiles + 2 * tsz;                                 // the updated tile (tile slots)
-  float* Bahi = reinterpret_cast<float*>(outt + tsz);
-  float* Balo = Bahi + 32 * 32;
-  __shared__ __align__(8) uint64_t mbar;
-  __shared__ uint32_t tmem_base;
-  __shared__ int s_err;
-  __shared__ double sred[64];
-  __shared__ int s_last;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  {
-    const double scale = f.spec_unit ? 1.0 : 1.0 / sqrt(*f.ap.N);
-    build_b(reinterpret_cast<const float2*>(f.ap.kraus) + (m ? 256 : 0), scale, Bahi, Balo, f.ap.w == 2);
-    if (tid == 0) {
-      s_err = 0;
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)));
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(&tmem_base)));
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  tc_sync();
-  const uint32_t tmem = tmem_base;
-  const uint32_t mb = smem_u32(&mbar);
-  int qa[4], qas[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    qa[j] = f.qa[j];
-    qas[j] = f.qa_s[j];
-  }
-  // tile slots and chunk offsets as in k_fused_tc
-  auto slot = [](uint32_t e) { return e ^ ((((e >> 4) ^ (e >> 7) ^ (e >> 10)) & 7u) << 1); };
-  uint32_t offa[C];
-#pragma unroll
-  for (int l = 0; l < C; ++l) offa[l] = slot(member_off<4>(l, qa));
-  uint32_t coff[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const uint32_t e = (uint32_t)tid * 2 + 512u * i, h = e >> f.lb;
-    uint32_t o = 0;
-    for (int j = 0; j < f.nt - f.lb; ++j) o |= ((h >> j) & 1u) << f.hbits[j];
-    coff[i] = o | (e & lmask);
-  }
-  const uint32_t sba = slot(local_base<4>((uint32_t)tid, qas));
-  uint32_t cd[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) cd[i] = slot((uint32_t)tid * 2 + 512u * i);
-  // Thread tid owns row tid: M-half tid / 128, TMEM lane tid % 128 (its warp's lane quarter).
-  const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-  const uint32_t taddr = tq + 32u * (warp >> 2);                 // D, this row
-  const uint32_t tA = tq + kTcColA2 + 64u * (warp >> 2);         // A of this row (hi; lo at +32)
-  const float2* src = reinterpret_cast<const float2*>(f.ap.src);
-  float2* dst = reinterpret_cast<float2*>(f.ap.dst);
-  const uint32_t ntile = 1u << f.nout;
-  double accI = 0.0, accO = 0.0;
-  uint32_t ph = 0;
-  const int obit = (threadIdx.x & 31) < (unsigned)f.nout ? f.obits[threadIdx.x & 31] : 0;
-  auto tile_base = [&](uint32_t tix) { return tile_base_warp(tix, f.nout, obit); };
-  // one commit group per call, empty past the last tile, so that wait_group<1> always means "all but
-  // the newest copy are in"
-  auto load_tile = [&](uint32_t tix, float2* buf) {
-    if (tix < ntile) {
-      const uint32_t tb = tile_base(tix);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) cp_async16(buf + cd[i], src + (tb | coff[i]));
-    }
-    cp_async_commit();
-  };
-  load_tile(blockIdx.x, tiles);
-  load_tile(blockIdx.x + gridDim.x, tiles + tsz);
-  int cur = 0;
-  for (uint32_t tix = blockIdx.x; tix < ntile; tix += gridDim.x) {
-    const uint32_t tb = tile_base(tix);
-    float2* tile = tiles + (cur ? tsz : 0u);
-    cp_async_wait<1>();
-    __syncthreads();   // this tile is in; the previous tile's readers of the updated tile are done
-    float sI = 0.f;
-#pragma unroll
-    for (int l = 0; l < C; l += 4) {
-      float hv[8], lv[8];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float2 v = tile[sba ^ offa[l + q]];
-        sI = fmaf(v.x, v.x, fmaf(v.y, v.y, sI));
-        hv[2 * q] = tf32_rna(v.x);
-        lv[2 * q] = tf32_rna(v.x - hv[2 * q]);
-        hv[2 * q + 1] = tf32_rna(v.y);
-        lv[2 * q + 1] = tf32_rna(v.y - hv[2 * q + 1]);
-      }
-      tmem_st8(tA + 2u * l, hv);
-      tmem_st8(tA + 32u + 2u * l, lv);
-    }
-    accI += (double)sI;
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    tc_sync();
-    load_tile(tix + 2 * gridDim.x, tile);   // every thread has read this tile: the copy two ahead
-    if (tid == 0) issue_gemm_ts(tmem, 0u, kTcColA2, Bahi, Balo, mb);
-    if (!mbar_wait(mb, ph & 1)) s_err = 1;
-    ++ph;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (s_err) break;
-    {
-      float d[32];
-      tmem_ld32(taddr, d);
-      float sO = 0.f;
-#pragma unroll
-      for (int r = 0; r < C; ++r) {
-        outt[sba ^ offa[r]] = make_float2(d[2 * r], d[2 * r + 1]);
-        sO = fmaf(d[2 * r], d[2 * r], fmaf(d[2 * r + 1], d[2 * r + 1], sO));
-      }
-      accO += (double)sO;
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-      *reinterpret_cast<float4*>(dst + (tb | coff[i])) = *reinterpret_cast<const float4*>(outt + cd[i]);
-    cur ^= 1;
-  }
-  cp_async_wait<0>();
-  tc_sync();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem));
-  if (s_err && tid == 0) atomicOr(&f.ap.ctl->status, 1u);
-  spec_finish<FIX>(f, gs, accI, 0.0, accO, 0.0, sred, &s_last, true);
 }
 
 // ---- complex128 passes, FP64-exact on the FP16 tensor cores (Ozaki slices) ---------------------
@@ -2253,7 +1929,8 @@ __global__ void __launch_bounds__(256) k_hist(ReadArgs a) {
   const int B = 1 << a.k1;
   const int nb = B >> 8;                 // bins per thread (B >= 256)
   const int64_t nchunk = 1ll << (a.D - a.k1);
-  const T2* src = reinterpret_cast<const T2*>(a.src);
+  const T2* src = reinterpret_cast<const T2*>(a.src) + blockIdx.y * a.src_stride;
+  double* part = a.hist_part + (size_t)blockIdx.y * a.grid_hist * B;
   double acc[16];
 #pragma unroll
   for (int j = 0; j < 16; ++j) acc[j] = 0.0;
@@ -2269,16 +1946,17 @@ __global__ void __launch_bounds__(256) k_hist(ReadArgs a) {
   }
 #pragma unroll
   for (int j = 0; j < 16; ++j)
-    if (j < nb) a.hist_part[(size_t)blockIdx.x * B + threadIdx.x + 256 * j] = acc[j];
+    if (j < nb) part[(size_t)blockIdx.x * B + threadIdx.x + 256 * j] = acc[j];
 }
 
 __global__ void __launch_bounds__(256) k_hist_reduce(ReadArgs a) {
   const int B = 1 << a.k1;
   const int bin = blockIdx.x * blockDim.x + threadIdx.x;
   if (bin >= B) return;
+  const double* part = a.hist_part + (size_t)blockIdx.y * a.grid_hist * B;
   double s = 0.0;
-  for (int c = 0; c < a.grid_hist; ++c) s += a.hist_part[(size_t)c * B + bin];
-  a.hist[bin] = s;
+  for (int c = 0; c < a.grid_hist; ++c) s += part[(size_t)c * B + bin];
+  a.hist[(size_t)blockIdx.y * B + bin] = s;
 }
 
 // Samples the bits [0, nbits) of the index over the weights w[0, n) (n = 2^nbits),
@@ -2317,25 +1995,29 @@ __global__ void __launch_bounds__(256) k_sample(ReadArgs a) {
   __shared__ double sred[64];
   __shared__ int sbit;
   const int B = 1 << a.k1;
-  const uint64_t seed = a.ctl->seed, traj = a.ctl->traj;
-  const unsigned long long t = traj - a.ctl->first;
+  // trajectory blockIdx.x of the launch: a graph's from the control word, else first, first + 1, ...
+  const uint64_t seed = a.direct ? a.seed : a.ctl->seed;
+  const uint64_t traj = a.direct ? a.first + blockIdx.x : a.ctl->traj;
+  const unsigned long long t = a.direct ? blockIdx.x : traj - a.ctl->first;
+  uint32_t flips = 0;   // the register holds data index x at x ^ flips
+  for (int r = 0; a.masks && r < a.rounds; ++r) flips ^= a.masks[(size_t)blockIdx.x * a.rounds + r];
   const uint64_t rnd = (uint64_t)a.rounds + 1;
   const int nd = a.D;   // data qubits = resident register bits
   uint8_t* bits = a.bits + t * (unsigned long long)nd;
   double tot = 0.0, dummy = 0.0;
   for (int i = threadIdx.x; i < B; i += blockDim.x) {
-    sh[i] = a.hist[i];
+    sh[i] = a.hist[(size_t)blockIdx.x * B + (i ^ (flips & (B - 1)))];
     tot += sh[i];
   }
   block_sum2(tot, dummy, sred);
-  if (threadIdx.x == 0) a.ctl->final_norm = tot;
+  if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) a.ctl->final_norm = tot;
   const int low = sample_bits(sh, a.k1, 0, seed, traj, rnd, bits, sred, &sbit);
   if (a.D > a.k1) {
     const int H = 1 << (a.D - a.k1);
-    const T2* src = reinterpret_cast<const T2*>(a.src);
+    const T2* src = reinterpret_cast<const T2*>(a.src) + blockIdx.x * a.src_stride;
     __syncthreads();
     for (int y = threadIdx.x; y < H; y += blockDim.x) {
-      const T2 v = src[((int64_t)y << a.k1) | low];
+      const T2 v = src[(((int64_t)y << a.k1) | low) ^ flips];
       sh[y] = (double)v.x * (double)v.x + (double)v.y * (double)v.y;
     }
     __syncthreads();
@@ -2347,7 +2029,7 @@ __global__ void __launch_bounds__(256) k_sample(ReadArgs a) {
     for (int c = 0; c < a.d; ++c) par ^= bits[c];   // Z_L: the first row (surface), the whole line (repetition)
     a.logical[t] = (uint8_t)par;
     for (int k = 0; k < a.nstab; ++k) a.syn[t * (unsigned long long)a.syn_stride + k] = 0;
-    a.ctl->traj = traj + 1;
+    if (!a.direct) a.ctl->traj = traj + 1;
   }
 }
 
@@ -2451,13 +2133,13 @@ cudaError_t launch_readout(int precision, const ReadArgs& a, cudaStream_t s) {
   const int B = 1 << a.k1;
   const size_t smem = sample_smem(a.D);
   if (is_f64(precision)) {
-    k_hist<double><<<a.grid_hist, 256, 0, s>>>(a);
-    k_hist_reduce<<<(B + 255) / 256, 256, 0, s>>>(a);
-    k_sample<double><<<1, 256, smem, s>>>(a);
+    k_hist<double><<<dim3(a.grid_hist, a.groups), 256, 0, s>>>(a);
+    k_hist_reduce<<<dim3((B + 255) / 256, a.groups), 256, 0, s>>>(a);
+    k_sample<double><<<a.groups, 256, smem, s>>>(a);
   } else {
-    k_hist<float><<<a.grid_hist, 256, 0, s>>>(a);
-    k_hist_reduce<<<(B + 255) / 256, 256, 0, s>>>(a);
-    k_sample<float><<<1, 256, smem, s>>>(a);
+    k_hist<float><<<dim3(a.grid_hist, a.groups), 256, 0, s>>>(a);
+    k_hist_reduce<<<dim3((B + 255) / 256, a.groups), 256, 0, s>>>(a);
+    k_sample<float><<<a.groups, 256, smem, s>>>(a);
   }
   return cudaGetLastError();
 }
@@ -2681,94 +2363,21 @@ static bool spec_args(const PassArgs& ap, double* n_next, bool unit_in, int num_
   return true;
 }
 
-// The FP64 CUDA-core speculative pass: grid-stride over groups, one wave of resident CTAs, 4 partial
-// sums per CTA.
-static bool spec_fp64_args(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, FusedArgs& f) {
-  if ((ap.w != 2 && ap.w != 4) || ap.src == ap.dst) return false;
-  f.ap = ap;
-  f.pr = ap;
-  f.n_next = n_next;
-  f.spec_unit = unit_in ? 1 : 0;
-  const void* fn = ap.w == 4 ? (const void*)k_apply_spec<4, false> : (const void*)k_apply_spec<2, false>;
-  f.grid = wave_grid(fn, 0, num_sms, ((1ll << (ap.D - ap.w)) + 255) / 256);
-  if (f.grid > MAX_PASS_GRID / 2) f.grid = MAX_PASS_GRID / 2;
-  return true;
-}
-
-// The complex64 speculative pass: k_fused's tile rule for block ap alone (low bits for 128-byte runs,
-// raised to at least 2^12 amplitudes), one wave of resident CTAs, 4 partial sums per CTA.
-static bool spec_c64_args(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, FusedArgs& f,
-                          size_t& smem) {
-  if ((ap.w != 2 && ap.w != 4) || ap.src == ap.dst) return false;
-  f.ap = ap;
-  f.pr = ap;
-  f.n_next = n_next;
-  f.spec_unit = unit_in ? 1 : 0;
-  block_tile(ap, ap, 4, 12, f);
-  smem = 2 * 8 * ((size_t)1 << f.nt) + sizeof(uint32_t) * ((size_t)1 << (f.nt - f.lb));
-  if (smem > (size_t)kFusedSmemMax) return false;
-  const void* fn = ap.w == 4 ? (const void*)k_fused_spec<4, false> : (const void*)k_fused_spec<2, false>;
-  f.grid = wave_grid(fn, smem, num_sms, 1ll << f.nout);
-  if (f.grid > MAX_PASS_GRID / 2) f.grid = MAX_PASS_GRID / 2;
-  return true;
-}
-
-// QEC_C64_TC: weight-4 blocks whose tile has 2^12 amplitudes on the tensor cores (k_fused_tc_spec, two
-// CTAs per SM), the rest as QEC_C64.
-template <bool FIX>
-static cudaError_t launch_spec_c64(int precision, const PassArgs& ap, double* n_next, bool unit_in, int num_sms,
-                                   cudaStream_t s) {
+cudaError_t launch_spec(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s) {
   FusedArgs f;
-  size_t smem = 0;
-  if (!spec_c64_args(ap, n_next, unit_in, num_sms, f, smem)) return cudaErrorInvalidValue;
-  if (precision == QEC_C64_TC && ap.w == 4 && f.nt == 12) {
-    oz_block_bits(ap.w, f.qa, f.qa_s, f.nt);
-    int64_t g = 2ll * num_sms;
-    if (g > (1ll << f.nout)) g = 1ll << f.nout;
-    if (g > MAX_PASS_GRID / 2) g = MAX_PASS_GRID / 2;
-    f.grid = (int)g;
-    k_fused_tc_spec<FIX><<<f.grid, 256, kTcSmem, s>>>(f);
-    return cudaGetLastError();
-  }
-  if (ap.w == 4) k_fused_spec<4, FIX><<<f.grid, 256, smem, s>>>(f);
-  else k_fused_spec<2, FIX><<<f.grid, 256, smem, s>>>(f);
+  if (!spec_args(ap, n_next, unit_in, num_sms, f)) return cudaErrorInvalidValue;
+  k_ozs<false><<<f.grid, 256, kOzsSmem, s>>>(f);
   return cudaGetLastError();
 }
 
-static bool spec_on_tensor_cores(int precision, const PassArgs& ap) {
-  return precision == QEC_C128_TC && apply_oz_applies(ap);
-}
-
-cudaError_t launch_spec(int precision, const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s) {
-  if (!is_f64(precision)) return launch_spec_c64<false>(precision, ap, n_next, unit_in, num_sms, s);
+cudaError_t launch_spec_fix(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s) {
   FusedArgs f;
-  if (spec_on_tensor_cores(precision, ap)) {
-    if (!spec_args(ap, n_next, unit_in, num_sms, f)) return cudaErrorInvalidValue;
-    k_ozs<false><<<f.grid, 256, kOzsSmem, s>>>(f);
-    return cudaGetLastError();
-  }
-  if (!is_f64(precision) || !spec_fp64_args(ap, n_next, unit_in, num_sms, f)) return cudaErrorInvalidValue;
-  if (ap.w == 4) k_apply_spec<4, false><<<f.grid, 256, 0, s>>>(f);
-  else k_apply_spec<2, false><<<f.grid, 256, 0, s>>>(f);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_spec_fix(int precision, const PassArgs& ap, double* n_next, bool unit_in, int num_sms,
-                            cudaStream_t s) {
-  if (!is_f64(precision)) return launch_spec_c64<true>(precision, ap, n_next, unit_in, num_sms, s);
-  FusedArgs f;
-  if (spec_on_tensor_cores(precision, ap)) {
-    if (!spec_args(ap, n_next, unit_in, num_sms, f)) return cudaErrorInvalidValue;
-    PassArgs a = ap;
-    a.store_n = 0;   // *N keeps the scale both applies of this block use
-    cudaError_t e = launch_oz(OZ_PROB, true, a, num_sms, s);
-    if (e != cudaSuccess) return e;
-    k_ozs<true><<<f.grid, 256, kOzsSmem, s>>>(f);
-    return cudaGetLastError();
-  }
-  if (!is_f64(precision) || !spec_fp64_args(ap, n_next, unit_in, num_sms, f)) return cudaErrorInvalidValue;
-  if (ap.w == 4) k_apply_spec<4, true><<<f.grid, 256, 0, s>>>(f);
-  else k_apply_spec<2, true><<<f.grid, 256, 0, s>>>(f);
+  if (!spec_args(ap, n_next, unit_in, num_sms, f)) return cudaErrorInvalidValue;
+  PassArgs a = ap;
+  a.store_n = 0;   // *N keeps the scale both applies of this block use
+  cudaError_t e = launch_oz(OZ_PROB, true, a, num_sms, s);
+  if (e != cudaSuccess) return e;
+  k_ozs<true><<<f.grid, 256, kOzsSmem, s>>>(f);
   return cudaGetLastError();
 }
 
@@ -2810,15 +2419,8 @@ cudaError_t setup_kernels(int precision, int D) {
   }
   cudaError_t e = cudaFuncSetAttribute(k_sample<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess) e = fused_attrs<float>();
-  for (const void* fn : {(const void*)k_fused_spec<2, false>, (const void*)k_fused_spec<2, true>,
-                         (const void*)k_fused_spec<4, false>, (const void*)k_fused_spec<4, true>}) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedSmemMax);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  }
-  for (const void* fn : {(const void*)k_fused_tc, (const void*)k_fused_tc_spec<false>, (const void*)k_fused_tc_spec<true>}) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedSmemMax);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  }
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)k_fused_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedSmemMax);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)k_fused_tc, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   return e;
 }
 

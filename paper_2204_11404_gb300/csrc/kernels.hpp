@@ -106,6 +106,12 @@ struct ReadArgs {
   uint8_t* syn;           // [traj][syn_stride]; round-0 row zeroed here
   int syn_stride;
   int nstab;
+  // Several trajectories at once: group g's state at src + g src_stride amplitudes, its outputs at row g.
+  int groups = 1;
+  size_t src_stride = 0;
+  int direct = 0;                   // 1: trajectories first, first + 1, ... of `seed` (else the control word's)
+  unsigned long long seed = 0, first = 0;
+  const uint32_t* masks = nullptr;  // [groups][rounds]: the register's index flips per round (null: none)
 };
 
 cudaError_t launch_instantiate(int precision, const InstArgs& a, cudaStream_t s);
@@ -129,17 +135,13 @@ bool fused_oz_applies(const PassArgs& ap, const PassArgs& pr);
 cudaError_t launch_fused_oz(const PassArgs& ap, const PassArgs& pr, int num_sms, cudaStream_t s);
 // The exact probability launch of block pr after a fused pass (returns at once unless needed).
 cudaError_t launch_prob_oz_check(const PassArgs& pr, int num_sms, cudaStream_t s);
-// Speculative complex128 pass of block ap (ap.src and ap.dst distinct buffers): applies K_g / sqrt(*ap.N)
-// (scale 1 with unit_in) for the guessed outcome g, decides the outcome (on the tensor cores where
-// its bound allows), and stores |output|^2 in *n_next (n_next may be null).  QEC_C128_TC blocks whose
-// tile fits (apply_oz_applies) run on the tensor cores, every other complex128 block on the FP64
-// CUDA cores; QEC_C64_TC weight-4 blocks whose tile has 2^12 amplitudes on the tensor cores (3xTF32),
-// every other complex64 block on the FP32 CUDA cores (shared-memory tiles).
-cudaError_t launch_spec(int precision, const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s);
-// Its completion: on the tensor cores the exact probability launch (returns at once unless the bound
-// left the outcome open); then the corrective apply (returns at once unless the outcome is not g).
-cudaError_t launch_spec_fix(int precision, const PassArgs& ap, double* n_next, bool unit_in, int num_sms,
-                            cudaStream_t s);
+// Speculative complex128 pass on the tensor cores of block ap (ap.src and ap.dst distinct buffers): applies
+// K_g / sqrt(*ap.N) (scale 1 with unit_in) for the guessed outcome g, decides the outcome where its
+// bound allows, and stores |output|^2 in *n_next (n_next may be null).
+cudaError_t launch_spec(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s);
+// Its completion: the exact probability launch (returns at once unless the bound left the outcome
+// open), then the corrective apply (returns at once unless the outcome is not g).
+cudaError_t launch_spec_fix(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s);
 int pass_grid(int D, int w, int num_sms);
 // One wave of resident CTAs for the probability (prob = true) or apply pass kernel.
 int pass_grid_for(int precision, bool prob, int D, int w, int num_sms);
