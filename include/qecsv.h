@@ -244,9 +244,9 @@ typedef struct qec_batch qec_batch;
 /*
  * Batched simulator for the d = 3 delayed-measurement register (9 data qubits
  * + reused ancilla, Sec. II.B), `rounds` noisy rounds, gate set `gates`.
- * One warp runs one trajectory in shared memory; a single graph-captured
- * persistent kernel processes a whole batch, taking trajectories from a
- * device work counter.  max_traj bounds n of every run.  Only d = 3 is
+ * A trajectory runs on chip, its blocks as rotations and diagonals: one warp
+ * each in a persistent launch that takes trajectories from a device work
+ * counter, or one CTA each where there are at most four per SM.  max_traj bounds n of every run.  Only d = 3 is
  * accepted (QEC_EUNSUPPORTED otherwise).  cuda_stream as in qec_create.
  */
 qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t max_traj, void* cuda_stream,
@@ -256,10 +256,11 @@ qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t m
  * Run n trajectories (Sec. III.B protocol, as qec_run_trajectories), each with
  * its own trajectory index traj[i], kind[i] = precision (QEC_C128 or QEC_C64)
  * + 2 * layout, and noise parameters noise[i] (Sec. III.A).  Layout
- * QEC_LAYOUT_REDUCED runs the 10-qubit delayed register (one warp, Sec. II.B);
- * QEC_LAYOUT_UNREDUCED runs all 17 qubits time-ordered, every ancilla of a part
- * active at once (one CTA; the other part's ancillas are |0>, so a
- * 2^13-amplitude slab holds the exact state).  Inputs and outputs are HOST
+ * QEC_LAYOUT_REDUCED runs the 10-qubit delayed register (Sec. II.B);
+ * QEC_LAYOUT_UNREDUCED runs all 17 qubits, every ancilla of a part active at
+ * once and measured at the part's end (one CTA; the other part's ancillas are
+ * |0>, so a 2^13-amplitude slab holds the exact state; each qubit meets its
+ * gates in time order).  Inputs and outputs are HOST
  * arrays: syndromes [n][rounds+1][8], data_bits [n][9], raw_logical [n] (any
  * output may be NULL).  Trajectory i equals qec_run_trajectories for
  * (noise[i], kind[i], seed, traj[i]).  Blocks until the outputs are on the host.
@@ -272,9 +273,8 @@ qec_status qec_batch_run(qec_batch* b, uint64_t seed, uint32_t n, const uint64_t
  * configuration of each engine, each timed on the sample's trajectories of its
  * register: the reduced-register engine's CTA shape (warps per CTA, one
  * resident wave per SM), then the unreduced engine's fusion width k (2..6 slab
- * bits per pass: consecutive gate units on disjoint bits, which commute, are
- * applied in one pass over the 2^13-amplitude slab) and threads per CTA (128,
- * 256).  *chosen_warps gets the reduced engine's warps per CTA, *best_ms the
+ * bits per sweep: above 4 a weight-4 stabilizer's four data qubits are rotated
+ * in one sweep, else two at a time) and threads per CTA (128, 256).  *chosen_warps gets the reduced engine's warps per CTA, *best_ms the
  * device time of the whole sample with the chosen configuration;
  * qec_batch_config reports all three choices.
  */
@@ -324,9 +324,9 @@ qec_status qec_debug_program(const qec_params* params, int32_t* ops, uint32_t ca
                              int32_t* block_info, uint32_t block_cap, uint32_t* n_blocks);
 
 /*
- * Host-only test hook (no GPU needed): the batched form's plan for one round
- * of the unreduced 17-qubit register (d = 3, gate set `gates`, every noise
- * site present), at fusion width k.  items: int32 quadruples (kind 0 = unit /
+ * Host-only hook (no GPU needed): a time-ordered gate plan for one round of
+ * the unreduced 17-qubit register (d = 3, gate set `gates`, every noise site
+ * present) in passes of at most k slab bits.  items: int32 quadruples (kind 0 = unit /
  * 1 = measurement, qubits 1 or 2, slab bit qa, slab bit qb or -1) in
  * execution order, *n_items of them.  pass_units: the unit items the passes
  * apply, in order (*n_pass_units).  absorbs: int32 triples (one-qubit item,

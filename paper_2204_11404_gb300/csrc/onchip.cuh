@@ -84,6 +84,16 @@ __device__ __forceinline__ void group_sum2(double& a, double& b, double* red, in
   b = __shfl_sync(0xffffffffu, v, 16);
 }
 
+// The register's scale is free (a probability is a ratio of sums over one state): where the kept part's
+// norm gets small, an exact power of two brings it back into range.
+__device__ __forceinline__ int norm_exp(double a) { return (int)((__double_as_longlong(a) >> 52) & 0x7FF) - 1023; }
+__device__ __forceinline__ bool small_norm(double a) { return norm_exp(a) < -20; }
+template <typename T>
+__device__ __forceinline__ T norm_scale(double a) {
+  const int e = norm_exp(a);
+  return (T)__longlong_as_double((long long)(1023 + (-(e < -1022 ? -1022 : e) >> 1)) << 52);
+}
+
 // A compiled block in shared memory.
 template <typename T>
 struct Compiled {
@@ -95,11 +105,11 @@ struct Compiled {
   uint8_t form[4];  // the rotations' forms
 };
 
-// One block on the group's register psi (2^D = 4 NT ITEMS amplitudes); returns the raw outcome.
-// red: 64 doubles (NT > 32), alternated between calls by `parity`.
+// One block on the group's register psi (2^D = 4 NT ITEMS amplitudes); returns the raw outcome (drawn, or
+// `forced` where that is not negative).  red: 64 doubles (NT > 32), alternated between calls by `parity`.
 template <typename T, int NT, int ITEMS>
 __device__ __forceinline__ int run_block(typename V2t<T>::t* psi, const FBlock& B, const Compiled<T>& C, double* red,
-                                         int parity, int rank) {
+                                         int parity, int rank, int forced = -1) {
   using T2 = typename V2t<T>::t;
   T2 v[ITEMS][4];
   uint32_t at[ITEMS];
@@ -155,13 +165,10 @@ __device__ __forceinline__ int run_block(typename V2t<T>::t* psi, const FBlock& 
   }
   double A0 = (double)s0, A1 = (double)s1;
   group_sum2<NT>(A0, A1, red + (parity & 1) * 64, rank);
-  const int m = C.u * (A0 + A1) < A1 ? 1 : 0;
+  const int m = forced >= 0 ? forced : C.u * (A0 + A1) < A1 ? 1 : 0;
   const double A = m ? A1 : A0;
-  // the register's scale is free (a probability is a ratio of sums over one state): an exact power of
-  // two keeps it in range
-  const int e = (int)((__double_as_longlong(A) >> 52) & 0x7FF) - 1023;
-  const bool rescale = e < -20;
-  const T sc = (T)__longlong_as_double((long long)(1023 + (-(e < -1022 ? -1022 : e) >> 1)) << 52);
+  const bool rescale = small_norm(A);
+  const T sc = norm_scale<T>(A);
   const uint32_t ma = 1u << qa, mb = 1u << qb;
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i)
