@@ -65,8 +65,12 @@ struct qec_sim {
   double fm[FM_COUNT][4][2] = {};
   // factored passes (rounds.cu): up to r_groups trajectories of r_G CTAs each
   int r_groups = 0, r_G = 0;
-  std::vector<ChainDesc> chains;
-  ChainDesc* d_chains = nullptr;
+  std::vector<ChainDesc> chains, small_chains;
+  ChainDesc* d_chains = nullptr;        // chains, then small_chains
+  int small_ctas = 0;                   // with small tiles: at most this many CTAs (0: never)
+  std::vector<DiagDesc> diags;
+  DiagDesc* d_diags = nullptr;
+  int n_x = 0;                          // blocks of X stabilizers (a round's first)
   void* d_cblocks = nullptr;
   unsigned char* d_scratch = nullptr;
   uint32_t* d_masks = nullptr;
@@ -273,23 +277,38 @@ PassArgs spec_pass(const qec_sim* s, int b) {
 
 // Registers of up to 13 qubits run whole trajectories on chip (onchip.cu), one SM each, unless the
 // passes that compute each probability first were asked for.  2^13 complex128 amplitudes are enough
-// FP64 work for one or two trajectories to be faster as passes over the whole GPU (three rounds of the
-// repetition code: 1.45 ms on one SM, 0.74 ms per trajectory in passes; 16 trajectories 1.46 and 10.9 ms).
+// FP64 work for few trajectories to be faster in passes over all SMs (five rounds of the repetition
+// code, 1, 32 and 64 trajectories: 2.2 ms each on chip, 0.69, 0.95 and 1.83 ms in passes).
 bool on_chip(const qec_sim* s, uint32_t n) {
-  return s->spec && onchip_applies(s->D) && (s->D < 13 || !is_f64(s->p.precision) || n >= 3);
+  return s->spec && onchip_applies(s->D) && (s->D < 13 || !is_f64(s->p.precision) || n > 64);
 }
 
-// Everything else runs in factored passes (rounds.cu), but for the tensor-core complex128 form on large
-// registers, where its dense slices beat the FP64 pipe (five rounds of the repetition code, 25 qubits:
-// 47.0 and 52.1 ms, 21 qubits: 5.1 and 6.2, 17 qubits: 2.0 and 0.89).
 // Blocks per pass.  complex64 passes are bound by memory and shared-memory sweeps: four blocks share a
 // read and a write.  complex128 ones are bound by the FP64 pipe, where a pass that runs again costs
 // all its blocks: one block each on large registers (d = 5, five rounds: 94.8, 101, 107, 112 ms for 1 to
 // 4); on small ones the barrier between passes counts (17 qubits: 1.25, 1.01, 0.94, 0.89 ms).
 int chain_limit(const qec_params& p, int D) { return is_f64(p.precision) && D > 21 ? 1 : 4; }
-bool rounds_apply(const qec_params& p, int D) {
-  if (D < 13 || (D == 13 && !is_f64(p.precision))) return false;   // on chip
-  return p.precision != QEC_C128_TC || D < 21;
+
+// Registers from here on are large enough that passes, not launches and barriers, take the time: a launch
+// per round and part, and the Z part in diagonal passes.
+constexpr int kLargeD = 21;
+
+// The factored engines (rounds.cu) have this register's buffers.
+bool rounds_size(const qec_params& p, int D) { return D > 13 || (D == 13 && is_f64(p.precision)); }
+
+// No touch of any block rotates: no X stabilizers, and the round-start terms are diagonal.
+bool all_diagonal(const qec_sim* s) {
+  const double (*m)[2] = s->fm[FM_ROUND];
+  return s->n_x == 0 && m[1][0] == 0.0 && m[1][1] == 0.0 && m[2][0] == 0.0 && m[2][1] == 0.0;
+}
+
+// Everything that is not on chip runs in factored passes.  The tensor-core complex128 form keeps its dense
+// slices on large registers for blocks that rotate (0.39 ms a block at 25 qubits; rotations and diagonals
+// on the FP64 pipe 0.75): the X part of the surface code, and the repetition code with round-start
+// rotations, which runs as before.
+bool rounds_apply(const qec_sim* s) {
+  if (!s->spec || !rounds_size(s->p, s->D)) return false;
+  return s->p.precision != QEC_C128_TC || s->D < kLargeD || s->n_x > 0 || all_diagonal(s);
 }
 
 // The state that a trajectory's graph ends in (the init state when there are no noisy rounds).
@@ -440,7 +459,7 @@ void drop_graph(qec_sim* s) {
 void free_all(qec_sim* s) {
   drop_graph(s);
   if (s->h_out) cudaFreeHost(s->h_out);
-  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_factor, s->d_chains, s->d_cblocks, s->d_scratch, s->d_masks,
+  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_factor, s->d_chains, s->d_diags, s->d_cblocks, s->d_scratch, s->d_masks,
                   s->d_norm, s->d_rparts, s->d_bar, s->d_kraus, s->d_u, s->d_A, s->d_N, s->d_m, s->d_partials, s->d_ctl,
                   s->d_hist_part, s->d_hist, s->d_syn, s->d_bits, s->d_log, s->d_events,
                   s->d_ops[0], s->d_ops[1], s->d_blocks[0], s->d_blocks[1], s->d_mats[0], s->d_mats[1]};
@@ -492,19 +511,25 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   const int k1 = hist_k1(s->D);
   s->spec = true;
   s->r_groups = 1;
-  if (rounds_apply(s->p, s->D)) {
+  if (rounds_size(s->p, s->D)) {
     if ((e = setup_rounds(s->p.precision)) != cudaSuccess)
       return bail(fail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e)));
-    const int wave = round_wave(s->p.precision, s->num_sms), tiles = round_ctas(s->D);
+    const bool early = s->D >= kLargeD && !s->init_prog.blocks.empty() && s->p.code == QEC_CODE_SURFACE;
+    const int wave = round_wave(s->p.precision, kTileBits, early, s->num_sms), tiles = 1 << (s->D - kTileBits);
+    // Small tiles while they leave the GPU far from full (five rounds of the repetition code, small and
+    // large tiles: 15 qubits complex128, 8 trajectories = 512 CTAs: 0.72 and 0.94 ms, 32: 2.74 and 2.63;
+    // 17 qubits complex64, 1 = 256 CTAs: 0.33 and 0.43, 3: 0.69 and 0.50)
+    if (s->p.code == QEC_CODE_REPETITION && s->D < kLargeD)
+      s->small_ctas = std::min(512, round_wave(s->p.precision, kSmallTileBits, false, s->num_sms));
     if (wave < 1) return bail(fail(QEC_ECUDA, "the factored pass does not fit an SM"));
     s->r_G = std::min(wave, tiles);
-    s->r_groups = s->D == 13 ? 2 : wave / s->r_G;   // trajectories side by side where one does not fill the GPU
+    s->r_groups = s->D == 13 ? 32 : wave / s->r_G;   // trajectories side by side where one does not fill the GPU
   }
   const size_t groups = (size_t)s->r_groups;
   if ((st = dmalloc(&s->psi2, state_bytes * groups)) || (st = dmalloc(&s->psi, state_bytes * groups)) || (st = dmalloc(&s->psi0, state_bytes)) ||
       (st = dmalloc(&s->d_kraus, (size_t)nblk * KRAUS_STRIDE * s->amp)) ||
       (st = dmalloc(&s->d_u, sizeof(double) * nblk)) || (st = dmalloc(&s->d_A, sizeof(double) * nblk)) ||
-      (st = dmalloc(&s->d_N, sizeof(double) * nblk)) || (st = dmalloc(&s->d_m, sizeof(int) * nblk)) ||
+      (st = dmalloc(&s->d_N, sizeof(double) * (nblk + 1))) || (st = dmalloc(&s->d_m, sizeof(int) * nblk)) ||
       (st = dmalloc(&s->d_partials, sizeof(double) * 2 * MAX_PASS_GRID)) ||
       (st = dmalloc(&s->d_ctl, sizeof(Ctl))) ||
       (st = dmalloc(&s->d_hist_part, sizeof(double) * groups * ((size_t)hist_grid(s->D, s->num_sms) << k1))) ||
@@ -522,20 +547,32 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   if ((st = upload_program(s, 0, s->init_prog)) || (st = upload_program(s, 1, s->prog))) return bail(st);
   size_t scratch = 0;
   if ((st = alloc_factor(s, &scratch)) || (st = upload_factor(s))) return bail(st);
-  if (rounds_apply(s->p, s->D)) {
-    s->chains = plan_chains(s->fprog, s->p.precision, chain_limit(s->p, s->D));
+  while (s->n_x < s->nstab && !s->fprog.blocks[s->n_x].z_type) ++s->n_x;
+  if (rounds_size(s->p, s->D)) {
+    const bool large = s->D >= kLargeD;
+    s->chains = plan_chains(s->fprog, s->p.precision, kTileBits, chain_limit(s->p, s->D), 0,
+                            large && s->n_x ? s->n_x : s->nstab);
+    if (s->small_ctas)
+      s->small_chains = plan_chains(s->fprog, s->p.precision, kSmallTileBits, kMaxChain, 0, s->nstab);
+    if (large) s->diags = plan_diagonals(s->fprog, s->p.precision, s->n_x, s->nstab);
     const size_t nr = groups * kMaxRounds;
-    if ((st = dmalloc(&s->d_chains, sizeof(ChainDesc) * s->chains.size())) ||
+    if ((st = dmalloc(&s->d_chains, sizeof(ChainDesc) * (s->chains.size() + s->small_chains.size()))) ||
         (st = dmalloc(&s->d_cblocks, nr * s->nstab * compiled_block_bytes(s->p.precision))) ||
         (st = dmalloc(&s->d_scratch, nr * scratch)) || (st = dmalloc(&s->d_masks, nr * sizeof(uint32_t))) ||
         (st = dmalloc(&s->d_norm, groups * sizeof(double))) ||
-        (st = dmalloc(&s->d_rparts, 2 * groups * s->r_G * kMaxChain * sizeof(double))) ||
+        (st = dmalloc(&s->d_diags, sizeof(DiagDesc) * (s->diags.size() + 1))) ||
+        (st = dmalloc(&s->d_rparts, 2 * (groups * s->r_G + 512 + s->num_sms) * (kMaxDiag + 1) * sizeof(double))) ||
         (st = dmalloc(&s->d_bar, 2 * groups * sizeof(unsigned int))))
       return bail(st);
     e = cudaMemsetAsync(s->d_bar, 0, 2 * groups * sizeof(unsigned int), s->work);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(s->d_chains, s->chains.data(), sizeof(ChainDesc) * s->chains.size(), cudaMemcpyHostToDevice,
                           s->work);
+    if (e == cudaSuccess && !s->small_chains.empty())
+      e = cudaMemcpyAsync(s->d_chains + s->chains.size(), s->small_chains.data(),
+                          sizeof(ChainDesc) * s->small_chains.size(), cudaMemcpyHostToDevice, s->work);
+    if (e == cudaSuccess && !s->diags.empty())
+      e = cudaMemcpyAsync(s->d_diags, s->diags.data(), sizeof(DiagDesc) * s->diags.size(), cudaMemcpyHostToDevice, s->work);
     if (e != cudaSuccess) return bail(fail(QEC_ECUDA, cudaGetErrorString(e)));
   }
   if (onchip_applies(s->D)) {
@@ -607,20 +644,31 @@ qec_status run_onchip(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uin
   return QEC_OK;
 }
 
-// A batch of `chunk` trajectories from `first` on, in factored passes, into the device output batch:
-// r_groups of them side by side, a launch per round (larger registers: other streams' work gets in
-// between) or for all rounds.
+// A batch of `chunk` trajectories from `first` on, in factored passes, into the device output batch: small
+// registers r_groups of them side by side with all rounds in one launch, large ones one by one with a
+// launch per round and part (other streams' work gets in between).
 qec_status run_rounds(qec_sim* s, uint64_t seed, uint64_t first, uint32_t chunk) {
+  const bool large = s->D >= kLargeD, f64 = is_f64(s->p.precision);
+  const bool tensor = large && s->p.precision == QEC_C128_TC && s->n_x > 0;   // the X part's dense blocks
   RoundArgs a;
   a.F = device_factor(s);
+  a.F.early = large && s->n_x > 0;
   for (int i = 0; i < PR_COUNT; ++i) a.thr[i] = fac::draw_threshold(s->prog.prob[i]);
   std::memcpy(a.fm, s->fm, sizeof(a.fm));
   a.seed = seed;
-  a.G = s->r_G;
+  const uint32_t side = std::min<uint32_t>((uint32_t)s->r_groups, chunk);
+  const bool small = s->small_ctas && ((uint64_t)side << (s->D - kSmallTileBits)) <= (uint64_t)s->small_ctas;
+  a.tb = small ? kSmallTileBits : kTileBits;
+  a.G = small ? 1 << (s->D - kSmallTileBits) : s->r_G;
   a.D = s->D;
   a.rounds = s->R;
-  a.chains = s->d_chains;
-  a.nc = (int)s->chains.size();
+  a.chains = s->d_chains + (small ? s->chains.size() : 0);
+  a.diags = s->d_diags;
+  const bool diagonal = large && all_diagonal(s);
+  a.nc = diagonal ? 0 : tensor ? s->n_x : (int)(small ? s->small_chains : s->chains).size();
+  a.nd = diagonal || a.F.early ? (int)s->diags.size() : 0;
+  a.steps = a.nc + a.nd;
+  a.step0 = a.nc;
   a.psi0 = s->psi0;
   a.buf[0] = s->psi;
   a.buf[1] = s->psi2;
@@ -628,40 +676,63 @@ qec_status run_rounds(qec_sim* s, uint64_t seed, uint64_t first, uint32_t chunk)
   a.scratch = s->d_scratch;
   a.masks = s->d_masks;
   a.norm = s->d_norm;
+  // the tensor-core passes keep a norm per block
+  a.diag_in = tensor ? s->d_N + s->n_x : nullptr;
+  a.diag_out = tensor ? s->d_N + s->nstab : nullptr;
+  a.diag_stride = tensor ? s->nstab : 0;
   a.partials = s->d_rparts;
   a.bar = s->d_bar;
   a.ctl = s->d_ctl;
   a.events = s->ev_cap ? s->d_events : nullptr;
   ReadArgs r = read_args(s);
-  r.direct = 1;
+  r.direct = tensor ? 0 : 1;   // (those take their trajectory from the control word, which the readout advances)
   r.seed = seed;
   if (s->R > 0) {
-    r.src = ((s->R * a.nc - 1) & 1) ? s->psi2 : s->psi;
+    r.src = ((s->R * a.steps - 1) & 1) ? s->psi2 : s->psi;
     r.src_stride = (size_t)1 << s->D;
     r.masks = s->d_masks;
   }
-  const int per = s->D >= 21 ? 1 : std::max(s->R, 1);   // rounds per launch
-  const int timed = s->timed_block < 0 ? 0 : 1 + s->timed_block / s->nstab;
+  const int prec = f64 ? QEC_C128 : QEC_C64;
+  const int per = large ? 1 : std::max(s->R, 1);   // rounds per launch
+  const int tb = s->timed_block, timed = tb < 0 ? 0 : 1 + tb / s->nstab;
+  qec_status st = QEC_OK;
+  auto record3 = [&]() {
+    for (int i = 0; i < 2 && st == QEC_OK; ++i)
+      if (cudaEventRecord(s->kev[i], s->work) != cudaSuccess) st = fail(QEC_ECUDA, "event record");
+  };
   for (uint32_t t = 0; t < chunk; t += (uint32_t)a.groups) {
     a.groups = (int)std::min<uint32_t>((uint32_t)s->r_groups, chunk - t);
     a.first = first + t;
     a.syn = s->d_syn + (size_t)t * s->syn_stride();
-    if (s->R > 0) QEC_CUDA(launch_compile(s->p.precision, a, s->work));
+    if (s->R > 0) QEC_CUDA(launch_compile(prec, a, s->work));
+    if (s->R > 0 && tensor) QEC_CUDA(launch_dense(a, s->n_x, s->d_kraus, s->d_u, s->work));
     for (int r0 = 1; r0 <= s->R; r0 += per) {
       const int r1 = std::min(s->R, r0 + per - 1);
-      const bool tm = t == 0 && timed >= r0 && timed <= r1;
-      if (tm) {
-        QEC_CUDA(cudaEventRecord(s->kev[0], s->work));
-        QEC_CUDA(cudaEventRecord(s->kev[1], s->work));
+      bool tm = t == 0 && timed >= r0 && timed <= r1;
+      const bool block = tensor && tb % s->nstab < s->n_x;   // the instrumented block has a pass of its own
+      if (tm && !block) record3();
+      for (int b = 0; b < s->n_x && tensor; ++b) {
+        const int k = (r0 - 1) * s->nstab + b, step = (r0 - 1) * a.steps + b;
+        PassArgs p = spec_pass(s, k);
+        p.src = step == 0 ? s->psi0 : a.buf[(step & 1) ^ 1];
+        p.dst = a.buf[step & 1];
+        if (tm && block && k == tb) record3();
+        QEC_CUDA(launch_spec(p, s->d_N + k + 1, step == 0, s->num_sms, s->work));
+        if (tm && block && k == tb) QEC_CUDA(cudaEventRecord(s->kev[2], s->work));
+        QEC_CUDA(launch_spec_fix(p, s->d_N + k + 1, step == 0, s->num_sms, s->work));
       }
-      QEC_CUDA(launch_rounds(s->p.precision, a, r0, r1, s->work));
-      if (tm) QEC_CUDA(cudaEventRecord(s->kev[2], s->work));
+      if (a.nc && !tensor) QEC_CUDA(launch_rounds(prec, a, r0, r1, s->work));
+      if (a.nd) QEC_CUDA(launch_diagonals(prec, a, r0, s->num_sms, s->work));
+      if (tm && !block) QEC_CUDA(cudaEventRecord(s->kev[2], s->work));
+      if (st) return st;
     }
     r.groups = a.groups;
     r.first = a.first;
-    r.syn = a.syn;
-    r.bits = s->d_bits + (size_t)t * s->D;
-    r.logical = s->d_log + t;
+    if (!tensor) {
+      r.syn = a.syn;
+      r.bits = s->d_bits + (size_t)t * s->D;
+      r.logical = s->d_log + t;
+    }
     QEC_CUDA(launch_readout(s->p.precision, r, s->work));
   }
   s->last_state = static_cast<const char*>(r.src) + (size_t)(a.groups - 1) * r.src_stride * s->amp;
@@ -672,7 +743,7 @@ qec_status run_rounds(qec_sim* s, uint64_t seed, uint64_t first, uint32_t chunk)
 qec_status run_impl(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8_t* syn, uint8_t* bits,
                     uint8_t* logical, bool host_out) {
   if (!s) return fail(QEC_EINVAL, "null handle");
-  const bool oc = on_chip(s, n), rd = !oc && s->spec && rounds_apply(s->p, s->D);
+  const bool oc = on_chip(s, n), rd = !oc && rounds_apply(s);
   qec_status st = oc || rd ? QEC_OK : ensure_graph(s);
   if (st) return st;
   if (s->user) {

@@ -13,6 +13,10 @@
 // round what remains on a qubit is a phase per value and a flip: both go into that block's diagonal
 // and F.  So the diagonal of block b for outcome m, as the passes use it, is
 //   D_m(z ^ f) prod_j lu_j(z_j) rw_j(z_j),  lu from the block's own touches, rw from the next ones.
+// FactorView::early: the rotations between a qubit's last X and first Z stabilizer of a round run in the
+// X stabilizer's pass, after its diagonal (their cosines then belong to that diagonal).  No later touch
+// of a Z stabilizer rotates (between them a qubit meets diagonal matrices and Paulis only), so the Z
+// part of a round is diagonal.
 #pragma once
 #include <math.h>
 #include <string.h>
@@ -228,6 +232,12 @@ QEC_HD int touch_merge(const FactorView& F, int t, Touch* T) {
 // times diagonal matrices: its zeros are exact).
 QEC_HD int touch_end_swap(const Touch& T) { return is_zero(T.post.a[0].x) && is_zero(T.post.a[0].y) ? 1 : 0; }
 
+// Whether touch t's rotation runs in the block of the qubit's previous touch.
+QEC_HD bool runs_early(const FactorView& F, int t) {
+  const int pv = F.touches[t].prev;
+  return F.early && pv >= 0 && F.blocks[t >> 2].z_type && !F.blocks[pv >> 2].z_type;
+}
+
 // Stage 3: rotation of touch t from G, the flips f' before and f after it; lu and the previous
 // touch's rw (or, at a round's last touch, its own rw from what remains on the qubit).
 QEC_HD double2 touch_rotation(const FactorView& F, int t, Touch* T, int f_before, int f_after) {
@@ -269,8 +279,16 @@ QEC_HD double2 touch_rotation(const FactorView& F, int t, Touch* T, int f_before
   }
   const double k = rsqrt_d(n00 * n10);
   tt.x = n10 * k;
-  lu[1] = c2(m.a[2].x * (n00 * k), m.a[2].y * (n00 * k));
   const double2 w = cmulc(m.a[3], m.a[2]);
+  if (runs_early(F, t)) {         // lu = u, the cosine in rw
+    const double c0 = rsqrt_d(n00), s0 = n00 * k * c0, c = n00 * c0;
+    lu[0] = c2(m.a[0].x * c0, m.a[0].y * c0);
+    lu[1] = c2(m.a[2].x * s0, m.a[2].y * s0);
+    T[pv].rw[0] = c2(c, 0.0);
+    T[pv].rw[1] = c2(w.x * (k * c), w.y * (k * c));
+    return tt;
+  }
+  lu[1] = c2(m.a[2].x * (n00 * k), m.a[2].y * (n00 * k));
   T[pv].rw[1] = c2(w.x * k, w.y * k);
   return tt;
 }

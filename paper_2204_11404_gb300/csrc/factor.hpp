@@ -80,6 +80,7 @@ struct FactorView {
   const FBlock* blocks;
   const uint16_t* order;
   int nsites, nstab, nd, n_touch, n_x;
+  int early = 0;   // see factor.cuh
 };
 
 inline FactorView view_of(const FactorProgram& F) {

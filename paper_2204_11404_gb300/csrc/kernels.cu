@@ -1940,7 +1940,7 @@ __global__ void __launch_bounds__(256) k_hist(ReadArgs a) {
     for (int j = 0; j < 16; ++j) {
       if (j < nb) {
         const T2 v = src[base + threadIdx.x + 256 * j];
-        acc[j] += (double)v.x * (double)v.x + (double)v.y * (double)v.y;
+        acc[j] = fma((double)v.x, (double)v.x, fma((double)v.y, (double)v.y, acc[j]));
       }
     }
   }
@@ -1949,51 +1949,55 @@ __global__ void __launch_bounds__(256) k_hist(ReadArgs a) {
     if (j < nb) part[(size_t)blockIdx.x * B + threadIdx.x + 256 * j] = acc[j];
 }
 
+// 32 bins per CTA, eight threads each over the partial histograms.
 __global__ void __launch_bounds__(256) k_hist_reduce(ReadArgs a) {
-  const int B = 1 << a.k1;
-  const int bin = blockIdx.x * blockDim.x + threadIdx.x;
-  if (bin >= B) return;
+  __shared__ double part_sum[8][32];
+  const int B = 1 << a.k1, lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+  const int bin = blockIdx.x * 32 + lane;
   const double* part = a.hist_part + (size_t)blockIdx.y * a.grid_hist * B;
   double s = 0.0;
-  for (int c = 0; c < a.grid_hist; ++c) s += part[(size_t)c * B + bin];
-  a.hist[(size_t)blockIdx.y * B + bin] = s;
+  if (bin < B)
+    for (int c = seg; c < a.grid_hist; c += 8) s += part[(size_t)c * B + bin];
+  part_sum[seg][lane] = s;
+  __syncthreads();
+  if (seg == 0 && bin < B) {
+    for (int i = 1; i < 8; ++i) s += part_sum[i][lane];
+    a.hist[(size_t)blockIdx.y * B + bin] = s;
+  }
 }
 
-// Samples the bits [0, nbits) of the index over the weights w[0, n) (n = 2^nbits),
-// qubit-by-qubit; bit j of the result goes to out_bits[bit_base + j].
-__device__ int sample_bits(const double* w, int nbits, int bit_base, uint64_t seed, uint64_t traj,
-                           uint64_t rnd, uint8_t* out_bits, double* sred, int* sbit) {
-  const int n = 1 << nbits;
-  int prefix = 0;
-  for (int j = 0; j < nbits; ++j) {
-    const int mask = (1 << j) - 1;
-    double s_all = 0.0, s_one = 0.0;
-    for (int x = threadIdx.x; x < n; x += blockDim.x) {
-      if ((x & mask) == prefix) {
-        s_all += w[x];
-        if ((x >> j) & 1) s_one += w[x];
-      }
-    }
-    block_sum2(s_all, s_one, sred);
-    if (threadIdx.x == 0) {
-      const double u = uniform53(draw(seed, traj, rnd, 0u, (uint32_t)(bit_base + j), TAG_READOUT).v[0]);
-      const int b = (u < s_one / s_all) ? 1 : 0;
-      *sbit = b;
-      out_bits[bit_base + j] = (uint8_t)b;
-    }
-    __syncthreads();
-    prefix |= (*sbit) << j;
+constexpr int kSampleThreads = 512;
+
+// Samples the bits [0, nbits) of the index over the weights w[0, 2^nbits), bit by bit: heap (2^nbits
+// doubles) gets, at 2^j + i, the weight of all indices equal to i modulo 2^j (one addition per entry, from
+// the top level down), and thread 0 walks it with the uniforms ur.  Every thread returns the index;
+// heap[1] is the total.
+__device__ int sample_bits(const double* w, int nbits, double* heap, const double* ur, int* out) {
+  for (int j = nbits - 1; j >= 0; --j) {
+    const int n = 1 << j;
+    const double* up = j == nbits - 1 ? w : heap + 2 * n;
+    for (int i = threadIdx.x; i < n; i += kSampleThreads) heap[n + i] = up[i] + up[i + n];
     __syncthreads();
   }
-  return prefix;
+  if (threadIdx.x == 0) {
+    int x = 0;
+    for (int j = 0; j < nbits; ++j) {
+      const int n = 1 << j;
+      const double one = j == nbits - 1 ? w[x + n] : heap[2 * n + x + n];
+      if (ur[j] * heap[n + x] < one) x |= n;
+    }
+    *out = x;
+  }
+  __syncthreads();
+  return *out;
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_sample(ReadArgs a) {
+__global__ void __launch_bounds__(kSampleThreads) k_sample(ReadArgs a) {
   using T2 = typename V2<T>::t;
-  extern __shared__ double sh[];
-  __shared__ double sred[64];
-  __shared__ int sbit;
+  extern __shared__ double sh[];   // weights, then their heap
+  __shared__ double ur[32];
+  __shared__ int s_low, s_high;
   const int B = 1 << a.k1;
   // trajectory blockIdx.x of the launch: a graph's from the control word, else first, first + 1, ...
   const uint64_t seed = a.direct ? a.seed : a.ctl->seed;
@@ -2004,31 +2008,29 @@ __global__ void __launch_bounds__(256) k_sample(ReadArgs a) {
   const uint64_t rnd = (uint64_t)a.rounds + 1;
   const int nd = a.D;   // data qubits = resident register bits
   uint8_t* bits = a.bits + t * (unsigned long long)nd;
-  double tot = 0.0, dummy = 0.0;
-  for (int i = threadIdx.x; i < B; i += blockDim.x) {
-    sh[i] = a.hist[(size_t)blockIdx.x * B + (i ^ (flips & (B - 1)))];
-    tot += sh[i];
-  }
-  block_sum2(tot, dummy, sred);
-  if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) a.ctl->final_norm = tot;
-  const int low = sample_bits(sh, a.k1, 0, seed, traj, rnd, bits, sred, &sbit);
+  if (threadIdx.x < nd) ur[threadIdx.x] = uniform53(draw(seed, traj, rnd, 0u, (uint32_t)threadIdx.x, TAG_READOUT).v[0]);
+  for (int i = threadIdx.x; i < B; i += kSampleThreads) sh[i] = a.hist[(size_t)blockIdx.x * B + (i ^ (flips & (B - 1)))];
+  __syncthreads();
+  const int low = sample_bits(sh, a.k1, sh + B, ur, &s_low);
+  const double total = sh[B + 1];
+  uint32_t x = (uint32_t)low;
   if (a.D > a.k1) {
     const int H = 1 << (a.D - a.k1);
     const T2* src = reinterpret_cast<const T2*>(a.src) + blockIdx.x * a.src_stride;
-    __syncthreads();
-    for (int y = threadIdx.x; y < H; y += blockDim.x) {
+    __syncthreads();   // total is read
+    for (int y = threadIdx.x; y < H; y += kSampleThreads) {
       const T2 v = src[(((int64_t)y << a.k1) | low) ^ flips];
       sh[y] = (double)v.x * (double)v.x + (double)v.y * (double)v.y;
     }
     __syncthreads();
-    sample_bits(sh, a.D - a.k1, a.k1, seed, traj, rnd, bits, sred, &sbit);
+    x |= (uint32_t)sample_bits(sh, a.D - a.k1, sh + H, ur + a.k1, &s_high) << a.k1;
   }
-  __syncthreads();
+  if (threadIdx.x < nd) bits[threadIdx.x] = (uint8_t)((x >> threadIdx.x) & 1u);
+  for (int k = threadIdx.x; k < a.nstab; k += kSampleThreads) a.syn[t * (unsigned long long)a.syn_stride + k] = 0;
   if (threadIdx.x == 0) {
-    int par = 0;
-    for (int c = 0; c < a.d; ++c) par ^= bits[c];   // Z_L: the first row (surface), the whole line (repetition)
-    a.logical[t] = (uint8_t)par;
-    for (int k = 0; k < a.nstab; ++k) a.syn[t * (unsigned long long)a.syn_stride + k] = 0;
+    if (blockIdx.x == gridDim.x - 1) a.ctl->final_norm = total;
+    // Z_L: the first row (surface), the whole line (repetition)
+    a.logical[t] = (uint8_t)(__popc(x & (a.d < 32 ? (1u << a.d) - 1u : ~0u)) & 1);
     if (!a.direct) a.ctl->traj = traj + 1;
   }
 }
@@ -2126,7 +2128,7 @@ cudaError_t launch_apply(int precision, const PassArgs& a, int grid, cudaStream_
 static size_t sample_smem(int D) {
   const int k1 = hist_k1(D);
   const size_t B = (size_t)1 << k1, H = D > k1 ? ((size_t)1 << (D - k1)) : 0;
-  return sizeof(double) * (B > H ? B : H);
+  return 2 * sizeof(double) * (B > H ? B : H);   // weights and their heap
 }
 
 cudaError_t launch_readout(int precision, const ReadArgs& a, cudaStream_t s) {
@@ -2134,12 +2136,12 @@ cudaError_t launch_readout(int precision, const ReadArgs& a, cudaStream_t s) {
   const size_t smem = sample_smem(a.D);
   if (is_f64(precision)) {
     k_hist<double><<<dim3(a.grid_hist, a.groups), 256, 0, s>>>(a);
-    k_hist_reduce<<<dim3((B + 255) / 256, a.groups), 256, 0, s>>>(a);
-    k_sample<double><<<a.groups, 256, smem, s>>>(a);
+    k_hist_reduce<<<dim3((B + 31) / 32, a.groups), 256, 0, s>>>(a);
+    k_sample<double><<<a.groups, kSampleThreads, smem, s>>>(a);
   } else {
     k_hist<float><<<dim3(a.grid_hist, a.groups), 256, 0, s>>>(a);
-    k_hist_reduce<<<dim3((B + 255) / 256, a.groups), 256, 0, s>>>(a);
-    k_sample<float><<<a.groups, 256, smem, s>>>(a);
+    k_hist_reduce<<<dim3((B + 31) / 32, a.groups), 256, 0, s>>>(a);
+    k_sample<float><<<a.groups, kSampleThreads, smem, s>>>(a);
   }
   return cudaGetLastError();
 }

@@ -31,11 +31,11 @@ template <typename T> struct Shape;
 // (85 registers: spills), 9.7 with runs of 128 bytes (11 passes a round instead of 9) and 9.5 with
 // 4096-amplitude tiles on 256 threads.
 template <> struct Shape<float> {
-  static constexpr int NT = 128, TB = kChainTileBits, BUF = 2, CTAS = 5, CHAIN = 4;
+  static constexpr int BUF = 2, CTAS = 5, CTAS_POST = 4, CHAIN = 4;
 };
 // complex128: three CTAs per SM; the FP64 pipe is the bound (one ready warp per scheduler keeps it busy).
 template <> struct Shape<double> {
-  static constexpr int NT = 128, TB = kChainTileBits, BUF = 2, CTAS = 3, CHAIN = 4;
+  static constexpr int BUF = 2, CTAS = 3, CTAS_POST = 3, CHAIN = 4;
 };
 
 __device__ __forceinline__ void cp16(void* smem, const void* gmem) {
@@ -156,59 +156,73 @@ __host__ __device__ __forceinline__ uint32_t slot_of(uint32_t e, const uint16_t*
   return e ^ (par(e & swz[0]) << P) ^ (par(e & swz[1]) << (P + 1)) ^ (par(e & swz[2]) << (P + 2));
 }
 
-template <typename T>
+// Groups of 2^GB amplitudes per thread: 16, or 4 on small registers (weight-2 blocks only), where a warp's
+// FP64 instructions, one every 64 cycles, are the pass's time and four times the warps share them.
+__host__ __device__ constexpr int group_bits(int TB) { return TB == 9 ? 2 : 4; }
+__host__ __device__ constexpr int round_threads(int TB) { return 1 << (TB - group_bits(TB)); }
+
+template <typename T, int TB>
 struct Smem {
-  static constexpr int NT = Shape<T>::NT, TS = 1 << Shape<T>::TB;
+  static constexpr int NT = round_threads(TB), TS = 1 << TB;
   using T2 = typename V2t<T>::t;
   T2 tile[Shape<T>::BUF][TS];
   T2 d[Shape<T>::CHAIN][16];
-  T2 rot[Shape<T>::CHAIN][4];
+  T2 rot[Shape<T>::CHAIN][8];              // before the diagonal, then (4 ..) after it
   uint32_t gen[Shape<T>::CHAIN][4];        // slots of a group's four tile bits
   typename Reg<T>::Acc acc[Shape<T>::CHAIN][NT];   // a thread's sums over the CTA's tiles
   uint16_t base[Shape<T>::CHAIN][NT];      // slot of a thread's group in each block
-  uint8_t form[Shape<T>::CHAIN][4];
+  alignas(8) uint8_t form[Shape<T>::CHAIN][8];
 };
 
-// One block on the thread's group of 16 amplitudes of a tile; returns its sum of squares after it.
+// One block on the thread's group of 2^GB amplitudes of a tile; returns its sum of squares after it.
 // PAIR (complex64): the group's first tile bit is bit 0, so its amplitudes come in 16-byte pairs.
-template <typename T, bool PAIR>
+// POST: rotations after the diagonal (those that run early) may be there.
+template <typename T, int GB, bool PAIR, bool POST>
 __device__ __forceinline__ typename Reg<T>::S run_group(typename V2t<T>::t* tile, uint32_t b0, const uint32_t* gen,
-                                                        const typename V2t<T>::t* rot, uint32_t forms,
+                                                        const typename V2t<T>::t* rot, uint2 forms,
                                                         const typename V2t<T>::t* d) {
   using R = Reg<T>;
-  typename R::A v[16];
-  const uint32_t g0 = gen[0], g1 = gen[1], g2 = gen[2], g3 = gen[3];
-  uint32_t at[16];
+  constexpr int NA = 1 << GB;
+  typename R::A v[NA];
+  uint32_t at[NA];
   at[0] = b0;
-  at[1] = b0 ^ g0;
 #pragma unroll
-  for (int l = 2; l < 16; ++l) at[l] = l >= 8 ? at[l - 8] ^ g3 : l >= 4 ? at[l - 4] ^ g2 : at[l - 2] ^ g1;
+  for (int j = 0; j < GB; ++j) {
+    const uint32_t g = gen[j];
+#pragma unroll
+    for (int l = 0; l < (1 << j); ++l) at[l | (1 << j)] = at[l] ^ g;
+  }
   if constexpr (PAIR) {
 #pragma unroll
-    for (int l = 0; l < 16; l += 2) R::load2(tile + at[l], v[l], v[l + 1]);
+    for (int l = 0; l < NA; l += 2) R::load2(tile + at[l], v[l], v[l + 1]);
   } else {
 #pragma unroll
-    for (int l = 0; l < 16; ++l) v[l] = R::load(tile + at[l]);
+    for (int l = 0; l < NA; ++l) v[l] = R::load(tile + at[l]);
   }
+  auto turn = [&](uint32_t f4, const typename V2t<T>::t* r4) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const uint32_t f = (forms >> (8 * j)) & 0xFFu;   // 0 also for a spectator
-    if (f == 0) continue;
-    const auto r = R::rot(rot[j]);
-    if (f == 1) {
+    for (int j = 0; j < GB; ++j) {
+      const uint32_t f = (f4 >> (8 * j)) & 0xFFu;   // 0 also for a spectator
+      if (f == 0) continue;
+      const auto r = R::rot(r4[j]);
+      if (f == 1) {
 #pragma unroll
-      for (int l = 0; l < 16; ++l)
-        if (!(l & (1 << j))) R::real(v[l], v[l | (1 << j)], r);
-    } else {
+        for (int l = 0; l < NA; ++l)
+          if (!(l & (1 << j))) R::real(v[l], v[l | (1 << j)], r);
+      } else {
 #pragma unroll
-      for (int l = 0; l < 16; ++l)
-        if (!(l & (1 << j))) R::cplx(v[l], v[l | (1 << j)], r);
+        for (int l = 0; l < NA; ++l)
+          if (!(l & (1 << j))) R::cplx(v[l], v[l | (1 << j)], r);
+      }
     }
-  }
+  };
+  turn(forms.x, rot);
+#pragma unroll
+  for (int l = 0; l < NA; l += 2) R::scale2(v[l], v[l + 1], d + l);
+  if (POST && forms.y) turn(forms.y, rot + 4);
   auto s = R::zero();
 #pragma unroll
-  for (int l = 0; l < 16; l += 2) {
-    R::scale2(v[l], v[l + 1], d + l);
+  for (int l = 0; l < NA; l += 2) {
     R::sq(s, v[l]);
     R::sq(s, v[l + 1]);
     if constexpr (PAIR) {
@@ -249,16 +263,13 @@ __device__ __forceinline__ bool group_barrier(unsigned int* bar, unsigned int ta
   return *s_ok != 0;
 }
 
-static_assert(Shape<float>::CHAIN <= Shape<float>::NT / 32 && Shape<double>::CHAIN <= Shape<double>::NT / 32,
-              "one warp sums one block of a pass");
-
-template <typename T>
-__global__ void __launch_bounds__(Shape<T>::NT, Shape<T>::CTAS) k_rounds(const __grid_constant__ RoundArgs a, int r0, int r1) {
+template <typename T, bool POST, int TB>
+__global__ void __launch_bounds__(round_threads(TB), (POST ? Shape<T>::CTAS_POST : Shape<T>::CTAS)) k_rounds(const __grid_constant__ RoundArgs a, int r0, int r1) {
   using T2 = typename V2t<T>::t;
   using SH = Shape<T>;
-  constexpr int NT = SH::NT, TB = SH::TB, CH = 16 / sizeof(T2), NCH = (1 << TB) / (NT * CH);
+  constexpr int GB = group_bits(TB), NT = round_threads(TB), NW = NT / 32, CH = 16 / sizeof(T2), NCH = (1 << TB) / (NT * CH);
   extern __shared__ __align__(16) unsigned char rsm[];
-  Smem<T>& S = *reinterpret_cast<Smem<T>*>(rsm);
+  Smem<T, TB>& S = *reinterpret_cast<Smem<T, TB>*>(rsm);
   __shared__ double s_sum[kMaxChain];
   __shared__ int s_ok, s_known, s_out;
   __shared__ ChainDesc C;
@@ -274,14 +285,14 @@ __global__ void __launch_bounds__(Shape<T>::NT, Shape<T>::CTAS) k_rounds(const _
   double N = r0 == 1 ? 1.0 : *(volatile double*)(a.norm + grp);
   unsigned int epoch = 0, misses = 0;
   bool ok = true;
-  if (tid < nstab) s_prev[tid] = r0 == 1 ? 0 : syn[(r0 - 1) * nstab + tid];
+  for (int i = tid; i < nstab; i += NT) s_prev[i] = r0 == 1 ? 0 : syn[(r0 - 1) * nstab + i];
   for (int rnd = r0; rnd <= r1 && ok; ++rnd) {
     for (int c = 0; c < a.nc && ok; ++c) {
       __syncthreads();
       for (int i = tid; i < (int)(sizeof(ChainDesc) / 4); i += NT)
         reinterpret_cast<uint32_t*>(&C)[i] = reinterpret_cast<const uint32_t*>(a.chains + c)[i];
       __syncthreads();
-      const int step = (rnd - 1) * a.nc + c, nb = C.nb;
+      const int step = (rnd - 1) * a.steps + c, nb = C.nb;
       const T2* src = step == 0 ? reinterpret_cast<const T2*>(a.psi0) : buf[(step & 1) ^ 1];
       T2* dst = buf[step & 1];
       const Compiled<T>* cb = blk + (size_t)(rnd - 1) * nstab + C.b0;
@@ -290,17 +301,22 @@ __global__ void __launch_bounds__(Shape<T>::NT, Shape<T>::CTAS) k_rounds(const _
         const int b = i / NT;
         uint32_t x = (uint32_t)(i - b * NT);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < GB; ++j) {
           const int q = C.bits[b][j];
           x = ((x >> q) << (q + 1)) | (x & ((1u << q) - 1u));
         }
         S.base[b][i - b * NT] = (uint16_t)slot_of<T>(x, C.swz);
       }
-      if (tid < 4 * nb) {
+      if (tid < 4 * nb && (tid & 3) < GB) {
         const int b = tid >> 2, j = tid & 3, q = C.qubit[b][j];
         S.gen[b][j] = slot_of<T>(1u << C.bits[b][j], C.swz);
         if (q < 4) S.rot[b][j] = cb[b].rot[q];
-        S.form[b][j] = q < 4 ? cb[b].form[q] : (uint8_t)0;
+        S.form[b][j] = q < 4 && !fac::runs_early(a.F, 4 * (C.b0 + b) + q) ? cb[b].form[q] : (uint8_t)0;
+        const int nx = q < 4 ? a.F.touches[4 * (C.b0 + b) + q].next : -1;
+        const bool after = POST && nx >= 0 && fac::runs_early(a.F, nx);
+        const Compiled<T>& cn = blk[(size_t)(rnd - 1) * nstab + (after ? nx >> 2 : 0)];
+        if (after) S.rot[b][4 + j] = cn.rot[nx & 3];
+        S.form[b][4 + j] = after ? cn.form[nx & 3] : (uint8_t)0;
       }
       // this thread's 16-byte chunks e = CH (tid + NT i): register offset and tile slot, both linear over XOR
       auto t2g = [&](uint32_t e) {
@@ -330,13 +346,13 @@ __global__ void __launch_bounds__(Shape<T>::NT, Shape<T>::CTAS) k_rounds(const _
       int known = 0, out = 0;   // outcomes decided so far: bits 0 .. known - 1 of out
       for (;;) {
         // the chosen outcomes' diagonals; the input's scale goes into the first
-        if (tid < 16 * nb) {
-          const int b = tid >> 4, l = tid & 15;
+        for (int i = tid; i < (nb << GB); i += NT) {
+          const int b = i >> GB, l = i & ((1 << GB) - 1);
           const int off = a.F.blocks[C.b0 + b].offset;
           const int m = b < known ? (out >> b) & 1 : s_prev[C.b0 + b] ^ off;
           int z = 0;
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
+          for (int j = 0; j < GB; ++j)
             if (C.qubit[b][j] < 4) z |= ((l >> j) & 1) << C.qubit[b][j];
           T2 v = cb[b].d[m][z];
           if (b == 0) {
@@ -358,12 +374,12 @@ __global__ void __launch_bounds__(Shape<T>::NT, Shape<T>::CTAS) k_rounds(const _
           const uint32_t nxt = cur == 0 ? SH::BUF - 1 : cur - 1;
           load_tile(t + (SH::BUF - 1) * a.G, S.tile[nxt]);
           for (int b = 0; b < nb; ++b) {
-            const uint32_t forms = *reinterpret_cast<const uint32_t*>(S.form[b]);
+            const uint2 forms = *reinterpret_cast<const uint2*>(S.form[b]);
             typename Reg<T>::S s;
             if (sizeof(T) == 4 && C.bits[b][0] == 0)
-              s = run_group<T, sizeof(T) == 4>(tile, S.base[b][tid], S.gen[b], S.rot[b], forms, S.d[b]);
+              s = run_group<T, GB, sizeof(T) == 4, POST>(tile, S.base[b][tid], S.gen[b], S.rot[b], forms, S.d[b]);
             else
-              s = run_group<T, false>(tile, S.base[b][tid], S.gen[b], S.rot[b], forms, S.d[b]);
+              s = run_group<T, GB, false, POST>(tile, S.base[b][tid], S.gen[b], S.rot[b], forms, S.d[b]);
             Reg<T>::add(S.acc[b][tid], s);
             __syncthreads();
           }
@@ -375,23 +391,23 @@ __global__ void __launch_bounds__(Shape<T>::NT, Shape<T>::CTAS) k_rounds(const _
         }
         cp_wait<0>();
         __syncthreads();
-        if (warp < nb) {   // block `warp`'s sum over the CTA
+        for (int b = warp; b < nb; b += NW) {   // block b's sum over the CTA
           double acc = 0.0;
 #pragma unroll
-          for (int i = 0; i < NT / 32; ++i) acc += Reg<T>::total(S.acc[warp][lane + 32 * i]);
+          for (int i = 0; i < NW; ++i) acc += Reg<T>::total(S.acc[b][lane + 32 * i]);
           acc = warp_total(acc);
-          if (lane == 0) a.partials[((size_t)(epoch & 1) * gridDim.x + blockIdx.x) * kMaxChain + warp] = acc;
+          if (lane == 0) a.partials[((size_t)(epoch & 1) * gridDim.x + blockIdx.x) * kMaxChain + b] = acc;
         }
         ++epoch;
         ok = group_barrier(bar, epoch * a.G, a.ctl, &s_ok);
         if (!ok) break;
         // every CTA sums the group's partials in the same order and decides alike
-        if (warp < nb) {
-          const double* p = a.partials + ((size_t)((epoch - 1) & 1) * gridDim.x + grp * a.G) * kMaxChain + warp;
+        for (int b = warp; b < nb; b += NW) {
+          const double* p = a.partials + ((size_t)((epoch - 1) & 1) * gridDim.x + grp * a.G) * kMaxChain + b;
           double s = 0.0;
           for (int i = lane; i < a.G; i += 32) s += __ldcg(p + (size_t)i * kMaxChain);
           s = warp_total(s);
-          if (lane == 0) s_sum[warp] = s;
+          if (lane == 0) s_sum[b] = s;
         }
         __syncthreads();
         if (tid == 0) {
@@ -442,6 +458,322 @@ __global__ void __launch_bounds__(Shape<T>::NT, Shape<T>::CTAS) k_rounds(const _
       bar[1] = 0;
     }
   }
+}
+
+// ---- diagonal passes ------------------------------------------------------------------------------------
+// A pass of blocks without rotations is phi(x) <- E(z(x)) phi(x), z the pass's data bits and E the product
+// of the chosen outcomes' diagonals, and every sum it needs is a weighted sum of h(z) = sum |phi|^2 over
+// the amplitudes with bits z.  A thread keeps the same tile positions in every tile, so its E and h are
+// in registers; amplitudes stream through a ring of thread-private 16-byte copies, without barriers: 6
+// multiply-adds each however many blocks the pass holds.  When the tiles are done, the sums for the
+// guessed outcomes decide the blocks up to the first wrong guess; those for the corrected path come
+// from the same h.  So the outcomes cost one pass whatever the guesses, and wrong ones one more without
+// sums.
+constexpr int kDiagThreads = 512;
+__host__ __device__ constexpr int diag_bits(bool f64) { return f64 ? 12 : 13; }
+
+template <typename T>
+struct DiagSmem {
+  using T2 = typename V2t<T>::t;
+  static constexpr int TB = diag_bits(sizeof(T) == 8), P = (1 << TB) / kDiagThreads;   // positions per thread
+  static constexpr int CH = 16 / sizeof(T2), NCH = P / CH, STAGES = 2;
+  union {
+    float4 ring[STAGES][NCH][kDiagThreads];
+    struct {                                   // after a pass
+      double pos[1 << TB];                     // h per tile position
+      double sum[kMaxDiag + 1][kDiagThreads];
+    } r;
+  };
+  T2 E[1 << kDiagUnion];
+  double h[1 << kDiagUnion];
+  double wd[kMaxDiag][2][16];                  // |D_m|^2
+  T2 d[kMaxDiag][2][16];
+  double u[kMaxDiag];
+  double scale;                                // of the input
+  uint8_t guess[kMaxDiag];
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kDiagThreads) k_diagonals(const __grid_constant__ RoundArgs a, int rnd) {
+  using T2 = typename V2t<T>::t;
+  using SM = DiagSmem<T>;
+  constexpr int NT = kDiagThreads, P = SM::P, CH = SM::CH, NCH = SM::NCH, ST = SM::STAGES;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  SM& S = *reinterpret_cast<SM*>(dsm);
+  __shared__ double s_sum[kMaxDiag + 1];
+  __shared__ int s_ok, s_known, s_out;
+  __shared__ DiagDesc C;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nstab = a.F.nstab, G = (int)gridDim.x;
+  uint8_t* syn = a.syn;
+  const Compiled<T>* blk = reinterpret_cast<const Compiled<T>*>(a.blocks) + (size_t)(rnd - 1) * nstab;
+  double N = a.diag_in ? *(volatile const double*)(a.diag_in + (size_t)(rnd - 1) * a.diag_stride)
+                       : rnd == 1 && a.step0 == 0 ? 1.0 : *(volatile double*)a.norm;
+  unsigned int epoch = 0, misses = 0;
+  bool ok = true;
+  for (int c = 0; c < a.nd && ok; ++c) {
+    __syncthreads();
+    for (int i = tid; i < (int)(sizeof(DiagDesc) / 4); i += NT)
+      reinterpret_cast<uint32_t*>(&C)[i] = reinterpret_cast<const uint32_t*>(a.diags + c)[i];
+    __syncthreads();
+    const int step = (rnd - 1) * a.steps + a.step0 + c, nb = C.nb;
+    const T2* src = reinterpret_cast<const T2*>(step == 0 ? a.psi0 : a.buf[(step & 1) ^ 1]);
+    T2* dst = reinterpret_cast<T2*>(a.buf[step & 1]);
+    const Compiled<T>* cb = blk + C.b0;
+    if (tid < nb) {
+      const int b = C.b0 + tid;
+      S.u[tid] = cb[tid].u;
+      S.guess[tid] = (uint8_t)((rnd == 1 ? 0 : syn[(rnd - 1) * nstab + b]) ^ a.F.blocks[b].offset);
+    }
+    if (tid == NT - 1) S.scale = rsqrt(N);
+    for (int i = tid; i < 32 * nb; i += NT) {
+      const int b = i >> 5, m = (i >> 4) & 1, z = i & 15;
+      if (z >> C.w[b]) continue;
+      const T2 d = cb[b].d[m][z];
+      S.d[b][m][z] = d;
+      S.wd[b][m][z] = fma((double)d.x, (double)d.x, (double)d.y * (double)d.y);
+    }
+    uint32_t coff[NCH];
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      const uint32_t e = (uint32_t)(CH * (tid + NT * i)), hi = e >> C.lb;
+      uint32_t o = 0;
+      for (int j = 0; j < C.nh; ++j) o |= ((hi >> j) & 1u) << C.hbits[j];
+      coff[i] = o | (e & ((1u << C.lb) - 1u));
+    }
+    auto bin_of = [&](uint32_t e) {   // the pass's data bits at tile index e
+      uint32_t z = 0;
+      for (int j = 0; j < C.nu; ++j) z |= ((e >> C.ubits[j]) & 1u) << j;
+      return z;
+    };
+    auto z_of = [&](int b, uint32_t bin) {   // block b's data bits
+      int z = 0;
+      for (int j = 0; j < C.w[b]; ++j) z |= (int)((bin >> C.at[b][j]) & 1u) << j;
+      return z;
+    };
+    const int nout = C.nout, obit = lane < nout ? C.obits[lane] : 0;
+    auto tile_base = [&](uint32_t t) {
+      return __reduce_or_sync(0xffffffffu, lane < nout ? ((t >> lane) & 1u) << obit : 0u);
+    };
+    const uint32_t ntile = 1u << nout, bins = 1u << C.nu;
+    auto load = [&](uint32_t t, int st) {
+      if (t < ntile) {
+        const T2* p = src + tile_base(t);
+#pragma unroll
+        for (int i = 0; i < NCH; ++i) cp16(&S.ring[st][i][tid], p + coff[i]);
+      }
+      cp_commit();
+    };
+    double h[P];
+    // one pass for the outcomes in `out`; SUM: |phi|^2 goes into h
+    auto pass = [&](int out, auto with_sums) {
+      constexpr bool SUM = decltype(with_sums)::value;
+      __syncthreads();   // S.d, S.wd are there; the ring's memory is free
+#pragma unroll
+      for (int i = 0; i < ST; ++i) load(blockIdx.x + i * G, i);
+      for (uint32_t z = tid; z < bins; z += NT) {
+        T2 e = make2<T2>(S.scale, 0.0);
+        for (int b = 0; b < nb; ++b) {
+          const T2 d = S.d[b][(out >> b) & 1][z_of(b, z)], x = e;
+          e.x = fma(-d.y, x.y, d.x * x.x);
+          e.y = fma(d.y, x.x, d.x * x.y);
+        }
+        S.E[z] = e;
+      }
+      __syncthreads();
+      T2 E[P];
+#pragma unroll
+      for (int k = 0; k < P; ++k) E[k] = S.E[bin_of((uint32_t)(CH * (tid + NT * (k / CH)) + k % CH))];
+      T part[P];   // complex64: FP32 over up to 16 tiles, then FP64
+      int run = 0, st = 0;
+#pragma unroll
+      for (int k = 0; k < P; ++k) {
+        part[k] = 0;
+        h[k] = SUM ? 0.0 : h[k];
+      }
+      for (uint32_t t = blockIdx.x; t < ntile; t += G) {
+        T2* o = dst + tile_base(t);
+        cp_wait<ST - 1>();
+#pragma unroll
+        for (int i = 0; i < NCH; ++i) {
+          T2 v[CH];
+          *reinterpret_cast<float4*>(v) = S.ring[st][i][tid];
+#pragma unroll
+          for (int k = 0; k < CH; ++k) {
+            const T2 x = v[k], e = E[CH * i + k];
+            if (SUM) part[CH * i + k] = fma(x.x, x.x, fma(x.y, x.y, part[CH * i + k]));
+            v[k].x = fma(-e.y, x.y, e.x * x.x);
+            v[k].y = fma(e.y, x.x, e.x * x.y);
+          }
+          *reinterpret_cast<float4*>(o + coff[i]) = *reinterpret_cast<const float4*>(v);
+        }
+        load(t + ST * G, st);   // this thread has consumed its copies of the stage
+        st = st + 1 == ST ? 0 : st + 1;
+        if (SUM && sizeof(T) == 4 && ++run == 16) {
+          run = 0;
+#pragma unroll
+          for (int k = 0; k < P; ++k) {
+            h[k] += (double)part[k];
+            part[k] = 0;
+          }
+        }
+      }
+      cp_wait<0>();
+      if (SUM)
+#pragma unroll
+        for (int k = 0; k < P; ++k) h[k] += (double)part[k];
+    };
+    int out = 0, known = 0;   // chosen outcomes; the first `known` are decided
+    __syncthreads();
+    for (int b = 0; b < nb; ++b) out |= S.guess[b] << b;
+    const int guess = out;
+    pass(out, std::true_type{});
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < P; ++k) S.r.pos[CH * (tid + NT * (k / CH)) + k % CH] = h[k];
+    __syncthreads();
+    for (uint32_t z = tid; z < bins; z += NT) {
+      uint32_t e0 = 0;
+      for (int j = 0; j < C.nu; ++j) e0 |= ((z >> j) & 1u) << C.ubits[j];
+      double s = 0.0;
+      for (uint32_t i = 0; i < (1u << (SM::TB - C.nu)); ++i) {
+        uint32_t e = e0;
+        for (int j = 0; j < SM::TB - C.nu; ++j) e |= ((i >> j) & 1u) << C.rbits[j];
+        s += S.r.pos[e];
+      }
+      S.h[z] = s;   // read by this thread alone
+    }
+    for (;;) {
+      // S_i of the chosen path, i = 0 (the input's norm) .. nb
+      double s[kMaxDiag + 1];
+#pragma unroll
+      for (int i = 0; i <= kMaxDiag; ++i) s[i] = 0.0;
+      for (uint32_t z = tid; z < bins; z += NT) {
+        double w = S.h[z];
+        s[0] += w;
+#pragma unroll
+        for (int b = 0; b < kMaxDiag; ++b)
+          if (b < nb) {
+            w *= S.wd[b][(out >> b) & 1][z_of(b, z)];
+            s[b + 1] += w;
+          }
+      }
+#pragma unroll
+      for (int i = 0; i <= kMaxDiag; ++i)
+        if (i <= nb) S.r.sum[i][tid] = s[i];
+      __syncthreads();
+      if (warp <= nb) {
+        double t = 0.0;
+        const uint32_t n = bins < NT ? bins : NT;
+        for (uint32_t i = lane; i < n; i += 32) t += S.r.sum[warp][i];
+        t = warp_total(t);
+        if (lane == 0) a.partials[((size_t)(epoch & 1) * G + blockIdx.x) * (kMaxDiag + 1) + warp] = t;
+      }
+      ++epoch;
+      ok = group_barrier(a.bar, epoch * G, a.ctl, &s_ok);
+      if (!ok) break;
+      if (warp <= nb) {
+        const double* p = a.partials + (size_t)((epoch - 1) & 1) * G * (kMaxDiag + 1) + warp;
+        double t = 0.0;
+        for (int i = lane; i < G; i += 32) t += __ldcg(p + (size_t)i * (kMaxDiag + 1));
+        t = warp_total(t);
+        if (lane == 0) s_sum[warp] = t;
+      }
+      __syncthreads();
+      if (tid == 0) {
+        int k = known, o = out;
+        bool hit = true;
+        while (k < nb && hit) {
+          const int g = (out >> k) & 1;
+          const double p1 = g ? s_sum[k + 1] : s_sum[k] - s_sum[k + 1];
+          const int m = S.u[k] * s_sum[k] < p1 ? 1 : 0;
+          hit = m == g;
+          if (!hit) o ^= 1 << k;
+          ++k;
+          misses += !hit;
+        }
+        s_known = hit ? nb + 1 : k;
+        s_out = o;
+      }
+      __syncthreads();
+      known = s_known;
+      out = s_out;
+      if (known > nb) break;   // the whole path holds
+    }
+    if (!ok) break;
+    const double total = s_sum[nb];
+    if (out != guess) pass(out, std::false_type{});
+    N = total / N;
+    if (blockIdx.x == 0 && tid < nb)
+      syn[rnd * nstab + C.b0 + tid] = (uint8_t)(((out >> tid) & 1) ^ a.F.blocks[C.b0 + tid].offset);
+    if (c + 1 < a.nd) {   // the next pass reads what every CTA wrote
+      ++epoch;
+      ok = group_barrier(a.bar, epoch * G, a.ctl, &s_ok);
+    }
+  }
+  if (tid == 0) {
+    if (blockIdx.x == 0) {
+      if (a.diag_out) a.diag_out[(size_t)(rnd - 1) * a.diag_stride] = N;
+      else a.norm[0] = N;
+      if (misses) atomicAdd(&a.ctl->spec_misses, (unsigned long long)misses);
+      if (a.ctl->prob_force_exact) {   // these sums are the exact evaluation that hook asks for
+        int n = 0;
+        for (int c = 0; c < a.nd; ++c) n += a.diags[c].nb;
+        atomicAdd(&a.ctl->prob_fallbacks, (unsigned long long)n);
+      }
+    }
+    __threadfence();
+    if (atomicAdd(a.bar + 1, 1u) == (unsigned)G - 1) {
+      a.bar[0] = 0;
+      a.bar[1] = 0;
+    }
+  }
+}
+
+// ---- dense blocks for the tensor-core passes ---------------------------------------------------------------
+// K_m = R_after D_m R_before of block b (the factored register's gauge), R the products of the rotations
+// before it and of those after it that run early (their cosines are in D_m).  One CTA per block, a
+// thread per entry.
+__global__ void __launch_bounds__(256) k_dense(const __grid_constant__ RoundArgs a, int nb, double2* kraus, double* u) {
+  const int b = blockIdx.x % nb, r = blockIdx.x / nb, nstab = a.F.nstab;
+  const Compiled<double>* blk = reinterpret_cast<const Compiled<double>*>(a.blocks) + (size_t)r * nstab;
+  const Compiled<double>& C = blk[b];
+  const FBlock B = a.F.blocks[b];
+  const int w = B.w, n = 1 << w, row = threadIdx.x >> 4, col = threadIdx.x & 15;
+  __shared__ double2 pre[4][4], post[4][4];
+  if (threadIdx.x < 8) {
+    const int j = threadIdx.x & 3;
+    const bool after = threadIdx.x >= 4;
+    double2 t = make_double2(0.0, 0.0);
+    if (j < w) {
+      const int tc = 4 * b + j, nx = a.F.touches[tc].next;
+      if (!after) {
+        if (!fac::runs_early(a.F, tc)) t = C.rot[j];
+      } else if (nx >= 0 && fac::runs_early(a.F, nx)) {
+        // the cosine is in D_m: the t form itself
+        t = blk[nx >> 2].rot[nx & 3];
+      }
+    }
+    double2* m = after ? post[j] : pre[j];
+    m[0] = m[3] = make_double2(1.0, 0.0);
+    m[1] = make_double2(-t.x, t.y);
+    m[2] = t;
+  }
+  __syncthreads();
+  double2 k0 = make_double2(0.0, 0.0), k1 = k0;
+  if (row < n && col < n)
+    for (int l = 0; l < n; ++l) {
+      double2 x = make_double2(1.0, 0.0);
+      for (int j = 0; j < w; ++j)
+        x = fac::cmul(x, fac::cmul(post[j][2 * ((row >> j) & 1) + ((l >> j) & 1)], pre[j][2 * ((l >> j) & 1) + ((col >> j) & 1)]));
+      const double2 x0 = fac::cmul(x, C.d[0][l]), x1 = fac::cmul(x, C.d[1][l]);
+      k0 = make_double2(k0.x + x0.x, k0.y + x0.y);
+      k1 = make_double2(k1.x + x1.x, k1.y + x1.y);
+    }
+  double2* out = kraus + ((size_t)r * nstab + b) * KRAUS_STRIDE;
+  out[threadIdx.x] = k0;
+  out[256 + threadIdx.x] = k1;
+  if (threadIdx.x == 0) u[(size_t)r * nstab + b] = C.u;
 }
 
 // ---- compile ------------------------------------------------------------------------------------------
@@ -515,12 +847,27 @@ __global__ void __launch_bounds__(128) k_compile_emit(const __grid_constant__ Ro
 
 }  // namespace
 
+// The kernel for a pass's tile bits and its shared memory; early: with the rotations that run early (large
+// registers only).
+struct RoundKernel {
+  const void* fn;
+  size_t smem;
+};
+template <typename T>
+static RoundKernel round_kernel_t(int tb, bool early) {
+  if (tb == 9) return {(const void*)k_rounds<T, false, 9>, sizeof(Smem<T, 9>)};
+  return {early ? (const void*)k_rounds<T, true, 11> : (const void*)k_rounds<T, false, 11>, sizeof(Smem<T, 11>)};
+}
+static RoundKernel round_kernel(int precision, int tb, bool early) {
+  return is_f64(precision) ? round_kernel_t<double>(tb, early) : round_kernel_t<float>(tb, early);
+}
+
 size_t compile_scratch_bytes(const FactorProgram& F) { return scratch_bytes(F.nstab, (int)F.sites.size()); }
 size_t compiled_block_bytes(int precision) { return is_f64(precision) ? sizeof(Compiled<double>) : sizeof(Compiled<float>); }
 
 // Shared-memory wavefronts of a warp's 16 group loads (32-bit banks; `wide`: bytes of one load), summed
 // over the pass's blocks.
-static int conflict_cost(const ChainDesc& c, int precision) {
+static int conflict_cost(const ChainDesc& c, int precision, int gb) {
   const bool f64 = is_f64(precision);
   int cost = 0;
   for (int i = 0; i < c.nb; ++i) {
@@ -530,7 +877,7 @@ static int conflict_cost(const ChainDesc& c, int precision) {
       int per_slot[16] = {}, worst = 0;
       for (int l = w; l < w + lanes; ++l) {
         uint32_t x = (uint32_t)l;
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < gb; ++j) {
           const int q = c.bits[i][j];
           x = ((x >> q) << (q + 1)) | (x & ((1u << q) - 1u));
         }
@@ -554,7 +901,7 @@ static void choose_swizzle(ChainDesc& c, int precision, int TB) {
     for (int b = lo + k; b < TB; b += 3) m |= 1u << b;
     c.swz[k] = best[k] = (uint16_t)m;
   }
-  int cost = conflict_cost(c, precision), floor = 0;
+  int cost = conflict_cost(c, precision, group_bits(TB)), floor = 0;
   for (int i = 0; i < c.nb; ++i) floor += !is_f64(precision) && c.bits[i][0] != 0 ? 4 : is_f64(precision) ? 8 : 4;
   uint64_t x = 0x9E3779B97F4A7C15ull;
   for (int t = 0; t < 300 && cost > floor; ++t) {
@@ -564,7 +911,7 @@ static void choose_swizzle(ChainDesc& c, int precision, int TB) {
       x ^= x << 17;
       c.swz[k] = (uint16_t)(x & all);
     }
-    const int n = conflict_cost(c, precision);
+    const int n = conflict_cost(c, precision, group_bits(TB));
     if (n < cost) {
       cost = n;
       std::copy(c.swz, c.swz + 3, best);
@@ -573,14 +920,14 @@ static void choose_swizzle(ChainDesc& c, int precision, int TB) {
   std::copy(best, best + 3, c.swz);
 }
 
-std::vector<ChainDesc> plan_chains(const FactorProgram& F, int precision, int most) {
-  constexpr int TB = kChainTileBits, low = 3;
+std::vector<ChainDesc> plan_chains(const FactorProgram& F, int precision, int TB, int most, int b0, int b1) {
+  constexpr int low = 3;
   most = std::min(most, is_f64(precision) ? Shape<double>::CHAIN : Shape<float>::CHAIN);
   std::vector<ChainDesc> out;
-  for (int b = 0; b < F.nstab;) {
+  for (int b = b0; b < b1;) {
     uint32_t mask = 0;
     int nb = 0;
-    while (b + nb < F.nstab && nb < most) {
+    while (b + nb < b1 && nb < most) {
       uint32_t m = mask;
       for (int j = 0; j < F.blocks[b + nb].w; ++j) m |= 1u << F.blocks[b + nb].q[j];
       if (nb && __builtin_popcount(m | ((1u << low) - 1u)) > TB) break;
@@ -615,17 +962,18 @@ std::vector<ChainDesc> plan_chains(const FactorProgram& F, int precision, int mo
       // spectators: tile bit 0 (complex64 amplitudes then come in pairs), then the highest tile bits
       // outside the block (a warp's groups lie side by side)
       auto used = [&](int x) { return std::find(q, q + n, x) != q + n; };
-      for (int x = TB; n < 4; --x) {
+      const int gb = group_bits(TB);
+      for (int x = TB; n < gb; --x) {
         const int y = x == TB ? 0 : x;
         if (used(y)) continue;
         q[n] = y;
         which[n++] = 4;
       }
-      int at[4] = {0, 1, 2, 3};
-      std::sort(at, at + 4, [&](int x, int y) { return q[x] < q[y]; });
-      for (int j = 0; j < 4; ++j) {
-        c.bits[i][j] = (uint8_t)q[at[j]];
-        c.qubit[i][j] = (uint8_t)which[at[j]];
+      for (int j = 0; j < gb; ++j) {   // ascending
+        int at = 0;
+        for (int k = 0; k < gb; ++k) at += q[k] < q[j];
+        c.bits[i][at] = (uint8_t)q[j];
+        c.qubit[i][at] = (uint8_t)which[j];
       }
     }
     choose_swizzle(c, precision, TB);
@@ -635,21 +983,72 @@ std::vector<ChainDesc> plan_chains(const FactorProgram& F, int precision, int mo
   return out;
 }
 
+std::vector<DiagDesc> plan_diagonals(const FactorProgram& F, int precision, int b0, int b1) {
+  const int TB = diag_bits(is_f64(precision)), low = is_f64(precision) ? 3 : 4;
+  std::vector<DiagDesc> out;
+  for (int b = b0; b < b1;) {
+    uint32_t mask = 0;
+    int nb = 0;
+    while (b + nb < b1 && nb < kMaxDiag) {
+      uint32_t m = mask;
+      for (int j = 0; j < F.blocks[b + nb].w; ++j) m |= 1u << F.blocks[b + nb].q[j];
+      if (nb && (__builtin_popcount(m | ((1u << low) - 1u)) > TB || __builtin_popcount(m) > kDiagUnion)) break;
+      mask = m;
+      ++nb;
+    }
+    DiagDesc c{};
+    c.b0 = b;
+    c.nb = nb;
+    int lb = low;
+    while (__builtin_popcount(mask | ((1u << lb) - 1u)) < TB) ++lb;
+    c.lb = lb;
+    int tile_bit[32];
+    for (int q = 0; q < F.nd; ++q) {
+      if (q < lb) tile_bit[q] = q;
+      else if (mask & (1u << q)) {
+        tile_bit[q] = lb + c.nh;
+        c.hbits[c.nh++] = (uint8_t)q;
+      } else {
+        c.obits[c.nout++] = (uint8_t)q;
+      }
+    }
+    int index[32], nr = 0;   // a data qubit's place among the pass's
+    uint32_t in_union = 0;
+    for (int q = 0; q < F.nd; ++q)
+      if (mask & (1u << q)) {
+        index[q] = c.nu;
+        c.ubits[c.nu++] = (uint8_t)tile_bit[q];
+        in_union |= 1u << tile_bit[q];
+      }
+    for (int t = 0; t < TB; ++t)
+      if (!(in_union & (1u << t))) c.rbits[nr++] = (uint8_t)t;
+    for (int i = 0; i < nb; ++i) {
+      c.w[i] = F.blocks[b + i].w;
+      for (int j = 0; j < c.w[i]; ++j) c.at[i][j] = (uint8_t)index[F.blocks[b + i].q[j]];
+    }
+    out.push_back(c);
+    b += nb;
+  }
+  return out;
+}
+
 cudaError_t setup_rounds(int precision) {
-  const void* fn = is_f64(precision) ? (const void*)k_rounds<double> : (const void*)k_rounds<float>;
-  const int smem = is_f64(precision) ? (int)sizeof(Smem<double>) : (int)sizeof(Smem<float>);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  cudaError_t e = cudaSuccess;
+  for (int v = 0; v < 3 && e == cudaSuccess; ++v) {
+    const RoundKernel k = round_kernel(precision, v == 0 ? 9 : 11, v == 2);
+    e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k.fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  }
+  const void* dg = is_f64(precision) ? (const void*)k_diagonals<double> : (const void*)k_diagonals<float>;
+  const int dsmem = is_f64(precision) ? (int)sizeof(DiagSmem<double>) : (int)sizeof(DiagSmem<float>);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(dg, cudaFuncAttributeMaxDynamicSharedMemorySize, dsmem);
   return e;
 }
 
-int round_ctas(int D) { return 1 << (D - kChainTileBits); }
-
-int round_wave(int precision, int num_sms) {
+int round_wave(int precision, int tb, bool early, int num_sms) {
   int occ = 0;
-  cudaError_t e = is_f64(precision)
-      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_rounds<double>, Shape<double>::NT, sizeof(Smem<double>))
-      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_rounds<float>, Shape<float>::NT, sizeof(Smem<float>));
+  const RoundKernel k = round_kernel(precision, tb, early);
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.fn, round_threads(tb), k.smem);
   return e == cudaSuccess && occ > 0 ? occ * num_sms : 0;
 }
 
@@ -662,13 +1061,26 @@ cudaError_t launch_compile(int precision, const RoundArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+cudaError_t launch_diagonals(int precision, const RoundArgs& a, int r, int num_sms, cudaStream_t s) {
+  RoundArgs b = a;
+  void* args[2] = {&b, &r};
+  const int64_t tiles = 1ll << (a.D - diag_bits(is_f64(precision)));
+  const dim3 grid((unsigned)(tiles < num_sms ? tiles : num_sms));
+  const void* fn = is_f64(precision) ? (const void*)k_diagonals<double> : (const void*)k_diagonals<float>;
+  return cudaLaunchCooperativeKernel(fn, grid, dim3(kDiagThreads), args, is_f64(precision) ? sizeof(DiagSmem<double>) : sizeof(DiagSmem<float>), s);
+}
+
+cudaError_t launch_dense(const RoundArgs& a, int nb, void* kraus, double* u, cudaStream_t s) {
+  k_dense<<<nb * a.rounds, 256, 0, s>>>(a, nb, static_cast<double2*>(kraus), u);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_rounds(int precision, const RoundArgs& a, int r0, int r1, cudaStream_t s) {
   RoundArgs b = a;
   void* args[3] = {&b, &r0, &r1};
   const dim3 grid((unsigned)(a.groups * a.G));
-  if (is_f64(precision))
-    return cudaLaunchCooperativeKernel((const void*)k_rounds<double>, grid, dim3(Shape<double>::NT), args, sizeof(Smem<double>), s);
-  return cudaLaunchCooperativeKernel((const void*)k_rounds<float>, grid, dim3(Shape<float>::NT), args, sizeof(Smem<float>), s);
+  const RoundKernel k = round_kernel(precision, a.tb, a.F.early != 0);
+  return cudaLaunchCooperativeKernel(k.fn, grid, dim3((unsigned)round_threads(a.tb)), args, k.smem, s);
 }
 
 }  // namespace qec
