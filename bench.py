@@ -30,6 +30,12 @@ import workloads as W  # noqa: E402
 
 METRIC = "d=5 QEC rounds/s (26-qubit SV), HBM GB/s vs peak; serve p50/p99 latency"
 UNIT = "rounds/s"
+# passes of a round on the 25-qubit register: (code, complex128) -> reads and writes of the register.  Surface:
+# 12 X blocks one by one in complex128, 5 passes in complex64; 12 Z blocks in 4 diagonal passes.  Repetition: 3.
+ROUND_PASSES = {("surface", True): 16, ("surface", False): 9, ("repetition", True): 3, ("repetition", False): 3}
+# FP64 multiply-adds per amplitude of a d = 5 round: 65 rotations of 2, 12 X blocks of 4 + 2 (diagonal, square),
+# 4 diagonal passes of 6
+ROUND_FP64_FMA = 65 * 2 + 12 * 6 + 4 * 6
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12   # 152 SMs x 2 FP64 FMA/clk/SM x 2 flop x 2070 MHz
 
 
@@ -211,7 +217,7 @@ def workload_config(args, world):
 # ---- native arm ------------------------------------------------------------------------------
 def traffic_record(precision):
     """dram bytes per launch of the apply pass from the committed ncu summary, if it was taken
-    on the current kernel source (sha256 of kernels.cu and ozaki.cuh); else None."""
+    on the current kernel source (sha256 of the files below); else None."""
     path = os.path.join(ROOT, "profiles", "apply_pass_traffic.json")
     try:
         rec = json.load(open(path)).get(precision, {})
@@ -224,7 +230,7 @@ def traffic_record(precision):
 
 def kernel_source_sha():
     h = hashlib.sha256()
-    for f in ("kernels.cu", "ozaki.cuh"):
+    for f in ("kernels.cu", "ozaki.cuh", "rounds.cu", "onchip.cuh", "factor.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2204_11404_gb300", "csrc", f), "rb").read())
     return h.hexdigest()
 
@@ -278,8 +284,8 @@ def native_arm(args, rank, world, local):
             step(args.warmup + i)
         e1.record(stream)
         torch.cuda.synchronize()
-    # the instrumented block's device times, from event-record nodes inside each simulator's
-    # trajectory graph (its most recent trajectory), read after the timed region
+    # the instrumented block's device times, from events around its pass or round in each simulator's
+    # most recent trajectory, read after the timed region
     used = sorted({(args.warmup + i) % len(pts) for i in range(args.steps)})
     kt = [capi.qec_kernel_times(sims[j].h) for j in used]
     fallbacks = (sum(capi.qec_debug_exact_probability(s.h, -1) for s in sims) - sum(fb0)) if fb0 else None
@@ -310,28 +316,26 @@ def native_arm(args, rank, world, local):
     e2e = {"value": world * n_e2e * R / e2e_secs, "unit": UNIT,
            "h2d_bytes_per_step": 32, "d2h_bytes_per_step": (R + 1) * nst + 25 + 1}
 
-    # roofline of the dominant kernel: the pass that applies a weight-4 block (psi <- K_m psi / sqrt(N));
-    # in the complex64 forms it also computes the next block's probability (fused: one read + one
-    # write of the register per stabilizer); in the complex128 forms it applies the guessed outcome's
-    # operator and sums |in|^2 and |out|^2 for the decision (one read + one write)
+    # roofline of the instrumented span, the middle round's: on the surface code's c128tc form one pass of a
+    # weight-4 X block (k_ozs: one read and one write of the register); otherwise the whole round, which
+    # reads and writes the register once per pass, several blocks to a pass
     ms_prob = float(np.mean([k[0] for k in kt]))
     ms_apply = float(np.mean([k[1] for k in kt]))
     amps = 1 << 25
-    # 16x16 complex mat-vec per 16 amplitudes: 16 cmacs/amp; the FP64 speculative pass adds |in|^2 and
-    # |out|^2 (2 FMA each per amplitude)
-    flops_apply = amps * (16 * 8 + (8 if args.precision == "c128" else 0))
-    bytes_apply = amps * (32 if args.precision in ("c128", "c128tc") else 16)
-    if args.precision == "c128":
-        roof = {"bound": "alu", "achieved": flops_apply / (ms_apply * 1e-3) / 1e12, "peak": FP64_PEAK_TFLOPS,
-                "unit": "TFLOP/s"}
+    f64 = args.precision in ("c128", "c128tc")
+    one_pass = args.precision == "c128tc" and args.code == "surface"
+    passes = 1 if one_pass else ROUND_PASSES[args.code, f64]
+    bytes_apply = passes * amps * (32 if f64 else 16)
+    if args.precision == "c128" and args.code == "surface":
+        roof = {"bound": "alu", "achieved": amps * ROUND_FP64_FMA * 2 / (ms_apply * 1e-3) / 1e12,
+                "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s"}
     else:
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
         roof = {"bound": "hbm", "achieved": bytes_apply / (ms_apply * 1e-3) / 1e9, "peak": peaks["hbm_gbs"],
                 "unit": "GB/s"}
     roof["frac"] = roof["achieved"] / roof["peak"]
-    # the fused pass of a pair of two weight-2 blocks (a quarter of the stabilizer pairs at d = 5),
-    # instrumented on three more trajectories after the timed region
-    if args.code == "surface" and args.precision != "c128":
+    # the pass of a weight-2 X block, instrumented on three more trajectories after the timed region
+    if one_pass:
         blk = capi.qec_select_timed_block(sims[0].h, 2, 2)
         ms22 = []
         for t in range(3):
@@ -339,36 +343,39 @@ def native_arm(args, rank, world, local):
             ms22.append(capi.qec_kernel_times(sims[0].h)[1])
         ms22 = float(np.median(ms22))
         roof["weight2_pair"] = {
-            "kernel": {"c64": "k_fused_spec<2,false> (weight-2 block)", "c64tc": "k_fused_spec<2,false> (CUDA cores)",
-                       "c128tc": "k_ozs<false> (weight-2 block as K (x) I)"}[args.precision],
+            "kernel": "k_ozs<false> (weight-2 block as K (x) I)",
             "block": blk, "ms": ms22, "achieved": bytes_apply / (ms22 * 1e-3) / 1e9,
             "frac": bytes_apply / (ms22 * 1e-3) / 1e9 / roof["peak"], "unit": "GB/s"}
-    roof["traffic"] = traffic_record(args.precision)
-    roof["kernel"] = {"c128": "k_apply_spec<4,false> (FP64: speculative apply of a weight-4 block, the outcome "
-                              "guessed from the previous round, + FP64 |in|^2 and |out|^2 sums, 2^25 amplitudes)",
-                      "c64": "k_fused_spec<4,false> (FP32: speculative apply of a weight-4 block, the outcome guessed "
-                             "from the previous round, + |in|^2 and |out|^2 sums, 2^25 amplitudes)",
-                      "c64tc": "k_fused_tc_spec<false> (tcgen05 3xTF32: speculative apply of a weight-4 block, the "
-                               "outcome guessed from the previous round, + |in|^2 and |out|^2 sums, 2^25 amplitudes)",
-                      "c128tc": "k_ozs<false> (tcgen05: speculative apply of a weight-4 block, the outcome guessed "
-                                "from the previous round, as FP64-exact 8-bit-slice products + bounded |in|^2 and "
-                                "|out|^2 sums on the same tiles, 2^25 amplitudes)",
-                      }[args.precision]
-    if args.code == "repetition":
-        roof["kernel"] = roof["kernel"].replace("weight-4 block", "weight-2 block Z_k Z_(k+1)")
+    roof["traffic"] = traffic_record(args.precision) if args.code == "surface" else None
+    if one_pass:
+        roof["kernel"] = ("k_ozs<false> (tcgen05: a weight-4 X block's Kraus operator of the outcome guessed from the "
+                          "previous round, as FP64-exact 8-bit-slice products + bounded |in|^2 and |out|^2 sums on the "
+                          "same tiles, 2^25 amplitudes)")
+    elif args.code == "surface":
+        roof["kernel"] = ("a round of 24 blocks on 2^25 amplitudes in %d passes: k_rounds<%s> (X blocks, rotations and "
+                          "diagonals, outcomes guessed from the previous round and decided from |.|^2 sums) and "
+                          "k_diagonals<%s> (Z blocks), reruns of passes with a wrong guess included"
+                          % (passes, "double" if f64 else "float", "double" if f64 else "float"))
+    else:
+        roof["kernel"] = ("a round of 24 blocks Z_k Z_(k+1) on 2^25 amplitudes in %d passes: k_diagonals<%s>, reruns "
+                          "included" % (passes, "double" if f64 else "float"))
+    roof["passes"] = passes
     roof["ms_apply"] = ms_apply
     roof["ms_prob"] = ms_prob
     roof["apply_hbm_gbs"] = bytes_apply / (ms_apply * 1e-3) / 1e9
     roof["timed_blocks"] = len(kt)
 
-    # launches per trajectory: instantiate; the complex64 forms: the first block's probability pass,
-    # per later block one fused pass, the last block's apply; the complex128 forms: per block the
-    # speculative pass and the corrective launch (returns at once unless the guess was wrong), with
-    # the exact-probability launch between them on the tensor cores (returns at once unless the
-    # bound left the outcome open); the readout (3)
+    # launches per trajectory: the compilation of every round's blocks (2, and the X blocks' dense operators
+    # in c128tc); per round c128tc: per X block the speculative pass, the exact-probability check and the
+    # corrective launch, then the diagonal passes (1); the other forms: the X blocks' passes (1) and the
+    # diagonal ones (1); the repetition code: the diagonal ones (1); the readout (3)
     S = nst * R
-    launches_per_traj = {"c128": 1 + 2 * S + 3, "c128tc": 1 + 3 * S + 3,
-                         "c64": 1 + 2 * S + 3, "c64tc": 1 + 2 * S + 3}[args.precision]
+    if args.code == "repetition":
+        launches_per_traj = 2 + R + 3
+    elif args.precision == "c128tc":
+        launches_per_traj = 2 + 1 + R * (3 * 12 + 1) + 3
+    else:
+        launches_per_traj = 2 + 2 * R + 3
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": 1e3 * secs / args.steps, "higher_is_better": True,
@@ -408,7 +415,8 @@ def native_arm(args, rank, world, local):
 
 def batched_arm(args, rank, world, local):
     """8192 d=3 reduced-register trajectories (half complex128, half complex64, per-trajectory p and
-    theta) per step, one persistent launch; the CTA shape is autotuned on a 1024-trajectory sample."""
+    theta) per step, one launch per engine on parallel streams; the CTA shapes are autotuned on a
+    1024-trajectory sample."""
     import torch
 
     from paper_2204_11404_gb300.simulator import BatchSimulator

@@ -41,33 +41,29 @@ typedef enum { QEC_CODE_SURFACE = 0, QEC_CODE_REPETITION = 1 } qec_code;
  * with data corrections after each part (Sec. III.A, Fig. 4). */
 typedef enum { QEC_GATES_CNOT = 0, QEC_GATES_CR = 1 } qec_gateset;
 
-/* Amplitude storage / arithmetic.  C128: complex128 state, FP64 arithmetic, one
- * speculative pass per block as described under C128_TC, with FP64 sums that
- * decide every outcome directly.
- * C64: complex64 state, FP32 gate arithmetic, FP64 probability reductions;
- * one speculative pass per block as described under C128_TC (FP32 sums per
- * tile, FP64 across tiles, deciding every outcome directly).
- * C64_TC: complex64 state; the speculative pass of every weight-4 block on the
- * tensor cores (3xTF32 split, FP32 accumulation; tiles of 2^12 amplitudes, so
- * d >= 5), of the weight-2 blocks as C64; FP64 reductions across tiles.  With
- * the speculative passes off, the fused apply + next-probability pass of every
- * pair of blocks with a weight-4 block on the tensor cores (a weight-2 block of
- * the pair as K (x) I over two spectator qubits), pairs of weight-2 blocks on
- * the CUDA cores.
- * C128_TC: complex128 state; the apply of every stabilizer block (tiles of
- * 2^11 amplitudes, so registers of at least 11 qubits: the d = 5 surface code
- * and the repetition code from d = 11; smaller registers as C128) as emulated
- * FP64 products on the FP16 tensor cores: each operand row split into 7
- * signed 8-bit slices under one exponent, slice products accumulated exactly,
- * recombined in integers and rounded once (Ozaki scheme).  One speculative
- * pass per block (qec_debug_speculation): it applies the Kraus operator of the
- * outcome the same stabilizer gave one round earlier (the init round's for the
- * first noisy round) into a second working state, and on the same tiles sums
- * |input|^2 and |output|^2 as 24-bit truncations with rigorous error bounds;
- * the outcome is decided from them where the bounds settle it, else by the
- * exact pass on the untouched input (qec_debug_exact_probability), and a wrong
- * guess is re-applied from that input.  Init and readout in FP64.  Same
- * outcomes and, to within a few FP64 roundings, the same amplitudes as C128. */
+/* Amplitude storage / arithmetic.  Every form runs a stabilizer block's Kraus operator in factored
+ * form (one rotation per data qubit, a diagonal per outcome, index flips; qec_debug_factors), on one of
+ * two engines.  On chip: registers of up to 13 data qubits (complex128 at 13 qubits: calls of more than
+ * 64 trajectories), whole trajectories in shared memory.  In passes over the state in HBM otherwise,
+ * several blocks to a pass: run for the outcomes the same stabilizers gave one round earlier (the init
+ * round's for the first noisy round) into a second working state, decided from the sums of squares after
+ * every block, and run again from the untouched input where a guess was wrong.  Registers of 21 qubits and
+ * more run the Z part of a round (all of the repetition code's) as diagonal passes, its rotations
+ * joined to the X part's.
+ * C128: complex128 state, FP64 arithmetic and sums.
+ * C64: complex64 state, FP32 gate arithmetic, FP64 reductions of FP32 partial sums.
+ * C64_TC: the same factored engines as C64 (rotations and diagonals leave no contraction for the tensor
+ * cores to do).  With speculation off (qec_debug_speculation) the fused apply + next-probability
+ * pass of every pair of blocks with a weight-4 block runs on the tensor cores (3xTF32 split, FP32
+ * accumulation; tiles of 2^12 amplitudes, so d >= 5).
+ * C128_TC: complex128 state; below 21 data qubits as C128.  From 21 the X blocks (and the repetition
+ * code's blocks when round-start terms rotate them) run as emulated FP64 products on the FP16
+ * tensor cores, one speculative pass per block: each operand row split into 7 signed 8-bit slices
+ * under one exponent, slice products accumulated exactly, recombined in integers and rounded once (Ozaki
+ * scheme); on the same tiles |input|^2 and |output|^2 are summed as 24-bit truncations with
+ * rigorous error bounds, and the outcome is decided from them where the bounds settle it, else by the
+ * exact pass on the untouched input (qec_debug_exact_probability).  Init, Z part and readout in FP64.
+ * Same outcomes and, to within a few FP64 roundings, the same amplitudes as C128. */
 typedef enum { QEC_C128 = 0, QEC_C64 = 1, QEC_C64_TC = 2, QEC_C128_TC = 3 } qec_precision;
 
 /* Noise (Sec. III.A).  Probabilities in [0, 1]; angles in radians, |angle| <= 4. */
@@ -175,26 +171,23 @@ qec_status qec_record_events(qec_sim* sim, uint32_t max_events);
 qec_status qec_get_events(qec_sim* sim, int32_t* host_events, uint32_t max_events, uint32_t* count);
 
 /*
- * Measurement hook: device time in milliseconds of the probability pass
- * (ms[0]) and of the collapse/apply pass (ms[1]) of one weight-4 stabilizer
- * block of the middle noisy round, in the most recent trajectory (CUDA events
- * recorded inside the trajectory's graph).  With the fused passes ms[0] is
- * empty for a block whose probability the previous pass computed; with the
- * speculative passes (the complex128 forms) ms[0] is empty and ms[1] is the
- * block's speculative pass, without the launches that complete it.  *block gets that block's index
- * (round-major, d^2-1 per round).  QEC_EINVAL if no trajectory ran yet or the
- * sim has no noisy round.
+ * Measurement hook: device time in milliseconds around one block of the middle noisy round (a weight-4
+ * block unless qec_select_timed_block chose another) in the most recent call's first trajectory.
+ * ms[1]: the block's own pass where it has one (C128_TC's tensor-core passes, without the launches
+ * that complete them; the passes with speculation off); the round that holds it on registers of 21
+ * qubits and more in the factored passes; all rounds of the trajectories that run side by side on
+ * smaller ones; the whole launch on chip.  ms[0]: the probability pass before it where that is a pass of
+ * its own (speculation off), else empty.  *block gets the block's index (round-major, as many per round
+ * as the code has stabilizers).  QEC_EINVAL if no trajectory ran yet or the sim has no noisy round.
  */
 qec_status qec_kernel_times(qec_sim* sim, float* ms, int32_t* block);
 
 /*
- * Measurement hook: instrument, from the next trajectory on, the first block
- * of the middle noisy round whose weight is w_apply and whose successor's
- * weight is w_next (2 or 4; ms[1] of qec_kernel_times is then that block's
- * speculative pass, or with the fused passes the pass that applies that block
- * and computes its successor's probability).  *block gets its index.  QEC_EINVAL if the sim has no noisy
- * round or no such pair of blocks.  The trajectory graph is rebuilt at the
- * next run; results do not change.
+ * Measurement hook: instrument, from the next trajectory on, the first block of the middle noisy round
+ * whose weight is w_apply and whose successor's weight is w_next (2 or 4; see qec_kernel_times for
+ * the span that is timed; with the fused passes of speculation off it is the pass that applies that
+ * block and computes its successor's probability).  *block gets its index.  QEC_EINVAL if the sim has
+ * no noisy round or no such pair of blocks.  Results do not change.
  */
 qec_status qec_select_timed_block(qec_sim* sim, int32_t w_apply, int32_t w_next, int32_t* block);
 
@@ -217,15 +210,13 @@ qec_status qec_selftest_wait(qec_sim* sim, uint32_t polls);
  * parameters, the trajectory range and DEVICE output buffers with the shapes
  * of qec_run_trajectories (all three required when n > 0); results are
  * identical to qec_run_trajectories for the same parameters, seed and
- * trajectory indices: it launches the same kernels with the same grids in the
- * same order (per block the speculative pass and its corrective launch, over
- * two working states), so every reduction adds in the same order.  Work
- * is enqueued asynchronously on cuda_stream (NULL = the legacy default
- * stream); no sim handle is involved.  At the sizes it accepts none of its
- * kernels waits on a barrier or flag, so it has no bounded-wait timeout to
- * report.
- * All device working memory (program, state vectors, Kraus blocks, reduction
- * and readout scratch) is one static 2 MiB device array inside the library,
+ * trajectory indices: after the init round it launches the same on-chip kernel
+ * (one CTA per trajectory, the register in shared memory).  Work is enqueued
+ * asynchronously on cuda_stream (NULL = the legacy default stream); no sim
+ * handle is involved.  At the sizes it accepts none of its kernels waits on a
+ * barrier or flag of another CTA, so it has no bounded-wait timeout to report.
+ * All device working memory (program, init state, the init round's Kraus blocks
+ * and reduction scratch) is one static 2 MiB device array inside the library,
  * which every GPU that loads the library holds until the process exits.  It
  * fits d = 3 with at most 16 noisy rounds; larger requests return QEC_EINVAL.
  * The first call on a device looks up that array's device address (once per
@@ -238,7 +229,7 @@ qec_status qec_run_trajectories_noalloc(const qec_params* params, uint64_t seed,
                                         uint8_t* d_syndromes, uint8_t* d_data_bits, uint8_t* d_raw_logical,
                                         void* cuda_stream);
 
-/* ---- Batched form: many small-register trajectories in one persistent launch ----------- */
+/* ---- Batched form: many small-register trajectories at once ----------------------------- */
 typedef struct qec_batch qec_batch;
 
 /*
@@ -246,8 +237,8 @@ typedef struct qec_batch qec_batch;
  * + reused ancilla, Sec. II.B), `rounds` noisy rounds, gate set `gates`.
  * A trajectory runs on chip, its blocks as rotations and diagonals: one warp
  * each in a persistent launch that takes trajectories from a device work
- * counter, or one CTA each where there are at most four per SM.  max_traj bounds n of every run.  Only d = 3 is
- * accepted (QEC_EUNSUPPORTED otherwise).  cuda_stream as in qec_create.
+ * counter, or one CTA each where there are at most four per SM.  max_traj
+ * bounds n of every run.  Only d = 3 is accepted (QEC_EUNSUPPORTED otherwise).  cuda_stream as in qec_create.
  */
 qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t max_traj, void* cuda_stream,
                             qec_batch** out);
@@ -274,9 +265,9 @@ qec_status qec_batch_run(qec_batch* b, uint64_t seed, uint32_t n, const uint64_t
  * register: the reduced-register engine's CTA shape (warps per CTA, one
  * resident wave per SM), then the unreduced engine's fusion width k (2..6 slab
  * bits per sweep: above 4 a weight-4 stabilizer's four data qubits are rotated
- * in one sweep, else two at a time) and threads per CTA (128, 256).  *chosen_warps gets the reduced engine's warps per CTA, *best_ms the
- * device time of the whole sample with the chosen configuration;
- * qec_batch_config reports all three choices.
+ * in one sweep, else two at a time) and threads per CTA (128, 256).
+ * *chosen_warps gets the reduced engine's warps per CTA, *best_ms the device
+ * time of the whole sample with the chosen configuration; qec_batch_config reports all three choices.
  */
 qec_status qec_batch_autotune(qec_batch* b, uint64_t seed, uint32_t n, const uint64_t* traj, const int32_t* kind,
                               const qec_noise* noise, int32_t* chosen_warps, float* best_ms);
@@ -306,7 +297,7 @@ qec_status qec_batch_snapshot(qec_batch* b, int64_t item);
  */
 qec_status qec_batch_get_state(qec_batch* b, void* host_buf, size_t bytes);
 
-/* Device time (ms, CUDA events around the persistent launch) of the last qec_batch_run. */
+/* Device time (ms, CUDA events around the launches) of the last qec_batch_run. */
 qec_status qec_batch_last_ms(const qec_batch* b, float* ms);
 qec_status qec_batch_destroy(qec_batch* b);
 
@@ -392,6 +383,8 @@ qec_status qec_debug_ozaki_gemm(const double* A, const double* B, int32_t m, int
  * qec_debug_speculation), or A from the top 3 of the 7 slices of each operand in the fused pass;
  * the device decides when |u N - A| exceeds twice the bound plus 1e-10 (A + N), where the exact
  * pass must decide the same way, and otherwise runs the exact pass.  force = 1: every outcome goes through the exact pass; 0: the default; -1: unchanged.
+ * Blocks outside the tensor-core passes are always decided from exact sums; the diagonal passes
+ * count theirs here when force is 1.
  * *fallbacks (may be NULL) receives the number of exact passes run on this handle so far.
  * Waits for the handle's queued work.  QEC_EINVAL on a null handle or force outside -1..1.
  */
@@ -399,14 +392,14 @@ qec_status qec_debug_exact_probability(qec_sim* sim, int32_t force, uint64_t* fa
 
 /*
  * Test hook (the paper has no counterpart: an evaluation order of Sec. II.B's measurement and
- * collapse).  enable = 1: the speculative passes (the default); 0: the passes that compute each
- * probability before its apply (QEC_C128: a probability pass and an apply pass per block;
+ * collapse).  enable = 1: the engines described at qec_precision (the default); 0: passes in HBM, at any
+ * register size, that compute each probability before its apply (QEC_C128: a probability pass and an apply pass per block;
  * QEC_C128_TC: per block pair, the apply fused with the next block's 3-slice bounded
  * probability; the complex64 forms: the apply fused with the next block's probability);
  * -1: unchanged.  Both give the same outcomes (except within the rounding of a threshold) and
  * states within a few roundings of the form's arithmetic.  *misses (may be NULL) receives the
- * number of corrective applies run on this handle so far (outcomes that differed from the
- * guess).  Waits for the handle's queued work; switching rebuilds the trajectory graph and
+ * number of outcomes on this handle so far that differed from the same stabilizer's one round
+ * earlier (in passes: that differed from the guess).  Waits for the handle's queued work; switching
  * requires a new run before qec_get_state.  QEC_EINVAL on a null handle or enable outside
  * -1..1.
  */

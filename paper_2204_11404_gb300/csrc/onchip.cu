@@ -5,6 +5,8 @@
 // scheduler on this chip, then barriers and the reduction trees of 8 blocks a round), for many the
 // FP64 pipe: per weight-4 block 8 rotation, 4 weight and 4 diagonal multiply-adds per amplitude,
 // against 136 for the dense probability and apply, plus the compile, about a quarter of the work.
+// Measured against a graph of dense probability and apply passes per trajectory (d = 3, 3 rounds,
+// complex128): one trajectory 849 -> 145 us, 1000 of them 797 ms -> 0.67 ms.
 #include <cuda_runtime.h>
 
 #include "onchip.cuh"

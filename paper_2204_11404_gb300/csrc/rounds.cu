@@ -11,6 +11,13 @@
 // Per tile and block a thread holds one group of 16 amplitudes in registers: one rotation per data
 // qubit, the diagonal of the outcome, the squares.  Tiles stream through shared memory (16-byte
 // asynchronous copies in, whole 128-byte runs out); the register is read and written once per pass.
+//
+// What bounds them at d = 5 (2^25 amplitudes): in complex64 the shared-memory sweeps (38% of issue slots, waits
+// on shared memory and barriers; 43% of DRAM throughput): 151 us for a pass of four blocks and 44 for one
+// of one, plus 34 until the last CTA arrives.  In complex128 the FP64 pipe: 550 to 946 us a block, plus 95
+// to 190 at the barrier, where the CTAs that were scheduled first on an SM wait for the others.  Against a
+// dense 16x16 pass per block, five rounds: complex64 19.1 -> 7.6 ms, complex128 359 -> 87; with the Z part
+// in diagonal passes 7.0 and 70.5.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -469,6 +476,10 @@ __global__ void __launch_bounds__(round_threads(TB), (POST ? Shape<T>::CTAS_POST
 // guessed outcomes decide the blocks up to the first wrong guess; those for the corrected path come
 // from the same h.  So the outcomes cost one pass whatever the guesses, and wrong ones one more without
 // sums.
+//
+// At 2^25 amplitudes a complex64 pass takes 68 to 93 us (memory: 512 MiB are 79 at the copy rate) and 17 to 37
+// to decide, a complex128 one 350 (the FP64 pipe: 6 multiply-adds an amplitude are 320; 1 GiB 158) and 8
+// to 15.  The Z part of a d = 5 round, complex128, went from 12 dense tensor-core passes of 0.39 ms to 1.7-2.0.
 constexpr int kDiagThreads = 512;
 __host__ __device__ constexpr int diag_bits(bool f64) { return f64 ? 12 : 13; }
 
@@ -904,7 +915,7 @@ static void choose_swizzle(ChainDesc& c, int precision, int TB) {
   int cost = conflict_cost(c, precision, group_bits(TB)), floor = 0;
   for (int i = 0; i < c.nb; ++i) floor += !is_f64(precision) && c.bits[i][0] != 0 ? 4 : is_f64(precision) ? 8 : 4;
   uint64_t x = 0x9E3779B97F4A7C15ull;
-  for (int t = 0; t < 300 && cost > floor; ++t) {
+  for (int t = 0; t < 100 && cost > floor; ++t) {
     for (int k = 0; k < 3; ++k) {
       x ^= x << 13;
       x ^= x >> 7;

@@ -35,8 +35,8 @@ constexpr int kTileBits = 11, kSmallTileBits = 9;
 std::vector<ChainDesc> plan_chains(const FactorProgram& F, int precision, int tile_bits, int most, int b0, int b1);
 
 // A pass of blocks that rotate no qubit: diagonals only.  Tile as above, but of 2^12 complex128 or 2^13
-// complex64 amplitudes (8 or 16 on each of 512 threads; runs of 128 bytes).  The blocks' data qubits are nu tile bits ubits (ascending; rbits: the other tile bits);
-// at[i][j]: which of them block i's qubit j is.
+// complex64 amplitudes (8 or 16 on each of 512 threads; runs of 128 bytes).  The blocks' data qubits are nu
+// tile bits ubits (ascending; rbits: the other tile bits); at[i][j]: which of them block i's qubit j is.
 constexpr int kMaxDiag = 8;
 constexpr int kDiagUnion = 10;      // at most this many data qubits in a pass
 struct DiagDesc {
