@@ -729,9 +729,9 @@ qec_status run_rounds(qec_sim* s, uint64_t seed, uint64_t first, uint32_t chunk)
         p.src = step == 0 ? s->psi0 : a.buf[(step & 1) ^ 1];
         p.dst = a.buf[step & 1];
         if (tm && block && k == tb) record3();
-        QEC_CUDA(launch_spec(p, s->d_N + k + 1, step == 0, s->num_sms, s->work));
+        QEC_CUDA(launch_spec(p, s->d_N + k + 1, step == 0, s->num_sms, s->work, b > 0));
         if (tm && block && k == tb) QEC_CUDA(cudaEventRecord(s->kev[2], s->work));
-        QEC_CUDA(launch_spec_fix(p, s->d_N + k + 1, step == 0, s->num_sms, s->work));
+        QEC_CUDA(launch_spec_fix(p, s->d_N + k + 1, step == 0, s->num_sms, s->work, true));
       }
       if (a.nc && !tensor) QEC_CUDA(launch_rounds(prec, a, r0, r1, s->work));
       if (a.nd) QEC_CUDA(launch_diagonals(prec, a, r0, s->num_sms, s->work));

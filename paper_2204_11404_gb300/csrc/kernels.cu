@@ -1086,6 +1086,15 @@ __device__ __forceinline__ void put_slices8(uint16_t* S, int slab, int row, int 
   put_digits8<NS>(S, slab, row, k0, X, hw);
 }
 
+// First thing in a kernel that may be launched while the one before it on the stream still runs (a
+// programmatic launch): waits until that one has completed and its writes are visible, after letting
+// the next launch in the same way.  Both do nothing after an ordinary launch.  A launch is let in when every
+// CTA here has started, so CTAs that wait never take the place of ones that they wait for.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // MODE 0 (OZ_APPLY): psi <- K_m psi / sqrt(N).  MODE 1 (OZ_PROB): A = sum |K_1 psi_g|^2 and
 // N = sum |psi|^2 over all groups, then the outcome (K_1^dagger K_1 is the operator M of the FP64
 // pass, so A is the same quantity).  MODE 2 (OZ_PROB_BOUND): the same N exactly, A from the top 3
@@ -1094,6 +1103,7 @@ __device__ __forceinline__ void put_slices8(uint16_t* S, int slab, int row, int 
 // f.skip_unless_uncertain (MODE 1): return at once unless that flag is set.
 template <int MODE>
 __global__ void __launch_bounds__(256, 2) k_oz(FusedArgs f) {
+  after_previous();
   constexpr bool PROB = MODE != OZ_APPLY;
   constexpr int NS = MODE == OZ_PROB_BOUND ? 3 : oz::kSlices;       // slices of each operand
   constexpr int ND = MODE == OZ_PROB_BOUND ? 2 * NS - 1 : oz::kSlices;   // diagonals accumulated
@@ -1697,6 +1707,7 @@ constexpr int kOzsSmem = 16 * (1 << kOzTileBits) + 2 * oz::kSlices * kOzSlab + 2
 
 template <bool FIX>
 __global__ void __launch_bounds__(256, 2) k_ozs(FusedArgs f) {
+  after_previous();
   const int g = spec_guess(f.ap);
   const int m = FIX ? *f.ap.m : g;   // the corrective pass applies the decided outcome ...
   if (FIX && m == g) return;         // ... only where the guess was wrong
@@ -2272,7 +2283,26 @@ bool apply_oz_applies(const PassArgs& ap) {
   return f.nt == kOzTileBits;
 }
 
-static cudaError_t launch_oz(int mode, bool skip_unless_uncertain, const PassArgs& ap, int num_sms, cudaStream_t s) {
+// overlap: a programmatic launch (after_previous): the CTAs are set up while the kernel before them on the
+// stream drains.  Two of a block's three launches usually return at once, so launches and gaps are the
+// cost: five d = 5 rounds 33.07 -> 32.76 ms.
+static cudaError_t launch_ozk(const void* fn, size_t smem, FusedArgs& f, bool overlap, cudaStream_t s) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)f.grid);
+  c.blockDim = dim3(256);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = overlap ? 1 : 0;
+  void* args[1] = {&f};
+  return cudaLaunchKernelExC(&c, fn, args);
+}
+
+static cudaError_t launch_oz(int mode, bool skip_unless_uncertain, const PassArgs& ap, int num_sms, cudaStream_t s,
+                             bool overlap = false) {
   FusedArgs f;
   f.ap = ap;
   f.pr = ap;
@@ -2291,10 +2321,9 @@ static cudaError_t launch_oz(int mode, bool skip_unless_uncertain, const PassArg
   if (g > MAX_PASS_GRID) g = MAX_PASS_GRID;
   if (mode == OZ_PROB_BOUND && 3 * g > 2 * MAX_PASS_GRID) g = 2 * MAX_PASS_GRID / 3;   // 3 partial sums per CTA
   f.grid = (int)g;
-  if (mode == OZ_APPLY) k_oz<OZ_APPLY><<<f.grid, 256, kOzSmem, s>>>(f);
-  else if (mode == OZ_PROB) k_oz<OZ_PROB><<<f.grid, 256, kOzSmem, s>>>(f);
-  else k_oz<OZ_PROB_BOUND><<<f.grid, 256, kOzSmem, s>>>(f);
-  return cudaGetLastError();
+  const void* fn = mode == OZ_APPLY ? (const void*)k_oz<OZ_APPLY>
+                   : mode == OZ_PROB ? (const void*)k_oz<OZ_PROB> : (const void*)k_oz<OZ_PROB_BOUND>;
+  return launch_ozk(fn, kOzSmem, f, overlap, s);
 }
 
 cudaError_t launch_apply_oz(const PassArgs& ap, int num_sms, cudaStream_t s) {
@@ -2367,22 +2396,20 @@ static bool spec_args(const PassArgs& ap, double* n_next, bool unit_in, int num_
   return true;
 }
 
-cudaError_t launch_spec(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s) {
+cudaError_t launch_spec(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s, bool overlap) {
   FusedArgs f;
   if (!spec_args(ap, n_next, unit_in, num_sms, f)) return cudaErrorInvalidValue;
-  k_ozs<false><<<f.grid, 256, kOzsSmem, s>>>(f);
-  return cudaGetLastError();
+  return launch_ozk((const void*)k_ozs<false>, kOzsSmem, f, overlap, s);
 }
 
-cudaError_t launch_spec_fix(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s) {
+cudaError_t launch_spec_fix(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s, bool overlap) {
   FusedArgs f;
   if (!spec_args(ap, n_next, unit_in, num_sms, f)) return cudaErrorInvalidValue;
   PassArgs a = ap;
   a.store_n = 0;   // *N keeps the scale both applies of this block use
-  cudaError_t e = launch_oz(OZ_PROB, true, a, num_sms, s);
+  cudaError_t e = launch_oz(OZ_PROB, true, a, num_sms, s, overlap);
   if (e != cudaSuccess) return e;
-  k_ozs<true><<<f.grid, 256, kOzsSmem, s>>>(f);
-  return cudaGetLastError();
+  return launch_ozk((const void*)k_ozs<true>, kOzsSmem, f, overlap, s);
 }
 
 cudaError_t launch_wait_selftest(unsigned int* status, long limit, cudaStream_t s) {

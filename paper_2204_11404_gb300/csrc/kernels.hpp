@@ -137,11 +137,14 @@ cudaError_t launch_fused_oz(const PassArgs& ap, const PassArgs& pr, int num_sms,
 cudaError_t launch_prob_oz_check(const PassArgs& pr, int num_sms, cudaStream_t s);
 // Speculative complex128 pass on the tensor cores of block ap (ap.src and ap.dst distinct buffers): applies
 // K_g / sqrt(*ap.N) (scale 1 with unit_in) for the guessed outcome g, decides the outcome where its
-// bound allows, and stores |output|^2 in *n_next (n_next may be null).
-cudaError_t launch_spec(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s);
+// bound allows, and stores |output|^2 in *n_next (n_next may be null).  overlap: a programmatic launch; the
+// kernel before it on the stream is a k_ozs or k_oz (any other completes first).
+cudaError_t launch_spec(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s,
+                        bool overlap = false);
 // Its completion: the exact probability launch (returns at once unless the bound left the outcome
 // open), then the corrective apply (returns at once unless the outcome is not g).
-cudaError_t launch_spec_fix(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s);
+cudaError_t launch_spec_fix(const PassArgs& ap, double* n_next, bool unit_in, int num_sms, cudaStream_t s,
+                            bool overlap = false);
 int pass_grid(int D, int w, int num_sms);
 // One wave of resident CTAs for the probability (prob = true) or apply pass kernel.
 int pass_grid_for(int precision, bool prob, int D, int w, int num_sms);
