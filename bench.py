@@ -230,7 +230,7 @@ def traffic_record(precision):
 
 def kernel_source_sha():
     h = hashlib.sha256()
-    for f in ("kernels.cu", "ozaki.cuh", "rounds.cu", "onchip.cuh", "factor.cuh"):
+    for f in ("kernels.cu", "ozaki.cuh", "rounds.cu", "onchip.cuh"):   # the passes and what they include
         h.update(open(os.path.join(ROOT, "paper_2204_11404_gb300", "csrc", f), "rb").read())
     return h.hexdigest()
 
