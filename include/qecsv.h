@@ -41,11 +41,13 @@ typedef enum { QEC_CODE_SURFACE = 0, QEC_CODE_REPETITION = 1 } qec_code;
  * with data corrections after each part (Sec. III.A, Fig. 4). */
 typedef enum { QEC_GATES_CNOT = 0, QEC_GATES_CR = 1 } qec_gateset;
 
-/* Amplitude storage / arithmetic.  Every form runs a stabilizer block's Kraus operator in factored
- * form (one rotation per data qubit, a diagonal per outcome, index flips; qec_debug_factors), on one of
- * two engines.  On chip: registers of up to 13 data qubits (complex128 at 13 qubits: calls of more than
- * 64 trajectories), whole trajectories in shared memory.  In passes over the state in HBM otherwise,
- * several blocks to a pass: run for the outcomes the same stabilizers gave one round earlier (the init
+/* Amplitude storage / arithmetic.  A stabilizer block's Kraus operator runs in factored form (one rotation per
+ * data qubit, a diagonal per outcome, index flips; qec_debug_factors) or as its dense matrix, on one of two
+ * engines.  On chip: registers of up to 13 data qubits (complex128 at 13 qubits: calls of more than
+ * 64 trajectories), whole trajectories in shared memory; complex128 factored, complex64 dense, whose
+ * states are the same to the last FP32 place from one version to the next (in the factored passes below
+ * a complex64 state is reproducible to FP32 rounding between versions).  In passes over the state in HBM otherwise,
+ * factored, several blocks to a pass: run for the outcomes the same stabilizers gave one round earlier (the init
  * round's for the first noisy round) into a second working state, decided from the sums of squares after
  * every block, and run again from the untouched input where a guess was wrong.  Registers of 21 qubits and
  * more run the Z part of a round (all of the repetition code's) as diagonal passes, its rotations
@@ -210,7 +212,7 @@ qec_status qec_selftest_wait(qec_sim* sim, uint32_t polls);
  * parameters, the trajectory range and DEVICE output buffers with the shapes
  * of qec_run_trajectories (all three required when n > 0); results are
  * identical to qec_run_trajectories for the same parameters, seed and
- * trajectory indices: after the init round it launches the same on-chip kernel
+ * trajectory indices: after the init round it launches the same on-chip kernels
  * (one CTA per trajectory, the register in shared memory).  Work is enqueued
  * asynchronously on cuda_stream (NULL = the legacy default stream); no sim
  * handle is involved.  At the sizes it accepts none of its kernels waits on a

@@ -13,6 +13,7 @@
 
 #include "../../include/qecsv.h"
 #include "common.cuh"
+#include "dense.hpp"
 #include "factor.cuh"
 #include "kernels.hpp"
 #include "onchip.hpp"
@@ -81,6 +82,11 @@ struct qec_sim {
   const void* last_state = nullptr;     // of the last run in factored passes: its state and flips
   const uint32_t* last_masks = nullptr;
   uint8_t* h_out = nullptr;             // pinned outputs of an on-chip batch, written by the kernel
+  // complex64 on chip (dense.cu): Kraus pairs and uniforms of up to dense_cap blocks
+  float2* d_dense = nullptr;
+  double* d_dense_u = nullptr;
+  uint32_t dense_cap = 0;
+  int dense_entries = 0;
   int D = 0, nstab = 0, R = 0, S = 0;
   size_t amp = 16;
   void* psi = nullptr;
@@ -461,7 +467,7 @@ void drop_graph(qec_sim* s) {
 void free_all(qec_sim* s) {
   drop_graph(s);
   if (s->h_out) cudaFreeHost(s->h_out);
-  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_factor, s->d_rounds, s->d_kraus, s->d_u, s->d_A, s->d_N, s->d_m,
+  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_factor, s->d_rounds, s->d_dense, s->d_dense_u, s->d_kraus, s->d_u, s->d_A, s->d_N, s->d_m,
                   s->d_partials, s->d_ctl,
                   s->d_hist_part, s->d_hist, s->d_syn, s->d_bits, s->d_log, s->d_events,
                   s->d_ops[0], s->d_ops[1], s->d_blocks[0], s->d_blocks[1], s->d_mats[0], s->d_mats[1]};
@@ -506,7 +512,8 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   for (int i = 0; i < kCtlRing && e == cudaSuccess; ++i)
     e = cudaEventCreateWithFlags(&s->ctl_ev[i], cudaEventDisableTiming);
   if (e == cudaSuccess) e = setup_kernels(s->p.precision, s->D);
-  if (e == cudaSuccess && onchip_applies(s->D)) e = setup_onchip();
+  if (e == cudaSuccess && dense_applies(s->p.precision, s->D)) e = setup_dense(s->D);
+  else if (e == cudaSuccess && onchip_applies(s->D)) e = setup_onchip();
   if (e != cudaSuccess) return bail(fail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e)));
   const size_t state_bytes = ((size_t)1 << s->D) * s->amp;
   const int nblk = s->nstab * kMaxRounds;   // room for any round count (qec_reconfigure)
@@ -587,6 +594,14 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
       e = cudaMemcpyAsync(s->d_diags, s->diags.data(), sizeof(DiagDesc) * s->diags.size(), cudaMemcpyHostToDevice, s->work);
     if (e != cudaSuccess) return bail(fail(QEC_ECUDA, cudaGetErrorString(e)));
   }
+  if (dense_applies(s->p.precision, s->D)) {
+    // 32 MiB of pairs with weight-4 blocks (340 trajectories of 3 rounds to a launch), 4 MiB without
+    s->dense_entries = dense_entries(s->prog);
+    s->dense_cap = s->dense_entries == 256 ? 8192u : 16384u;
+    if ((st = dmalloc(&s->d_dense, sizeof(float2) * 2 * s->dense_entries * s->dense_cap)) ||
+        (st = dmalloc(&s->d_dense_u, sizeof(double) * s->dense_cap)))
+      return bail(st);
+  }
   if (onchip_applies(s->D)) {
     e = cudaMallocHost((void**)&s->h_out, (size_t)kBatchCap * (s->syn_cap + s->D + 1));
     if (e != cudaSuccess) return bail(fail(QEC_ENOMEM, "pinned allocation failed"));
@@ -615,45 +630,82 @@ qec_status send_header(qec_sim* s, uint64_t seed, uint64_t first, bool reset_eve
   return QEC_OK;
 }
 
-// Trajectories on chip: one launch per kBatchCap of them.  Host outputs are written by the kernel
-// straight into pinned memory, device outputs into the caller's buffers.
-qec_status run_onchip(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8_t* syn, uint8_t* bits,
-                      uint8_t* logical, bool host_out) {
-  const size_t ss = (size_t)s->syn_stride(), bs = (size_t)s->D;
+// The arguments of the on-chip engines: factored blocks (complex128), dense ones (complex64).
+OnchipArgs onchip_args(const qec_sim* s) {
   OnchipArgs a;
   a.F = device_factor(s);
   for (int i = 0; i < PR_COUNT; ++i) a.thr[i] = fac::draw_threshold(s->prog.prob[i]);
   std::memcpy(a.fm, s->fm, sizeof(a.fm));
+  return a;
+}
+DenseArgs dense_args(const qec_sim* s) {
+  DenseArgs a;
+  a.ops = s->d_ops[1];
+  a.blocks = s->d_blocks[1];
+  a.mats = s->d_mats[1];
+  for (int i = 0; i < PR_COUNT; ++i) a.prob[i] = s->prog.prob[i];
+  a.nstab = s->nstab;
+  a.nd = s->D;
+  a.entries = s->dense_entries;
+  a.kraus = s->d_dense;
+  a.u = s->d_dense_u;
+  return a;
+}
+
+// Trajectories on chip, up to `most` to a launch.  Host outputs are written by the kernel straight into
+// pinned memory, kBatchCap trajectories at a time, device outputs into the caller's buffers.
+template <typename A, typename L>
+qec_status run_chunks(qec_sim* s, A a, uint32_t most, L launch, uint64_t seed, uint64_t first, uint32_t n, uint8_t* syn,
+                      uint8_t* bits, uint8_t* logical, bool host_out) {
+  const size_t ss = (size_t)s->syn_stride(), bs = (size_t)s->D;
   a.seed = seed;
   a.rounds = s->R;
   a.nl = s->p.d;
   a.psi0 = s->psi0;
   a.ctl = s->d_ctl;
   a.events = s->ev_cap ? s->d_events : nullptr;
-  for (uint32_t done = 0; done < n;) {
-    const uint32_t chunk = host_out && n - done > kBatchCap ? kBatchCap : n - done;
-    if (s->ev_cap && done == 0) {
-      qec_status st = send_header(s, seed, first, true);
-      if (st) return st;
+  if (s->ev_cap && n) {
+    qec_status st = send_header(s, seed, first, true);
+    if (st) return st;
+  }
+  for (uint32_t done = 0; done < n;) {   // (a call's host outputs: a group of chunks at a time)
+    const uint32_t group = host_out && n - done > kBatchCap ? kBatchCap : n - done;
+    uint8_t* const to[3] = {!syn ? nullptr : host_out ? s->h_out : syn + done * ss,
+                            !bits ? nullptr : host_out ? s->h_out + group * ss : bits + done * bs,
+                            !logical ? nullptr : host_out ? s->h_out + group * (ss + bs) : logical + done};
+    for (uint32_t at = 0; at < group; at += a.n) {
+      a.n = group - at < most ? group - at : most;
+      a.first = first + done + at;
+      a.psi_out = done + at + a.n == n ? s->psi : nullptr;
+      a.syn = to[0] ? to[0] + at * ss : nullptr;
+      a.bits = to[1] ? to[1] + at * bs : nullptr;
+      a.logical = to[2] ? to[2] + at : nullptr;
+      const bool timed = done + at == 0;
+      if (timed) QEC_CUDA(cudaEventRecord(s->kev[1], s->work));
+      QEC_CUDA(launch(a));
+      if (timed) QEC_CUDA(cudaEventRecord(s->kev[2], s->work));
     }
-    a.first = first + done;
-    a.n = chunk;
-    a.psi_out = done + chunk == n ? s->psi : nullptr;
-    a.syn = !syn ? nullptr : host_out ? s->h_out : syn + done * ss;
-    a.bits = !bits ? nullptr : host_out ? s->h_out + chunk * ss : bits + done * bs;
-    a.logical = !logical ? nullptr : host_out ? s->h_out + chunk * (ss + bs) : logical + done;
-    if (done == 0) QEC_CUDA(cudaEventRecord(s->kev[1], s->work));
-    QEC_CUDA(launch_onchip(s->p.precision, a, s->num_sms, s->work));
-    if (done == 0) QEC_CUDA(cudaEventRecord(s->kev[2], s->work));
     if (host_out) {
       QEC_CUDA(cudaStreamSynchronize(s->work));
-      if (syn) std::memcpy(syn + done * ss, a.syn, chunk * ss);
-      if (bits) std::memcpy(bits + done * bs, a.bits, chunk * bs);
-      if (logical) std::memcpy(logical + done, a.logical, chunk);
+      if (syn) std::memcpy(syn + done * ss, to[0], group * ss);
+      if (bits) std::memcpy(bits + done * bs, to[1], group * bs);
+      if (logical) std::memcpy(logical + done, to[2], group);
     }
-    done += chunk;
+    done += group;
   }
   return QEC_OK;
+}
+
+qec_status run_onchip(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8_t* syn, uint8_t* bits,
+                      uint8_t* logical, bool host_out) {
+  if (!dense_applies(s->p.precision, s->D))
+    return run_chunks(s, onchip_args(s), 0xffffffffu,
+                      [&](const OnchipArgs& a) { return launch_onchip(a, s->num_sms, s->work); }, seed, first, n, syn,
+                      bits, logical, host_out);
+  const uint32_t most = std::max<uint32_t>(s->dense_cap / (uint32_t)std::max(s->S, 1), 1);   // kMaxRounds rounds fit
+  return run_chunks(s, dense_args(s), std::min<uint32_t>(most, 65535u),
+                    [&](const DenseArgs& a) { return launch_dense_runs(a, s->num_sms, s->work); }, seed, first, n, syn,
+                    bits, logical, host_out);
 }
 
 // A batch of `chunk` trajectories from `first` on, in factored passes, into the device output batch: small

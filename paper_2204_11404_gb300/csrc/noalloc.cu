@@ -5,7 +5,8 @@
 // latency-critical path where cudaMalloc's implicit device synchronisation is
 // not acceptable, or plug-ins that are handed a stream and output buffers but
 // no allocator.  All device working memory of the call (circuit program, init
-// state, the init round's Kraus blocks and reduction partials, control word) lives in one file-scope static device array below; the caller passes
+// state, the init round's Kraus blocks and reduction partials, the Kraus blocks of a few
+// complex64 trajectories, control word) lives in one file-scope static device array below; the caller passes
 // only the inputs (parameters, seed, trajectory range) and the device output
 // buffers.  The array is sized for the d = 3 register (2^9 amplitudes) with at
 // most kNoAllocMaxRounds noisy rounds, and every GPU that loads this library
@@ -19,6 +20,7 @@
 
 #include "../../include/qecsv.h"
 #include "common.cuh"
+#include "dense.hpp"
 #include "factor.cuh"
 #include "kernels.hpp"
 #include "onchip.hpp"
@@ -98,6 +100,9 @@ qec_status run_noalloc(const qec_params* params, uint64_t seed, uint64_t first_t
   int pgrid = pass_grid(D, 2, sms);
   const int pg4 = pass_grid(D, 4, sms);
   if (pg4 > pgrid) pgrid = pg4;
+  const bool dense = dense_applies(prec, D);   // complex64: blocks' Kraus pairs, for as many trajectories as 1 MiB holds
+  const size_t entries = (size_t)dense_entries(prog), blocks = (size_t)nstab * R;
+  const uint32_t most = blocks ? (uint32_t)((1u << 20) / (blocks * 2 * entries * sizeof(float2))) : 65535u;
   Carve c;
   const size_t o_psi0 = c.take(((size_t)1 << D) * amp);
   const size_t o_ops = c.take(sizeof(ProgOp) * (init_prog.ops.size() + 1));
@@ -114,6 +119,10 @@ qec_status run_noalloc(const qec_params* params, uint64_t seed, uint64_t first_t
   const size_t o_N = c.take(sizeof(double) * nstab), o_m = c.take(sizeof(int) * nstab);
   const size_t o_part = c.take(sizeof(double) * 2 * (pgrid > MAX_PASS_GRID ? pgrid : MAX_PASS_GRID));
   const size_t o_ctl = c.take(sizeof(Ctl));
+  const size_t o_nops = c.take(dense ? sizeof(ProgOp) * (prog.ops.size() + 1) : 0);
+  const size_t o_nblk = c.take(dense ? sizeof(BlockInfo) * nstab : 0), o_nmat = c.take(dense ? sizeof(prog.mats) : 0);
+  const size_t o_pair = c.take(dense ? most * blocks * 2 * entries * sizeof(float2) : 0);
+  const size_t o_nu = c.take(dense ? most * blocks * sizeof(double) : 0);
   if (c.off > kNoAllocBytes) return nfail(QEC_EINVAL, "request does not fit the 2 MiB static scratch");
 
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
@@ -128,6 +137,13 @@ qec_status run_noalloc(const qec_params* params, uint64_t seed, uint64_t first_t
   if (e == cudaSuccess) e = cudaMemcpyAsync(mats, init_prog.mats, sizeof(init_prog.mats), cudaMemcpyHostToDevice, st);
   for (int i = 0; i < 5 && e == cudaSuccess; ++i)
     if (fac_bytes[i]) e = cudaMemcpyAsync(base + o_fac[i], fac_src[i], fac_bytes[i], cudaMemcpyHostToDevice, st);
+  if (dense) {
+    if (e == cudaSuccess && !prog.ops.empty())
+      e = cudaMemcpyAsync(base + o_nops, prog.ops.data(), sizeof(ProgOp) * prog.ops.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(base + o_nblk, prog.blocks.data(), sizeof(BlockInfo) * nstab, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_nmat, prog.mats, sizeof(prog.mats), cudaMemcpyHostToDevice, st);
+  }
   // The control word is the only scratch that must start from known values (the reduction
   // ticket at 0); everything else is written before it is read.
   Ctl h_ctl;
@@ -180,7 +196,7 @@ qec_status run_noalloc(const qec_params* params, uint64_t seed, uint64_t first_t
   };
 
   // The same launches and kernels as qec_create / qec_run_trajectories, so that the results are
-  // identical: the init round's passes, then every trajectory on chip in one launch.
+  // identical: the init round's passes, then every trajectory on chip.
   auto prob = [&](const PassArgs& a) { return launch_prob(prec, a, pass_grid_for(prec, true, D, a.w, sms), st); };
   auto apply = [&](const PassArgs& a) { return launch_apply(prec, a, pass_grid_for(prec, false, D, a.w, sms), st); };
   // Noise-free init round with outcomes forced to the zero syndrome (Sec. III.B), in psi0.
@@ -191,8 +207,34 @@ qec_status run_noalloc(const qec_params* params, uint64_t seed, uint64_t first_t
     e = prob(a);
     if (e == cudaSuccess) e = apply(a);
   }
-  if (e == cudaSuccess) e = setup_onchip();
-  if (e == cudaSuccess) {
+  if (e == cudaSuccess) e = dense ? setup_dense(D) : setup_onchip();
+  if (e == cudaSuccess && dense) {
+    DenseArgs a;
+    a.ops = reinterpret_cast<const ProgOp*>(base + o_nops);
+    a.blocks = reinterpret_cast<const BlockInfo*>(base + o_nblk);
+    a.mats = reinterpret_cast<const double*>(base + o_nmat);
+    for (int i = 0; i < PR_COUNT; ++i) a.prob[i] = prog.prob[i];
+    a.nstab = nstab;
+    a.nd = D;
+    a.rounds = R;
+    a.nl = params->d;
+    a.entries = (int)entries;
+    a.seed = seed;
+    a.psi0 = psi0;
+    a.kraus = reinterpret_cast<float2*>(base + o_pair);
+    a.u = reinterpret_cast<double*>(base + o_nu);
+    a.psi_out = nullptr;
+    a.ctl = nullptr;
+    a.events = nullptr;
+    for (uint32_t at = 0; at < n && e == cudaSuccess; at += a.n) {
+      a.n = n - at < most ? n - at : most;
+      a.first = first_traj + at;
+      a.syn = d_syndromes + (size_t)at * (R + 1) * nstab;
+      a.bits = d_data_bits + (size_t)at * D;
+      a.logical = d_raw_logical + at;
+      e = launch_dense_runs(a, sms, st);
+    }
+  } else if (e == cudaSuccess) {
     OnchipArgs a;
     a.F = view_of(fprog);
     a.F.sites = reinterpret_cast<const FSite*>(base + o_fac[0]);
@@ -214,7 +256,7 @@ qec_status run_noalloc(const qec_params* params, uint64_t seed, uint64_t first_t
     a.logical = d_raw_logical;
     a.ctl = nullptr;
     a.events = nullptr;
-    e = launch_onchip(prec, a, sms, st);
+    e = launch_onchip(a, sms, st);
   }
   if (e != cudaSuccess) return nfail(QEC_ECUDA, std::string("launch: ") + cudaGetErrorString(e));
   return QEC_OK;

@@ -1,5 +1,5 @@
-// On-chip trajectories: registers of up to 13 data qubits (the d = 3 surface code, the repetition
-// code up to d = 13), one CTA per trajectory, the whole trajectory in one launch.
+// On-chip complex128 trajectories: registers of up to 13 data qubits (the d = 3 surface code, the
+// repetition code up to d = 13), one CTA per trajectory, the whole trajectory in one launch.
 //
 // What bounds it: for one trajectory latency (FP64 instructions issue at 64 cycles per warp and
 // scheduler on this chip, then barriers and the reduction trees of 8 blocks a round), for many the
@@ -18,7 +18,7 @@ namespace {
 using namespace oc;
 
 // Rounds compiled together, and the shared memory of one trajectory.
-template <typename T, int NT, int ITEMS>
+template <int NT, int ITEMS>
 struct Layout {
   static constexpr int kAmps = 4 * NT * ITEMS;
   static constexpr int kD = kAmps == 512 ? 9 : kAmps == 2048 ? 11 : 13;
@@ -28,15 +28,16 @@ struct Layout {
   static constexpr int kSites = 384;                          // draws of a round, at most
   static constexpr size_t kScratch = kRounds * (sizeof(fac::Touch) * kTouches + kTouches + kSites);
   static constexpr size_t kUnion = ((kScratch > 8 * (size_t)kAmps ? kScratch : 8 * (size_t)kAmps) + 15) / 16 * 16;
-  static constexpr size_t kPsi = sizeof(typename V2t<T>::t) * (size_t)kAmps;
-  static constexpr size_t kBlocks = sizeof(Compiled<T>) * kRounds * kStab;
+  static constexpr size_t kPsi = sizeof(double2) * (size_t)kAmps;
+  static constexpr size_t kBlocks = sizeof(Compiled<double>) * kRounds * kStab;
   static constexpr size_t kSmem = kPsi + kUnion + kBlocks;
 };
 
-template <typename T, int NT, int ITEMS>
+template <int NT, int ITEMS>
 __global__ void __launch_bounds__(NT) k_onchip(const __grid_constant__ OnchipArgs a) {
-  using T2 = typename V2t<T>::t;
-  using L = Layout<T, NT, ITEMS>;
+  using T = double;
+  using T2 = double2;
+  using L = Layout<NT, ITEMS>;
   constexpr int D = L::kD;
   extern __shared__ __align__(16) unsigned char osm[];
   T2* psi = reinterpret_cast<T2*>(osm);
@@ -132,32 +133,21 @@ __global__ void __launch_bounds__(NT) k_onchip(const __grid_constant__ OnchipArg
   }
 }
 
-template <typename T, int NT, int ITEMS>
+template <int NT, int ITEMS>
 cudaError_t launch_t(const OnchipArgs& a, int num_sms, cudaStream_t s) {
-  constexpr size_t smem = Layout<T, NT, ITEMS>::kSmem;
+  constexpr size_t smem = Layout<NT, ITEMS>::kSmem;
   int occ = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_onchip<T, NT, ITEMS>, NT, smem);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_onchip<NT, ITEMS>, NT, smem);
   if (e != cudaSuccess) return e;
   const uint32_t wave = (uint32_t)(num_sms * (occ < 1 ? 1 : occ));
-  k_onchip<T, NT, ITEMS><<<a.n < wave ? a.n : wave, NT, smem, s>>>(a);
+  k_onchip<NT, ITEMS><<<a.n < wave ? a.n : wave, NT, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T, int NT, int ITEMS>
+template <int NT, int ITEMS>
 cudaError_t attr_t() {
-  return cudaFuncSetAttribute(k_onchip<T, NT, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)Layout<T, NT, ITEMS>::kSmem);
-}
-
-// Threads: one group of four amplitudes each up to 2^11 amplitudes (two at 2^13): a single trajectory's
-// latency is a chain of sweeps, and its FP64 work spreads over the SM's four schedulers.
-template <typename T>
-cudaError_t launch_p(const OnchipArgs& a, int num_sms, cudaStream_t s) {
-  switch (a.F.nd) {
-    case 9: return launch_t<T, 128, 1>(a, num_sms, s);
-    case 11: return launch_t<T, 512, 1>(a, num_sms, s);
-    default: return launch_t<T, 1024, 2>(a, num_sms, s);
-  }
+  return cudaFuncSetAttribute(k_onchip<NT, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)Layout<NT, ITEMS>::kSmem);
 }
 
 }  // namespace
@@ -165,19 +155,22 @@ cudaError_t launch_p(const OnchipArgs& a, int num_sms, cudaStream_t s) {
 bool onchip_applies(int nd) { return nd == 9 || nd == 11 || nd == 13; }
 
 cudaError_t setup_onchip() {
-  cudaError_t e = attr_t<double, 128, 1>();
-  if (e == cudaSuccess) e = attr_t<double, 512, 1>();
-  if (e == cudaSuccess) e = attr_t<double, 1024, 2>();
-  if (e == cudaSuccess) e = attr_t<float, 128, 1>();
-  if (e == cudaSuccess) e = attr_t<float, 512, 1>();
-  if (e == cudaSuccess) e = attr_t<float, 1024, 2>();
+  cudaError_t e = attr_t<128, 1>();
+  if (e == cudaSuccess) e = attr_t<512, 1>();
+  if (e == cudaSuccess) e = attr_t<1024, 2>();
   return e;
 }
 
-cudaError_t launch_onchip(int precision, const OnchipArgs& a, int num_sms, cudaStream_t s) {
-  if (!onchip_applies(a.F.nd) || a.F.nsites > Layout<double, 128, 1>::kSites) return cudaErrorInvalidValue;
+// Threads: one group of four amplitudes each up to 2^11 amplitudes (two at 2^13): a single trajectory's
+// latency is a chain of sweeps, and its FP64 work spreads over the SM's four schedulers.
+cudaError_t launch_onchip(const OnchipArgs& a, int num_sms, cudaStream_t s) {
+  if (!onchip_applies(a.F.nd) || a.F.nsites > Layout<128, 1>::kSites) return cudaErrorInvalidValue;
   if (a.n == 0) return cudaSuccess;
-  return is_f64(precision) ? launch_p<double>(a, num_sms, s) : launch_p<float>(a, num_sms, s);
+  switch (a.F.nd) {
+    case 9: return launch_t<128, 1>(a, num_sms, s);
+    case 11: return launch_t<512, 1>(a, num_sms, s);
+    default: return launch_t<1024, 2>(a, num_sms, s);
+  }
 }
 
 }  // namespace qec

@@ -24,9 +24,9 @@ struct OnchipArgs {
   int32_t* events;        // [ev_cap][5], null = not recorded
 };
 
-// Registers of 9, 11 and 13 data qubits run on chip: complex128 or complex64 amplitudes (is_f64).
+// Registers of 9, 11 and 13 data qubits run on chip: complex128 here, complex64 in dense blocks (dense.hpp).
 bool onchip_applies(int nd);
 cudaError_t setup_onchip();
-cudaError_t launch_onchip(int precision, const OnchipArgs& a, int num_sms, cudaStream_t s);
+cudaError_t launch_onchip(const OnchipArgs& a, int num_sms, cudaStream_t s);
 
 }  // namespace qec
