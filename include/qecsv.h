@@ -237,9 +237,11 @@ typedef struct qec_batch qec_batch;
 /*
  * Batched simulator for the d = 3 delayed-measurement register (9 data qubits
  * + reused ancilla, Sec. II.B), `rounds` noisy rounds, gate set `gates`.
- * A trajectory runs on chip, its blocks as rotations and diagonals: one warp
- * each in a persistent launch that takes trajectories from a device work
- * counter, or one CTA each where there are at most four per SM.  max_traj
+ * A trajectory runs on chip, complex128 with its blocks as rotations and
+ * diagonals, complex64 with dense blocks (states the same to the last FP32
+ * place from one version to the next): one warp each in a persistent launch
+ * that takes trajectories from a device work counter, or, complex128, one CTA
+ * each where there are at most four per SM.  max_traj
  * bounds n of every run.  Only d = 3 is accepted (QEC_EUNSUPPORTED otherwise).  cuda_stream as in qec_create.
  */
 qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t max_traj, void* cuda_stream,
@@ -265,9 +267,10 @@ qec_status qec_batch_run(qec_batch* b, uint64_t seed, uint32_t n, const uint64_t
  * Autotuner: times qec_batch_run on the given sample and keeps the fastest
  * configuration of each engine, each timed on the sample's trajectories of its
  * register: the reduced-register engine's CTA shape (warps per CTA, one
- * resident wave per SM), then the unreduced engine's fusion width k (2..6 slab
- * bits per sweep: above 4 a weight-4 stabilizer's four data qubits are rotated
- * in one sweep, else two at a time) and threads per CTA (128, 256).
+ * resident wave per SM), then the unreduced engines' fusion width k (2..6 slab
+ * bits: complex64 gate units applied in one pass; complex128 rotates a weight-4
+ * stabilizer's four data qubits in one sweep above 4, else two at a time) and
+ * threads per CTA (128, 256).
  * *chosen_warps gets the reduced engine's warps per CTA, *best_ms the device
  * time of the whole sample with the chosen configuration; qec_batch_config reports all three choices.
  */

@@ -6,13 +6,15 @@
 // are active together; the other part's are |0> throughout (reset after their measurement, untouched
 // before their part), so a slab of 2^13 amplitudes holds the exact state.  Warps and CTAs take
 // trajectories from device work counters, so precisions and noise parameters mix freely in one
-// launch.  The circuit program is built once with every noise and coherent slot present; a
+// run.  The circuit program is built once with every noise and coherent slot present; a
 // trajectory's own matrices and draw thresholds follow from its noise input (a zero angle is the
 // identity, a zero probability never fires).
 //
-// The FP64 pipe bounds the complex128 trajectories, the compile and the sweeps' latency the complex64 ones.
-// 2048 trajectories of 3 rounds, dense blocks and gate units before: reduced register 8.24 -> 1.43 ms
-// complex128, 2.20 -> 0.61 complex64; unreduced 33.3 -> 3.58 and 10.0 -> 1.17.
+// complex64 trajectories of both registers have engines of their own, in dense blocks and gate units
+// (batch_dense.cu); each engine is a launch of its own, side by side.
+//
+// The FP64 pipe bounds the complex128 trajectories.  2048 trajectories of 3 rounds, dense blocks and gate
+// units before: reduced register 8.24 -> 1.43 ms, unreduced 33.3 -> 3.58.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -22,6 +24,7 @@
 #include <vector>
 
 #include "../../include/qecsv.h"
+#include "batch_dense.hpp"
 #include "onchip.cuh"
 #include "kernels.hpp"
 #include "program.hpp"
@@ -37,65 +40,30 @@ constexpr int kNStab = kND - 1;          // 8 stabilizers
 constexpr int kNAnc = kNStab / 2;        // ancillas of one part
 constexpr int kTouches = 4 * kNStab;
 constexpr int kSites = 224;              // draws of a round, every slot present (checked at creation)
-constexpr int kUMaxFusionDecl = 6;       // widest sweep a configuration may ask for (slab bits)
+constexpr int kKinds = 4;                // precision + 2 for the unreduced register
 
 struct BatchCtl {
   uint64_t seed;
-  uint32_t n;                 // reduced-register (10-qubit) trajectories in this run
-  unsigned int counter;       // their work queue head (zeroed before every run)
-  uint32_t n_u[2];            // unreduced-register (17-qubit) trajectories in this run: complex128, complex64
-  unsigned int counter_u[2];  // their work queue heads
-  uint32_t snap_item;         // item whose final data-register state goes to snap (~0u = none)
-};
-
-// One pass of the unreduced engine over the slab: kind 0 applies the units punits[u0, u1) (disjoint
-// slab bits, together `nbits` bits listed in bits[]); kind 1 measures the ancilla of items[item].
-struct UPass {
-  int32_t kind;
-  int32_t item;
-  int32_t u0, u1;
-  int32_t nbits;
-  int32_t bits[kUMaxFusionDecl];
-};
-
-// A unit inside a pass: items[item] on slab bits qa (, qb), and the pass's other bits.  A two-qubit
-// unit also carries the one-qubit units folded into its matrix: entries abs0 .. abs0 + nabs - 1 of
-// the program's UAbs list.
-struct UPassUnit {
-  int32_t item;
-  int32_t nq, qa, qb;
-  int32_t nother;
-  int32_t other[kUMaxFusionDecl];
-  int32_t abs0, nabs;
-};
-
-// A one-qubit unit folded into a two-qubit unit's matrix: item1's matrix on the unit's local bit
-// (mode bit 1: 1 = qa, 0 = qb), multiplied from the left (mode bit 0 = 1: it follows the unit) or
-// from the right (it precedes).  A unit's entries list the right factors latest first, then the
-// left factors in program order.
-struct UAbs {
-  int32_t item1;
-  int32_t mode;
+  uint32_t n[kKinds];             // trajectories of each kind in this run
+  unsigned int counter[kKinds];   // their work queue heads (zeroed before every run)
+  uint32_t snap_item;             // item whose final data-register state goes to snap (~0u = none)
 };
 
 struct BatchArgs {
   FactorView F;               // noisy program (all slots present), or the init program
   const qec_noise* noise;     // [n]
-  const int32_t* kind;        // [n]: bit 0 = complex64 (else complex128), bit 1 = unreduced register
-  const uint32_t* idx;        // reduced-register items of this run
-  const uint32_t* idx_u;      // unreduced-register items of this run
+  const uint32_t* idx;        // reduced-register complex128 items of this run
+  const uint32_t* idx_u;      // unreduced-register ones
   const uint64_t* traj;       // [n]
   BatchCtl* ctl;
   int rounds, cr;
   int width;                  // unreduced register: slab bits a sweep may hold (see u_sweep)
-  const void* psi0[2];        // init code state per precision
+  const double2* psi0;        // init code state
   uint8_t* syn;               // [n][rounds+1][8]
   uint8_t* bits;              // [n][9]
   uint8_t* logical;           // [n]
   double2* snap;              // [512] data-register state of ctl->snap_item after its last round
-  int init_mode;              // 1: compute the init state of precision init_prec into init_out
-  int init_prec;
-  void* init_out;
+  double2* init_out;          // not null: compute the init state into it
 };
 
 using namespace oc;
@@ -103,7 +71,7 @@ using namespace oc;
 // Shared memory of one trajectory besides its amplitudes; NR rounds are compiled together.
 template <int NR>
 struct Mem {
-  static constexpr int kRounds = NR;
+  enum : int { kRounds = NR };
   double2 fm[FM_COUNT][4];
   uint64_t thr[PR_COUNT];
   uint32_t bits, mask[NR];
@@ -202,10 +170,9 @@ __device__ void trajectory_noise(const G& g, const qec_noise& nz, bool cr, Mem& 
 }
 
 // Compiles rounds rnd .. rnd + nr - 1 into blk[nr][kNStab]; returns the flips in force after them.
-template <typename T, class G, class Mem>
-__device__ uint32_t compile_rounds(const G& g, const FactorView& F, Mem& M, Compiled<T>* blk, uint64_t seed, uint64_t traj,
+template <class G, class Mem>
+__device__ uint32_t compile_rounds(const G& g, const FactorView& F, Mem& M, Compiled<double>* blk, uint64_t seed, uint64_t traj,
                                    int rnd, int nr, uint32_t flips) {
-  using T2 = typename V2t<T>::t;
   if (g.rank < nr) M.mask[g.rank] = 0;
   g.sync();
   fac::Rounds R;
@@ -217,16 +184,16 @@ __device__ uint32_t compile_rounds(const G& g, const FactorView& F, Mem& M, Comp
   fac::compile_merge(g, F, M.thr, seed, traj, (uint64_t)rnd, M.fm, R, [](int, int, int) {});
   fac::compile_emit(g, F, M.fm, R, flips,
                     [&](int k, int i, double2 v) {
-                      Compiled<T>& c = blk[k * kNStab + (i >> 2)];
-                      c.rot[i & 3] = make2<T2>(v.x, v.y);
+                      Compiled<double>& c = blk[k * kNStab + (i >> 2)];
+                      c.rot[i & 3] = v;
                       c.form[i & 3] = rotation_form(v);
                     },
                     [&](int k, int b, int z, double2 d0, double2 d1) {
-                      Compiled<T>& c = blk[k * kNStab + b];
-                      c.d[0][z] = make2<T2>(d0.x, d0.y);
-                      c.d[1][z] = make2<T2>(d1.x, d1.y);
-                      c.wt[0][z] = (T)fac::cnorm(d0);
-                      c.wt[1][z] = (T)fac::cnorm(d1);
+                      Compiled<double>& c = blk[k * kNStab + b];
+                      c.d[0][z] = d0;
+                      c.d[1][z] = d1;
+                      c.wt[0][z] = fac::cnorm(d0);
+                      c.wt[1][z] = fac::cnorm(d1);
                     });
   for (int i = g.rank; i < nr * kNStab; i += g.size)
     blk[i].u = uniform53(draw(seed, traj, (uint64_t)(rnd + i / kNStab), 0u, (uint32_t)(kND + i % kNStab), TAG_MEASURE).v[0]);
@@ -236,68 +203,64 @@ __device__ uint32_t compile_rounds(const G& g, const FactorView& F, Mem& M, Comp
 }
 
 // Samples the final readout and writes the bits and the raw logical; the state to snap where asked.
-template <typename T, int NT, class Mem>
-__device__ void finish(const BatchArgs& a, const typename V2t<T>::t* psi, uint32_t flips, Mem& M, uint32_t item,
+template <int NT, class Mem>
+__device__ void finish(const BatchArgs& a, const double2* psi, uint32_t flips, Mem& M, uint32_t item,
                        uint64_t seed, uint64_t traj, int rank) {
   const Group<NT> g{rank};
   g.sync();   // the compile's memory is reused
   if (rank < kND)
     M.r.ur[rank] = uniform53(draw(seed, traj, (uint64_t)a.rounds + 1, 0u, (uint32_t)rank, TAG_READOUT).v[0]);
-  readout<T, NT>(psi, kND, flips, M.r.heap, M.r.ur, &M.bits, rank);
+  readout<double, NT>(psi, kND, flips, M.r.heap, M.r.ur, &M.bits, rank);
   const uint32_t x = M.bits;
   if (rank < kND) a.bits[(size_t)item * kND + rank] = (uint8_t)((x >> rank) & 1u);
   if (rank == 0) a.logical[item] = (uint8_t)(__popc(x & ((1u << kD) - 1u)) & 1);
   if (item == a.ctl->snap_item)
-    for (int i = rank; i < kNAmp; i += NT) a.snap[i] = make_double2((double)psi[i ^ flips].x, (double)psi[i ^ flips].y);
+    for (int i = rank; i < kNAmp; i += NT) a.snap[i] = psi[i ^ flips];
   g.sync();
 }
 
 // ---- reduced register: one warp per trajectory, or one CTA of four where there are few ------------------
-// What bounds it: the FP64 pipe (complex128: per round 1840 FP64 instructions a warp for the blocks, about
-// 700 for their compile, which complex64 trajectories run too).  A warp's FP64 instructions issue at its
-// scheduler's rate, a quarter of the SM's, so up to four trajectories per SM run on CTAs of four warps
-// (301 trajectories of 5 rounds, half complex128, with their host copies: 1.84 -> 0.84 ms).
+// What bounds it: the FP64 pipe (per round 1840 FP64 instructions a warp for the blocks, about 700 for their
+// compile).  A warp's FP64 instructions issue at its scheduler's rate, a quarter of the SM's, so up to four
+// trajectories per SM run on CTAs of four warps (150 trajectories of 5 rounds: 0.30 ms).
 using WMem = Mem<1>;
 constexpr size_t kGroupSmem = sizeof(WMem) + 16 * (size_t)kNAmp + sizeof(Compiled<double>) * kNStab;
 constexpr size_t kWarpSmem = kGroupSmem;
 static_assert(sizeof(WMem) % 16 == 0 && kWarpSmem % 16 == 0, "16-byte aligned amplitudes");
 
-template <typename T, int NT>
+template <int NT>
 __device__ void run_group(const BatchArgs& a, unsigned char* wsm, double* red, uint32_t item, int rank) {
-  using T2 = typename V2t<T>::t;
   const Group<NT> g{rank};
   WMem& M = *reinterpret_cast<WMem*>(wsm);
-  T2* psi = reinterpret_cast<T2*>(wsm + sizeof(WMem));
-  Compiled<T>* blk = reinterpret_cast<Compiled<T>*>(wsm + sizeof(WMem) + 16 * (size_t)kNAmp);
-  const bool init = a.init_mode != 0;
+  double2* psi = reinterpret_cast<double2*>(wsm + sizeof(WMem));
+  Compiled<double>* blk = reinterpret_cast<Compiled<double>*>(wsm + sizeof(WMem) + 16 * (size_t)kNAmp);
+  const bool init = a.init_out != nullptr;
   const qec_noise nz = init ? qec_noise{} : a.noise[item];
   const uint64_t traj = init ? 0ull : a.traj[item], seed = a.ctl->seed;
   trajectory_noise(g, nz, a.cr != 0, M);
-  const T2* p0 = reinterpret_cast<const T2*>(a.psi0[sizeof(T) == 4]);
-  for (int i = rank; i < kNAmp; i += NT) psi[i] = init ? make2<T2>(i == 0 ? 1.0 : 0.0, 0.0) : p0[i];
+  for (int i = rank; i < kNAmp; i += NT) psi[i] = init ? make_double2(i == 0 ? 1.0 : 0.0, 0.0) : a.psi0[i];
   uint8_t* syn = init ? nullptr : a.syn + (size_t)item * (a.rounds + 1) * kNStab;
   if (syn && rank < kNStab) syn[rank] = 0;
   uint32_t flips = 0;
   int parity = 0;
   for (int rnd = init ? 0 : 1; rnd <= (init ? 0 : a.rounds); ++rnd) {
-    flips = compile_rounds<T>(g, a.F, M, blk, seed, traj, rnd, 1, flips);
+    flips = compile_rounds(g, a.F, M, blk, seed, traj, rnd, 1, flips);
     for (int b = 0; b < kNStab; ++b) {
       const FBlock B = a.F.blocks[b];
-      const int m = run_block<T, NT, kNAmp / (4 * NT)>(psi, B, blk[b], red, parity++, rank, init ? B.offset : -1);
+      const int m = run_block<double, NT, kNAmp / (4 * NT)>(psi, B, blk[b], red, parity++, rank, init ? B.offset : -1);
       if (syn && rank == 0) syn[rnd * kNStab + b] = (uint8_t)(m ^ B.offset);
     }
   }
   if (init) {   // one warp
     double s = 0.0;
-    for (int i = rank; i < kNAmp; i += NT) s += (double)psi[i].x * psi[i].x + (double)psi[i].y * psi[i].y;
+    for (int i = rank; i < kNAmp; i += NT) s += psi[i].x * psi[i].x + psi[i].y * psi[i].y;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     const double sc = rsqrt(s);
-    T2* out = reinterpret_cast<T2*>(a.init_out);
-    for (int i = rank; i < kNAmp; i += NT) out[i] = make2<T2>(psi[i ^ flips].x * sc, psi[i ^ flips].y * sc);
+    for (int i = rank; i < kNAmp; i += NT) a.init_out[i] = make_double2(psi[i ^ flips].x * sc, psi[i ^ flips].y * sc);
     return;
   }
-  finish<T, NT>(a, psi, flips, M, item, seed, traj, rank);
+  finish<NT>(a, psi, flips, M, item, seed, traj, rank);
 }
 
 // Warps: the first trajectory of each by its place (warp 0 of every CTA, then warp 1, ...: few
@@ -306,19 +269,14 @@ __global__ void k_batch(const __grid_constant__ BatchArgs a) {
   extern __shared__ __align__(16) unsigned char bsm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned char* wsm = bsm + (size_t)warp * kWarpSmem;
-  if (a.init_mode) {
-    if (blockIdx.x == 0 && warp == 0) {
-      if (a.init_prec == 0) run_group<double, 32>(a, wsm, nullptr, 0, lane);
-      else run_group<float, 32>(a, wsm, nullptr, 0, lane);
-    }
+  if (a.init_out) {
+    if (blockIdx.x == 0 && warp == 0) run_group<32>(a, wsm, nullptr, 0, lane);
     return;
   }
-  const uint32_t all = gridDim.x * (blockDim.x >> 5), n = a.ctl->n;
+  const uint32_t all = gridDim.x * (blockDim.x >> 5), n = a.ctl->n[QEC_C128];
   for (uint32_t pos = (uint32_t)warp * gridDim.x + blockIdx.x; pos < n;) {
-    const uint32_t item = a.idx[pos];
-    if ((a.kind[item] & 1) == 0) run_group<double, 32>(a, wsm, nullptr, item, lane);
-    else run_group<float, 32>(a, wsm, nullptr, item, lane);
-    if (lane == 0) pos = all + atomicAdd(&a.ctl->counter, 1u);
+    run_group<32>(a, wsm, nullptr, a.idx[pos], lane);
+    if (lane == 0) pos = all + atomicAdd(&a.ctl->counter[QEC_C128], 1u);
     pos = __shfl_sync(0xffffffffu, pos, 0);
   }
 }
@@ -327,9 +285,7 @@ __global__ void k_batch(const __grid_constant__ BatchArgs a) {
 __global__ void __launch_bounds__(128) k_batch_cta(const __grid_constant__ BatchArgs a) {
   extern __shared__ __align__(16) unsigned char bsm[];
   __shared__ double red[2 * 64];
-  const uint32_t item = a.idx[blockIdx.x];
-  if ((a.kind[item] & 1) == 0) run_group<double, 128>(a, bsm, red, item, (int)threadIdx.x);
-  else run_group<float, 128>(a, bsm, red, item, (int)threadIdx.x);
+  run_group<128>(a, bsm, red, a.idx[blockIdx.x], (int)threadIdx.x);
 }
 
 // ---- unreduced register: one CTA per 17-qubit trajectory ------------------------------------------------
@@ -341,23 +297,19 @@ __global__ void __launch_bounds__(128) k_batch_cta(const __grid_constant__ Batch
 // entered, the norms of the 16 ancilla configurations give their measurements in order, and the
 // measured configuration's data is the register for the next part.
 constexpr int kUAmp = kNAmp << kNAnc;          // 8192 amplitudes
-template <typename T>
 struct UMem {
-  Mem<sizeof(T) == 8 ? 4 : 1> m;   // complex128: one CTA per SM, whose compile nothing else hides: four rounds together
+  Mem<4> m;   // one CTA per SM, whose compile nothing else hides: four rounds together
   double norm[1 << kNAnc];
 };
-static_assert(sizeof(UMem<double>) % 16 == 0 && sizeof(UMem<float>) % 16 == 0, "16-byte aligned amplitudes");
-template <typename T>
-constexpr size_t u_smem() {
-  return sizeof(UMem<T>) + sizeof(typename V2t<T>::t) * kUAmp + sizeof(Compiled<T>) * kNStab * decltype(UMem<T>::m)::kRounds;
-}
+static_assert(sizeof(UMem) % 16 == 0, "16-byte aligned amplitudes");
+constexpr size_t kUSmem = sizeof(UMem) + sizeof(double2) * kUAmp + sizeof(Compiled<double>) * kNStab * decltype(UMem::m)::kRounds;
 
 // Rotations of data qubits j0 .. j0 + W - 1 of a block on 2^nb amplitudes in groups of 2^W; with `enter`,
 // the block's ancilla enters at bit nb.  Two qubits a sweep are the faster choice (2048 complex128
 // trajectories of 3 rounds: 3.58 ms, 3.96 with four): the early ancillas' slabs then fill the CTA.
-template <typename T, int W>
-__device__ void u_sweep(typename V2t<T>::t* slab, int nb, const FBlock& B, const Compiled<T>& C, int j0, bool enter) {
-  using T2 = typename V2t<T>::t;
+template <int W>
+__device__ void u_sweep(double2* slab, int nb, const FBlock& B, const Compiled<double>& C, int j0, bool enter) {
+  using T2 = double2;
   constexpr int N = 1 << W;
   int q[W];
 #pragma unroll
@@ -413,51 +365,47 @@ struct CtaGroup {
   __device__ __forceinline__ void sync() const { __syncthreads(); }
 };
 
-template <typename T, int NT>
+template <int NT>
 __device__ void run_cta_u(const BatchArgs& a, unsigned char* sm, uint32_t item) {
-  using T2 = typename V2t<T>::t;
   const int tid = threadIdx.x;
   const CtaGroup g{tid, NT};
-  UMem<T>& U = *reinterpret_cast<UMem<T>*>(sm);
-  T2* slab = reinterpret_cast<T2*>(sm + sizeof(UMem<T>));
-  Compiled<T>* compiled = reinterpret_cast<Compiled<T>*>(sm + sizeof(UMem<T>) + sizeof(T2) * kUAmp);
-  constexpr int NR = decltype(UMem<T>::m)::kRounds;
+  UMem& U = *reinterpret_cast<UMem*>(sm);
+  double2* slab = reinterpret_cast<double2*>(sm + sizeof(UMem));
+  Compiled<double>* compiled = reinterpret_cast<Compiled<double>*>(sm + sizeof(UMem) + sizeof(double2) * kUAmp);
+  constexpr int NR = decltype(UMem::m)::kRounds;
   const qec_noise nz = a.noise[item];
   const uint64_t traj = a.traj[item], seed = a.ctl->seed;
   trajectory_noise(g, nz, a.cr != 0, U.m);
-  const T2* p0 = reinterpret_cast<const T2*>(a.psi0[sizeof(T) == 4]);
-  for (int i = tid; i < kNAmp; i += NT) slab[i] = p0[i];
+  for (int i = tid; i < kNAmp; i += NT) slab[i] = a.psi0[i];
   uint8_t* syn = a.syn + (size_t)item * (a.rounds + 1) * kNStab;
   if (tid < kNStab) syn[tid] = 0;
   uint32_t flips = 0;
   for (int rnd = 1; rnd <= a.rounds; ++rnd) {
     const int k = (rnd - 1) % NR;
-    if (k == 0) flips = compile_rounds<T>(g, a.F, U.m, compiled, seed, traj, rnd, min(NR, a.rounds + 1 - rnd), flips);
-    const Compiled<T>* blk = compiled + k * kNStab;
+    if (k == 0) flips = compile_rounds(g, a.F, U.m, compiled, seed, traj, rnd, min(NR, a.rounds + 1 - rnd), flips);
+    const Compiled<double>* blk = compiled + k * kNStab;
     for (int part = 0; part < 2; ++part) {
       for (int j = 0; j < kNAnc; ++j) {
         const FBlock B = a.F.blocks[part * kNAnc + j];
-        const Compiled<T>& C = blk[part * kNAnc + j];
+        const Compiled<double>& C = blk[part * kNAnc + j];
         const int nb = kND + j;
         if (B.w == 2) {
-          u_sweep<T, 2>(slab, nb, B, C, 0, true);
+          u_sweep<2>(slab, nb, B, C, 0, true);
         } else if (a.width > 4) {
-          u_sweep<T, 4>(slab, nb, B, C, 0, true);
+          u_sweep<4>(slab, nb, B, C, 0, true);
         } else {
-          if (C.form[0] | C.form[1]) u_sweep<T, 2>(slab, nb, B, C, 0, false);
-          u_sweep<T, 2>(slab, nb, B, C, 2, true);
+          if (C.form[0] | C.form[1]) u_sweep<2>(slab, nb, B, C, 0, false);
+          u_sweep<2>(slab, nb, B, C, 2, true);
         }
       }
-      // the 16 configurations' norms: 16 lanes each, the squares of a lane's amplitudes in the state's
-      // precision, then FP64 (lane l of a configuration takes data indices l, l + 16, ...: the sums do
-      // not depend on the CTA's size)
+      // the 16 configurations' norms: 16 lanes each (lane l of a configuration takes data indices l,
+      // l + 16, ...: the sums do not depend on the CTA's size)
       for (int c = tid >> 4; c < (1 << kNAnc); c += NT >> 4) {
-        T s = 0;
+        double w = 0.0;
         for (int i = tid & 15; i < kNAmp; i += 16) {
-          const T2 v = slab[c * kNAmp + i];
-          s = fma(v.x, v.x, fma(v.y, v.y, s));
+          const double2 v = slab[c * kNAmp + i];
+          w = fma(v.x, v.x, fma(v.y, v.y, w));
         }
-        double w = (double)s;
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
         if ((tid & 15) == 0) U.norm[c] = w;
@@ -478,10 +426,10 @@ __device__ void run_cta_u(const BatchArgs& a, unsigned char* sm, uint32_t item) 
         norm = one ? s1 : s0;
       }
       const bool rescale = small_norm(norm);
-      const T sc = norm_scale<T>(norm);
+      const double sc = norm_scale<double>(norm);
       if (m || rescale)
         for (int i = tid; i < kNAmp; i += NT) {
-          T2 v = slab[m * kNAmp + i];
+          double2 v = slab[m * kNAmp + i];
           if (rescale) {
             v.x *= sc;
             v.y *= sc;
@@ -495,33 +443,29 @@ __device__ void run_cta_u(const BatchArgs& a, unsigned char* sm, uint32_t item) 
       __syncthreads();
     }
   }
-  finish<T, NT>(a, slab, flips, U.m, item, seed, traj, tid);
+  finish<NT>(a, slab, flips, U.m, item, seed, traj, tid);
 }
 
-// One precision's trajectories (a launch of its own: a complex64 slab is half the size, so that two or
-// three CTAs share an SM).  idx_u lists the complex128 items, then the complex64 ones.
-template <typename T, int NT>
+template <int NT>
 __global__ void __launch_bounds__(NT) k_batch_u(const __grid_constant__ BatchArgs a) {
   extern __shared__ __align__(16) unsigned char usm[];
   __shared__ uint32_t s_pos;
-  constexpr int P = sizeof(T) == 4;
-  const uint32_t n = a.ctl->n_u[P], base = P ? a.ctl->n_u[0] : 0u;
+  constexpr int kind = QEC_C128 + 2;
+  const uint32_t n = a.ctl->n[kind];
   for (;;) {
-    if (threadIdx.x == 0) s_pos = atomicAdd(&a.ctl->counter_u[P], 1u);
+    if (threadIdx.x == 0) s_pos = atomicAdd(&a.ctl->counter[kind], 1u);
     __syncthreads();
     const uint32_t pos = s_pos;
     __syncthreads();
     if (pos >= n) return;
-    run_cta_u<T, NT>(a, usm, a.idx_u[base + pos]);
+    run_cta_u<NT>(a, usm, a.idx_u[pos]);
     __syncthreads();
   }
 }
 
-const void* u_kernel(int prec, int threads) {
-  if (prec) return threads == 128 ? (const void*)k_batch_u<float, 128> : threads == 256 ? (const void*)k_batch_u<float, 256> : (const void*)k_batch_u<float, 512>;
-  return threads == 128 ? (const void*)k_batch_u<double, 128> : threads == 256 ? (const void*)k_batch_u<double, 256> : (const void*)k_batch_u<double, 512>;
+const void* u_kernel(int threads) {
+  return threads == 128 ? (const void*)k_batch_u<128> : threads == 256 ? (const void*)k_batch_u<256> : (const void*)k_batch_u<512>;
 }
-constexpr size_t u_smem_of(int prec) { return prec ? u_smem<float>() : u_smem<double>(); }
 
 }  // namespace
 
@@ -534,15 +478,22 @@ struct qec_batch {
   FactorProgram fac[2];              // [0] noisy program, every slot present; [1] init program
   unsigned char* d_fac[2] = {nullptr, nullptr};
   size_t fac_off[2][5] = {};
-  void* d_psi0[2] = {nullptr, nullptr};
-  uint32_t* d_idx = nullptr;
-  uint32_t* d_idx_u = nullptr;
-  std::vector<uint32_t> h_idx, h_idx_u;
-  cudaStream_t side[2] = {nullptr, nullptr};   // the unreduced engine's launches, per precision
-  cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
-  int u_ctas_per_sm[2] = {1, 1};
+  // the complex64 engines' programs, again noisy and init: ops, blocks, then the unreduced register's ops, items,
+  // passes, pass units and folded units at off64
+  Program prog[2];
+  UProgram uprog[2];
+  unsigned char* d_prog64[2] = {nullptr, nullptr};
+  size_t off64[2][7] = {};
+  int n_upasses[2] = {0, 0}, n_upunits[2] = {0, 0};
+  int u_items = 0;                   // unit matrices a CTA of theirs holds
+  double* d_mats = nullptr;
+  double2* d_psi0 = nullptr;
+  float2* d_psi0_64 = nullptr;       // 2^9, then the unreduced register's slab
+  uint32_t* d_idx = nullptr;         // a run's items by kind, one kind after the other
+  std::vector<uint32_t> h_idx;
+  cudaStream_t side[kKinds - 1] = {};   // launches besides the work stream's
+  cudaEvent_t fork = nullptr, join[kKinds - 1] = {};
   qec_noise* d_noise = nullptr;
-  int32_t* d_kind = nullptr;
   uint64_t* d_traj = nullptr;
   BatchCtl* d_ctl = nullptr;
   BatchCtl* h_ctl = nullptr;   // pinned
@@ -550,13 +501,13 @@ struct qec_batch {
   uint8_t* d_bits = nullptr;
   uint8_t* d_log = nullptr;
   int warps_per_cta = 8;
-  int ctas_per_sm = 1;
+  int ctas_per_sm[kKinds] = {1, 1, 1, 1};
   float last_ms = 0.f;
   double2* d_snap = nullptr;
   int64_t snap_item = -1;   // for the next run
   bool snap_valid = false;  // a completed run recorded a snapshot
-  int fusion_k = 4;         // unreduced engine: slab bits a sweep may hold
-  int u_threads = 256;      // unreduced engine: threads per CTA
+  int fusion_k = 0;         // unreduced engines: slab bits a sweep or pass may hold (0: no plan yet)
+  int u_threads = 256;      // unreduced engines: threads per CTA
 };
 
 namespace {
@@ -575,11 +526,11 @@ qec_status bfail(qec_status s, const std::string& m) {
   } while (0)
 
 void batch_free(qec_batch* b) {
-  void* ptrs[] = {b->d_fac[0], b->d_fac[1], b->d_psi0[0], b->d_psi0[1], b->d_noise, b->d_kind, b->d_traj, b->d_ctl,
-                  b->d_syn, b->d_bits, b->d_log, b->d_idx, b->d_idx_u, b->d_snap};
+  void* ptrs[] = {b->d_fac[0], b->d_fac[1], b->d_prog64[0], b->d_prog64[1], b->d_mats, b->d_psi0, b->d_psi0_64, b->d_noise,
+                  b->d_traj, b->d_ctl, b->d_syn, b->d_bits, b->d_log, b->d_idx, b->d_snap};
   for (void* p : ptrs) if (p) cudaFree(p);
   if (b->fork) cudaEventDestroy(b->fork);
-  for (int i = 0; i < 2; ++i) {
+  for (int i = 0; i < kKinds - 1; ++i) {
     if (b->join[i]) cudaEventDestroy(b->join[i]);
     if (b->side[i]) cudaStreamDestroy(b->side[i]);
   }
@@ -605,202 +556,146 @@ BatchArgs batch_args(const qec_batch* b) {
   BatchArgs a;
   a.F = batch_program(b, 0);
   a.noise = b->d_noise;
-  a.kind = b->d_kind;
   a.traj = b->d_traj;
   a.ctl = b->d_ctl;
   a.rounds = b->rounds;
   a.cr = b->gates == QEC_GATES_CR;
   a.width = b->fusion_k;
-  a.psi0[0] = b->d_psi0[0];
-  a.psi0[1] = b->d_psi0[1];
-  a.idx = b->d_idx;
-  a.idx_u = b->d_idx_u;
+  a.psi0 = b->d_psi0;
+  a.idx = a.idx_u = b->d_idx;
   a.syn = b->d_syn;
   a.bits = b->d_bits;
   a.logical = b->d_log;
   a.snap = b->d_snap;
-  a.init_mode = 0;
-  a.init_prec = 0;
   a.init_out = nullptr;
   return a;
 }
 
+// which: the noisy program or the init round's.
+Batch64Args batch64_args(const qec_batch* b, int which) {
+  const unsigned char* d = b->d_prog64[which];
+  const size_t* off = b->off64[which];
+  Batch64Args a{};
+  a.ops = reinterpret_cast<const ProgOp*>(d + off[0]);
+  a.blocks = reinterpret_cast<const BlockInfo*>(d + off[1]);
+  a.n_ops = (int)b->prog[which].ops.size();
+  a.uops = reinterpret_cast<const ProgOp*>(d + off[2]);
+  a.uitems = reinterpret_cast<const UItem*>(d + off[3]);
+  a.upasses = reinterpret_cast<const UPass*>(d + off[4]);
+  a.upunits = reinterpret_cast<const UPassUnit*>(d + off[5]);
+  a.uabs = reinterpret_cast<const UAbs*>(d + off[6]);
+  a.n_uitems = (int)b->uprog[which].items.size();
+  a.n_upasses = b->n_upasses[which];
+  a.n_upunits = b->n_upunits[which];
+  a.mats = b->d_mats;
+  a.rounds = b->rounds;
+  a.snap_item = ~0u;
+  if (which) return a;
+  a.noise = b->d_noise;
+  a.traj = b->d_traj;
+  a.seed = b->h_ctl->seed;
+  a.snap_item = b->h_ctl->snap_item;
+  a.syn = b->d_syn;
+  a.bits = b->d_bits;
+  a.logical = b->d_log;
+  a.snap = b->d_snap;
+  return a;
+}
+
+// Function attributes are the process's, not a handle's: the ceiling, so that handles of different shapes coexist; the
+// largest carveout, so that engines side by side fit the same SMs (batch_dense.cu).
+constexpr int kSmemCeiling = 226 * 1024;
+cudaError_t set_attributes(const void* fn) {
+  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCeiling);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
 size_t smem_for(int warps) { return (size_t)warps * kWarpSmem; }
 
 // The run's launches: each engine that has trajectories, side by side (one CTA wave each at most, pulling
 // trajectories from the control word's counters).
-qec_status launch_batch(qec_batch* b, uint32_t n, uint32_t n_u128, uint32_t n_u64) {
+qec_status launch_batch(qec_batch* b) {
+  const uint32_t* n = b->h_ctl->n;
   BatchArgs a = batch_args(b);
-  const uint32_t n_u[2] = {n_u128, n_u64};
-  bool busy = n > 0;   // something runs on the work stream itself
-  if (n_u128 || n_u64) QEC_BCUDA(cudaEventRecord(b->fork, b->work));
-  if (n > 0) {
-    // up to four trajectories per SM: a CTA of four warps each (see above)
-    if (n <= 4u * (uint32_t)b->num_sms) {
-      k_batch_cta<<<n, 128, kGroupSmem, b->work>>>(a);
+  Batch64Args a64 = batch64_args(b, 0);
+  QEC_BCUDA(cudaEventRecord(b->fork, b->work));
+  uint32_t base = 0;
+  for (int kind = 0, used = 0; kind < kKinds; base += n[kind++]) {
+    if (!n[kind]) continue;
+    cudaStream_t s = used ? b->side[used - 1] : b->work;
+    if (used) QEC_BCUDA(cudaStreamWaitEvent(s, b->fork, 0));
+    const uint32_t wave = (uint32_t)(b->num_sms * b->ctas_per_sm[kind]);
+    const bool u = kind >= 2;
+    const uint32_t ctas = u ? n[kind] : (n[kind] + b->warps_per_cta - 1) / b->warps_per_cta, grid = ctas < wave ? ctas : wave;
+    if (kind & 1) {
+      a64.idx = b->d_idx + base;
+      a64.n = n[kind];
+      a64.counter = &b->d_ctl->counter[kind];
+      a64.psi0 = u ? b->d_psi0_64 + kNAmp : b->d_psi0_64;
+      // few trajectories: fewer warps on an SM each
+      const uint32_t per = (n[kind] + b->num_sms - 1) / b->num_sms;
+      if (u) QEC_BCUDA(launch_batch64_u(a64, b->u_threads, b->u_items, (int)grid, s));
+      else if (per < (uint32_t)b->warps_per_cta) QEC_BCUDA(launch_batch64(a64, (int)per, (int)((n[kind] + per - 1) / per), s));
+      else QEC_BCUDA(launch_batch64(a64, b->warps_per_cta, (int)grid, s));
+    } else if (u) {
+      a.idx_u = b->d_idx + base;
+      void* args[1] = {&a};
+      QEC_BCUDA(cudaLaunchKernel(u_kernel(b->u_threads), dim3(grid), dim3((unsigned)b->u_threads), args, kUSmem, s));
     } else {
-      const uint32_t ctas = (n + b->warps_per_cta - 1) / b->warps_per_cta, wave = (uint32_t)(b->num_sms * b->ctas_per_sm);
-      k_batch<<<ctas < wave ? ctas : wave, 32 * b->warps_per_cta, smem_for(b->warps_per_cta), b->work>>>(a);
+      a.idx = b->d_idx + base;
+      // up to four trajectories per SM: a CTA of four warps each (see above)
+      if (n[kind] <= 4u * (uint32_t)b->num_sms) k_batch_cta<<<n[kind], 128, kGroupSmem, s>>>(a);
+      else k_batch<<<grid, 32 * b->warps_per_cta, smem_for(b->warps_per_cta), s>>>(a);
+      QEC_BCUDA(cudaGetLastError());
     }
-    QEC_BCUDA(cudaGetLastError());
-  }
-  for (int i = 0; i < 2; ++i) {
-    if (!n_u[i]) continue;
-    cudaStream_t s = busy ? b->side[i] : b->work;
-    if (busy) QEC_BCUDA(cudaStreamWaitEvent(s, b->fork, 0));
-    const uint32_t wave = (uint32_t)(b->num_sms * b->u_ctas_per_sm[i]);
-    void* args[1] = {&a};
-    QEC_BCUDA(cudaLaunchKernel(u_kernel(i, b->u_threads), dim3(n_u[i] < wave ? n_u[i] : wave), dim3((unsigned)b->u_threads),
-                               args, u_smem_of(i), s));
-    if (busy) {
-      QEC_BCUDA(cudaEventRecord(b->join[i], s));
-      QEC_BCUDA(cudaStreamWaitEvent(b->work, b->join[i], 0));
+    if (used) {
+      QEC_BCUDA(cudaEventRecord(b->join[used - 1], s));
+      QEC_BCUDA(cudaStreamWaitEvent(b->work, b->join[used - 1], 0));
     }
-    busy = true;
+    ++used;
   }
   return QEC_OK;
 }
 
-// Time-ordered plan of one round of the unreduced register (qec_debug_unreduced_plan) for fusion width k: consecutive units whose slab bits
-// are disjoint from those already in the pass (they commute with them) join it while the pass has at
-// most k bits; a unit on a bit already in the pass, or a measurement, closes it.
-// One-qubit units folded into two-qubit units: on each slab bit, a run of consecutive one-qubit units
-// (nothing else on that bit between them) directly before a two-qubit unit on the bit goes into that
-// unit's matrix from the right, a run directly after one from the left (between two, into the one
-// whose second qubit is the bit).  Moving the run next to the unit is exact: the run acts on its bit alone, and nothing else
-// acts on that bit in between.  absorbed[it] marks the folded units; pre/post list them per
-// two-qubit unit in program order.
-void plan_absorb(const UProgram& U, std::vector<char>& absorbed, std::vector<std::vector<UAbs>>& pre,
-                 std::vector<std::vector<UAbs>>& post) {
-  const int n = (int)U.items.size();
-  absorbed.assign(n, 0);
-  pre.assign(n, {});
-  post.assign(n, {});
-  auto is1 = [&](int it) { return U.items[it].kind == 0 && U.items[it].nq == 1; };
-  auto is2 = [&](int it) { return U.items[it].kind == 0 && U.items[it].nq == 2; };
-  for (int b = 0; b < U.nbits; ++b) {
-    std::vector<int> seq;   // items acting on bit b, in order
-    for (int it = 0; it < n; ++it) {
-      const UItem& u = U.items[it];
-      if (u.qa == b || (u.kind == 0 && u.nq == 2 && u.qb == b)) seq.push_back(it);
-    }
-    for (size_t i = 0; i < seq.size();) {
-      if (!is1(seq[i])) { ++i; continue; }
-      size_t j = i;
-      while (j < seq.size() && is1(seq[j])) ++j;
-      int target = -1;
-      bool after = false;
-      const bool next2 = j < seq.size() && is2(seq[j]), prev2 = i > 0 && is2(seq[i - 1]);
-      // between two two-qubit units, the one in which b is the second qubit (the gate's target) takes
-      // the run: a one-qubit matrix there keeps that unit block-diagonal in its first qubit
-      if (next2 && (!prev2 || U.items[seq[j]].qb == b || U.items[seq[i - 1]].qb != b)) {
-        target = seq[j];
-      } else if (prev2) {
-        target = seq[i - 1];
-        after = true;
-      }
-      if (target >= 0) {
-        const int bit = U.items[target].qa == b ? 2 : 0;
-        for (size_t r = i; r < j; ++r) {
-          absorbed[seq[r]] = 1;
-          (after ? post : pre)[target].push_back({seq[r], bit | (after ? 1 : 0)});
-        }
-      }
-      i = j;
-    }
-  }
-}
-
-void build_passes(const UProgram& U, int k, std::vector<UPass>& passes, std::vector<UPassUnit>& punits,
-                  std::vector<UAbs>& uabs) {
-  passes.clear();
-  punits.clear();
-  uabs.clear();
-  std::vector<char> absorbed;
-  std::vector<std::vector<UAbs>> pre, post;
-  plan_absorb(U, absorbed, pre, post);
-  UPass cur{};
-  uint32_t mask = 0;
-  auto close = [&]() {
-    if (cur.u1 == cur.u0) return;
-    cur.nbits = 0;
-    for (int q = 0; q < 32; ++q)
-      if (mask & (1u << q)) cur.bits[cur.nbits++] = q;
-    for (int i = cur.u0; i < cur.u1; ++i) {
-      UPassUnit& pu = punits[i];
-      const uint32_t um = (1u << pu.qa) | (pu.nq == 2 ? (1u << pu.qb) : 0u);
-      pu.nother = 0;
-      for (int j = 0; j < cur.nbits; ++j)
-        if (!(um & (1u << cur.bits[j]))) pu.other[pu.nother++] = cur.bits[j];
-    }
-    passes.push_back(cur);
-  };
-  auto open = [&]() {
-    cur = UPass{};
-    cur.kind = 0;
-    cur.u0 = cur.u1 = (int32_t)punits.size();
-    mask = 0;
-  };
-  open();
-  for (int it = 0; it < (int)U.items.size(); ++it) {
-    const UItem& u = U.items[it];
-    if (u.kind == 1) {
-      close();
-      UPass m{};
-      m.kind = 1;
-      m.item = it;
-      passes.push_back(m);
-      open();
-      continue;
-    }
-    if (absorbed[it]) continue;
-    const uint32_t um = (1u << u.qa) | (u.nq == 2 ? (1u << u.qb) : 0u);
-    if ((mask & um) || __builtin_popcount(mask | um) > k) {
-      close();
-      open();
-    }
-    UPassUnit pu{};
-    pu.item = it;
-    pu.nq = u.nq;
-    pu.qa = u.qa;
-    pu.qb = u.nq == 2 ? u.qb : 0;
-    pu.abs0 = (int32_t)uabs.size();
-    for (auto r = pre[it].rbegin(); r != pre[it].rend(); ++r) uabs.push_back(*r);   // right factors, latest first
-    for (const UAbs& x : post[it]) uabs.push_back(x);                              // left factors, in order
-    pu.nabs = (int32_t)uabs.size() - pu.abs0;
-    punits.push_back(pu);
-    cur.u1 = (int32_t)punits.size();
-    mask |= um;
-  }
-  close();
-}
-
-// Sweep width (2..6 slab bits: with more than 4 a weight-4 block's four data qubits go in one sweep, with the
-// ancilla that enters; else two at a time) and threads per CTA (128..512)
-// of the unreduced engine.
+// Threads per CTA (128..512) of the unreduced engines and their width in slab bits (2..6): the complex64
+// engine's passes hold that many, the complex128 one rotates a weight-4 block's four data qubits in one sweep
+// from 5 on, with the ancilla that enters, else two at a time.
 qec_status set_fusion(qec_batch* b, int k, int threads) {
-  if (k < 2 || k > kUMaxFusionDecl || (threads != 128 && threads != 256 && threads != 512))
+  if (k < 2 || k > kUMaxFusion || (threads != 128 && threads != 256 && threads != 512))
     return bfail(QEC_EINVAL, "fusion width must be in [2, 6] and threads 128, 256 or 512");
   int occ[2] = {0, 0};
-  for (int i = 0; i < 2; ++i) {
-    QEC_BCUDA(cudaFuncSetAttribute(u_kernel(i, threads), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)u_smem_of(i)));
-    QEC_BCUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[i], u_kernel(i, threads), threads, u_smem_of(i)));
-    if (occ[i] < 1) return bfail(QEC_EUNSUPPORTED, "unreduced batched kernel does not fit an SM with this shape");
+  QEC_BCUDA(set_attributes(u_kernel(threads)));
+  QEC_BCUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[0], u_kernel(threads), threads, kUSmem));
+  QEC_BCUDA(setup_batch64_u(threads, b->u_items, &occ[1]));
+  if (occ[0] < 1 || occ[1] < 1) return bfail(QEC_EUNSUPPORTED, "unreduced batched kernel does not fit an SM with this shape");
+  for (int w = 0; w < 2 && k != b->fusion_k; ++w) {
+    std::vector<UPass> passes;
+    std::vector<UPassUnit> punits;
+    std::vector<UAbs> uabs;
+    build_passes(b->uprog[w], k, passes, punits, uabs);
+    const void* src[3] = {passes.data(), punits.data(), uabs.data()};
+    const size_t bytes[3] = {sizeof(UPass) * passes.size(), sizeof(UPassUnit) * punits.size(), sizeof(UAbs) * uabs.size()};
+    for (int i = 0; i < 3; ++i)
+      if (bytes[i]) QEC_BCUDA(cudaMemcpy(b->d_prog64[w] + b->off64[w][4 + i], src[i], bytes[i], cudaMemcpyHostToDevice));
+    b->n_upasses[w] = (int)passes.size();
+    b->n_upunits[w] = (int)punits.size();
   }
   b->fusion_k = k;
   b->u_threads = threads;
-  b->u_ctas_per_sm[0] = occ[0];
-  b->u_ctas_per_sm[1] = occ[1];
+  b->ctas_per_sm[QEC_C128 + 2] = occ[0];
+  b->ctas_per_sm[QEC_C64 + 2] = occ[1];
   return QEC_OK;
 }
 
 qec_status set_shape(qec_batch* b, int warps) {
-  QEC_BCUDA(cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_for(warps)));
-  int occ = 0;
-  QEC_BCUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch, 32 * warps, smem_for(warps)));
-  if (occ < 1) return bfail(QEC_EUNSUPPORTED, "batched kernel does not fit an SM with this shape");
+  int occ[2] = {0, 0};
+  QEC_BCUDA(set_attributes((const void*)k_batch));
+  QEC_BCUDA(set_attributes((const void*)k_batch_cta));
+  QEC_BCUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[0], k_batch, 32 * warps, smem_for(warps)));
+  QEC_BCUDA(setup_batch64(warps, &occ[1]));
+  if (occ[0] < 1 || occ[1] < 1) return bfail(QEC_EUNSUPPORTED, "batched kernel does not fit an SM with this shape");
   b->warps_per_cta = warps;
-  b->ctas_per_sm = occ;
+  b->ctas_per_sm[QEC_C128] = occ[0];
+  b->ctas_per_sm[QEC_C64] = occ[1];
   return QEC_OK;
 }
 
@@ -812,7 +707,7 @@ qec_status qec_debug_unreduced_plan(int32_t gates, int32_t k, int32_t* items, ui
                                     int32_t* pass_units, uint32_t* n_pass_units, int32_t* absorbs, uint32_t* n_absorbs) {
   if (!items || !n_items || !pass_units || !n_pass_units || !absorbs || !n_absorbs)
     return bfail(QEC_EINVAL, "null argument");
-  if (k < 2 || k > kUMaxFusionDecl) return bfail(QEC_EINVAL, "fusion width must be in [2, 6]");
+  if (k < 2 || k > kUMaxFusion) return bfail(QEC_EINVAL, "fusion width must be in [2, 6]");
   try {
     qec_params p{};
     p.d = kD;
@@ -880,10 +775,14 @@ qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t m
   b->cap = max_traj;
   b->user = static_cast<cudaStream_t>(cuda_stream);
   for (int w = 0; w < 2; ++w) {
-    Program P;
-    if (!build_program(p, w == 0, P, err, w == 0) || !build_factor(P, b->fac[w], err)) return bail(bfail(QEC_EINVAL, err));
-    if (b->fac[w].sites.size() > (size_t)kSites)
-      return bail(bfail(QEC_EUNSUPPORTED, "a round has more draws than the engine's table"));
+    Program& P = b->prog[w];
+    UProgram& U = b->uprog[w];
+    if (!build_program(p, w == 0, P, err, w == 0) || !build_factor(P, b->fac[w], err) ||
+        !build_unreduced_program(p, w == 0, U, err, w == 0))
+      return bail(bfail(QEC_EINVAL, err));
+    if (b->fac[w].sites.size() > (size_t)kSites || P.ops.size() > (size_t)kBatchOps || U.items.size() > (size_t)kUMaxItems)
+      return bail(bfail(QEC_EUNSUPPORTED, "a round has more draws, ops or units than the engines' tables"));
+    if ((int)U.items.size() > b->u_items) b->u_items = (int)U.items.size();
   }
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -894,42 +793,51 @@ qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t m
   if (e == cudaSuccess) e = cudaEventCreate(&b->t0);
   if (e == cudaSuccess) e = cudaEventCreate(&b->t1);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-  for (int i = 0; i < 2; ++i) {
+  for (int i = 0; i < kKinds - 1; ++i) {
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming);
   }
   if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e)));
   const size_t syn_bytes = (size_t)max_traj * (rounds + 1) * kNStab;
-  const void* src[2][5];
-  size_t bytes[2][5], total[2];
+  const void* src[2][12];
+  size_t bytes[2][12], total[2] = {0, 0}, total64[2] = {0, 0};
   for (int w = 0; w < 2; ++w) {
     const FactorProgram& F = b->fac[w];
-    const void* s[5] = {F.sites.data(), F.items.data(), F.touches.data(), F.blocks.data(), F.order.data()};
-    const size_t n[5] = {sizeof(FSite) * F.sites.size(), sizeof(FItem) * F.items.size(), sizeof(FTouch) * F.touches.size(),
-                         sizeof(FBlock) * F.blocks.size(), sizeof(uint16_t) * F.order.size()};
-    total[w] = 0;
-    for (int i = 0; i < 5; ++i) {
+    const Program& P = b->prog[w];
+    const UProgram& U = b->uprog[w];
+    const size_t items = U.items.size();   // at least as many as there are passes, pass units or folded units
+    const void* s[12] = {F.sites.data(), F.items.data(), F.touches.data(), F.blocks.data(), F.order.data(),
+                         P.ops.data(), P.blocks.data(), U.ops.data(), U.items.data(), nullptr, nullptr, nullptr};
+    const size_t n[12] = {sizeof(FSite) * F.sites.size(), sizeof(FItem) * F.items.size(), sizeof(FTouch) * F.touches.size(),
+                          sizeof(FBlock) * F.blocks.size(), sizeof(uint16_t) * F.order.size(),
+                          sizeof(ProgOp) * P.ops.size(), sizeof(BlockInfo) * P.blocks.size(), sizeof(ProgOp) * U.ops.size(),
+                          sizeof(UItem) * items, sizeof(UPass) * items, sizeof(UPassUnit) * items, sizeof(UAbs) * items};
+    for (int i = 0; i < 12; ++i) {
+      size_t& at = i < 5 ? total[w] : total64[w];
       src[w][i] = s[i];
       bytes[w][i] = n[i];
-      b->fac_off[w][i] = total[w];
-      total[w] += (n[i] + 255) / 256 * 256;
+      (i < 5 ? b->fac_off[w][i] : b->off64[w][i - 5]) = at;
+      at += (n[i] + 255) / 256 * 256;
     }
   }
-  void** allocs[] = {(void**)&b->d_fac[0], (void**)&b->d_fac[1], &b->d_psi0[0], &b->d_psi0[1], (void**)&b->d_noise,
-                     (void**)&b->d_kind, (void**)&b->d_traj, (void**)&b->d_ctl, (void**)&b->d_syn, (void**)&b->d_bits,
-                     (void**)&b->d_log, (void**)&b->d_idx, (void**)&b->d_idx_u, (void**)&b->d_snap};
-  const size_t sizes[] = {total[0], total[1], (size_t)kNAmp * 16, (size_t)kNAmp * 8, sizeof(qec_noise) * max_traj,
-                          sizeof(int32_t) * max_traj, sizeof(uint64_t) * max_traj, sizeof(BatchCtl), syn_bytes,
-                          (size_t)max_traj * kND, (size_t)max_traj, sizeof(uint32_t) * max_traj,
-                          sizeof(uint32_t) * max_traj, sizeof(double2) * kNAmp};
+  void** allocs[] = {(void**)&b->d_fac[0], (void**)&b->d_fac[1], (void**)&b->d_prog64[0], (void**)&b->d_prog64[1],
+                     (void**)&b->d_mats, (void**)&b->d_psi0, (void**)&b->d_psi0_64, (void**)&b->d_noise, (void**)&b->d_traj,
+                     (void**)&b->d_ctl, (void**)&b->d_syn, (void**)&b->d_bits, (void**)&b->d_log, (void**)&b->d_idx,
+                     (void**)&b->d_snap};
+  const size_t sizes[] = {total[0], total[1], total64[0], total64[1], sizeof(b->prog[0].mats), sizeof(double2) * kNAmp,
+                          sizeof(float2) * (kNAmp + kSlabAmps), sizeof(qec_noise) * max_traj, sizeof(uint64_t) * max_traj,
+                          sizeof(BatchCtl), syn_bytes, (size_t)max_traj * kND, (size_t)max_traj, sizeof(uint32_t) * max_traj,
+                          sizeof(double2) * kNAmp};
   for (size_t i = 0; i < sizeof(sizes) / sizeof(sizes[0]); ++i) {
     e = cudaMalloc(allocs[i], sizes[i]);
     if (e != cudaSuccess) return bail(bfail(QEC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e)));
   }
   for (int w = 0; w < 2; ++w)
-    for (int i = 0; i < 5 && e == cudaSuccess; ++i)
-      if (bytes[w][i])
-        e = cudaMemcpy(b->d_fac[w] + b->fac_off[w][i], src[w][i], bytes[w][i], cudaMemcpyHostToDevice);
+    for (int i = 0; i < 12 && e == cudaSuccess; ++i)
+      if (src[w][i] && bytes[w][i])
+        e = cudaMemcpy(i < 5 ? b->d_fac[w] + b->fac_off[w][i] : b->d_prog64[w] + b->off64[w][i - 5], src[w][i], bytes[w][i],
+                       cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(b->d_mats, b->prog[0].mats, sizeof(b->prog[0].mats), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, std::string("upload: ") + cudaGetErrorString(e)));
   e = cudaMallocHost((void**)&b->h_ctl, sizeof(BatchCtl));
   if (e != cudaSuccess) return bail(bfail(QEC_ENOMEM, "pinned allocation failed"));
@@ -939,16 +847,18 @@ qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t m
   qec_status st = set_shape(b, 10);
   if (st) return bail(st);
   if ((st = set_fusion(b, 4, 256))) return bail(st);
-  for (int prec = 0; prec < 2; ++prec) {   // the noise-free init round, once per precision
-    BatchArgs a = batch_args(b);
-    a.F = batch_program(b, 1);
-    a.init_mode = 1;
-    a.init_prec = prec;
-    a.init_out = b->d_psi0[prec];
-    k_batch<<<1, 32, smem_for(1), b->work>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, std::string("init round: ") + cudaGetErrorString(e)));
-  }
+  // the noise-free init round, once per precision, in complex64 once per register
+  BatchArgs a = batch_args(b);
+  a.F = batch_program(b, 1);
+  a.init_out = b->d_psi0;
+  k_batch<<<1, 32, smem_for(1), b->work>>>(a);
+  e = cudaGetLastError();
+  Batch64Args a64 = batch64_args(b, 1);
+  a64.out = b->d_psi0_64;
+  if (e == cudaSuccess) e = launch_batch64(a64, 1, 1, b->work);
+  a64.out = b->d_psi0_64 + kNAmp;
+  if (e == cudaSuccess) e = launch_batch64_u(a64, 256, b->u_items, 1, b->work);
+  if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, std::string("init round: ") + cudaGetErrorString(e)));
   e = cudaStreamSynchronize(b->work);
   if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, std::string("init round: ") + cudaGetErrorString(e)));
   *out = b;
@@ -979,37 +889,26 @@ qec_status qec_batch_run(qec_batch* b, uint64_t seed, uint32_t n, const uint64_t
     QEC_BCUDA(cudaStreamWaitEvent(b->work, b->ev_in, 0));
   }
   QEC_BCUDA(cudaMemcpyAsync(b->d_traj, traj, sizeof(uint64_t) * n, cudaMemcpyHostToDevice, b->work));
-  QEC_BCUDA(cudaMemcpyAsync(b->d_kind, kind, sizeof(int32_t) * n, cudaMemcpyHostToDevice, b->work));
   QEC_BCUDA(cudaMemcpyAsync(b->d_noise, noise, sizeof(qec_noise) * n, cudaMemcpyHostToDevice, b->work));
-  b->h_idx.clear();
-  b->h_idx_u.clear();
-  // each engine's items complex128 first, then complex64: the warps (CTAs) then run one precision's
-  // code at a time instead of interleaving both instantiations, and the longer items start first.
-  // Every trajectory's result is independent of the order.
-  uint32_t n_u128 = 0;
-  for (int prec = 0; prec < 2; ++prec) {
-    for (uint32_t i = 0; i < n; ++i)
-      if ((kind[i] & 1) == prec) ((kind[i] & 2) ? b->h_idx_u : b->h_idx).push_back(i);
-    if (prec == 0) n_u128 = (uint32_t)b->h_idx_u.size();
-  }
-  if (!b->h_idx.empty())
-    QEC_BCUDA(cudaMemcpyAsync(b->d_idx, b->h_idx.data(), sizeof(uint32_t) * b->h_idx.size(), cudaMemcpyHostToDevice, b->work));
-  if (!b->h_idx_u.empty())
-    QEC_BCUDA(cudaMemcpyAsync(b->d_idx_u, b->h_idx_u.data(), sizeof(uint32_t) * b->h_idx_u.size(),
-                              cudaMemcpyHostToDevice, b->work));
+  uint32_t count[kKinds] = {0, 0, 0, 0}, at[kKinds];
+  for (uint32_t i = 0; i < n; ++i) ++count[kind[i]];
+  at[0] = 0;
+  for (int k = 1; k < kKinds; ++k) at[k] = at[k - 1] + count[k - 1];
+  b->h_idx.resize(n);
+  for (uint32_t i = 0; i < n; ++i) b->h_idx[at[kind[i]]++] = i;
+  QEC_BCUDA(cudaMemcpyAsync(b->d_idx, b->h_idx.data(), sizeof(uint32_t) * n, cudaMemcpyHostToDevice, b->work));
   QEC_BCUDA(cudaStreamSynchronize(b->work));   // h_ctl is reused
   b->h_ctl->seed = seed;
-  b->h_ctl->n = (uint32_t)b->h_idx.size();
-  b->h_ctl->counter = 0;
-  b->h_ctl->n_u[0] = n_u128;
-  b->h_ctl->n_u[1] = (uint32_t)b->h_idx_u.size() - n_u128;
-  b->h_ctl->counter_u[0] = b->h_ctl->counter_u[1] = 0;
+  for (int k = 0; k < kKinds; ++k) {
+    b->h_ctl->n[k] = count[k];
+    b->h_ctl->counter[k] = 0;
+  }
   const bool snap = b->snap_item >= 0 && b->snap_item < (int64_t)n;
   b->h_ctl->snap_item = snap ? (uint32_t)b->snap_item : ~0u;
   b->snap_valid = false;
   QEC_BCUDA(cudaMemcpyAsync(b->d_ctl, b->h_ctl, sizeof(BatchCtl), cudaMemcpyHostToDevice, b->work));
   QEC_BCUDA(cudaEventRecord(b->t0, b->work));
-  qec_status st = launch_batch(b, b->h_ctl->n, b->h_ctl->n_u[0], b->h_ctl->n_u[1]);
+  qec_status st = launch_batch(b);
   if (st) return st;
   QEC_BCUDA(cudaEventRecord(b->t1, b->work));
   const size_t ss = (size_t)(b->rounds + 1) * kNStab;
@@ -1070,7 +969,7 @@ qec_status qec_batch_autotune(qec_batch* b, uint64_t seed, uint32_t n, const uin
   // unreduced register: sweep width (slab bits) x threads per CTA
   int bk = -1, bthr = 256;
   float bu = 0.f;
-  for (int k : {4, 6})
+  for (int k = 2; k <= kUMaxFusion; ++k)
     for (int thr : {128, 256}) {
       if (set_fusion(b, k, thr) != QEC_OK) continue;
       float t;

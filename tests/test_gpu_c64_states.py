@@ -14,7 +14,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
-from paper_2204_11404_gb300.simulator import Simulator  # noqa: E402
+from paper_2204_11404_gb300.simulator import BatchSimulator, Simulator  # noqa: E402
 
 ALL = dict(p1=0.01, p2=0.012, p_idle=0.008, theta_rx=0.05, theta_rz=0.04, theta_rzx=0.03, phi_zz=0.02, round_rz=0.03, round_rx=0.02)
 NOISE = {"all": ALL, "cr": dict(p1=3e-3, p2=3e-3, p_idle=3e-3, theta_rx=0.03, phi_zz=0.02),
@@ -41,3 +41,18 @@ def test_handle_state(key):
         if n > 1:                      # whatever the call holds besides
             sim.run(1000 + rounds, 17 + n - 1, 1)
             check(sim.state(), GOLDEN[key])
+
+
+@pytest.mark.parametrize("key", [k for k in GOLDEN if k.startswith("batch/")])
+def test_batch_state(key):
+    _, kind, gates, noise, rounds = key.split("/")
+    rounds, nz = int(rounds), NOISE[noise]
+    with BatchSimulator(rounds, gates, max_traj=64) as b:
+        b.snapshot(1)
+        b.run(40 + rounds, [3, 900 + rounds, 7], ["c128", kind, "c64"], [nz] * 3)
+        check(b.state(), GOLDEN[key])
+        b.snapshot(40)                 # whatever the run holds besides, and in any configuration
+        b.set_config(4, 2, 128)
+        traj = [900 + rounds if i == 40 else i for i in range(64)]
+        b.run(40 + rounds, traj, [kind if i == 40 else ("c64", "c128", "c64u", "c128u")[i % 4] for i in range(64)], [nz] * 64)
+        check(b.state(), GOLDEN[key])
