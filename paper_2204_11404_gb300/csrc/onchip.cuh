@@ -84,6 +84,26 @@ __device__ __forceinline__ void group_sum2(double& a, double& b, double* red, in
   b = __shfl_sync(0xffffffffu, v, 16);
 }
 
+// The same sums over 128 places, four on a lane (place 32 i + lane) instead of one on each of 128 threads: the same
+// tree as group_sum2<128>, so that one warp and a CTA of four decide alike.  Each step of a warp's tree
+// halves the values that a lane carries: 11 additions, 5 for one value each.
+__device__ __forceinline__ void warp_sum4(const double (&a)[4], const double (&b)[4], double& A, double& B) {
+  const int lane = threadIdx.x & 31;
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+  double r[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) r[i] = (h16 ? b[i] : a[i]) + __shfl_xor_sync(0xffffffffu, h16 ? a[i] : b[i], 16);
+  double p0 = (h8 ? r[2] : r[0]) + __shfl_xor_sync(0xffffffffu, h8 ? r[0] : r[2], 8);
+  double p1 = (h8 ? r[3] : r[1]) + __shfl_xor_sync(0xffffffffu, h8 ? r[1] : r[3], 8);
+  double v = (h4 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, h4 ? p0 : p1, 4);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  v += __shfl_xor_sync(0xffffffffu, v, 8);   // the four warps' sums
+  v += __shfl_xor_sync(0xffffffffu, v, 4);
+  A = __shfl_sync(0xffffffffu, v, 0);
+  B = __shfl_sync(0xffffffffu, v, 16);
+}
+
 // The register's scale is free (a probability is a ratio of sums over one state): where the kept part's
 // norm gets small, an exact power of two brings it back into range.
 __device__ __forceinline__ int norm_exp(double a) { return (int)((__double_as_longlong(a) >> 52) & 0x7FF) - 1023; }
@@ -150,21 +170,33 @@ __device__ __forceinline__ int run_block(typename V2t<T>::t* psi, const FBlock& 
     qb = B.q[3];
   }
   sweep(qa, qb, w4 ? 2 : 0, false);
-  T s0 = 0, s1 = 0;   // the thread's share: at most 16 amplitudes
+  T s0[ITEMS], s1[ITEMS];
   int z0[ITEMS];
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     z0[i] = w4 ? (int)(((at[i] >> B.q[0]) & 1u) | (((at[i] >> B.q[1]) & 1u) << 1)) : 0;
+    s0[i] = s1[i] = 0;
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
       const int z = w4 ? z0[i] | (l << 2) : l;
       const T sq = fma(v[i][l].x, v[i][l].x, v[i][l].y * v[i][l].y);
-      s0 = fma(C.wt[0][z], sq, s0);
-      s1 = fma(C.wt[1][z], sq, s1);
+      s0[i] = fma(C.wt[0][z], sq, s0[i]);
+      s1[i] = fma(C.wt[1][z], sq, s1[i]);
     }
   }
-  double A0 = (double)s0, A1 = (double)s1;
-  group_sum2<NT>(A0, A1, red + (parity & 1) * 64, rank);
+  double A0, A1;
+  if constexpr (NT == 32 && ITEMS == 4) {
+    warp_sum4(s0, s1, A0, A1);
+  } else {
+    A0 = (double)s0[0];
+    A1 = (double)s1[0];
+#pragma unroll
+    for (int i = 1; i < ITEMS; ++i) {
+      A0 += (double)s0[i];
+      A1 += (double)s1[i];
+    }
+    group_sum2<NT>(A0, A1, red + (parity & 1) * 64, rank);
+  }
   const int m = forced >= 0 ? forced : C.u * (A0 + A1) < A1 ? 1 : 0;
   const double A = m ? A1 : A0;
   const bool rescale = small_norm(A);
