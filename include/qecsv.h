@@ -43,8 +43,8 @@ typedef enum { QEC_GATES_CNOT = 0, QEC_GATES_CR = 1 } qec_gateset;
 
 /* Amplitude storage / arithmetic.  A stabilizer block's Kraus operator runs in factored form (one rotation per
  * data qubit, a diagonal per outcome, index flips; qec_debug_factors) or as its dense matrix, on one of two
- * engines.  On chip: registers of up to 13 data qubits (complex128 at 13 qubits: calls of more than
- * 64 trajectories), whole trajectories in shared memory; complex128 factored, complex64 dense, whose
+ * engines.  On chip: registers of 9 and 11 data qubits, complex64 ones of 13 too: whole
+ * trajectories in shared memory; complex128 factored, complex64 dense, whose
  * states are the same to the last FP32 place from one version to the next (in the factored passes below
  * a complex64 state is reproducible to FP32 rounding between versions).  In passes over the state in HBM otherwise,
  * factored, several blocks to a pass: run for the outcomes the same stabilizers gave one round earlier (the init

@@ -65,10 +65,9 @@ struct qec_sim {
   size_t factor_off[5] = {};
   double fm[FM_COUNT][4][2] = {};
   // factored passes (rounds.cu): up to r_groups trajectories of r_G CTAs each
-  int r_groups = 0, r_G = 0;
-  std::vector<ChainDesc> chains, small_chains;
-  ChainDesc* d_chains = nullptr;        // chains, then small_chains
-  int small_ctas = 0;                   // with small tiles: at most this many CTAs (0: never)
+  int r_groups = 0, r_G = 0, r_tb = 0;  // r_tb: tile bits
+  std::vector<ChainDesc> chains;
+  ChainDesc* d_chains = nullptr;
   std::vector<DiagDesc> diags;
   DiagDesc* d_diags = nullptr;
   int n_x = 0;                          // blocks of X stabilizers (a round's first)
@@ -283,12 +282,22 @@ PassArgs spec_pass(const qec_sim* s, int b) {
   return a;
 }
 
-// Registers of up to 13 qubits run whole trajectories on chip (onchip.cu), one SM each, unless the
-// passes that compute each probability first were asked for.  2^13 complex128 amplitudes are enough
-// FP64 work for few trajectories to be faster in passes over all SMs (five rounds of the repetition
-// code, 1, 32 and 64 trajectories: 2.2 ms each on chip, 0.69, 0.95 and 1.83 ms in passes).
-bool on_chip(const qec_sim* s, uint32_t n) {
-  return s->spec && onchip_applies(s->D) && (s->D < 13 || !is_f64(s->p.precision) || n > 64);
+// Registers of up to 13 qubits run whole trajectories on chip, one SM each (onchip.cu; complex64: dense.cu), unless
+// the passes that compute each probability first were asked for.  2^13 complex128 amplitudes are enough FP64
+// work to be faster in passes over all SMs (five rounds of the repetition code, 1, 32 and 128 trajectories: 2.2 ms
+// each on chip, 0.27, 0.48 and 1.8 ms in passes; 1000: 14.5 and 14.2).  The engine, like the tile below, follows from
+// the register alone: it is part of the order of evaluation, so a trajectory's bits must not depend on the call's size.
+bool on_chip(const qec_sim* s) {
+  return s->spec && (onchip_applies(s->D) || dense_applies(s->p.precision, s->D));
+}
+
+// Small tiles (512 amplitudes, four on a thread) on the complex128 registers of 13 and 15 qubits: a pass's time there
+// is one warp's FP64 instructions, which four times the warps share.  Five rounds, 1, 8, 32 and 128 trajectories, small
+// and large tiles: 13 qubits 0.27, 0.30, 0.48, 1.8 and 0.46, 0.54, 0.59, 2.3 ms; 15 qubits 0.32, 0.55, 1.5, 5.8 and 0.54,
+// 0.63, 1.7, 5.3; 17 qubits 0.45, 1.7, 7.1, 29 and 0.62, 1.8, 5.9, 23.  complex64, 15 qubits: 0.27, 0.34, 0.99, 3.8 and
+// 0.30, 0.32, 0.40, 1.2.
+int tile_bits(const qec_params& p, int D) {
+  return p.code == QEC_CODE_REPETITION && is_f64(p.precision) && D <= 15 ? kSmallTileBits : kTileBits;
 }
 
 // Blocks per pass.  complex64 passes are bound by memory and shared-memory sweeps: four blocks share a
@@ -524,15 +533,11 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
     if ((e = setup_rounds(s->p.precision)) != cudaSuccess)
       return bail(fail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e)));
     const bool early = s->D >= kLargeD && !s->init_prog.blocks.empty() && s->p.code == QEC_CODE_SURFACE;
-    const int wave = round_wave(s->p.precision, kTileBits, early, s->num_sms), tiles = 1 << (s->D - kTileBits);
-    // Small tiles while they leave the GPU far from full (five rounds of the repetition code, small and
-    // large tiles: 15 qubits complex128, 8 trajectories = 512 CTAs: 0.72 and 0.94 ms, 32: 2.74 and 2.63;
-    // 17 qubits complex64, 1 = 256 CTAs: 0.33 and 0.43, 3: 0.69 and 0.50)
-    if (s->p.code == QEC_CODE_REPETITION && s->D < kLargeD)
-      s->small_ctas = std::min(512, round_wave(s->p.precision, kSmallTileBits, false, s->num_sms));
+    s->r_tb = tile_bits(s->p, s->D);
+    const int wave = round_wave(s->p.precision, s->r_tb, early, s->num_sms), tiles = 1 << (s->D - s->r_tb);
     if (wave < 1) return bail(fail(QEC_ECUDA, "the factored pass does not fit an SM"));
     s->r_G = std::min(wave, tiles);
-    s->r_groups = s->D == 13 ? 32 : wave / s->r_G;   // trajectories side by side where one does not fill the GPU
+    s->r_groups = s->D == 13 ? std::min(32, wave / s->r_G) : wave / s->r_G;   // trajectories side by side where one does not fill the GPU
   }
   const size_t groups = (size_t)s->r_groups;
   if ((st = dmalloc(&s->psi2, state_bytes * groups)) || (st = dmalloc(&s->psi, state_bytes * groups)) || (st = dmalloc(&s->psi0, state_bytes)) ||
@@ -559,15 +564,13 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   while (s->n_x < s->nstab && !s->fprog.blocks[s->n_x].z_type) ++s->n_x;
   if (rounds_size(s->p, s->D)) {
     const bool large = s->D >= kLargeD;
-    s->chains = plan_chains(s->fprog, s->p.precision, kTileBits, chain_limit(s->p, s->D), 0,
+    s->chains = plan_chains(s->fprog, s->p.precision, s->r_tb, chain_limit(s->p, s->D), 0,
                             large && s->n_x ? s->n_x : s->nstab);
-    if (s->small_ctas)
-      s->small_chains = plan_chains(s->fprog, s->p.precision, kSmallTileBits, kMaxChain, 0, s->nstab);
     if (large) s->diags = plan_diagonals(s->fprog, s->p.precision, s->n_x, s->nstab);
-    const size_t nr = groups * kMaxRounds, parts = 2 * (groups * s->r_G + 512 + s->num_sms) * (kMaxDiag + 1);
+    const size_t nr = groups * kMaxRounds, parts = 2 * (groups * s->r_G + s->num_sms) * (kMaxDiag + 1);
     const size_t bytes[8] = {nr * s->nstab * compiled_block_bytes(s->p.precision), nr * scratch, nr * sizeof(uint32_t),
                              groups * sizeof(double), parts * sizeof(double), 2 * groups * sizeof(unsigned int),
-                             sizeof(ChainDesc) * (s->chains.size() + s->small_chains.size()),
+                             sizeof(ChainDesc) * s->chains.size(),
                              sizeof(DiagDesc) * s->diags.size()};
     size_t off[8], total = 0;
     for (int i = 0; i < 8; ++i) {
@@ -587,9 +590,6 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(s->d_chains, s->chains.data(), sizeof(ChainDesc) * s->chains.size(), cudaMemcpyHostToDevice,
                           s->work);
-    if (e == cudaSuccess && !s->small_chains.empty())
-      e = cudaMemcpyAsync(s->d_chains + s->chains.size(), s->small_chains.data(),
-                          sizeof(ChainDesc) * s->small_chains.size(), cudaMemcpyHostToDevice, s->work);
     if (e == cudaSuccess && !s->diags.empty())
       e = cudaMemcpyAsync(s->d_diags, s->diags.data(), sizeof(DiagDesc) * s->diags.size(), cudaMemcpyHostToDevice, s->work);
     if (e != cudaSuccess) return bail(fail(QEC_ECUDA, cudaGetErrorString(e)));
@@ -602,7 +602,7 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
         (st = dmalloc(&s->d_dense_u, sizeof(double) * s->dense_cap)))
       return bail(st);
   }
-  if (onchip_applies(s->D)) {
+  if (onchip_applies(s->D) || s->dense_cap) {
     e = cudaMallocHost((void**)&s->h_out, (size_t)kBatchCap * (s->syn_cap + s->D + 1));
     if (e != cudaSuccess) return bail(fail(QEC_ENOMEM, "pinned allocation failed"));
   }
@@ -720,16 +720,14 @@ qec_status run_rounds(qec_sim* s, uint64_t seed, uint64_t first, uint32_t chunk)
   for (int i = 0; i < PR_COUNT; ++i) a.thr[i] = fac::draw_threshold(s->prog.prob[i]);
   std::memcpy(a.fm, s->fm, sizeof(a.fm));
   a.seed = seed;
-  const uint32_t side = std::min<uint32_t>((uint32_t)s->r_groups, chunk);
-  const bool small = s->small_ctas && ((uint64_t)side << (s->D - kSmallTileBits)) <= (uint64_t)s->small_ctas;
-  a.tb = small ? kSmallTileBits : kTileBits;
-  a.G = small ? 1 << (s->D - kSmallTileBits) : s->r_G;
+  a.tb = s->r_tb;
+  a.G = s->r_G;
   a.D = s->D;
   a.rounds = s->R;
-  a.chains = s->d_chains + (small ? s->chains.size() : 0);
+  a.chains = s->d_chains;
   a.diags = s->d_diags;
   const bool diagonal = large && all_diagonal(s);
-  a.nc = diagonal ? 0 : tensor ? s->n_x : (int)(small ? s->small_chains : s->chains).size();
+  a.nc = diagonal ? 0 : tensor ? s->n_x : (int)s->chains.size();
   a.nd = diagonal || a.F.early ? (int)s->diags.size() : 0;
   a.steps = a.nc + a.nd;
   a.step0 = a.nc;
@@ -807,7 +805,7 @@ qec_status run_rounds(qec_sim* s, uint64_t seed, uint64_t first, uint32_t chunk)
 qec_status run_impl(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8_t* syn, uint8_t* bits,
                     uint8_t* logical, bool host_out) {
   if (!s) return fail(QEC_EINVAL, "null handle");
-  const bool oc = on_chip(s, n), rd = !oc && rounds_apply(s);
+  const bool oc = on_chip(s), rd = !oc && rounds_apply(s);
   qec_status st = oc || rd ? QEC_OK : ensure_graph(s);
   if (st) return st;
   if (s->user) {

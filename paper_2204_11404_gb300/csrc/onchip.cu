@@ -1,5 +1,5 @@
-// On-chip complex128 trajectories: registers of up to 13 data qubits (the d = 3 surface code, the
-// repetition code up to d = 13), one CTA per trajectory, the whole trajectory in one launch.
+// On-chip complex128 trajectories: registers of 9 and 11 data qubits (the d = 3 surface code, the
+// repetition code of d = 9 and 11), one CTA per trajectory, the whole trajectory in one launch.
 //
 // What bounds it: for one trajectory latency (FP64 instructions issue at 64 cycles per warp and
 // scheduler on this chip, then barriers and the reduction trees of 8 blocks a round), for many the
@@ -21,9 +21,9 @@ using namespace oc;
 template <int NT, int ITEMS>
 struct Layout {
   static constexpr int kAmps = 4 * NT * ITEMS;
-  static constexpr int kD = kAmps == 512 ? 9 : kAmps == 2048 ? 11 : 13;
-  static constexpr int kStab = kD == 9 ? 8 : kD - 1;        // 8 (both codes), 10, 12
-  static constexpr int kRounds = kD == 13 ? 2 : 4;
+  static constexpr int kD = kAmps == 512 ? 9 : 11;
+  static constexpr int kStab = kD - 1;                        // 8 (both codes), 10
+  static constexpr int kRounds = 4;
   static constexpr int kTouches = 4 * kStab;
   static constexpr int kSites = 384;                          // draws of a round, at most
   static constexpr size_t kScratch = kRounds * (sizeof(fac::Touch) * kTouches + kTouches + kSites);
@@ -152,25 +152,20 @@ cudaError_t attr_t() {
 
 }  // namespace
 
-bool onchip_applies(int nd) { return nd == 9 || nd == 11 || nd == 13; }
+bool onchip_applies(int nd) { return nd == 9 || nd == 11; }
 
 cudaError_t setup_onchip() {
   cudaError_t e = attr_t<128, 1>();
   if (e == cudaSuccess) e = attr_t<512, 1>();
-  if (e == cudaSuccess) e = attr_t<1024, 2>();
   return e;
 }
 
-// Threads: one group of four amplitudes each up to 2^11 amplitudes (two at 2^13): a single trajectory's
-// latency is a chain of sweeps, and its FP64 work spreads over the SM's four schedulers.
+// Threads: one group of four amplitudes each: a single trajectory's latency is a chain of sweeps, and its
+// FP64 work spreads over the SM's four schedulers.
 cudaError_t launch_onchip(const OnchipArgs& a, int num_sms, cudaStream_t s) {
   if (!onchip_applies(a.F.nd) || a.F.nsites > Layout<128, 1>::kSites) return cudaErrorInvalidValue;
   if (a.n == 0) return cudaSuccess;
-  switch (a.F.nd) {
-    case 9: return launch_t<128, 1>(a, num_sms, s);
-    case 11: return launch_t<512, 1>(a, num_sms, s);
-    default: return launch_t<1024, 2>(a, num_sms, s);
-  }
+  return a.F.nd == 9 ? launch_t<128, 1>(a, num_sms, s) : launch_t<512, 1>(a, num_sms, s);
 }
 
 }  // namespace qec

@@ -24,7 +24,7 @@ struct OnchipArgs {
   int32_t* events;        // [ev_cap][5], null = not recorded
 };
 
-// Registers of 9, 11 and 13 data qubits run on chip: complex128 here, complex64 in dense blocks (dense.hpp).
+// complex128 registers of 9 and 11 data qubits run on chip (complex64 ones of 9 to 13: dense.hpp).
 bool onchip_applies(int nd);
 cudaError_t setup_onchip();
 cudaError_t launch_onchip(const OnchipArgs& a, int num_sms, cudaStream_t s);

@@ -163,8 +163,9 @@ __host__ __device__ __forceinline__ uint32_t slot_of(uint32_t e, const uint16_t*
   return e ^ (par(e & swz[0]) << P) ^ (par(e & swz[1]) << (P + 1)) ^ (par(e & swz[2]) << (P + 2));
 }
 
-// Groups of 2^GB amplitudes per thread: 16, or 4 on small registers (weight-2 blocks only), where a warp's
-// FP64 instructions, one every 64 cycles, are the pass's time and four times the warps share them.
+// Groups of 2^GB amplitudes per thread: 16, or 4 on small complex128 registers (weight-2 blocks only), where a
+// warp's FP64 instructions, one every 64 cycles, are the pass's time and four times the warps share them.  Eight
+// CTAs per SM (15 qubits, five rounds, 128 trajectories: 7.5, 6.9, 6.4 and 5.8 ms with 4, 5, 6 and 8).
 __host__ __device__ constexpr int group_bits(int TB) { return TB == 9 ? 2 : 4; }
 __host__ __device__ constexpr int round_threads(int TB) { return 1 << (TB - group_bits(TB)); }
 
@@ -271,7 +272,7 @@ __device__ __forceinline__ bool group_barrier(unsigned int* bar, unsigned int ta
 }
 
 template <typename T, bool POST, int TB>
-__global__ void __launch_bounds__(round_threads(TB), (POST ? Shape<T>::CTAS_POST : Shape<T>::CTAS)) k_rounds(const __grid_constant__ RoundArgs a, int r0, int r1) {
+__global__ void __launch_bounds__(round_threads(TB), (TB == kSmallTileBits ? 8 : POST ? Shape<T>::CTAS_POST : Shape<T>::CTAS)) k_rounds(const __grid_constant__ RoundArgs a, int r0, int r1) {
   using T2 = typename V2t<T>::t;
   using SH = Shape<T>;
   constexpr int GB = group_bits(TB), NT = round_threads(TB), NW = NT / 32, CH = 16 / sizeof(T2), NCH = (1 << TB) / (NT * CH);
@@ -866,7 +867,8 @@ struct RoundKernel {
 };
 template <typename T>
 static RoundKernel round_kernel_t(int tb, bool early) {
-  if (tb == 9) return {(const void*)k_rounds<T, false, 9>, sizeof(Smem<T, 9>)};
+  if constexpr (sizeof(T) == 8)
+    if (tb == kSmallTileBits) return {(const void*)k_rounds<T, false, kSmallTileBits>, sizeof(Smem<T, kSmallTileBits>)};
   return {early ? (const void*)k_rounds<T, true, 11> : (const void*)k_rounds<T, false, 11>, sizeof(Smem<T, 11>)};
 }
 static RoundKernel round_kernel(int precision, int tb, bool early) {
@@ -1045,8 +1047,8 @@ std::vector<DiagDesc> plan_diagonals(const FactorProgram& F, int precision, int 
 
 cudaError_t setup_rounds(int precision) {
   cudaError_t e = cudaSuccess;
-  for (int v = 0; v < 3 && e == cudaSuccess; ++v) {
-    const RoundKernel k = round_kernel(precision, v == 0 ? 9 : 11, v == 2);
+  for (int v = is_f64(precision) ? 0 : 1; v < 3 && e == cudaSuccess; ++v) {
+    const RoundKernel k = round_kernel(precision, v == 0 ? kSmallTileBits : kTileBits, v == 2);
     e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k.fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   }

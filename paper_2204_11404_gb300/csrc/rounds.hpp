@@ -27,8 +27,8 @@ struct ChainDesc {
   uint8_t bits[kMaxChain][4], qubit[kMaxChain][4];
 };
 
-// Tile bits of a rotating pass: 11 (2048 amplitudes, 16 on each of 128 threads), or, for few CTAs of
-// weight-2 blocks, 9 (512, 4 on each); runs of at least 8 amplitudes either way.
+// Tile bits of a rotating pass: 11 (2048 amplitudes, 16 on each of 128 threads), or, on small complex128
+// registers of weight-2 blocks, 9 (512, 4 on each); runs of at least 8 amplitudes either way.
 constexpr int kTileBits = 11, kSmallTileBits = 9;
 
 // Splits blocks [b0, b1) of a round into passes: as many consecutive blocks as one tile holds, at most `most`.
@@ -67,7 +67,7 @@ struct RoundArgs {
   const double* diag_in;            // the diagonal passes' own (default: norm), in and out; [rounds] strides
   double* diag_out;
   int diag_stride;
-  double* partials;                 // [2][groups G][kMaxChain]
+  double* partials;                 // [2][groups G][kMaxChain]; diagonal passes: [2][CTAs][kMaxDiag + 1]
   unsigned int* bar;                // [groups][2]: arrivals, departures (both 0 between launches)
   uint8_t* syn;                     // [groups][(rounds + 1) nstab]
   Ctl* ctl;

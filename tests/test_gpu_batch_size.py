@@ -1,5 +1,5 @@
-"""A trajectory's result is a function of its own inputs: the same bits from a run of few trajectories (one CTA
-each), of many (one warp each) and in any place, complex128 included."""
+"""A trajectory's result is a function of its own inputs: the same bits from a call of few trajectories and of
+many and in any place, complex128 included."""
 import numpy as np
 import pytest
 
@@ -11,7 +11,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
-from paper_2204_11404_gb300.simulator import BatchSimulator  # noqa: E402
+from paper_2204_11404_gb300.simulator import BatchSimulator, Simulator  # noqa: E402
 
 
 @pytest.mark.parametrize("gates", ["cr", "cnot"])
@@ -27,3 +27,21 @@ def test_same_state_bits_in_small_and_large_batches(kind, gates):
                 states.append(b.state())
             for s in states[1:]:
                 assert np.array_equal(s.view(np.uint64), states[0].view(np.uint64))
+
+
+@pytest.mark.parametrize("code,d,prec", [("surface", 3, "c128"), ("surface", 3, "c64"), ("repetition", 11, "c128"),
+                                         ("repetition", 13, "c128"), ("repetition", 13, "c64"), ("repetition", 15, "c128"),
+                                         ("repetition", 15, "c64"), ("repetition", 17, "c128tc"), ("repetition", 17, "c64")])
+def test_same_state_bits_in_short_and_long_calls(code, d, prec):
+    with Simulator(d, 3, "cr", prec, code=code, **W.STRESS) as sim:
+        ref = {}
+        for n in (1, 2, 3, 9, 40, 70):
+            out = sim.run(23, 200 - n, n)                     # the last trajectory is 199 every time
+            psi = sim.state()
+            for x, y in zip(out, ref.setdefault("out", out)):
+                assert (x[-1] == y[-1]).all()
+            assert np.array_equal(psi.view(np.uint64), ref.setdefault("psi", psi).view(np.uint64)), n
+        singles = [sim.run(23, 130 + i, 1) for i in (0, 31, 32, 69)]
+        for s, i in zip(singles, (0, 31, 32, 69)):
+            for x, y in zip(s, out):
+                assert (x[0] == y[i]).all()
