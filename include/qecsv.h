@@ -266,7 +266,8 @@ qec_status qec_batch_run(qec_batch* b, uint64_t seed, uint32_t n, const uint64_t
 /*
  * Autotuner: times qec_batch_run on the given sample and keeps the fastest
  * configuration of each engine, each timed on the sample's trajectories of its
- * register: the reduced-register engine's CTA shape (warps per CTA, one
+ * register, repeated until they fill the GPU twice or the handle's max_traj (an
+ * engine without any keeps its configuration), on the kernels of large runs: the reduced-register engine's CTA shape (warps per CTA, one
  * resident wave per SM), then the unreduced engines' fusion width k (2..6 slab
  * bits: complex64 gate units applied in one pass; complex128 rotates a weight-4
  * stabilizer's four data qubits in one sweep above 4, else two at a time) and

@@ -17,6 +17,7 @@
 // units before: reduced register 8.24 -> 1.43 ms, unreduced 33.3 -> 3.58.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -508,6 +509,7 @@ struct qec_batch {
   bool snap_valid = false;  // a completed run recorded a snapshot
   int fusion_k = 0;         // unreduced engines: slab bits a sweep or pass may hold (0: no plan yet)
   int u_threads = 256;      // unreduced engines: threads per CTA
+  bool tuning = false;      // runs use the configured warps however few trajectories they hold
 };
 
 namespace {
@@ -634,7 +636,7 @@ qec_status launch_batch(qec_batch* b) {
       // few trajectories: fewer warps on an SM each
       const uint32_t per = (n[kind] + b->num_sms - 1) / b->num_sms;
       if (u) QEC_BCUDA(launch_batch64_u(a64, b->u_threads, b->u_items, (int)grid, s));
-      else if (per < (uint32_t)b->warps_per_cta) QEC_BCUDA(launch_batch64(a64, (int)per, (int)((n[kind] + per - 1) / per), s));
+      else if (per < (uint32_t)b->warps_per_cta && !b->tuning) QEC_BCUDA(launch_batch64(a64, (int)per, (int)((n[kind] + per - 1) / per), s));
       else QEC_BCUDA(launch_batch64(a64, b->warps_per_cta, (int)grid, s));
     } else if (u) {
       a.idx_u = b->d_idx + base;
@@ -643,7 +645,7 @@ qec_status launch_batch(qec_batch* b) {
     } else {
       a.idx = b->d_idx + base;
       // up to four trajectories per SM: a CTA of four warps each (see above)
-      if (n[kind] <= 4u * (uint32_t)b->num_sms) k_batch_cta<<<n[kind], 128, kGroupSmem, s>>>(a);
+      if (n[kind] <= 4u * (uint32_t)b->num_sms && !b->tuning) k_batch_cta<<<n[kind], 128, kGroupSmem, s>>>(a);
       else k_batch<<<grid, 32 * b->warps_per_cta, smem_for(b->warps_per_cta), s>>>(a);
       QEC_BCUDA(cudaGetLastError());
     }
@@ -928,7 +930,8 @@ qec_status qec_batch_run(qec_batch* b, uint64_t seed, uint32_t n, const uint64_t
 qec_status qec_batch_autotune(qec_batch* b, uint64_t seed, uint32_t n, const uint64_t* traj, const int32_t* kind,
                               const qec_noise* noise, int32_t* chosen_warps, float* best_ms) {
   if (!b || !chosen_warps || !best_ms || !traj || !kind || !noise) return bfail(QEC_EINVAL, "null argument");
-  // the sample split by register: each engine is tuned on its own trajectories
+  // the sample split by register: each engine is tuned on its own trajectories, on the kernels that large runs
+  // take, repeated until they fill the GPU twice (or the handle); without any its configuration stays
   std::vector<uint64_t> tr[2];
   std::vector<int32_t> kd[2];
   std::vector<qec_noise> nz[2];
@@ -938,56 +941,68 @@ qec_status qec_batch_autotune(qec_batch* b, uint64_t seed, uint32_t n, const uin
     kd[u].push_back(kind[i]);
     nz[u].push_back(noise[i]);
   }
+  for (int u = 0; u < 2; ++u) {
+    const size_t own = tr[u].size(), want = std::min<size_t>(b->cap, (u ? 4 : 40) * (size_t)b->num_sms);
+    for (size_t i = 0; own && i + own < want; ++i) {
+      tr[u].push_back(tr[u][i]);
+      kd[u].push_back(kd[u][i]);
+      nz[u].push_back(nz[u][i]);
+    }
+  }
+  struct Tuning {
+    qec_batch* b;
+    explicit Tuning(qec_batch* x) : b(x) { b->tuning = true; }
+    ~Tuning() { b->tuning = false; }
+  };
   auto time_run = [&](int u, float& t) -> qec_status {
-    t = 1e30f;
-    if (tr[u].empty()) return QEC_OK;
-    for (int rep = 0; rep < 2; ++rep) {   // first run warms up
+    const Tuning on(b);
+    for (int rep = 0; rep < 3; ++rep) {   // first run warms up, the faster of the others counts
       qec_status st = qec_batch_run(b, seed, (uint32_t)tr[u].size(), tr[u].data(), kd[u].data(), nz[u].data(),
                                     nullptr, nullptr, nullptr);
       if (st) return st;
-      if (rep) t = b->last_ms;
+      if (rep) t = rep == 1 || b->last_ms < t ? b->last_ms : t;
     }
     return QEC_OK;
   };
-  // reduced register: warps per CTA
-  const int cand[] = {2, 4, 6, 8, 10};
-  int best = -1;
-  float best_t = 0.f;
-  for (int w : cand) {
-    if (set_shape(b, w) != QEC_OK) continue;
-    float t;
-    qec_status st = time_run(0, t);
-    if (st) return st;
-    if (best < 0 || t < best_t) {
-      best = w;
-      best_t = t;
-    }
-  }
-  if (best < 0) return bfail(QEC_EUNSUPPORTED, "no batched kernel shape fits");
-  qec_status st = set_shape(b, best);
-  if (st) return st;
-  // unreduced register: sweep width (slab bits) x threads per CTA
-  int bk = -1, bthr = 256;
-  float bu = 0.f;
-  for (int k = 2; k <= kUMaxFusion; ++k)
-    for (int thr : {128, 256}) {
-      if (set_fusion(b, k, thr) != QEC_OK) continue;
-      float t;
-      if ((st = time_run(1, t))) return st;
-      if (bk < 0 || t < bu) {
-        bk = k;
-        bthr = thr;
-        bu = t;
+  qec_status st;
+  if (!tr[0].empty()) {   // reduced register: warps per CTA
+    int best = -1;
+    float best_t = 0.f;
+    for (int w : {2, 4, 6, 8, 10}) {
+      if (set_shape(b, w) != QEC_OK) continue;
+      float t = 0.f;
+      if ((st = time_run(0, t))) return st;
+      if (best < 0 || t < best_t) {
+        best = w;
+        best_t = t;
       }
     }
-  if (bk < 0) return bfail(QEC_EUNSUPPORTED, "no unreduced engine shape fits");
-  if ((st = set_fusion(b, bk, bthr))) return st;
+    if (best < 0) return bfail(QEC_EUNSUPPORTED, "no batched kernel shape fits");
+    if ((st = set_shape(b, best))) return st;
+  }
+  if (!tr[1].empty()) {   // unreduced register: width in slab bits x threads per CTA
+    int bk = -1, bthr = 256;
+    float bu = 0.f;
+    for (int k = 2; k <= kUMaxFusion; ++k)
+      for (int thr : {128, 256}) {
+        if (set_fusion(b, k, thr) != QEC_OK) continue;
+        float t = 0.f;
+        if ((st = time_run(1, t))) return st;
+        if (bk < 0 || t < bu) {
+          bk = k;
+          bthr = thr;
+          bu = t;
+        }
+      }
+    if (bk < 0) return bfail(QEC_EUNSUPPORTED, "no unreduced engine shape fits");
+    if ((st = set_fusion(b, bk, bthr))) return st;
+  }
   float t_all = 0.f;   // the whole sample with the chosen configuration
   for (int rep = 0; rep < 2; ++rep) {
     if ((st = qec_batch_run(b, seed, n, traj, kind, noise, nullptr, nullptr, nullptr))) return st;
     t_all = b->last_ms;
   }
-  *chosen_warps = best;
+  *chosen_warps = b->warps_per_cta;
   *best_ms = t_all;
   return QEC_OK;
 }
