@@ -103,8 +103,7 @@ class BatchSimulator:
         nz = np.zeros((max(n, 1), len(capi.NOISE_FIELDS)))   # rows of qec_noise
         if not cls._noise_columns(nz, noise):
             for i, d in enumerate(noise):
-                for j, f in enumerate(capi.NOISE_FIELDS):
-                    nz[i, j] = float(d.get(f, 0.0))
+                nz[i] = [float(d.get(f, 0.0)) for f in capi.NOISE_FIELDS]
         return n, t, k, nz
 
     @staticmethod
