@@ -101,26 +101,31 @@ class BatchSimulator:
         except (KeyError, TypeError):   # numeric codes among them
             k = np.ascontiguousarray([cls._CODES.get(x, x) for x in kind], dtype=np.int32)
         nz = np.zeros((max(n, 1), len(capi.NOISE_FIELDS)))   # rows of qec_noise
-        if not cls._noise_columns(nz, noise):
+        if not cls._noise_dicts(nz, noise):
             for i, d in enumerate(noise):
                 nz[i] = [float(d.get(f, 0.0)) for f in capi.NOISE_FIELDS]
         return n, t, k, nz
 
     @staticmethod
-    def _noise_columns(nz, noise):
-        """A list of plain dicts with the same fields, one per row, a column at a time (8192 dicts of four
-        fields: 1.5 ms, 11.3 ms value by value).  False: it is something else, and nz holds zeros."""
-        if not isinstance(noise, (list, tuple)) or len(noise) != len(nz) or set(map(type, noise)) != {dict}:
+    def _noise_dicts(nz, noise):
+        """A list of plain dicts, at most one per row: a column at a time where they all have the same fields (8192
+        dicts of four fields: 1.5 ms, 11.3 ms value by value), else in one array.  False: it is something else, or
+        holds a value that only float() can judge; nz holds zeros."""
+        if not isinstance(noise, (list, tuple)) or not 0 < len(noise) <= len(nz) or set(map(type, noise)) != {dict}:
             return False
-        keys = list(noise[0])
-        if set(map(len, noise)) != {len(keys)} or not all(f in capi.NOISE_FIELDS for f in keys):
-            return False
+        keys, n = list(noise[0]), len(noise)
+        same = set(map(len, noise)) == {len(keys)} and all(f in capi.NOISE_FIELDS for f in keys)
         try:
-            for f in keys:
-                nz[:, capi.NOISE_FIELDS.index(f)] = np.fromiter(map(operator.itemgetter(f), noise), float, len(noise))
-            if not np.isnan(nz).any():   # (fromiter takes None for a nan)
+            try:
+                for f in keys if same else ():
+                    nz[:n, capi.NOISE_FIELDS.index(f)] = np.fromiter(map(operator.itemgetter(f), noise), float, n)
+            except KeyError:
+                same = False
+            if not same:
+                nz[:n] = np.array([[d.get(f, 0.0) for f in capi.NOISE_FIELDS] for d in noise], dtype=float)
+            if not np.isnan(nz).any():   # (numpy takes None for a nan)
                 return True
-        except (KeyError, TypeError, ValueError):
+        except (TypeError, ValueError):
             pass
         nz[:] = 0.0
         return False
