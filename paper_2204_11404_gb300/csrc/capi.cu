@@ -7,6 +7,7 @@
 #include <cstddef>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -71,8 +72,8 @@ struct qec_sim {
   std::vector<DiagDesc> diags;
   DiagDesc* d_diags = nullptr;
   int n_x = 0;                          // blocks of X stabilizers (a round's first)
-  unsigned char* d_rounds = nullptr;    // one allocation: the arrays below and the plans above
-  void* d_cblocks = nullptr;
+  unsigned char* d_all = nullptr;       // the allocation that holds every device buffer but d_events
+  unsigned char* d_cblocks = nullptr;
   unsigned char* d_scratch = nullptr;
   uint32_t* d_masks = nullptr;
   double* d_norm = nullptr;
@@ -80,7 +81,7 @@ struct qec_sim {
   unsigned int* d_bar = nullptr;
   const void* last_state = nullptr;     // of the last run in factored passes: its state and flips
   const uint32_t* last_masks = nullptr;
-  uint8_t* h_out = nullptr;             // pinned outputs of an on-chip batch, written by the kernel
+  uint8_t* h_out = nullptr;             // pinned outputs of an on-chip batch, written by the kernel (behind h_ctl)
   // complex64 on chip (dense.cu): Kraus pairs and uniforms of up to dense_cap blocks
   float2* d_dense = nullptr;
   double* d_dense_u = nullptr;
@@ -133,37 +134,32 @@ qec_status dmalloc(T** p, size_t bytes) {
   return QEC_OK;
 }
 
-qec_status upload_program(qec_sim* s, int which, const Program& P) {
-  qec_status st;
-  size_t cap = P.ops.size() + 1;
-  if (which == 1) {   // room for every noise site and coherent op, so qec_reconfigure never reallocates
-    qec_params full = s->p;
-    full.noise = qec_noise{1, 1, 1, 1, 1, 1, 1, 1, 1, 0};
-    Program F;
-    std::string err;
-    if (build_program(full, true, F, err, true) && F.ops.size() + 1 > cap) cap = F.ops.size() + 1;
-    s->ops_cap = cap;
+// A handle's device buffers, in one allocation (an allocation each took 0.3 to 0.6 ms of creating one).
+struct Buffers {
+  std::vector<std::pair<void**, size_t>> parts;
+  size_t total = 0;
+  template <typename T>
+  void add(T** p, size_t bytes) {
+    parts.emplace_back((void**)p, total);
+    total += (bytes + 255) / 256 * 256;
   }
-  if ((st = dmalloc(&s->d_ops[which], sizeof(ProgOp) * cap)) != QEC_OK) return st;
-  if ((st = dmalloc(&s->d_blocks[which], sizeof(BlockInfo) * P.blocks.size())) != QEC_OK) return st;
-  if ((st = dmalloc(&s->d_mats[which], sizeof(P.mats))) != QEC_OK) return st;
+  qec_status allocate(unsigned char** base) {
+    const qec_status st = dmalloc(base, total);
+    for (auto& p : parts) *p.first = st == QEC_OK ? *base + p.second : nullptr;
+    return st;
+  }
+};
+
+qec_status upload_program(qec_sim* s, int which, const Program& P) {
   if (!P.ops.empty())
-    QEC_CUDA(cudaMemcpy(s->d_ops[which], P.ops.data(), sizeof(ProgOp) * P.ops.size(), cudaMemcpyHostToDevice));
-  QEC_CUDA(cudaMemcpy(s->d_blocks[which], P.blocks.data(), sizeof(BlockInfo) * P.blocks.size(), cudaMemcpyHostToDevice));
-  QEC_CUDA(cudaMemcpy(s->d_mats[which], P.mats, sizeof(P.mats), cudaMemcpyHostToDevice));
+    QEC_CUDA(cudaMemcpyAsync(s->d_ops[which], P.ops.data(), sizeof(ProgOp) * P.ops.size(), cudaMemcpyHostToDevice, s->work));
+  QEC_CUDA(cudaMemcpyAsync(s->d_blocks[which], P.blocks.data(), sizeof(BlockInfo) * P.blocks.size(), cudaMemcpyHostToDevice, s->work));
+  QEC_CUDA(cudaMemcpyAsync(s->d_mats[which], P.mats, sizeof(P.mats), cudaMemcpyHostToDevice, s->work));
   return QEC_OK;
 }
 
-// The factored program's arrays behind each other; room for every noise site, so that qec_reconfigure
-// never reallocates.
-qec_status alloc_factor(qec_sim* s, size_t* scratch) {
-  qec_params full = s->p;
-  full.noise = qec_noise{1, 1, 1, 1, 1, 1, 1, 1, 1, 0};
-  Program P;
-  FactorProgram F;
-  std::string err;
-  if (!build_program(full, true, P, err, true) || !build_factor(P, F, err)) return fail(QEC_EINVAL, err);
-  *scratch = compile_scratch_bytes(F);
+// Where the factored program's arrays lie in d_factor; returns their size.
+size_t place_factor(qec_sim* s, const FactorProgram& F) {
   const size_t bytes[5] = {sizeof(FSite) * F.sites.size(), sizeof(FItem) * F.items.size(),
                            sizeof(FTouch) * F.touches.size(), sizeof(FBlock) * F.blocks.size(),
                            sizeof(uint16_t) * F.order.size()};
@@ -172,13 +168,11 @@ qec_status alloc_factor(qec_sim* s, size_t* scratch) {
     s->factor_off[i] = off;
     off += (bytes[i] + 255) / 256 * 256;
   }
-  return dmalloc(&s->d_factor, off);
+  return off;
 }
 
-// Builds prog's factored form and uploads it on the work stream (the caller waits before s->fprog changes).
+// Uploads prog's factored form on the work stream (the caller waits before s->fprog changes).
 qec_status upload_factor(qec_sim* s) {
-  std::string err;
-  if (!build_factor(s->prog, s->fprog, err)) return fail(QEC_EINVAL, err);
   factor_mats(s->prog.mats, s->p.gates == QEC_GATES_CR, s->p.noise.twirl != 0.0, s->fm);
   const FactorProgram& F = s->fprog;
   const void* src[5] = {F.sites.data(), F.items.data(), F.touches.data(), F.blocks.data(), F.order.data()};
@@ -475,12 +469,8 @@ void drop_graph(qec_sim* s) {
 
 void free_all(qec_sim* s) {
   drop_graph(s);
-  if (s->h_out) cudaFreeHost(s->h_out);
-  void* ptrs[] = {s->psi, s->psi0, s->psi2, s->d_factor, s->d_rounds, s->d_dense, s->d_dense_u, s->d_kraus, s->d_u, s->d_A, s->d_N, s->d_m,
-                  s->d_partials, s->d_ctl,
-                  s->d_hist_part, s->d_hist, s->d_syn, s->d_bits, s->d_log, s->d_events,
-                  s->d_ops[0], s->d_ops[1], s->d_blocks[0], s->d_blocks[1], s->d_mats[0], s->d_mats[1]};
-  for (void* p : ptrs) if (p) cudaFree(p);
+  if (s->d_all) cudaFree(s->d_all);
+  if (s->d_events) cudaFree(s->d_events);
   if (s->h_ctl) cudaFreeHost(s->h_ctl);
   for (cudaEvent_t ev : s->kev) if (ev) cudaEventDestroy(ev);
   for (cudaEvent_t ev : s->ctl_ev) if (ev) cudaEventDestroy(ev);
@@ -498,12 +488,15 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
     return fail(QEC_EUNSUPPORTED, "only the reduced (d^2+1 qubit) register runs on the GPU");
   qec_sim* s = new (std::nothrow) qec_sim();
   if (!s) return fail(QEC_ENOMEM, "host allocation failed");
+  struct Free {
+    void operator()(qec_sim* x) const { free_all(x); delete x; }
+  };
+  std::unique_ptr<qec_sim, Free> owner(s);
   qec_status st = QEC_OK;
-  auto bail = [&](qec_status x) { free_all(s); delete s; return x; };
   s->p = *params;
   s->user = static_cast<cudaStream_t>(stream);
   if (!build_program(s->p, false, s->init_prog, err) || !build_program(s->p, true, s->prog, err))
-    return bail(fail(QEC_EINVAL, err));
+    return fail(QEC_EINVAL, err);
   s->D = s->prog.nd;
   s->nstab = s->prog.nstab;
   s->R = s->p.rounds;
@@ -523,7 +516,7 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   if (e == cudaSuccess) e = setup_kernels(s->p.precision, s->D);
   if (e == cudaSuccess && dense_applies(s->p.precision, s->D)) e = setup_dense(s->D);
   else if (e == cudaSuccess && onchip_applies(s->D)) e = setup_onchip();
-  if (e != cudaSuccess) return bail(fail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e)));
+  if (e != cudaSuccess) return fail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e));
   const size_t state_bytes = ((size_t)1 << s->D) * s->amp;
   const int nblk = s->nstab * kMaxRounds;   // room for any round count (qec_reconfigure)
   const int k1 = hist_k1(s->D);
@@ -531,83 +524,89 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   s->r_groups = 1;
   if (rounds_size(s->p, s->D)) {
     if ((e = setup_rounds(s->p.precision)) != cudaSuccess)
-      return bail(fail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e)));
+      return fail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e));
     const bool early = s->D >= kLargeD && !s->init_prog.blocks.empty() && s->p.code == QEC_CODE_SURFACE;
     s->r_tb = tile_bits(s->p, s->D);
     const int wave = round_wave(s->p.precision, s->r_tb, early, s->num_sms), tiles = 1 << (s->D - s->r_tb);
-    if (wave < 1) return bail(fail(QEC_ECUDA, "the factored pass does not fit an SM"));
+    if (wave < 1) return fail(QEC_ECUDA, "the factored pass does not fit an SM");
     s->r_G = std::min(wave, tiles);
     s->r_groups = s->D == 13 ? std::min(32, wave / s->r_G) : wave / s->r_G;   // trajectories side by side where one does not fill the GPU
   }
-  const size_t groups = (size_t)s->r_groups;
-  if ((st = dmalloc(&s->psi2, state_bytes * groups)) || (st = dmalloc(&s->psi, state_bytes * groups)) || (st = dmalloc(&s->psi0, state_bytes)) ||
-      (st = dmalloc(&s->d_kraus, (size_t)nblk * KRAUS_STRIDE * s->amp)) ||
-      (st = dmalloc(&s->d_u, sizeof(double) * nblk)) || (st = dmalloc(&s->d_A, sizeof(double) * nblk)) ||
-      (st = dmalloc(&s->d_N, sizeof(double) * (nblk + 1))) || (st = dmalloc(&s->d_m, sizeof(int) * nblk)) ||
-      (st = dmalloc(&s->d_partials, sizeof(double) * 2 * MAX_PASS_GRID)) ||
-      (st = dmalloc(&s->d_ctl, sizeof(Ctl))) ||
-      (st = dmalloc(&s->d_hist_part, sizeof(double) * groups * ((size_t)hist_grid(s->D, s->num_sms) << k1))) ||
-      (st = dmalloc(&s->d_hist, (sizeof(double) * groups) << k1)) ||
-      (st = dmalloc(&s->d_syn, (size_t)kBatchCap * (kMaxRounds + 1) * s->nstab)) ||
-      (st = dmalloc(&s->d_bits, (size_t)kBatchCap * s->D)) || (st = dmalloc(&s->d_log, kBatchCap)))
-    return bail(st);
-  s->blk_cap = nblk;
-  s->syn_cap = (kMaxRounds + 1) * s->nstab;
-  e = cudaMallocHost((void**)&s->h_ctl, sizeof(Ctl) * kCtlRing);
-  if (e != cudaSuccess) return bail(fail(QEC_ENOMEM, "pinned allocation failed"));
-  std::memset(s->h_ctl, 0, sizeof(Ctl) * kCtlRing);
-  e = cudaMemcpy(s->d_ctl, s->h_ctl, sizeof(Ctl), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return bail(fail(QEC_ECUDA, cudaGetErrorString(e)));
-  if ((st = upload_program(s, 0, s->init_prog)) || (st = upload_program(s, 1, s->prog))) return bail(st);
-  size_t scratch = 0;
-  if ((st = alloc_factor(s, &scratch)) || (st = upload_factor(s))) return bail(st);
+  // room for every noise site and coherent op, and for any round count: qec_reconfigure never allocates
+  qec_params full = s->p;
+  full.noise = qec_noise{1, 1, 1, 1, 1, 1, 1, 1, 1, 0};
+  Program all;
+  FactorProgram fall;
+  if (!build_program(full, true, all, err, true) || !build_factor(all, fall, err) || !build_factor(s->prog, s->fprog, err))
+    return fail(QEC_EINVAL, err);
+  s->ops_cap = std::max(all.ops.size(), s->prog.ops.size()) + 1;
   while (s->n_x < s->nstab && !s->fprog.blocks[s->n_x].z_type) ++s->n_x;
-  if (rounds_size(s->p, s->D)) {
-    const bool large = s->D >= kLargeD;
+  const size_t groups = (size_t)s->r_groups;
+  Buffers B;
+  B.add(&s->psi2, state_bytes * groups);
+  B.add(&s->psi, state_bytes * groups);
+  B.add(&s->psi0, state_bytes);
+  B.add(&s->d_kraus, (size_t)nblk * KRAUS_STRIDE * s->amp);
+  B.add(&s->d_u, sizeof(double) * nblk);
+  B.add(&s->d_A, sizeof(double) * nblk);
+  B.add(&s->d_N, sizeof(double) * (nblk + 1));
+  B.add(&s->d_m, sizeof(int) * nblk);
+  B.add(&s->d_partials, sizeof(double) * 2 * MAX_PASS_GRID);
+  B.add(&s->d_ctl, sizeof(Ctl));
+  B.add(&s->d_hist_part, sizeof(double) * groups * ((size_t)hist_grid(s->D, s->num_sms) << k1));
+  B.add(&s->d_hist, (sizeof(double) * groups) << k1);
+  B.add(&s->d_syn, (size_t)kBatchCap * (kMaxRounds + 1) * s->nstab);
+  B.add(&s->d_bits, (size_t)kBatchCap * s->D);
+  B.add(&s->d_log, kBatchCap);
+  for (int w = 0; w < 2; ++w) {
+    B.add(&s->d_ops[w], sizeof(ProgOp) * (w ? s->ops_cap : s->init_prog.ops.size() + 1));
+    B.add(&s->d_blocks[w], sizeof(BlockInfo) * s->nstab);
+    B.add(&s->d_mats[w], sizeof(s->prog.mats));
+  }
+  B.add(&s->d_factor, place_factor(s, fall));
+  const bool passes = rounds_size(s->p, s->D), large = s->D >= kLargeD;
+  if (passes) {
     s->chains = plan_chains(s->fprog, s->p.precision, s->r_tb, chain_limit(s->p, s->D), 0,
                             large && s->n_x ? s->n_x : s->nstab);
     if (large) s->diags = plan_diagonals(s->fprog, s->p.precision, s->n_x, s->nstab);
-    const size_t nr = groups * kMaxRounds, parts = 2 * (groups * s->r_G + s->num_sms) * (kMaxDiag + 1);
-    const size_t bytes[8] = {nr * s->nstab * compiled_block_bytes(s->p.precision), nr * scratch, nr * sizeof(uint32_t),
-                             groups * sizeof(double), parts * sizeof(double), 2 * groups * sizeof(unsigned int),
-                             sizeof(ChainDesc) * s->chains.size(),
-                             sizeof(DiagDesc) * s->diags.size()};
-    size_t off[8], total = 0;
-    for (int i = 0; i < 8; ++i) {
-      off[i] = total;
-      total += (bytes[i] + 255) / 256 * 256;
-    }
-    if ((st = dmalloc(&s->d_rounds, total))) return bail(st);
-    s->d_cblocks = s->d_rounds + off[0];
-    s->d_scratch = s->d_rounds + off[1];
-    s->d_masks = reinterpret_cast<uint32_t*>(s->d_rounds + off[2]);
-    s->d_norm = reinterpret_cast<double*>(s->d_rounds + off[3]);
-    s->d_rparts = reinterpret_cast<double*>(s->d_rounds + off[4]);
-    s->d_bar = reinterpret_cast<unsigned int*>(s->d_rounds + off[5]);
-    s->d_chains = reinterpret_cast<ChainDesc*>(s->d_rounds + off[6]);
-    s->d_diags = reinterpret_cast<DiagDesc*>(s->d_rounds + off[7]);
-    e = cudaMemsetAsync(s->d_bar, 0, 2 * groups * sizeof(unsigned int), s->work);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(s->d_chains, s->chains.data(), sizeof(ChainDesc) * s->chains.size(), cudaMemcpyHostToDevice,
-                          s->work);
-    if (e == cudaSuccess && !s->diags.empty())
-      e = cudaMemcpyAsync(s->d_diags, s->diags.data(), sizeof(DiagDesc) * s->diags.size(), cudaMemcpyHostToDevice, s->work);
-    if (e != cudaSuccess) return bail(fail(QEC_ECUDA, cudaGetErrorString(e)));
+    const size_t nr = groups * kMaxRounds;
+    B.add(&s->d_cblocks, nr * s->nstab * compiled_block_bytes(s->p.precision));
+    B.add(&s->d_scratch, nr * compile_scratch_bytes(fall));
+    B.add(&s->d_masks, nr * sizeof(uint32_t));
+    B.add(&s->d_norm, groups * sizeof(double));
+    B.add(&s->d_rparts, sizeof(double) * 2 * (groups * s->r_G + s->num_sms) * (kMaxDiag + 1));
+    B.add(&s->d_bar, 2 * groups * sizeof(unsigned int));
+    B.add(&s->d_chains, sizeof(ChainDesc) * s->chains.size());
+    B.add(&s->d_diags, sizeof(DiagDesc) * s->diags.size());
   }
   if (dense_applies(s->p.precision, s->D)) {
     // 32 MiB of pairs with weight-4 blocks (340 trajectories of 3 rounds to a launch), 4 MiB without
+    if (!dense_fits(s->prog)) return fail(QEC_EUNSUPPORTED, "a block has more ops than the engine's table");
     s->dense_entries = dense_entries(s->prog);
     s->dense_cap = s->dense_entries == 256 ? 8192u : 16384u;
-    if ((st = dmalloc(&s->d_dense, sizeof(float2) * 2 * s->dense_entries * s->dense_cap)) ||
-        (st = dmalloc(&s->d_dense_u, sizeof(double) * s->dense_cap)))
-      return bail(st);
+    B.add(&s->d_dense, sizeof(float2) * 2 * s->dense_entries * s->dense_cap);
+    B.add(&s->d_dense_u, sizeof(double) * s->dense_cap);
   }
-  if (onchip_applies(s->D) || s->dense_cap) {
-    e = cudaMallocHost((void**)&s->h_out, (size_t)kBatchCap * (s->syn_cap + s->D + 1));
-    if (e != cudaSuccess) return bail(fail(QEC_ENOMEM, "pinned allocation failed"));
+  if ((st = B.allocate(&s->d_all))) return st;
+  s->blk_cap = nblk;
+  s->syn_cap = (kMaxRounds + 1) * s->nstab;
+  const size_t ctl_bytes = sizeof(Ctl) * kCtlRing, out_bytes = (size_t)kBatchCap * (s->syn_cap + s->D + 1);
+  const bool chip = onchip_applies(s->D) || s->dense_cap;
+  e = cudaMallocHost((void**)&s->h_ctl, ctl_bytes + (chip ? out_bytes : 0));
+  if (e != cudaSuccess) return fail(QEC_ENOMEM, "pinned allocation failed");
+  std::memset(s->h_ctl, 0, ctl_bytes);
+  if (chip) s->h_out = reinterpret_cast<uint8_t*>(s->h_ctl) + ctl_bytes;
+  QEC_CUDA(cudaMemcpyAsync(s->d_ctl, s->h_ctl, sizeof(Ctl), cudaMemcpyHostToDevice, s->work));
+  QEC_CUDA(cudaEventRecord(s->ctl_ev[0], s->work));   // (send_header reuses the slot)
+  if ((st = upload_program(s, 0, s->init_prog)) || (st = upload_program(s, 1, s->prog)) || (st = upload_factor(s))) return st;
+  if (passes) {
+    QEC_CUDA(cudaMemsetAsync(s->d_bar, 0, 2 * groups * sizeof(unsigned int), s->work));
+    QEC_CUDA(cudaMemcpyAsync(s->d_chains, s->chains.data(), sizeof(ChainDesc) * s->chains.size(), cudaMemcpyHostToDevice, s->work));
+    if (!s->diags.empty())
+      QEC_CUDA(cudaMemcpyAsync(s->d_diags, s->diags.data(), sizeof(DiagDesc) * s->diags.size(), cudaMemcpyHostToDevice, s->work));
   }
-  if ((st = run_init_round(s))) return bail(st);
-  *out = s;
+  if ((st = run_init_round(s))) return st;
+  *out = owner.release();
   return QEC_OK;
 }
 
@@ -957,13 +956,16 @@ qec_status qec_reconfigure(qec_sim* s, const qec_params* params) {
       params->layout != s->p.layout || params->code != s->p.code)
     return fail(QEC_EINVAL, "qec_reconfigure keeps d, gate set, precision, layout and code");
   Program P;
-  if (!build_program(*params, true, P, err)) return fail(QEC_EINVAL, err);
+  FactorProgram F;
+  if (!build_program(*params, true, P, err) || !build_factor(P, F, err)) return fail(QEC_EINVAL, err);
   if (params->rounds > kMaxRounds) return fail(QEC_EINVAL, "rounds exceed the simulator's capacity");
+  if (s->dense_cap && !dense_fits(P)) return fail(QEC_EUNSUPPORTED, "a block has more ops than the engine's table");
   if (P.ops.size() + 1 > s->ops_cap) return fail(QEC_EINVAL, "program larger than the simulator's capacity");
   QEC_CUDA(cudaStreamSynchronize(s->work));   // in-flight work still reads the old program
   drop_graph(s);
   const int S = s->nstab * params->rounds;
   s->prog = P;
+  s->fprog = F;
   if (!P.ops.empty())
     QEC_CUDA(cudaMemcpyAsync(s->d_ops[1], s->prog.ops.data(), sizeof(ProgOp) * P.ops.size(), cudaMemcpyHostToDevice,
                              s->work));

@@ -101,6 +101,7 @@ qec_status run_noalloc(const qec_params* params, uint64_t seed, uint64_t first_t
   const int pg4 = pass_grid(D, 4, sms);
   if (pg4 > pgrid) pgrid = pg4;
   const bool dense = dense_applies(prec, D);   // complex64: blocks' Kraus pairs, for as many trajectories as 1 MiB holds
+  if (dense && !dense_fits(prog)) return nfail(QEC_EUNSUPPORTED, "a block has more ops than the engine's table");
   const size_t entries = (size_t)dense_entries(prog), blocks = (size_t)nstab * R;
   const uint32_t most = blocks ? (uint32_t)((1u << 20) / (blocks * 2 * entries * sizeof(float2))) : 65535u;
   Carve c;
