@@ -476,6 +476,7 @@ struct qec_batch {
   cudaStream_t work = nullptr;
   cudaStream_t user = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr, t0 = nullptr, t1 = nullptr;
+  unsigned char* d_all = nullptr;    // the allocation that holds every device buffer
   FactorProgram fac[2];              // [0] noisy program, every slot present; [1] init program
   unsigned char* d_fac[2] = {nullptr, nullptr};
   size_t fac_off[2][5] = {};
@@ -528,9 +529,7 @@ qec_status bfail(qec_status s, const std::string& m) {
   } while (0)
 
 void batch_free(qec_batch* b) {
-  void* ptrs[] = {b->d_fac[0], b->d_fac[1], b->d_prog64[0], b->d_prog64[1], b->d_mats, b->d_psi0, b->d_psi0_64, b->d_noise,
-                  b->d_traj, b->d_ctl, b->d_syn, b->d_bits, b->d_log, b->d_idx, b->d_snap};
-  for (void* p : ptrs) if (p) cudaFree(p);
+  if (b->d_all) cudaFree(b->d_all);
   if (b->fork) cudaEventDestroy(b->fork);
   for (int i = 0; i < kKinds - 1; ++i) {
     if (b->join[i]) cudaEventDestroy(b->join[i]);
@@ -830,16 +829,20 @@ qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t m
                           sizeof(float2) * (kNAmp + kSlabAmps), sizeof(qec_noise) * max_traj, sizeof(uint64_t) * max_traj,
                           sizeof(BatchCtl), syn_bytes, (size_t)max_traj * kND, (size_t)max_traj, sizeof(uint32_t) * max_traj,
                           sizeof(double2) * kNAmp};
-  for (size_t i = 0; i < sizeof(sizes) / sizeof(sizes[0]); ++i) {
-    e = cudaMalloc(allocs[i], sizes[i]);
-    if (e != cudaSuccess) return bail(bfail(QEC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e)));
-  }
+  // one allocation, the programs and matrices (the first five) first: one copy
+  constexpr int kUploads = 5, kParts = sizeof(sizes) / sizeof(sizes[0]);
+  size_t off[kParts + 1] = {0};
+  for (int i = 0; i < kParts; ++i) off[i + 1] = off[i] + (sizes[i] + 255) / 256 * 256;
+  e = cudaMalloc((void**)&b->d_all, off[kParts]);
+  if (e != cudaSuccess) return bail(bfail(QEC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e)));
+  for (int i = 0; i < kParts; ++i) *allocs[i] = b->d_all + off[i];
+  std::vector<unsigned char> stage(off[kUploads]);
   for (int w = 0; w < 2; ++w)
-    for (int i = 0; i < 12 && e == cudaSuccess; ++i)
+    for (int i = 0; i < 12; ++i)
       if (src[w][i] && bytes[w][i])
-        e = cudaMemcpy(i < 5 ? b->d_fac[w] + b->fac_off[w][i] : b->d_prog64[w] + b->off64[w][i - 5], src[w][i], bytes[w][i],
-                       cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(b->d_mats, b->prog[0].mats, sizeof(b->prog[0].mats), cudaMemcpyHostToDevice);
+        std::memcpy(stage.data() + (i < 5 ? off[w] + b->fac_off[w][i] : off[2 + w] + b->off64[w][i - 5]), src[w][i], bytes[w][i]);
+  std::memcpy(stage.data() + off[4], b->prog[0].mats, sizeof(b->prog[0].mats));
+  e = cudaMemcpy(b->d_all, stage.data(), stage.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, std::string("upload: ") + cudaGetErrorString(e)));
   e = cudaMallocHost((void**)&b->h_ctl, sizeof(BatchCtl));
   if (e != cudaSuccess) return bail(bfail(QEC_ENOMEM, "pinned allocation failed"));
