@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -702,14 +703,24 @@ qec_status set_shape(qec_batch* b, int warps) {
 
 }  // namespace
 
+// Nothing throws across the C entries: what their host containers or strings may throw becomes a status.
+template <class F>
+static qec_status guarded(F f) {
+  try {
+    return f();
+  } catch (...) {
+    return bfail(QEC_ENOMEM, "host allocation failed");
+  }
+}
+
 extern "C" {
 
 qec_status qec_debug_unreduced_plan(int32_t gates, int32_t k, int32_t* items, uint32_t cap, uint32_t* n_items,
                                     int32_t* pass_units, uint32_t* n_pass_units, int32_t* absorbs, uint32_t* n_absorbs) {
-  if (!items || !n_items || !pass_units || !n_pass_units || !absorbs || !n_absorbs)
-    return bfail(QEC_EINVAL, "null argument");
-  if (k < 2 || k > kUMaxFusion) return bfail(QEC_EINVAL, "fusion width must be in [2, 6]");
-  try {
+  return guarded([&]() -> qec_status {
+    if (!items || !n_items || !pass_units || !n_pass_units || !absorbs || !n_absorbs)
+      return bfail(QEC_EINVAL, "null argument");
+    if (k < 2 || k > kUMaxFusion) return bfail(QEC_EINVAL, "fusion width must be in [2, 6]");
     qec_params p{};
     p.d = kD;
     p.rounds = 1;
@@ -747,267 +758,274 @@ qec_status qec_debug_unreduced_plan(int32_t gates, int32_t k, int32_t* items, ui
     *n_pass_units = (uint32_t)punits.size();
     *n_absorbs = na;
     return QEC_OK;
-  } catch (...) {
-    return bfail(QEC_ENOMEM, "host allocation failed");
-  }
+  });
 }
 
 qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t max_traj, void* cuda_stream,
                             qec_batch** out) {
-  if (!out) return bfail(QEC_EINVAL, "null output handle");
-  *out = nullptr;
-  if (d != kD) return bfail(QEC_EUNSUPPORTED, "the batched form runs the d = 3 reduced register");
-  if (rounds < 0 || rounds > 64 || max_traj == 0 || max_traj > (1u << 24))
-    return bfail(QEC_EINVAL, "rounds must be in [0, 64] and max_traj in [1, 2^24]");
-  qec_params p{};
-  p.d = d;
-  p.rounds = rounds;
-  p.layout = QEC_LAYOUT_REDUCED;
-  p.gates = gates;
-  p.precision = QEC_C128;
-  // every noise site and coherent op present; the per-trajectory values decide what they do
-  p.noise = qec_noise{1, 1, 1, 1, 1, 1, 1, 1, 1, 0};
-  std::string err;
-  qec_batch* b = new (std::nothrow) qec_batch();
-  if (!b) return bfail(QEC_ENOMEM, "host allocation failed");
-  auto bail = [&](qec_status s) { batch_free(b); delete b; return s; };
-  b->rounds = rounds;
-  b->gates = gates;
-  b->cap = max_traj;
-  b->user = static_cast<cudaStream_t>(cuda_stream);
-  for (int w = 0; w < 2; ++w) {
-    Program& P = b->prog[w];
-    UProgram& U = b->uprog[w];
-    if (!build_program(p, w == 0, P, err, w == 0) || !build_factor(P, b->fac[w], err) ||
-        !build_unreduced_program(p, w == 0, U, err, w == 0))
-      return bail(bfail(QEC_EINVAL, err));
-    if (b->fac[w].sites.size() > (size_t)kSites || P.ops.size() > (size_t)kBatchOps || U.items.size() > (size_t)kUMaxItems)
-      return bail(bfail(QEC_EUNSUPPORTED, "a round has more draws, ops or units than the engines' tables"));
-    if ((int)U.items.size() > b->u_items) b->u_items = (int)U.items.size();
-  }
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->work, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreate(&b->t0);
-  if (e == cudaSuccess) e = cudaEventCreate(&b->t1);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-  for (int i = 0; i < kKinds - 1; ++i) {
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming);
-  }
-  if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e)));
-  const size_t syn_bytes = (size_t)max_traj * (rounds + 1) * kNStab;
-  const void* src[2][12];
-  size_t bytes[2][12], total[2] = {0, 0}, total64[2] = {0, 0};
-  for (int w = 0; w < 2; ++w) {
-    const FactorProgram& F = b->fac[w];
-    const Program& P = b->prog[w];
-    const UProgram& U = b->uprog[w];
-    const size_t items = U.items.size();   // at least as many as there are passes, pass units or folded units
-    const void* s[12] = {F.sites.data(), F.items.data(), F.touches.data(), F.blocks.data(), F.order.data(),
-                         P.ops.data(), P.blocks.data(), U.ops.data(), U.items.data(), nullptr, nullptr, nullptr};
-    const size_t n[12] = {sizeof(FSite) * F.sites.size(), sizeof(FItem) * F.items.size(), sizeof(FTouch) * F.touches.size(),
-                          sizeof(FBlock) * F.blocks.size(), sizeof(uint16_t) * F.order.size(),
-                          sizeof(ProgOp) * P.ops.size(), sizeof(BlockInfo) * P.blocks.size(), sizeof(ProgOp) * U.ops.size(),
-                          sizeof(UItem) * items, sizeof(UPass) * items, sizeof(UPassUnit) * items, sizeof(UAbs) * items};
-    for (int i = 0; i < 12; ++i) {
-      size_t& at = i < 5 ? total[w] : total64[w];
-      src[w][i] = s[i];
-      bytes[w][i] = n[i];
-      (i < 5 ? b->fac_off[w][i] : b->off64[w][i - 5]) = at;
-      at += (n[i] + 255) / 256 * 256;
+  return guarded([&]() -> qec_status {
+    if (!out) return bfail(QEC_EINVAL, "null output handle");
+    *out = nullptr;
+    if (d != kD) return bfail(QEC_EUNSUPPORTED, "the batched form runs the d = 3 reduced register");
+    if (rounds < 0 || rounds > 64 || max_traj == 0 || max_traj > (1u << 24))
+      return bfail(QEC_EINVAL, "rounds must be in [0, 64] and max_traj in [1, 2^24]");
+    qec_params p{};
+    p.d = d;
+    p.rounds = rounds;
+    p.layout = QEC_LAYOUT_REDUCED;
+    p.gates = gates;
+    p.precision = QEC_C128;
+    // every noise site and coherent op present; the per-trajectory values decide what they do
+    p.noise = qec_noise{1, 1, 1, 1, 1, 1, 1, 1, 1, 0};
+    std::string err;
+    qec_batch* b = new (std::nothrow) qec_batch();
+    if (!b) return bfail(QEC_ENOMEM, "host allocation failed");
+    struct Free {
+      void operator()(qec_batch* x) const { batch_free(x); delete x; }
+    };
+    std::unique_ptr<qec_batch, Free> owner(b);
+    b->rounds = rounds;
+    b->gates = gates;
+    b->cap = max_traj;
+    b->user = static_cast<cudaStream_t>(cuda_stream);
+    for (int w = 0; w < 2; ++w) {
+      Program& P = b->prog[w];
+      UProgram& U = b->uprog[w];
+      if (!build_program(p, w == 0, P, err, w == 0) || !build_factor(P, b->fac[w], err) ||
+          !build_unreduced_program(p, w == 0, U, err, w == 0))
+        return bfail(QEC_EINVAL, err);
+      if (b->fac[w].sites.size() > (size_t)kSites || P.ops.size() > (size_t)kBatchOps || U.items.size() > (size_t)kUMaxItems)
+        return bfail(QEC_EUNSUPPORTED, "a round has more draws, ops or units than the engines' tables");
+      if ((int)U.items.size() > b->u_items) b->u_items = (int)U.items.size();
     }
-  }
-  void** allocs[] = {(void**)&b->d_fac[0], (void**)&b->d_fac[1], (void**)&b->d_prog64[0], (void**)&b->d_prog64[1],
-                     (void**)&b->d_mats, (void**)&b->d_psi0, (void**)&b->d_psi0_64, (void**)&b->d_noise, (void**)&b->d_traj,
-                     (void**)&b->d_ctl, (void**)&b->d_syn, (void**)&b->d_bits, (void**)&b->d_log, (void**)&b->d_idx,
-                     (void**)&b->d_snap};
-  const size_t sizes[] = {total[0], total[1], total64[0], total64[1], sizeof(b->prog[0].mats), sizeof(double2) * kNAmp,
-                          sizeof(float2) * (kNAmp + kSlabAmps), sizeof(qec_noise) * max_traj, sizeof(uint64_t) * max_traj,
-                          sizeof(BatchCtl), syn_bytes, (size_t)max_traj * kND, (size_t)max_traj, sizeof(uint32_t) * max_traj,
-                          sizeof(double2) * kNAmp};
-  // one allocation, the programs and matrices (the first five) first: one copy
-  constexpr int kUploads = 5, kParts = sizeof(sizes) / sizeof(sizes[0]);
-  size_t off[kParts + 1] = {0};
-  for (int i = 0; i < kParts; ++i) off[i + 1] = off[i] + (sizes[i] + 255) / 256 * 256;
-  e = cudaMalloc((void**)&b->d_all, off[kParts]);
-  if (e != cudaSuccess) return bail(bfail(QEC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e)));
-  for (int i = 0; i < kParts; ++i) *allocs[i] = b->d_all + off[i];
-  std::vector<unsigned char> stage(off[kUploads]);
-  for (int w = 0; w < 2; ++w)
-    for (int i = 0; i < 12; ++i)
-      if (src[w][i] && bytes[w][i])
-        std::memcpy(stage.data() + (i < 5 ? off[w] + b->fac_off[w][i] : off[2 + w] + b->off64[w][i - 5]), src[w][i], bytes[w][i]);
-  std::memcpy(stage.data() + off[4], b->prog[0].mats, sizeof(b->prog[0].mats));
-  e = cudaMemcpy(b->d_all, stage.data(), stage.size(), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, std::string("upload: ") + cudaGetErrorString(e)));
-  e = cudaMallocHost((void**)&b->h_ctl, sizeof(BatchCtl));
-  if (e != cudaSuccess) return bail(bfail(QEC_ENOMEM, "pinned allocation failed"));
-  std::memset(b->h_ctl, 0, sizeof(BatchCtl));
-  e = cudaMemcpy(b->d_ctl, b->h_ctl, sizeof(BatchCtl), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, cudaGetErrorString(e)));
-  qec_status st = set_shape(b, 10);
-  if (st) return bail(st);
-  if ((st = set_fusion(b, 4, 256))) return bail(st);
-  // the noise-free init round, once per precision, in complex64 once per register
-  BatchArgs a = batch_args(b);
-  a.F = batch_program(b, 1);
-  a.init_out = b->d_psi0;
-  k_batch<<<1, 32, smem_for(1), b->work>>>(a);
-  e = cudaGetLastError();
-  Batch64Args a64 = batch64_args(b, 1);
-  a64.out = b->d_psi0_64;
-  if (e == cudaSuccess) e = launch_batch64(a64, 1, 1, b->work);
-  a64.out = b->d_psi0_64 + kNAmp;
-  if (e == cudaSuccess) e = launch_batch64_u(a64, 256, b->u_items, 1, b->work);
-  if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, std::string("init round: ") + cudaGetErrorString(e)));
-  e = cudaStreamSynchronize(b->work);
-  if (e != cudaSuccess) return bail(bfail(QEC_ECUDA, std::string("init round: ") + cudaGetErrorString(e)));
-  *out = b;
-  return QEC_OK;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->work, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreate(&b->t0);
+    if (e == cudaSuccess) e = cudaEventCreate(&b->t1);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+    for (int i = 0; i < kKinds - 1; ++i) {
+      if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming);
+    }
+    if (e != cudaSuccess) return bfail(QEC_ECUDA, std::string("CUDA setup: ") + cudaGetErrorString(e));
+    const size_t syn_bytes = (size_t)max_traj * (rounds + 1) * kNStab;
+    const void* src[2][12];
+    size_t bytes[2][12], total[2] = {0, 0}, total64[2] = {0, 0};
+    for (int w = 0; w < 2; ++w) {
+      const FactorProgram& F = b->fac[w];
+      const Program& P = b->prog[w];
+      const UProgram& U = b->uprog[w];
+      const size_t items = U.items.size();   // at least as many as there are passes, pass units or folded units
+      const void* s[12] = {F.sites.data(), F.items.data(), F.touches.data(), F.blocks.data(), F.order.data(),
+                           P.ops.data(), P.blocks.data(), U.ops.data(), U.items.data(), nullptr, nullptr, nullptr};
+      const size_t n[12] = {sizeof(FSite) * F.sites.size(), sizeof(FItem) * F.items.size(), sizeof(FTouch) * F.touches.size(),
+                            sizeof(FBlock) * F.blocks.size(), sizeof(uint16_t) * F.order.size(),
+                            sizeof(ProgOp) * P.ops.size(), sizeof(BlockInfo) * P.blocks.size(), sizeof(ProgOp) * U.ops.size(),
+                            sizeof(UItem) * items, sizeof(UPass) * items, sizeof(UPassUnit) * items, sizeof(UAbs) * items};
+      for (int i = 0; i < 12; ++i) {
+        size_t& at = i < 5 ? total[w] : total64[w];
+        src[w][i] = s[i];
+        bytes[w][i] = n[i];
+        (i < 5 ? b->fac_off[w][i] : b->off64[w][i - 5]) = at;
+        at += (n[i] + 255) / 256 * 256;
+      }
+    }
+    void** allocs[] = {(void**)&b->d_fac[0], (void**)&b->d_fac[1], (void**)&b->d_prog64[0], (void**)&b->d_prog64[1],
+                       (void**)&b->d_mats, (void**)&b->d_psi0, (void**)&b->d_psi0_64, (void**)&b->d_noise, (void**)&b->d_traj,
+                       (void**)&b->d_ctl, (void**)&b->d_syn, (void**)&b->d_bits, (void**)&b->d_log, (void**)&b->d_idx,
+                       (void**)&b->d_snap};
+    const size_t sizes[] = {total[0], total[1], total64[0], total64[1], sizeof(b->prog[0].mats), sizeof(double2) * kNAmp,
+                            sizeof(float2) * (kNAmp + kSlabAmps), sizeof(qec_noise) * max_traj, sizeof(uint64_t) * max_traj,
+                            sizeof(BatchCtl), syn_bytes, (size_t)max_traj * kND, (size_t)max_traj, sizeof(uint32_t) * max_traj,
+                            sizeof(double2) * kNAmp};
+    // one allocation, the programs and matrices (the first five) first: one copy
+    constexpr int kUploads = 5, kParts = sizeof(sizes) / sizeof(sizes[0]);
+    size_t off[kParts + 1] = {0};
+    for (int i = 0; i < kParts; ++i) off[i + 1] = off[i] + (sizes[i] + 255) / 256 * 256;
+    e = cudaMalloc((void**)&b->d_all, off[kParts]);
+    if (e != cudaSuccess) return bfail(QEC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    for (int i = 0; i < kParts; ++i) *allocs[i] = b->d_all + off[i];
+    std::vector<unsigned char> stage(off[kUploads]);
+    for (int w = 0; w < 2; ++w)
+      for (int i = 0; i < 12; ++i)
+        if (src[w][i] && bytes[w][i])
+          std::memcpy(stage.data() + (i < 5 ? off[w] + b->fac_off[w][i] : off[2 + w] + b->off64[w][i - 5]), src[w][i], bytes[w][i]);
+    std::memcpy(stage.data() + off[4], b->prog[0].mats, sizeof(b->prog[0].mats));
+    e = cudaMemcpy(b->d_all, stage.data(), stage.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return bfail(QEC_ECUDA, std::string("upload: ") + cudaGetErrorString(e));
+    e = cudaMallocHost((void**)&b->h_ctl, sizeof(BatchCtl));
+    if (e != cudaSuccess) return bfail(QEC_ENOMEM, "pinned allocation failed");
+    std::memset(b->h_ctl, 0, sizeof(BatchCtl));
+    e = cudaMemcpy(b->d_ctl, b->h_ctl, sizeof(BatchCtl), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return bfail(QEC_ECUDA, cudaGetErrorString(e));
+    qec_status st = set_shape(b, 10);
+    if (st) return st;
+    if ((st = set_fusion(b, 4, 256))) return st;
+    // the noise-free init round, once per precision, in complex64 once per register
+    BatchArgs a = batch_args(b);
+    a.F = batch_program(b, 1);
+    a.init_out = b->d_psi0;
+    k_batch<<<1, 32, smem_for(1), b->work>>>(a);
+    e = cudaGetLastError();
+    Batch64Args a64 = batch64_args(b, 1);
+    a64.out = b->d_psi0_64;
+    if (e == cudaSuccess) e = launch_batch64(a64, 1, 1, b->work);
+    a64.out = b->d_psi0_64 + kNAmp;
+    if (e == cudaSuccess) e = launch_batch64_u(a64, 256, b->u_items, 1, b->work);
+    if (e != cudaSuccess) return bfail(QEC_ECUDA, std::string("init round: ") + cudaGetErrorString(e));
+    e = cudaStreamSynchronize(b->work);
+    if (e != cudaSuccess) return bfail(QEC_ECUDA, std::string("init round: ") + cudaGetErrorString(e));
+    *out = owner.release();
+    return QEC_OK;
+  });
 }
 
 qec_status qec_batch_run(qec_batch* b, uint64_t seed, uint32_t n, const uint64_t* traj, const int32_t* kind,
                          const qec_noise* noise, uint8_t* syndromes, uint8_t* data_bits, uint8_t* raw_logical) {
-  if (!b) return bfail(QEC_EINVAL, "null handle");
-  if (n > b->cap) return bfail(QEC_EINVAL, "n exceeds the batch capacity given at creation");
-  if (n == 0) return QEC_OK;
-  if (!traj || !kind || !noise) return bfail(QEC_EINVAL, "null input array");
-  for (uint32_t i = 0; i < n; ++i) {
-    if (kind[i] < 0 || kind[i] > 3)
-      return bfail(QEC_EINVAL, "kind must be precision (QEC_C128 or QEC_C64) | 2 * layout (QEC_LAYOUT_*)");
-    const qec_noise& z = noise[i];
-    const double pr[3] = {z.p1, z.p2, z.p_idle};
-    for (double v : pr)
-      if (!(v >= 0.0 && v <= 1.0)) return bfail(QEC_EINVAL, "noise probabilities must be in [0, 1]");
-    const double an[6] = {z.theta_rx, z.theta_rz, z.theta_rzx, z.phi_zz, z.round_rz, z.round_rx};
-    for (double v : an)
-      if (!(std::fabs(v) <= 4.0)) return bfail(QEC_EINVAL, "angles must be finite with |angle| <= 4");
-    if (z.twirl != 0.0 && z.twirl != 1.0) return bfail(QEC_EINVAL, "twirl must be 0 or 1");
-    if (z.overrot_follows != 0.0 && z.overrot_follows != 1.0) return bfail(QEC_EINVAL, "overrot_follows must be 0 or 1");
-  }
-  if (b->user) {
-    QEC_BCUDA(cudaEventRecord(b->ev_in, b->user));
-    QEC_BCUDA(cudaStreamWaitEvent(b->work, b->ev_in, 0));
-  }
-  QEC_BCUDA(cudaMemcpyAsync(b->d_traj, traj, sizeof(uint64_t) * n, cudaMemcpyHostToDevice, b->work));
-  QEC_BCUDA(cudaMemcpyAsync(b->d_noise, noise, sizeof(qec_noise) * n, cudaMemcpyHostToDevice, b->work));
-  uint32_t count[kKinds] = {0, 0, 0, 0}, at[kKinds];
-  for (uint32_t i = 0; i < n; ++i) ++count[kind[i]];
-  at[0] = 0;
-  for (int k = 1; k < kKinds; ++k) at[k] = at[k - 1] + count[k - 1];
-  b->h_idx.resize(n);
-  for (uint32_t i = 0; i < n; ++i) b->h_idx[at[kind[i]]++] = i;
-  QEC_BCUDA(cudaMemcpyAsync(b->d_idx, b->h_idx.data(), sizeof(uint32_t) * n, cudaMemcpyHostToDevice, b->work));
-  QEC_BCUDA(cudaStreamSynchronize(b->work));   // h_ctl is reused
-  b->h_ctl->seed = seed;
-  for (int k = 0; k < kKinds; ++k) {
-    b->h_ctl->n[k] = count[k];
-    b->h_ctl->counter[k] = 0;
-  }
-  const bool snap = b->snap_item >= 0 && b->snap_item < (int64_t)n;
-  b->h_ctl->snap_item = snap ? (uint32_t)b->snap_item : ~0u;
-  b->snap_valid = false;
-  QEC_BCUDA(cudaMemcpyAsync(b->d_ctl, b->h_ctl, sizeof(BatchCtl), cudaMemcpyHostToDevice, b->work));
-  QEC_BCUDA(cudaEventRecord(b->t0, b->work));
-  qec_status st = launch_batch(b);
-  if (st) return st;
-  QEC_BCUDA(cudaEventRecord(b->t1, b->work));
-  const size_t ss = (size_t)(b->rounds + 1) * kNStab;
-  if (syndromes) QEC_BCUDA(cudaMemcpyAsync(syndromes, b->d_syn, n * ss, cudaMemcpyDeviceToHost, b->work));
-  if (data_bits) QEC_BCUDA(cudaMemcpyAsync(data_bits, b->d_bits, (size_t)n * kND, cudaMemcpyDeviceToHost, b->work));
-  if (raw_logical) QEC_BCUDA(cudaMemcpyAsync(raw_logical, b->d_log, n, cudaMemcpyDeviceToHost, b->work));
-  if (b->user) {
-    QEC_BCUDA(cudaEventRecord(b->ev_out, b->work));
-    QEC_BCUDA(cudaStreamWaitEvent(b->user, b->ev_out, 0));
-  }
-  QEC_BCUDA(cudaStreamSynchronize(b->work));
-  QEC_BCUDA(cudaEventElapsedTime(&b->last_ms, b->t0, b->t1));
-  b->snap_valid = snap;
-  return QEC_OK;
+  return guarded([&]() -> qec_status {
+    if (!b) return bfail(QEC_EINVAL, "null handle");
+    if (n > b->cap) return bfail(QEC_EINVAL, "n exceeds the batch capacity given at creation");
+    if (n == 0) return QEC_OK;
+    if (!traj || !kind || !noise) return bfail(QEC_EINVAL, "null input array");
+    for (uint32_t i = 0; i < n; ++i) {
+      if (kind[i] < 0 || kind[i] > 3)
+        return bfail(QEC_EINVAL, "kind must be precision (QEC_C128 or QEC_C64) | 2 * layout (QEC_LAYOUT_*)");
+      const qec_noise& z = noise[i];
+      const double pr[3] = {z.p1, z.p2, z.p_idle};
+      for (double v : pr)
+        if (!(v >= 0.0 && v <= 1.0)) return bfail(QEC_EINVAL, "noise probabilities must be in [0, 1]");
+      const double an[6] = {z.theta_rx, z.theta_rz, z.theta_rzx, z.phi_zz, z.round_rz, z.round_rx};
+      for (double v : an)
+        if (!(std::fabs(v) <= 4.0)) return bfail(QEC_EINVAL, "angles must be finite with |angle| <= 4");
+      if (z.twirl != 0.0 && z.twirl != 1.0) return bfail(QEC_EINVAL, "twirl must be 0 or 1");
+      if (z.overrot_follows != 0.0 && z.overrot_follows != 1.0) return bfail(QEC_EINVAL, "overrot_follows must be 0 or 1");
+    }
+    if (b->user) {
+      QEC_BCUDA(cudaEventRecord(b->ev_in, b->user));
+      QEC_BCUDA(cudaStreamWaitEvent(b->work, b->ev_in, 0));
+    }
+    QEC_BCUDA(cudaMemcpyAsync(b->d_traj, traj, sizeof(uint64_t) * n, cudaMemcpyHostToDevice, b->work));
+    QEC_BCUDA(cudaMemcpyAsync(b->d_noise, noise, sizeof(qec_noise) * n, cudaMemcpyHostToDevice, b->work));
+    uint32_t count[kKinds] = {0, 0, 0, 0}, at[kKinds];
+    for (uint32_t i = 0; i < n; ++i) ++count[kind[i]];
+    at[0] = 0;
+    for (int k = 1; k < kKinds; ++k) at[k] = at[k - 1] + count[k - 1];
+    b->h_idx.resize(n);
+    for (uint32_t i = 0; i < n; ++i) b->h_idx[at[kind[i]]++] = i;
+    QEC_BCUDA(cudaMemcpyAsync(b->d_idx, b->h_idx.data(), sizeof(uint32_t) * n, cudaMemcpyHostToDevice, b->work));
+    QEC_BCUDA(cudaStreamSynchronize(b->work));   // h_ctl is reused
+    b->h_ctl->seed = seed;
+    for (int k = 0; k < kKinds; ++k) {
+      b->h_ctl->n[k] = count[k];
+      b->h_ctl->counter[k] = 0;
+    }
+    const bool snap = b->snap_item >= 0 && b->snap_item < (int64_t)n;
+    b->h_ctl->snap_item = snap ? (uint32_t)b->snap_item : ~0u;
+    b->snap_valid = false;
+    QEC_BCUDA(cudaMemcpyAsync(b->d_ctl, b->h_ctl, sizeof(BatchCtl), cudaMemcpyHostToDevice, b->work));
+    QEC_BCUDA(cudaEventRecord(b->t0, b->work));
+    qec_status st = launch_batch(b);
+    if (st) return st;
+    QEC_BCUDA(cudaEventRecord(b->t1, b->work));
+    const size_t ss = (size_t)(b->rounds + 1) * kNStab;
+    if (syndromes) QEC_BCUDA(cudaMemcpyAsync(syndromes, b->d_syn, n * ss, cudaMemcpyDeviceToHost, b->work));
+    if (data_bits) QEC_BCUDA(cudaMemcpyAsync(data_bits, b->d_bits, (size_t)n * kND, cudaMemcpyDeviceToHost, b->work));
+    if (raw_logical) QEC_BCUDA(cudaMemcpyAsync(raw_logical, b->d_log, n, cudaMemcpyDeviceToHost, b->work));
+    if (b->user) {
+      QEC_BCUDA(cudaEventRecord(b->ev_out, b->work));
+      QEC_BCUDA(cudaStreamWaitEvent(b->user, b->ev_out, 0));
+    }
+    QEC_BCUDA(cudaStreamSynchronize(b->work));
+    QEC_BCUDA(cudaEventElapsedTime(&b->last_ms, b->t0, b->t1));
+    b->snap_valid = snap;
+    return QEC_OK;
+  });
 }
 
 qec_status qec_batch_autotune(qec_batch* b, uint64_t seed, uint32_t n, const uint64_t* traj, const int32_t* kind,
                               const qec_noise* noise, int32_t* chosen_warps, float* best_ms) {
-  if (!b || !chosen_warps || !best_ms || !traj || !kind || !noise) return bfail(QEC_EINVAL, "null argument");
-  // the sample split by register: each engine is tuned on its own trajectories, on the kernels that large runs
-  // take, repeated until they fill the GPU twice (or the handle); without any its configuration stays
-  std::vector<uint64_t> tr[2];
-  std::vector<int32_t> kd[2];
-  std::vector<qec_noise> nz[2];
-  for (uint32_t i = 0; i < n; ++i) {
-    const int u = (kind[i] & 2) ? 1 : 0;
-    tr[u].push_back(traj[i]);
-    kd[u].push_back(kind[i]);
-    nz[u].push_back(noise[i]);
-  }
-  for (int u = 0; u < 2; ++u) {
-    const size_t own = tr[u].size(), want = std::min<size_t>(b->cap, (u ? 4 : 40) * (size_t)b->num_sms);
-    for (size_t i = 0; own && i + own < want; ++i) {
-      tr[u].push_back(tr[u][i]);
-      kd[u].push_back(kd[u][i]);
-      nz[u].push_back(nz[u][i]);
+  return guarded([&]() -> qec_status {
+    if (!b || !chosen_warps || !best_ms || !traj || !kind || !noise) return bfail(QEC_EINVAL, "null argument");
+    // the sample split by register: each engine is tuned on its own trajectories, on the kernels that large runs
+    // take, repeated until they fill the GPU twice (or the handle); without any its configuration stays
+    std::vector<uint64_t> tr[2];
+    std::vector<int32_t> kd[2];
+    std::vector<qec_noise> nz[2];
+    for (uint32_t i = 0; i < n; ++i) {
+      const int u = (kind[i] & 2) ? 1 : 0;
+      tr[u].push_back(traj[i]);
+      kd[u].push_back(kind[i]);
+      nz[u].push_back(noise[i]);
     }
-  }
-  struct Tuning {
-    qec_batch* b;
-    explicit Tuning(qec_batch* x) : b(x) { b->tuning = true; }
-    ~Tuning() { b->tuning = false; }
-  };
-  auto time_run = [&](int u, float& t) -> qec_status {
-    const Tuning on(b);
-    for (int rep = 0; rep < 3; ++rep) {   // first run warms up, the faster of the others counts
-      qec_status st = qec_batch_run(b, seed, (uint32_t)tr[u].size(), tr[u].data(), kd[u].data(), nz[u].data(),
-                                    nullptr, nullptr, nullptr);
-      if (st) return st;
-      if (rep) t = rep == 1 || b->last_ms < t ? b->last_ms : t;
-    }
-    return QEC_OK;
-  };
-  qec_status st;
-  if (!tr[0].empty()) {   // reduced register: warps per CTA
-    int best = -1;
-    float best_t = 0.f;
-    for (int w : {2, 4, 6, 8, 10}) {
-      if (set_shape(b, w) != QEC_OK) continue;
-      float t = 0.f;
-      if ((st = time_run(0, t))) return st;
-      if (best < 0 || t < best_t) {
-        best = w;
-        best_t = t;
+    for (int u = 0; u < 2; ++u) {
+      const size_t own = tr[u].size(), want = std::min<size_t>(b->cap, (u ? 4 : 40) * (size_t)b->num_sms);
+      for (size_t i = 0; own && i + own < want; ++i) {
+        tr[u].push_back(tr[u][i]);
+        kd[u].push_back(kd[u][i]);
+        nz[u].push_back(nz[u][i]);
       }
     }
-    if (best < 0) return bfail(QEC_EUNSUPPORTED, "no batched kernel shape fits");
-    if ((st = set_shape(b, best))) return st;
-  }
-  if (!tr[1].empty()) {   // unreduced register: width in slab bits x threads per CTA
-    int bk = -1, bthr = 256;
-    float bu = 0.f;
-    for (int k = 2; k <= kUMaxFusion; ++k)
-      for (int thr : {128, 256}) {
-        if (set_fusion(b, k, thr) != QEC_OK) continue;
+    struct Tuning {
+      qec_batch* b;
+      explicit Tuning(qec_batch* x) : b(x) { b->tuning = true; }
+      ~Tuning() { b->tuning = false; }
+    };
+    auto time_run = [&](int u, float& t) -> qec_status {
+      const Tuning on(b);
+      for (int rep = 0; rep < 3; ++rep) {   // first run warms up, the faster of the others counts
+        qec_status st = qec_batch_run(b, seed, (uint32_t)tr[u].size(), tr[u].data(), kd[u].data(), nz[u].data(),
+                                      nullptr, nullptr, nullptr);
+        if (st) return st;
+        if (rep) t = rep == 1 || b->last_ms < t ? b->last_ms : t;
+      }
+      return QEC_OK;
+    };
+    qec_status st;
+    if (!tr[0].empty()) {   // reduced register: warps per CTA
+      int best = -1;
+      float best_t = 0.f;
+      for (int w : {2, 4, 6, 8, 10}) {
+        if (set_shape(b, w) != QEC_OK) continue;
         float t = 0.f;
-        if ((st = time_run(1, t))) return st;
-        if (bk < 0 || t < bu) {
-          bk = k;
-          bthr = thr;
-          bu = t;
+        if ((st = time_run(0, t))) return st;
+        if (best < 0 || t < best_t) {
+          best = w;
+          best_t = t;
         }
       }
-    if (bk < 0) return bfail(QEC_EUNSUPPORTED, "no unreduced engine shape fits");
-    if ((st = set_fusion(b, bk, bthr))) return st;
-  }
-  float t_all = 0.f;   // the whole sample with the chosen configuration
-  for (int rep = 0; rep < 2; ++rep) {
-    if ((st = qec_batch_run(b, seed, n, traj, kind, noise, nullptr, nullptr, nullptr))) return st;
-    t_all = b->last_ms;
-  }
-  *chosen_warps = b->warps_per_cta;
-  *best_ms = t_all;
-  return QEC_OK;
+      if (best < 0) return bfail(QEC_EUNSUPPORTED, "no batched kernel shape fits");
+      if ((st = set_shape(b, best))) return st;
+    }
+    if (!tr[1].empty()) {   // unreduced register: width in slab bits x threads per CTA
+      int bk = -1, bthr = 256;
+      float bu = 0.f;
+      for (int k = 2; k <= kUMaxFusion; ++k)
+        for (int thr : {128, 256}) {
+          if (set_fusion(b, k, thr) != QEC_OK) continue;
+          float t = 0.f;
+          if ((st = time_run(1, t))) return st;
+          if (bk < 0 || t < bu) {
+            bk = k;
+            bthr = thr;
+            bu = t;
+          }
+        }
+      if (bk < 0) return bfail(QEC_EUNSUPPORTED, "no unreduced engine shape fits");
+      if ((st = set_fusion(b, bk, bthr))) return st;
+    }
+    float t_all = 0.f;   // the whole sample with the chosen configuration
+    for (int rep = 0; rep < 2; ++rep) {
+      if ((st = qec_batch_run(b, seed, n, traj, kind, noise, nullptr, nullptr, nullptr))) return st;
+      t_all = b->last_ms;
+    }
+    *chosen_warps = b->warps_per_cta;
+    *best_ms = t_all;
+    return QEC_OK;
+  });
 }
 
 qec_status qec_batch_config(const qec_batch* b, int32_t* warps_per_cta, int32_t* fusion_width, int32_t* u_threads) {
@@ -1019,10 +1037,12 @@ qec_status qec_batch_config(const qec_batch* b, int32_t* warps_per_cta, int32_t*
 }
 
 qec_status qec_batch_set_config(qec_batch* b, int32_t warps_per_cta, int32_t fusion_width, int32_t u_threads) {
-  if (!b) return bfail(QEC_EINVAL, "null handle");
-  qec_status st = set_shape(b, warps_per_cta);
-  if (st) return st;
-  return set_fusion(b, fusion_width, u_threads);
+  return guarded([&]() -> qec_status {
+    if (!b) return bfail(QEC_EINVAL, "null handle");
+    qec_status st = set_shape(b, warps_per_cta);
+    if (st) return st;
+    return set_fusion(b, fusion_width, u_threads);
+  });
 }
 
 qec_status qec_batch_snapshot(qec_batch* b, int64_t item) {

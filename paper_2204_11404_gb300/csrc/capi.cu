@@ -848,75 +848,75 @@ qec_status run_impl(qec_sim* s, uint64_t seed, uint64_t first, uint32_t n, uint8
 
 }  // namespace
 
+// Nothing throws across the C entries: what their host containers or strings may throw becomes a status.
+template <class F>
+static qec_status guarded(F f) {
+  try {
+    return f();
+  } catch (...) {
+    return fail(QEC_ENOMEM, "host allocation failed");
+  }
+}
+
 extern "C" {
 
 qec_status qec_create(const qec_params* params, void* cuda_stream, qec_sim** out) {
-  try {
-    return create_impl(params, cuda_stream, out);
-  } catch (...) {
-    return fail(QEC_ENOMEM, "exception in qec_create");
-  }
+  return guarded([&] { return create_impl(params, cuda_stream, out); });
 }
 
 qec_status qec_run_trajectories(qec_sim* sim, uint64_t seed, uint64_t first_traj, uint32_t n,
                                 uint8_t* syndromes, uint8_t* data_bits, uint8_t* raw_logical) {
-  try {
-    return run_impl(sim, seed, first_traj, n, syndromes, data_bits, raw_logical, true);
-  } catch (...) {
-    return fail(QEC_ENOMEM, "exception in qec_run_trajectories");
-  }
+  return guarded([&] { return run_impl(sim, seed, first_traj, n, syndromes, data_bits, raw_logical, true); });
 }
 
 qec_status qec_run_trajectories_device(qec_sim* sim, uint64_t seed, uint64_t first_traj, uint32_t n,
                                        uint8_t* d_syndromes, uint8_t* d_data_bits, uint8_t* d_raw_logical) {
-  try {
-    return run_impl(sim, seed, first_traj, n, d_syndromes, d_data_bits, d_raw_logical, false);
-  } catch (...) {
-    return fail(QEC_ENOMEM, "exception in qec_run_trajectories_device");
-  }
+  return guarded([&] { return run_impl(sim, seed, first_traj, n, d_syndromes, d_data_bits, d_raw_logical, false); });
 }
 
 uint64_t qec_state_len(const qec_sim* sim) { return sim ? (1ull << sim->D) : 0ull; }
 
 qec_status qec_get_state(qec_sim* s, void* host_buf, size_t bytes) {
-  if (!s || !host_buf) return fail(QEC_EINVAL, "null argument");
-  const size_t n = (size_t)1 << s->D;
-  if (bytes < 16 * n) return fail(QEC_EINVAL, "host buffer too small");
-  if (!s->ran) return fail(QEC_EINVAL, "no trajectory has run yet");
-  QEC_CUDA(cudaStreamSynchronize(s->work));
-  Ctl c;
-  QEC_CUDA(cudaMemcpy(&c, s->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
-  const void* src = final_state(s);
-  uint32_t flips = 0;   // the register holds data index x at x ^ flips
-  if (s->ran_on == qec_sim::ROUNDS && s->last_masks) {
-    std::vector<uint32_t> masks(s->R);
-    QEC_CUDA(cudaMemcpy(masks.data(), s->last_masks, sizeof(uint32_t) * masks.size(), cudaMemcpyDeviceToHost));
-    for (uint32_t m : masks) flips ^= m;
-  }
-  double* out = static_cast<double*>(host_buf);
-  const double scale = 1.0 / std::sqrt(c.final_norm);
-  if (is_f64(s->p.precision)) {
-    QEC_CUDA(cudaMemcpy(out, src, 16 * n, cudaMemcpyDeviceToHost));
-    // one pass: each amplitude scaled and, with flips, exchanged with its partner (d = 5 complex128: 53 ms, 94 in two passes)
-    size_t top = flips;   // their highest bit
-    while (top & (top - 1)) top &= top - 1;
-    if (!flips)
-      for (size_t i = 0; i < 2 * n; ++i) out[i] *= scale;
-    for (size_t base = 0; base < n && flips; base += 2 * top)
-      for (size_t i = base; i < base + top; ++i) {
-        double *a = out + 2 * i, *b = out + 2 * (i ^ flips);
-        const double re = a[0] * scale, im = a[1] * scale;
-        a[0] = b[0] * scale;
-        a[1] = b[1] * scale;
-        b[0] = re;
-        b[1] = im;
-      }
-  } else {
-    std::vector<float> tmp(2 * n);
-    QEC_CUDA(cudaMemcpy(tmp.data(), src, 8 * n, cudaMemcpyDeviceToHost));
-    for (size_t i = 0; i < 2 * n; ++i) out[i] = (double)tmp[i ^ (2 * (size_t)flips)] * scale;
-  }
-  return QEC_OK;
+  return guarded([&]() -> qec_status {
+    if (!s || !host_buf) return fail(QEC_EINVAL, "null argument");
+    const size_t n = (size_t)1 << s->D;
+    if (bytes < 16 * n) return fail(QEC_EINVAL, "host buffer too small");
+    if (!s->ran) return fail(QEC_EINVAL, "no trajectory has run yet");
+    QEC_CUDA(cudaStreamSynchronize(s->work));
+    Ctl c;
+    QEC_CUDA(cudaMemcpy(&c, s->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
+    const void* src = final_state(s);
+    uint32_t flips = 0;   // the register holds data index x at x ^ flips
+    if (s->ran_on == qec_sim::ROUNDS && s->last_masks) {
+      std::vector<uint32_t> masks(s->R);
+      QEC_CUDA(cudaMemcpy(masks.data(), s->last_masks, sizeof(uint32_t) * masks.size(), cudaMemcpyDeviceToHost));
+      for (uint32_t m : masks) flips ^= m;
+    }
+    double* out = static_cast<double*>(host_buf);
+    const double scale = 1.0 / std::sqrt(c.final_norm);
+    if (is_f64(s->p.precision)) {
+      QEC_CUDA(cudaMemcpy(out, src, 16 * n, cudaMemcpyDeviceToHost));
+      // one pass: each amplitude scaled and, with flips, exchanged with its partner (d = 5 complex128: 53 ms, 94 in two passes)
+      size_t top = flips;   // their highest bit
+      while (top & (top - 1)) top &= top - 1;
+      if (!flips)
+        for (size_t i = 0; i < 2 * n; ++i) out[i] *= scale;
+      for (size_t base = 0; base < n && flips; base += 2 * top)
+        for (size_t i = base; i < base + top; ++i) {
+          double *a = out + 2 * i, *b = out + 2 * (i ^ flips);
+          const double re = a[0] * scale, im = a[1] * scale;
+          a[0] = b[0] * scale;
+          a[1] = b[1] * scale;
+          b[0] = re;
+          b[1] = im;
+        }
+    } else {
+      std::vector<float> tmp(2 * n);
+      QEC_CUDA(cudaMemcpy(tmp.data(), src, 8 * n, cudaMemcpyDeviceToHost));
+      for (size_t i = 0; i < 2 * n; ++i) out[i] = (double)tmp[i ^ (2 * (size_t)flips)] * scale;
+    }
+    return QEC_OK;
+  });
 }
 
 qec_status qec_record_events(qec_sim* s, uint32_t max_events) {
@@ -949,38 +949,40 @@ qec_status qec_get_events(qec_sim* s, int32_t* host_events, uint32_t max_events,
 }
 
 qec_status qec_reconfigure(qec_sim* s, const qec_params* params) {
-  if (!s || !params) return fail(QEC_EINVAL, "null argument");
-  std::string err;
-  if (!validate_params(*params, err)) return fail(QEC_EINVAL, err);
-  if (params->d != s->p.d || params->gates != s->p.gates || params->precision != s->p.precision ||
-      params->layout != s->p.layout || params->code != s->p.code)
-    return fail(QEC_EINVAL, "qec_reconfigure keeps d, gate set, precision, layout and code");
-  Program P;
-  FactorProgram F;
-  if (!build_program(*params, true, P, err) || !build_factor(P, F, err)) return fail(QEC_EINVAL, err);
-  if (params->rounds > kMaxRounds) return fail(QEC_EINVAL, "rounds exceed the simulator's capacity");
-  if (s->dense_cap && !dense_fits(P)) return fail(QEC_EUNSUPPORTED, "a block has more ops than the engine's table");
-  if (P.ops.size() + 1 > s->ops_cap) return fail(QEC_EINVAL, "program larger than the simulator's capacity");
-  QEC_CUDA(cudaStreamSynchronize(s->work));   // in-flight work still reads the old program
-  drop_graph(s);
-  const int S = s->nstab * params->rounds;
-  s->prog = P;
-  s->fprog = F;
-  if (!P.ops.empty())
-    QEC_CUDA(cudaMemcpyAsync(s->d_ops[1], s->prog.ops.data(), sizeof(ProgOp) * P.ops.size(), cudaMemcpyHostToDevice,
-                             s->work));
-  QEC_CUDA(cudaMemcpyAsync(s->d_blocks[1], s->prog.blocks.data(), sizeof(BlockInfo) * P.blocks.size(),
-                           cudaMemcpyHostToDevice, s->work));
-  QEC_CUDA(cudaMemcpyAsync(s->d_mats[1], s->prog.mats, sizeof(P.mats), cudaMemcpyHostToDevice, s->work));
-  s->p = *params;
-  qec_status fst = upload_factor(s);
-  if (fst) return fst;
-  QEC_CUDA(cudaStreamSynchronize(s->work));   // the host copies in s->prog must outlive the uploads
-  s->R = params->rounds;
-  s->S = S;
-  s->timed_block = s->R > 0 ? pick_timed_block(s) : -1;
-  s->ran = false;
-  return QEC_OK;
+  return guarded([&]() -> qec_status {
+    if (!s || !params) return fail(QEC_EINVAL, "null argument");
+    std::string err;
+    if (!validate_params(*params, err)) return fail(QEC_EINVAL, err);
+    if (params->d != s->p.d || params->gates != s->p.gates || params->precision != s->p.precision ||
+        params->layout != s->p.layout || params->code != s->p.code)
+      return fail(QEC_EINVAL, "qec_reconfigure keeps d, gate set, precision, layout and code");
+    Program P;
+    FactorProgram F;
+    if (!build_program(*params, true, P, err) || !build_factor(P, F, err)) return fail(QEC_EINVAL, err);
+    if (params->rounds > kMaxRounds) return fail(QEC_EINVAL, "rounds exceed the simulator's capacity");
+    if (s->dense_cap && !dense_fits(P)) return fail(QEC_EUNSUPPORTED, "a block has more ops than the engine's table");
+    if (P.ops.size() + 1 > s->ops_cap) return fail(QEC_EINVAL, "program larger than the simulator's capacity");
+    QEC_CUDA(cudaStreamSynchronize(s->work));   // in-flight work still reads the old program
+    drop_graph(s);
+    const int S = s->nstab * params->rounds;
+    s->prog = P;
+    s->fprog = F;
+    if (!P.ops.empty())
+      QEC_CUDA(cudaMemcpyAsync(s->d_ops[1], s->prog.ops.data(), sizeof(ProgOp) * P.ops.size(), cudaMemcpyHostToDevice,
+                               s->work));
+    QEC_CUDA(cudaMemcpyAsync(s->d_blocks[1], s->prog.blocks.data(), sizeof(BlockInfo) * P.blocks.size(),
+                             cudaMemcpyHostToDevice, s->work));
+    QEC_CUDA(cudaMemcpyAsync(s->d_mats[1], s->prog.mats, sizeof(P.mats), cudaMemcpyHostToDevice, s->work));
+    s->p = *params;
+    qec_status fst = upload_factor(s);
+    if (fst) return fst;
+    QEC_CUDA(cudaStreamSynchronize(s->work));   // the host copies in s->prog must outlive the uploads
+    s->R = params->rounds;
+    s->S = S;
+    s->timed_block = s->R > 0 ? pick_timed_block(s) : -1;
+    s->ran = false;
+    return QEC_OK;
+  });
 }
 
 qec_status qec_selftest_wait(qec_sim* s, uint32_t polls) {
@@ -1038,27 +1040,29 @@ const char* qec_last_error(void) { return g_err.c_str(); }
 
 qec_status qec_debug_program(const qec_params* params, int32_t* ops, uint32_t cap, uint32_t* n_ops,
                              int32_t* block_info, uint32_t block_cap, uint32_t* n_blocks) {
-  if (!params || !n_ops || !n_blocks) return fail(QEC_EINVAL, "null argument");
-  std::string err;
-  Program P;
-  if (!build_program(*params, true, P, err)) return fail(QEC_EINVAL, err);
-  *n_ops = (uint32_t)P.ops.size();
-  *n_blocks = (uint32_t)P.blocks.size();
-  for (size_t b = 0; b < P.blocks.size(); ++b) {
-    const BlockInfo& bi = P.blocks[b];
-    if (block_info && b < block_cap) {
-      int32_t* o = block_info + 6 * b;
-      o[0] = bi.w; o[1] = bi.q[0]; o[2] = bi.q[1]; o[3] = bi.q[2]; o[4] = bi.q[3]; o[5] = bi.offset;
-    }
-    for (int i = bi.op_begin; i < bi.op_end; ++i) {
-      if (ops && (uint32_t)i < cap) {
-        const ProgOp& op = P.ops[i];
-        int32_t* o = ops + 6 * i;
-        o[0] = (int32_t)b; o[1] = op.kind; o[2] = op.q0; o[3] = op.q1; o[4] = op.step; o[5] = (int32_t)op.site;
+  return guarded([&]() -> qec_status {
+    if (!params || !n_ops || !n_blocks) return fail(QEC_EINVAL, "null argument");
+    std::string err;
+    Program P;
+    if (!build_program(*params, true, P, err)) return fail(QEC_EINVAL, err);
+    *n_ops = (uint32_t)P.ops.size();
+    *n_blocks = (uint32_t)P.blocks.size();
+    for (size_t b = 0; b < P.blocks.size(); ++b) {
+      const BlockInfo& bi = P.blocks[b];
+      if (block_info && b < block_cap) {
+        int32_t* o = block_info + 6 * b;
+        o[0] = bi.w; o[1] = bi.q[0]; o[2] = bi.q[1]; o[3] = bi.q[2]; o[4] = bi.q[3]; o[5] = bi.offset;
+      }
+      for (int i = bi.op_begin; i < bi.op_end; ++i) {
+        if (ops && (uint32_t)i < cap) {
+          const ProgOp& op = P.ops[i];
+          int32_t* o = ops + 6 * i;
+          o[0] = (int32_t)b; o[1] = op.kind; o[2] = op.q0; o[3] = op.q1; o[4] = op.step; o[5] = (int32_t)op.site;
+        }
       }
     }
-  }
-  return QEC_OK;
+    return QEC_OK;
+  });
 }
 
 // Variant 4: the fused pass's probability arithmetic on the CPU, A as one tile (one exponent for all
@@ -1140,96 +1144,98 @@ static void ozaki_spec_sums(const double* A, int m, double* out) {
 }
 
 qec_status qec_debug_ozaki_gemm(const double* A, const double* B, int32_t m, int32_t variant, double* out) {
-  if (!A || !B || !out || m <= 0 || variant < 0 || variant > 5) return fail(QEC_EINVAL, "bad argument");
-  if (variant == 4) {
-    ozaki_fused_prob(A, B, m, out);
-    return QEC_OK;
-  }
-  if (variant == 5) {
-    ozaki_spec_sums(A, m, out);
-    return QEC_OK;
-  }
-  std::vector<int> ea(m), eb(32);
-  std::vector<int> da((size_t)m * 32 * oz::kSlices), db(32 * 32 * oz::kSlices);
-  for (int r = 0; r < m; ++r) {
-    int E = 0;
-    for (int k = 0; k < 32; ++k) E = std::max(E, oz::bexp(A[r * 32 + k]));
-    ea[r] = E;
-    for (int k = 0; k < 32; ++k) oz::split7(A[r * 32 + k], E, &da[((size_t)r * 32 + k) * oz::kSlices]);
-  }
-  int EB = 0;   // variant 2 (probability pass): one exponent for all of B
-  for (int i = 0; i < 32 * 32; ++i) EB = std::max(EB, oz::bexp(B[i]));
-  for (int n = 0; n < 32; ++n) {
-    int E = 0;
-    for (int k = 0; k < 32; ++k) E = std::max(E, oz::bexp(B[n * 32 + k]));
-    eb[n] = (variant == 2 || variant == 3) ? EB : E;
-    for (int k = 0; k < 32; ++k) oz::split7(B[n * 32 + k], eb[n], &db[((size_t)n * 32 + k) * oz::kSlices]);
-  }
-  for (int r = 0; r < m; ++r) {
-    oz::SqAcc sa, sn;   // variants 2, 3: parts of kPart reals of a row, as the pass's threads hold them
-    oz::SqAccS ss;
-    double A2 = 0.0, N2 = 0.0, E3 = 0.0;
+  return guarded([&]() -> qec_status {
+    if (!A || !B || !out || m <= 0 || variant < 0 || variant > 5) return fail(QEC_EINVAL, "bad argument");
+    if (variant == 4) {
+      ozaki_fused_prob(A, B, m, out);
+      return QEC_OK;
+    }
+    if (variant == 5) {
+      ozaki_spec_sums(A, m, out);
+      return QEC_OK;
+    }
+    std::vector<int> ea(m), eb(32);
+    std::vector<int> da((size_t)m * 32 * oz::kSlices), db(32 * 32 * oz::kSlices);
+    for (int r = 0; r < m; ++r) {
+      int E = 0;
+      for (int k = 0; k < 32; ++k) E = std::max(E, oz::bexp(A[r * 32 + k]));
+      ea[r] = E;
+      for (int k = 0; k < 32; ++k) oz::split7(A[r * 32 + k], E, &da[((size_t)r * 32 + k) * oz::kSlices]);
+    }
+    int EB = 0;   // variant 2 (probability pass): one exponent for all of B
+    for (int i = 0; i < 32 * 32; ++i) EB = std::max(EB, oz::bexp(B[i]));
     for (int n = 0; n < 32; ++n) {
-      if (variant == 3) {   // the bounded pass: 3 slices each, every product, diagonals 0..4
-        float D5[5];
-        for (int t = 0; t < 5; ++t) {
-          float acc = 0.f;
-          for (int p = 0; p < 3; ++p) {
-            const int q = t - p;
-            if (q < 0 || q > 2) continue;
-            for (int k = 0; k < 32; ++k)
-              acc += (float)(da[((size_t)r * 32 + k) * oz::kSlices + p] * db[((size_t)n * 32 + k) * oz::kSlices + q]);
+      int E = 0;
+      for (int k = 0; k < 32; ++k) E = std::max(E, oz::bexp(B[n * 32 + k]));
+      eb[n] = (variant == 2 || variant == 3) ? EB : E;
+      for (int k = 0; k < 32; ++k) oz::split7(B[n * 32 + k], eb[n], &db[((size_t)n * 32 + k) * oz::kSlices]);
+    }
+    for (int r = 0; r < m; ++r) {
+      oz::SqAcc sa, sn;   // variants 2, 3: parts of kPart reals of a row, as the pass's threads hold them
+      oz::SqAccS ss;
+      double A2 = 0.0, N2 = 0.0, E3 = 0.0;
+      for (int n = 0; n < 32; ++n) {
+        if (variant == 3) {   // the bounded pass: 3 slices each, every product, diagonals 0..4
+          float D5[5];
+          for (int t = 0; t < 5; ++t) {
+            float acc = 0.f;
+            for (int p = 0; p < 3; ++p) {
+              const int q = t - p;
+              if (q < 0 || q > 2) continue;
+              for (int k = 0; k < 32; ++k)
+                acc += (float)(da[((size_t)r * 32 + k) * oz::kSlices + p] * db[((size_t)n * 32 + k) * oz::kSlices + q]);
+            }
+            D5[t] = acc;
           }
-          D5[t] = acc;
+          ss.add(oz::combine5(D5));
+          if (n % oz::kPart == oz::kPart - 1) {
+            const double ah = (ea[r] && EB) ? ss.take(2 * (ea[r] + EB - 2092)) : ss.take(-4000);
+            A2 += ah;
+            if (ea[r] && EB) E3 += oz::part_bound(ah, ea[r] + EB);
+          }
+          continue;
         }
-        ss.add(oz::combine5(D5));
-        if (n % oz::kPart == oz::kPart - 1) {
-          const double ah = (ea[r] && EB) ? ss.take(2 * (ea[r] + EB - 2092)) : ss.take(-4000);
-          A2 += ah;
-          if (ea[r] && EB) E3 += oz::part_bound(ah, ea[r] + EB);
+        float D[oz::kSlices];
+        for (int t = 0; t < oz::kSlices; ++t) {
+          float acc = 0.f;   // exact: every partial sum is an integer below 2^24
+          for (int p = 0; p <= t; ++p)
+            for (int k = 0; k < 32; ++k)
+              acc += (float)(da[((size_t)r * 32 + k) * oz::kSlices + p] * db[((size_t)n * 32 + k) * oz::kSlices + (t - p)]);
+          D[t] = acc;
         }
-        continue;
-      }
-      float D[oz::kSlices];
-      for (int t = 0; t < oz::kSlices; ++t) {
-        float acc = 0.f;   // exact: every partial sum is an integer below 2^24
-        for (int p = 0; p <= t; ++p)
-          for (int k = 0; k < 32; ++k)
-            acc += (float)(da[((size_t)r * 32 + k) * oz::kSlices + p] * db[((size_t)n * 32 + k) * oz::kSlices + (t - p)]);
-        D[t] = acc;
+        if (variant == 2) {
+          const int64_t z = oz::combine7(D);
+          sa.add((uint64_t)(z < 0 ? -z : z));
+          sn.add(ea[r] ? oz::mag56(A[r * 32 + n], ea[r]) : 0ull);
+          if (n % oz::kPart == oz::kPart - 1) {
+            A2 += (ea[r] && EB) ? sa.take(2 * (ea[r] + EB - 2098)) : sa.take(-4000);
+            N2 += sn.take(2 * (ea[r] - 1078));
+          }
+          continue;
+        }
+        if (variant == 1) {   // the apply pass's choice: checked only when the row may leave the range
+          int cmin = 4095, cmax = 0;
+          for (int j = 0; j < 32; ++j) {
+            if (eb[j]) cmin = std::min(cmin, eb[j]);
+            cmax = std::max(cmax, eb[j]);
+          }
+          const bool in_range = ea[r] == 0 || (ea[r] + cmin >= 1076 && ea[r] + cmax <= 2980);
+          out[r * 32 + n] = in_range ? oz::assemble7_cvt_inrange(D, ea[r], eb[n]) : oz::assemble7_cvt(D, ea[r], eb[n]);
+        } else {
+          out[r * 32 + n] = oz::assemble7(D, ea[r], eb[n]);
+        }
       }
       if (variant == 2) {
-        const int64_t z = oz::combine7(D);
-        sa.add((uint64_t)(z < 0 ? -z : z));
-        sn.add(ea[r] ? oz::mag56(A[r * 32 + n], ea[r]) : 0ull);
-        if (n % oz::kPart == oz::kPart - 1) {
-          A2 += (ea[r] && EB) ? sa.take(2 * (ea[r] + EB - 2098)) : sa.take(-4000);
-          N2 += sn.take(2 * (ea[r] - 1078));
-        }
-        continue;
+        out[r * 32] = A2;
+        out[r * 32 + 1] = N2;
       }
-      if (variant == 1) {   // the apply pass's choice: checked only when the row may leave the range
-        int cmin = 4095, cmax = 0;
-        for (int j = 0; j < 32; ++j) {
-          if (eb[j]) cmin = std::min(cmin, eb[j]);
-          cmax = std::max(cmax, eb[j]);
-        }
-        const bool in_range = ea[r] == 0 || (ea[r] + cmin >= 1076 && ea[r] + cmax <= 2980);
-        out[r * 32 + n] = in_range ? oz::assemble7_cvt_inrange(D, ea[r], eb[n]) : oz::assemble7_cvt(D, ea[r], eb[n]);
-      } else {
-        out[r * 32 + n] = oz::assemble7(D, ea[r], eb[n]);
+      if (variant == 3) {
+        out[r * 32] = A2;
+        out[r * 32 + 1] = E3;
       }
     }
-    if (variant == 2) {
-      out[r * 32] = A2;
-      out[r * 32 + 1] = N2;
-    }
-    if (variant == 3) {
-      out[r * 32] = A2;
-      out[r * 32 + 1] = E3;
-    }
-  }
-  return QEC_OK;
+    return QEC_OK;
+  });
 }
 
 qec_status qec_debug_exact_probability(qec_sim* sim, int32_t force, uint64_t* fallbacks) {
@@ -1271,56 +1277,60 @@ qec_status qec_debug_speculation(qec_sim* sim, int32_t enable, uint64_t* misses)
 
 qec_status qec_debug_factors(const qec_params* params, uint64_t seed, uint64_t traj, int32_t round, uint32_t* flips,
                              double* rot, double* diag) {
-  if (!params || !flips || !rot || !diag) return fail(QEC_EINVAL, "null argument");
-  std::string err;
-  Program P;
-  FactorProgram FP;
-  if (round < 1 || !build_program(*params, true, P, err) || !build_factor(P, FP, err))
-    return fail(QEC_EINVAL, err.empty() ? "bad round" : err);
-  double2 fm[FM_COUNT][4];
-  factor_mats(P.mats, params->gates == QEC_GATES_CR, params->noise.twirl != 0.0,
-              reinterpret_cast<double (*)[4][2]>(&fm[0][0]));
-  const size_t nt = 4 * (size_t)P.nstab;
-  std::vector<uint8_t> code(FP.sites.size() + 1), swap(nt);
-  std::vector<fac::Touch> T(nt);
-  uint32_t mask = 0;
-  const fac::Rounds R{1, code.data(), T.data(), swap.data(), &mask};
-  std::memset(rot, 0, sizeof(double) * 2 * nt);
-  std::memset(diag, 0, sizeof(double) * 64 * P.nstab);
-  const FactorView F = view_of(FP);
-  uint64_t thr[PR_COUNT];
-  for (int i = 0; i < PR_COUNT; ++i) thr[i] = fac::draw_threshold(P.prob[i]);
-  fac::compile_merge(fac::OneThread{}, F, thr, seed, traj, (uint64_t)round, fm, R, [](int, int, int) {});
-  fac::compile_emit(fac::OneThread{}, F, fm, R, *flips,
-                    [&](int, int t, double2 v) { rot[2 * t] = v.x; rot[2 * t + 1] = v.y; },
-                    [&](int, int b, int z, double2 d0, double2 d1) {
-                      double* o = diag + 64 * (size_t)b + 2 * z;
-                      o[0] = d0.x; o[1] = d0.y; o[32] = d1.x; o[33] = d1.y;
-                    });
-  *flips ^= mask;
-  return QEC_OK;
+  return guarded([&]() -> qec_status {
+    if (!params || !flips || !rot || !diag) return fail(QEC_EINVAL, "null argument");
+    std::string err;
+    Program P;
+    FactorProgram FP;
+    if (round < 1 || !build_program(*params, true, P, err) || !build_factor(P, FP, err))
+      return fail(QEC_EINVAL, err.empty() ? "bad round" : err);
+    double2 fm[FM_COUNT][4];
+    factor_mats(P.mats, params->gates == QEC_GATES_CR, params->noise.twirl != 0.0,
+                reinterpret_cast<double (*)[4][2]>(&fm[0][0]));
+    const size_t nt = 4 * (size_t)P.nstab;
+    std::vector<uint8_t> code(FP.sites.size() + 1), swap(nt);
+    std::vector<fac::Touch> T(nt);
+    uint32_t mask = 0;
+    const fac::Rounds R{1, code.data(), T.data(), swap.data(), &mask};
+    std::memset(rot, 0, sizeof(double) * 2 * nt);
+    std::memset(diag, 0, sizeof(double) * 64 * P.nstab);
+    const FactorView F = view_of(FP);
+    uint64_t thr[PR_COUNT];
+    for (int i = 0; i < PR_COUNT; ++i) thr[i] = fac::draw_threshold(P.prob[i]);
+    fac::compile_merge(fac::OneThread{}, F, thr, seed, traj, (uint64_t)round, fm, R, [](int, int, int) {});
+    fac::compile_emit(fac::OneThread{}, F, fm, R, *flips,
+                      [&](int, int t, double2 v) { rot[2 * t] = v.x; rot[2 * t + 1] = v.y; },
+                      [&](int, int b, int z, double2 d0, double2 d1) {
+                        double* o = diag + 64 * (size_t)b + 2 * z;
+                        o[0] = d0.x; o[1] = d0.y; o[32] = d1.x; o[33] = d1.y;
+                      });
+    *flips ^= mask;
+    return QEC_OK;
+  });
 }
 
 qec_status qec_debug_blocks(const qec_params* params, uint64_t seed, uint64_t traj, int32_t round,
                             double* kraus, double* u) {
-  if (!params || !kraus || !u) return fail(QEC_EINVAL, "null argument");
-  std::string err;
-  Program P;
-  if (round < 0 || !build_program(*params, round > 0, P, err)) return fail(QEC_EINVAL, err.empty() ? "bad round" : err);
-  InstArgs a;
-  a.ops = P.ops.data();
-  a.blocks = P.blocks.data();
-  a.mats = &P.mats[0][0][0];
-  for (int i = 0; i < PR_COUNT; ++i) a.prob[i] = P.prob[i];
-  a.nstab = P.nstab;
-  a.nd = P.nd;
-  a.round_base = round;
-  a.nblk = P.nstab;
-  for (int k = 0; k < P.nstab; ++k) {
-    double2* k0 = reinterpret_cast<double2*>(kraus) + (size_t)k * 512;
-    instantiate_block_host(a, k, seed, traj, k0, k0 + 256, u + k);
-  }
-  return QEC_OK;
+  return guarded([&]() -> qec_status {
+    if (!params || !kraus || !u) return fail(QEC_EINVAL, "null argument");
+    std::string err;
+    Program P;
+    if (round < 0 || !build_program(*params, round > 0, P, err)) return fail(QEC_EINVAL, err.empty() ? "bad round" : err);
+    InstArgs a;
+    a.ops = P.ops.data();
+    a.blocks = P.blocks.data();
+    a.mats = &P.mats[0][0][0];
+    for (int i = 0; i < PR_COUNT; ++i) a.prob[i] = P.prob[i];
+    a.nstab = P.nstab;
+    a.nd = P.nd;
+    a.round_base = round;
+    a.nblk = P.nstab;
+    for (int k = 0; k < P.nstab; ++k) {
+      double2* k0 = reinterpret_cast<double2*>(kraus) + (size_t)k * 512;
+      instantiate_block_host(a, k, seed, traj, k0, k0 + 256, u + k);
+    }
+    return QEC_OK;
+  });
 }
 
 }  // extern "C"
