@@ -9,7 +9,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libqecsv.so")
 SOURCES = ["program.cpp", "factor.cpp", "kernels.cu", "onchip.cu", "dense.cu", "rounds.cu", "capi.cu", "noalloc.cu", "batch.cu", "batch_dense.cu"]
-HEADERS = ["program.hpp", "factor.hpp", "factor.cuh", "onchip.cuh", "onchip.hpp", "dense.hpp", "batch_dense.hpp", "rounds.hpp", "common.cuh", "kernels.hpp", "ozaki.cuh"]
+HEADERS = ["program.hpp", "factor.hpp", "factor.cuh", "gate_eigen.hpp", "onchip.cuh", "onchip.hpp", "dense.hpp", "batch_dense.hpp", "rounds.hpp", "common.cuh", "kernels.hpp", "ozaki.cuh"]
 NVCC_FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_103a,code=sm_103a",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall"]
 

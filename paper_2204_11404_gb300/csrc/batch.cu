@@ -27,6 +27,7 @@
 
 #include "../../include/qecsv.h"
 #include "batch_dense.hpp"
+#include "gate_eigen.hpp"
 #include "onchip.cuh"
 #include "kernels.hpp"
 #include "program.hpp"
@@ -115,7 +116,7 @@ __device__ void trajectory_noise(const G& g, const qec_noise& nz, bool cr, Mem& 
     M.cs[l] = make_double2(c, s);
   }
   g.sync();
-  if (g.rank < FM_COUNT) {
+  if (g.rank < FM_SH) {
     const int id = g.rank;
     auto C = [&](int k) { return M.cs[k].x; };
     auto S = [&](int k) { return M.cs[k].y; };
@@ -168,6 +169,8 @@ __device__ void trajectory_noise(const G& g, const qec_noise& nz, bool cr, Mem& 
     const double p = g.rank == PR_P1 ? nz.p1 : g.rank == PR_P2 ? nz.p2 : g.rank == PR_IDLE ? nz.p_idle : tw ? s * s : 0.0;
     M.thr[g.rank] = fac::draw_threshold(p);
   }
+  g.sync();
+  if (g.rank == 0) gate_eigen<double2, double>(M.fm[FM_G0], M.fm[FM_G1], M.fm[FM_SH], M.fm[FM_A0], M.fm[FM_A1], M.fm[FM_LAM]);
   g.sync();
 }
 

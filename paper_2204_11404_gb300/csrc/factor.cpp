@@ -1,6 +1,8 @@
 // Builds the factored program (see factor.hpp) from the block program.
 #include "factor.hpp"
 
+#include "gate_eigen.hpp"
+
 
 namespace qec {
 
@@ -196,6 +198,16 @@ void factor_mats(const double (*mats)[16][2], bool cr, bool twirl, double (*out)
     f[FM_G0 + c] = cr ? mul(zz, mul(c2(M_ROT_RZX, c), block_of(mats[M_RZX90], c)))
                       : mul(zz, block_of(mats[M_CNOT], c));
   }
+  struct C { long double x, y; };
+  C g[2][4], r[4][4];
+  for (int i = 0; i < 4; ++i)
+    for (int c = 0; c < 2; ++c) g[c][i] = {f[FM_G0 + c].m[i][0], f[FM_G0 + c].m[i][1]};
+  gate_eigen<C, long double>(g[0], g[1], r[0], r[1], r[2], r[3]);
+  for (int j = 0; j < 4; ++j)   // FM_SH, FM_A0, FM_A1, FM_LAM
+    for (int i = 0; i < 4; ++i) {
+      f[FM_SH + j].m[i][0] = r[j][i].x;
+      f[FM_SH + j].m[i][1] = r[j][i].y;
+    }
   for (int i = 0; i < FM_COUNT; ++i)
     for (int k = 0; k < 4; ++k)
       for (int c = 0; c < 2; ++c) out[i][k][c] = (double)f[i].m[k][c];

@@ -89,6 +89,16 @@ QEC_HD uint64_t bits_of(double x) {
   return u;
 #endif
 }
+QEC_HD double signed_by(double x, int minus) {   // minus ? -x : x
+  const uint64_t u = bits_of(x) ^ ((uint64_t)minus << 63);
+#if defined(__CUDA_ARCH__)
+  return __longlong_as_double((long long)u);
+#else
+  double r;
+  memcpy(&r, &u, 8);
+  return r;
+#endif
+}
 QEC_HD bool below(double a, double b) { return bits_of(a) < bits_of(b); }
 QEC_HD bool is_zero(double x) { return (bits_of(x) << 1) == 0; }
 
@@ -118,12 +128,12 @@ QEC_HD int item_pauli(const FItem& it, const uint8_t* code, bool anc) {
 struct Touch {
   M2 g;          // stage 1: B; stage 2: G
   M2 post;       // A
-  double2 lam[2];   // X stabilizer: the eigenvalues
+  int flip;         // X stabilizer: the ancilla is flipped before the gate (G_1 meets its |0>)
   double2 ph[2];    // stage 3: lu, then lu rw
   double2 rw[2];
 };
 
-// Stage 1: B and A of touch t (and lambda for an X stabilizer).
+// Stage 1: B and A of touch t (and its flip for an X stabilizer).
 QEC_HD void touch_factors(const FactorView& F, int t, const uint8_t* code, const double2 (*fm)[4], Touch& out) {
   const FBlock& b = F.blocks[t >> 2];
   const FTouch& tc = F.touches[t];
@@ -169,55 +179,15 @@ QEC_HD void touch_factors(const FactorView& F, int t, const uint8_t* code, const
     const int p = item_pauli(it, code, true);
     flip ^= (p == 1 || p == 2);
   }
-  M2 g0, g1;
+  out.flip = flip;
+  M2 S, A;
   for (int k = 0; k < 4; ++k) {
-    g0.a[k] = fm[FM_G0][k];
-    g1.a[k] = fm[FM_G1][k];
+    S.a[k] = fm[FM_SH][k];
+    A.a[k] = fm[flip ? FM_A1 : FM_A0][k];
   }
-  M2 V0 = mul(flip ? g1 : g0, P), V1 = mul(flip ? g0 : g1, P);
-  for (++i; i < tc.end; ++i) {
-    const int p = item_pauli(F.items[i], code, false);   // after an X gate: Paulis only
-    pauli_left(p, V0);
-    pauli_left(p, V1);
-  }
-  // T = V0^dagger V1 (unitary) = S diag(lambda) S^dagger.  The traceless part of T is a phase times
-  // n . sigma with a real n; the phase is read off its largest component.
-  M2 T;
-  T.a[0] = cmulc2(V1.a[0], V0.a[0], V1.a[2], V0.a[2]);
-  T.a[1] = cmulc2(V1.a[1], V0.a[0], V1.a[3], V0.a[2]);
-  T.a[2] = cmulc2(V1.a[0], V0.a[1], V1.a[2], V0.a[3]);
-  T.a[3] = cmulc2(V1.a[1], V0.a[1], V1.a[3], V0.a[3]);
-  const double2 vz = c2(0.5 * (T.a[0].x - T.a[3].x), 0.5 * (T.a[0].y - T.a[3].y));
-  const double2 vx = c2(0.5 * (T.a[1].x + T.a[2].x), 0.5 * (T.a[1].y + T.a[2].y));
-  const double2 vy = times_i(c2(0.5 * (T.a[1].x - T.a[2].x), 0.5 * (T.a[1].y - T.a[2].y)), false);
-  const double lx = cnorm(vx), ly = cnorm(vy), lz = cnorm(vz);
-  const double2 ph = below(lx, ly) ? (below(ly, lz) ? vz : vy) : (below(lx, lz) ? vz : vx);
-  double nx = cmulc(vx, ph).x, ny = cmulc(vy, ph).x, nz = cmulc(vz, ph).x;
-  const double len2 = nx * nx + ny * ny + nz * nz;
-  double p = 1.0;
-  double2 q = c2(0.0, 0.0);
-  if (below(1e-280, len2)) {
-    const double k0 = rsqrt_d(len2), s = (bits_of(nz) >> 63) ? -k0 : k0;
-    nx *= s;
-    ny *= s;
-    nz *= s;
-    const double k = rsqrt_d(2.0 * (1.0 + nz));
-    p = (1.0 + nz) * k;
-    q = c2(nx * k, ny * k);
-  }
-  M2 S;   // columns: the eigenvectors
-  S.a[0] = c2(p, 0.0);
-  S.a[1] = c2(-q.x, q.y);
-  S.a[2] = q;
-  S.a[3] = c2(p, 0.0);
-  const M2 TS = mul(T, S);
-  out.lam[0] = cmulc2(TS.a[0], S.a[0], TS.a[2], S.a[2]);
-  out.lam[1] = cmulc2(TS.a[1], S.a[1], TS.a[3], S.a[3]);
-  out.g.a[0] = S.a[0];
-  out.g.a[1] = c2(q.x, -q.y);
-  out.g.a[2] = neg(q);
-  out.g.a[3] = S.a[3];
-  out.post = mul(V0, S);
+  out.g = mul(S, P);
+  for (++i; i < tc.end; ++i) pauli_left(item_pauli(F.items[i], code, false), A);   // after an X gate: Paulis only
+  out.post = A;
 }
 
 // Stage 2: G of touch t = B A_prev, and whether it swaps (its larger column-0 entry is G_10).  Reads
@@ -315,7 +285,10 @@ QEC_HD void block_diagonal(const FactorView& F, int b, int z, int f, const uint8
     }
   } else {
     double2 l = c2(1.0, 0.0);
-    for (int j = 0; j < B.w; ++j) l = cmul(l, T[4 * b + j].lam[(zl >> j) & 1]);
+    for (int j = 0; j < B.w; ++j) {
+      const double2 lm = fm[FM_LAM][3 * ((zl >> j) & 1)];
+      l = cmul(l, c2(lm.x, signed_by(lm.y, T[4 * b + j].flip)));
+    }
     v0 = c2(1.0, 0.0);
     v1 = c2(0.0, 0.0);
     // the branch that leaves the preparation with the ancilla in |1> carries l

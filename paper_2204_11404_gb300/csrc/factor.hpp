@@ -9,8 +9,9 @@
 //   Z stabilizer: B_j / A_j are qubit j's ops before / after its gate, and D_m(z) = <m| ancilla ops and
 //     the gates' blocks W_{z_j} in time order |0>.
 //   X stabilizer: the ancilla's Z value selects one of two branches (Paulis on it only swap them), so
-//     K_m = sum_a Q_ma (x)_j V_j^(a); with V_j^(0)+ V_j^(1) = S_j diag(lambda_j) S_j+ (both unitary),
-//     B_j = S_j+, A_j = V_j^(0) S_j, D_m(z) = Q_m0 + Q_m1 prod_j lambda_j(z_j).
+//     K_m = sum_a Q_ma (x)_j V_j^(a), V_j^(a) = L_j G_a P_j with the qubit's ops before and after its gate; with
+//     G_0+ G_1 = S Lambda S+ (the same for every gate), B_j = S+ P_j, A_j = L_j G_0 S, D_m(z) = Q_m0 + Q_m1 prod_j
+//     lambda(z_j); a flip of the ancilla before the gate exchanges G_0 and G_1, so lambda is conjugate.
 // Consecutive blocks' A and B on a qubit merge into one 2x2 unitary, itself a diagonal times a real
 // rotation times a diagonal; the diagonals go into the neighbouring D's (factor.cuh).  A dense 16x16
 // block costs 64 real multiply-adds per amplitude; its factored form 2 per qubit (a real rotation)
@@ -46,9 +47,12 @@ struct FItem {
 };
 
 // Matrices of the factored program (2x2, row-major): the round-start terms, the data corrections
-// with their over-rotations, the ancilla's preparation and final rotation, and the two blocks of the
-// gate with its coherent terms (control 0, control 1).
-enum FMatId : uint8_t { FM_ROUND = 0, FM_RX1, FM_RX2, FM_RZ1, FM_RZ2, FM_PREP, FM_POST, FM_G0, FM_G1, FM_COUNT };
+// with their over-rotations, the ancilla's preparation and final rotation, the two blocks G_0, G_1 of the
+// gate with its coherent terms (control 0, control 1), and what an X stabilizer makes of them: with
+// G_0+ G_1 = S Lambda S+, S+ (FM_SH), G_0 S and G_1 S (FM_A0, FM_A1) and Lambda (FM_LAM).
+enum FMatId : uint8_t {
+  FM_ROUND = 0, FM_RX1, FM_RX2, FM_RZ1, FM_RZ2, FM_PREP, FM_POST, FM_G0, FM_G1, FM_SH, FM_A0, FM_A1, FM_LAM, FM_COUNT
+};
 
 // A touch: data qubit j of block b, index 4 b + j.
 struct FTouch {
