@@ -379,7 +379,7 @@ def native_arm(args, rank, world, local):
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": 1e3 * secs / args.steps, "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": {"c128": "f64", "c64": "f32", "c64tc": "tf32x3",
+        "scaling": "weak", "vs_baseline": None, "dtype": {"c128": "f64", "c64": "f32", "c64tc": "f32",
                                                                  "c128tc": "f64 (fp16 slices)"}[args.precision],
         "data": "synthetic", "config": workload_config(args, world), "clocks": clk.summary(),
         "e2e": e2e, "gpu_launches": launches_per_traj * args.steps, "roofline": roof,
@@ -414,8 +414,8 @@ def native_arm(args, rank, world, local):
 
 
 def batched_arm(args, rank, world, local):
-    """8192 d=3 reduced-register trajectories (half complex128, half complex64, per-trajectory p and
-    theta) per step, one launch per engine on parallel streams; the CTA shapes are autotuned on a
+    """8192 d=3 trajectories (quarters of reduced and unreduced register x complex128 and complex64,
+    per-trajectory p and theta) per step, one launch per engine on parallel streams; the CTA shapes are autotuned on a
     1024-trajectory sample."""
     import torch
 
@@ -457,13 +457,13 @@ def batched_arm(args, rank, world, local):
                        "reduced_warps_per_cta": warps, "unreduced_fusion_width": fusion_k,
                        "unreduced_threads_per_cta": u_threads,
                        "sample": "--config" if args.config else
-                                 "the first 1024 trajectories, each engine on its own register's"},
+                                 "the first 1024 trajectories, each engine on its own register's, repeated"},
                    "kinds": args.kinds,
                    "rounds_per_s": world * n * rounds * args.steps / dev},
         "clocks": clk.summary(),
         "e2e": {"value": world * n * args.steps / wall, "unit": "trajectories/s",
-                "h2d_bytes_per_step": n * (8 + 4 + 72) + 16, "d2h_bytes_per_step": n * ((rounds + 1) * 8 + 9 + 1)},
-        "gpu_launches": 2 * args.steps,   # per step: the 10-qubit and the 17-qubit persistent kernels
+                "h2d_bytes_per_step": n * (8 + 4 + 88) + 48, "d2h_bytes_per_step": n * ((rounds + 1) * 8 + 9 + 1)},
+        "gpu_launches": len(set(kinds)) * args.steps,   # per step: a launch per register and precision
     }
     if rank == 0:
         print(json.dumps(out))

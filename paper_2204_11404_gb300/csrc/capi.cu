@@ -297,11 +297,16 @@ int tile_bits(const qec_params& p, int D) {
 // Blocks per pass.  complex64 passes are bound by memory and shared-memory sweeps: four blocks share a
 // read and a write.  complex128 ones are bound by the FP64 pipe, where a pass that runs again costs
 // all its blocks: one block each on large registers (d = 5, five rounds: 94.8, 101, 107, 112 ms for 1 to
-// 4); on small ones the barrier between passes counts (17 qubits: 1.25, 1.01, 0.94, 0.89 ms).
+// 4); on small ones the barrier between passes counts.  Five rounds of the repetition code whose blocks rotate, 1, 2 and
+// 4 blocks: complex128 17 qubits 1.23, 0.96, 0.83 ms, 19 qubits 1.94, 1.58, 1.46, 21 qubits 6.3, 5.8, 5.8 (six
+// trajectories 38.9, 37.2, 39.3), 23 qubits 18.8, 17.9, 18.0 (118, 116, 124); complex64 19 qubits 0.88, 0.58, 0.45, 21
+// qubits 1.73, 1.10, 0.89, 23 qubits 3.6, 2.3, 1.8.
 int chain_limit(const qec_params& p, int D) { return is_f64(p.precision) && D > 21 ? 1 : 4; }
 
 // Registers from here on are large enough that passes, not launches and barriers, take the time: a launch
-// per round and part, and the Z part in diagonal passes.
+// per round and part, and the Z part in diagonal passes.  Five rounds of the repetition code, diagonal throughout, in
+// diagonal passes and in rotating ones: 19 qubits complex64 1.70 and 0.43 ms, complex128 1.12 and 1.08; 21 qubits 0.85 and
+// 0.85, 1.07 and 3.7; 23 qubits 0.97 and 1.67, 2.0 and 11.6.
 constexpr int kLargeD = 21;
 
 // The factored engines (rounds.cu) have this register's buffers.

@@ -12,10 +12,10 @@
 // qubit, the diagonal of the outcome, the squares.  Tiles stream through shared memory (16-byte
 // asynchronous copies in, whole 128-byte runs out); the register is read and written once per pass.
 //
-// What bounds them at d = 5 (2^25 amplitudes): in complex64 the shared-memory sweeps (38% of issue slots, waits
-// on shared memory and barriers; 43% of DRAM throughput): 151 us for a pass of four blocks and 44 for one
-// of one, plus 34 until the last CTA arrives.  In complex128 the FP64 pipe: 550 to 946 us a block, plus 95
-// to 190 at the barrier, where the CTAs that were scheduled first on an SM wait for the others.  Against a
+// What bounds them at d = 5 (2^25 amplitudes): in complex64 the shared-memory sweeps and their barriers (52% of issue
+// slots, 0.54 of the copy bandwidth; per issue 1.6 cycles fixed latency, 1.4 shared memory, 1.2 barriers): 151 us for a
+// pass of four blocks and 44 for one of one, plus 34 until the last CTA arrives.  In complex128 the FP64 pipe: 550 to 946
+// us a block, plus 95 to 190 at the barrier, where the CTAs that were scheduled first on an SM wait for the others.  Against a
 // dense 16x16 pass per block, five rounds: complex64 19.1 -> 7.6 ms, complex128 359 -> 87; with the Z part
 // in diagonal passes 7.0 and 70.5.
 #include <cuda_runtime.h>

@@ -76,10 +76,10 @@ class Slot:
 
 class Server:
     """fp64_on_tensor_cores: complex128 jobs with d >= 5 run on the tensor-core complex128 engine
-    ("c128tc": the same outcomes, amplitudes within a few FP64 roundings, about 10x faster); False
-    keeps them on the FP64 CUDA-core engine.  fp32_on_tensor_cores: complex64 jobs with d >= 5 run on
-    the tensor-core complex64 engine ("c64tc": 3xTF32 products with FP32 accumulation, within the
-    complex64 tolerance of the oracle, about 1.2x faster); False keeps them on the FP32 CUDA cores.
+    ("c128tc": the same outcomes, amplitudes within a few FP64 roundings, 2.2 times as fast); False
+    keeps them on the FP64 CUDA-core engine.  fp32_on_tensor_cores: complex64 jobs with d >= 5 run as
+    "c64tc", False as "c64"; both are the same factored engine by now (without speculation, "c64tc" has
+    3xTF32 products), so the switch changes a slot's key only.
     policy: the order in which waiting jobs are admitted as slots and memory free up: "sjf" (shortest
     estimated work first, `work`, aged: a job's work counts divided by 1 + its wait / sjf_aging_s, so
     that long jobs are not held back indefinitely by a stream of short ones) or "fifo" (arrival
