@@ -527,9 +527,11 @@ qec_status bfail(qec_status s, const std::string& m) {
 #define QEC_BCUDA(call)                                                                   \
   do {                                                                                    \
     cudaError_t e_ = (call);                                                              \
-    if (e_ != cudaSuccess)                                                                \
+    if (e_ != cudaSuccess) {                                                              \
+      cudaGetLastError(); /* reported here, not by the next launch */                     \
       return bfail(e_ == cudaErrorMemoryAllocation ? QEC_ENOMEM : QEC_ECUDA,              \
                    std::string(#call) + ": " + cudaGetErrorString(e_));                   \
+    }                                                                                     \
   } while (0)
 
 void batch_free(qec_batch* b) {
@@ -692,6 +694,7 @@ qec_status set_fusion(qec_batch* b, int k, int threads) {
 }
 
 qec_status set_shape(qec_batch* b, int warps) {
+  if (warps < 1 || warps > 10) return bfail(QEC_EINVAL, "warps per CTA must be in [1, 10]");
   int occ[2] = {0, 0};
   QEC_BCUDA(set_attributes((const void*)k_batch));
   QEC_BCUDA(set_attributes((const void*)k_batch_cta));

@@ -37,6 +37,7 @@ qec_status fail(qec_status s, const std::string& msg) {
   do {                                                                                   \
     cudaError_t e_ = (call);                                                             \
     if (e_ != cudaSuccess) {                                                             \
+      cudaGetLastError(); /* reported here, not by a later call's check */               \
       return fail(e_ == cudaErrorMemoryAllocation ? QEC_ENOMEM : QEC_ECUDA,              \
                   std::string(#call) + ": " + cudaGetErrorString(e_));                   \
     }                                                                                    \
@@ -598,7 +599,10 @@ qec_status create_impl(const qec_params* params, void* stream, qec_sim** out) {
   const size_t ctl_bytes = sizeof(Ctl) * kCtlRing, out_bytes = (size_t)kBatchCap * (s->syn_cap + s->D + 1);
   const bool chip = onchip_applies(s->D) || s->dense_cap;
   e = cudaMallocHost((void**)&s->h_ctl, ctl_bytes + (chip ? out_bytes : 0));
-  if (e != cudaSuccess) return fail(QEC_ENOMEM, "pinned allocation failed");
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(QEC_ENOMEM, "pinned allocation failed");
+  }
   std::memset(s->h_ctl, 0, ctl_bytes);
   if (chip) s->h_out = reinterpret_cast<uint8_t*>(s->h_ctl) + ctl_bytes;
   QEC_CUDA(cudaMemcpyAsync(s->d_ctl, s->h_ctl, sizeof(Ctl), cudaMemcpyHostToDevice, s->work));

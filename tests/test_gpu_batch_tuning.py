@@ -32,3 +32,19 @@ def test_small_sample_does_not_settle_on_a_shape_that_starves_large_runs():
         for seed in range(4):
             warps, _ = b.autotune(seed, list(range(n)), ["c128"] * n, [dict(W.STRESS)] * n)
             assert warps != 6
+
+
+def test_a_refused_configuration_leaves_no_trace():
+    from paper_2204_11404_gb300 import capi
+
+    n = 8
+    args = (5, list(range(n)), ["c128", "c64", "c128u", "c64u"] * 2, [dict(W.STRESS)] * n)
+    with BatchSimulator(2, "cr", max_traj=16) as b:
+        ref = b.run(*args)
+        for bad in ((0, 4, 256), (-3, 4, 256), (11, 4, 256), (64, 4, 256), (8, 1, 256), (8, 7, 256), (8, 4, 100)):
+            before = b.config()
+            with pytest.raises(capi.QecError):
+                b.set_config(*bad)
+            assert b.config()[1:] == before[1:]
+            for x, y in zip(b.run(*args), ref):      # the refusal is not reported again by the next run
+                assert (x == y).all()
