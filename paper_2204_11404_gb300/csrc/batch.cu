@@ -871,7 +871,7 @@ qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t m
     qec_status st = set_shape(b, 10);
     if (st) return st;
     if ((st = set_fusion(b, 4, 256))) return st;
-    // the noise-free init round, once per precision, in complex64 once per register
+    // the noise-free init round, once per precision, in complex64 once per register, side by side
     BatchArgs a = batch_args(b);
     a.F = batch_program(b, 1);
     a.init_out = b->d_psi0;
@@ -879,11 +879,11 @@ qec_status qec_batch_create(int32_t d, int32_t rounds, int32_t gates, uint32_t m
     e = cudaGetLastError();
     Batch64Args a64 = batch64_args(b, 1);
     a64.out = b->d_psi0_64;
-    if (e == cudaSuccess) e = launch_batch64(a64, 1, 1, b->work);
+    if (e == cudaSuccess) e = launch_batch64(a64, 1, 1, b->side[0]);
     a64.out = b->d_psi0_64 + kNAmp;
-    if (e == cudaSuccess) e = launch_batch64_u(a64, 256, b->u_items, 1, b->work);
-    if (e != cudaSuccess) return bfail(QEC_ECUDA, std::string("init round: ") + cudaGetErrorString(e));
-    e = cudaStreamSynchronize(b->work);
+    if (e == cudaSuccess) e = launch_batch64_u(a64, 256, b->u_items, 1, b->side[1]);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->work);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaStreamSynchronize(b->side[i]);
     if (e != cudaSuccess) return bfail(QEC_ECUDA, std::string("init round: ") + cudaGetErrorString(e));
     *out = owner.release();
     return QEC_OK;
